@@ -134,20 +134,21 @@ attn_umma_kernel(const __grid_constant__ AttnLayers<NL> layers, const sd_batch b
     const int num_blocks = ly.num_blocks;
     const int G = bt.Hq / bt.Hkv;
     const int T = bt.T_max;
+    const int n = min(max(__ldg(bt.n_nodes + b), 0), T);
+    const int len = max(__ldg(bt.len + b), 0);
+    // Rows of this sequence: its own nodes only (rows are node-major, so they are the first n * G).  A tree
+    // smaller than T_max pays for the row tiles it fills: the rows behind them only get their zeros.  (A
+    // batch of 16 trees of 30 to 60 nodes, T_max = 60: 2.9 of 4 row tiles run.)
+    const int rows = n * G;
     // A last row tile of at most 64 rows (420 rows = 3 x 128 + 36) runs its MMAs with M = 64: the
     // accumulator rows then sit in lanes 0..15 of each 32-lane TMEM quadrant (row = 16 * quadrant + lane),
     // the tensor cores work at half width and only 64 rows of Q are staged and re-read per key tile.
-    const bool m64 = (plan.rows - rt * kRowTile) <= 64;
-    // The softmax threads request their row of Q together with the lengths, before anything waits for
-    // either.  A node index below T_max always addresses memory of q; rows of unused nodes are replaced
-    // by zeros when staged.
+    const bool m64 = (rows - rt * kRowTile) <= 64;
     const int q_tid = warp * 32 + lane;
     const int q_row_in_tile = (warp >= 4) ? -1 : (m64 ? (lane < 16 ? warp * 16 + lane : -1) : q_tid);   // -1: no row
-    const int q_row = (q_row_in_tile >= 0) ? rt * kRowTile + q_row_in_tile : plan.rows;
-    const int n = min(max(__ldg(bt.n_nodes + b), 0), T);      // (requested before the row, needed before it)
-    const int len = max(__ldg(bt.len + b), 0);
+    const int q_row = (q_row_in_tile >= 0) ? rt * kRowTile + q_row_in_tile : rows;
     uint4 q_regs[16];
-    if (q_row < plan.rows) {
+    if (q_row < rows) {
         const int node = q_row / G;
         const uint4* src = reinterpret_cast<const uint4*>(
             q + (((size_t)b * T + node) * bt.Hq + kvh * G + (q_row - node * G)) * kD);
@@ -166,9 +167,21 @@ attn_umma_kernel(const __grid_constant__ AttnLayers<NL> layers, const sd_batch b
     const int t1 = min(t0 + tpc, tiles_total);
     const bool has_tree = (chunk == plan.n_chunks - 1);
     const int nt = (t1 - t0) + (has_tree ? 1 : 0);
-    // A CTA without key tiles has nothing to compute, but it still takes part in the cluster barriers.
-    const bool active = (nt > 0) && aligned;
-    const bool clustered = (plan.n_chunks > 1);            // cluster = the chunks of one (b, kvh, row tile)
+    // A CTA without key tiles has nothing to compute, but it still takes part in the cluster barriers; a
+    // row tile without rows is skipped by every CTA of its cluster.
+    const bool has_rows = rt * kRowTile < rows;
+    const bool active = (nt > 0) && aligned && has_rows;
+    const bool clustered = (plan.n_chunks > 1) && has_rows;   // cluster = the chunks of one (b, kvh, row tile)
+    // rows of unused nodes are zeroed by the first chunk's CTA, 16 bytes per lane
+    if (chunk == 0) {
+        const int z0 = max(rows, rt * kRowTile), z1 = min(plan.rows, (rt + 1) * kRowTile);
+        for (int i = z0 * 16 + (int)threadIdx.x; i < z1 * 16; i += kAttThreads) {
+            const int row = i >> 4, node = row / G;
+            const size_t orow = ((size_t)b * T + node) * bt.Hq + kvh * G + (row - node * G);
+            reinterpret_cast<uint4*>(out + orow * kD)[i & 15] = make_uint4(0, 0, 0, 0);
+            if (lse && (i & 15) == 0) lse[orow] = 0.f;
+        }
+    }
     float m_used = -INFINITY, l = 0.f;                     // softmax state of this thread's row (warps 0-3)
     bool rows_ready = false;                               // ... and whether it completed (clustered launches)
 
@@ -299,10 +312,10 @@ attn_umma_kernel(const __grid_constant__ AttnLayers<NL> layers, const sd_batch b
         // ------------------------------------------------------------ softmax: one thread per row
         const int tid = warp * 32 + lane;
         const int row_in_tile = m64 ? (lane < 16 ? warp * 16 + lane : -1) : tid;   // -1: a TMEM lane without a row
-        const int row = (row_in_tile >= 0) ? rt * kRowTile + row_in_tile : plan.rows;
+        const int row = (row_in_tile >= 0) ? rt * kRowTile + row_in_tile : rows;
         const int node = row / G;
         const int g = row - node * G;
-        const bool row_ok = (row < plan.rows) && (node < n);
+        const bool row_ok = row < rows;
         {   // stage this row of Q (zeros for padding rows) in the swizzled K-major layout
 #pragma unroll
             for (int c = 0; c < 16; ++c) {
@@ -456,13 +469,11 @@ attn_umma_kernel(const __grid_constant__ AttnLayers<NL> layers, const sd_batch b
                 uint32_t o[32];
                 tmem_ld32(tmem_o + lane_field + cc * 32, o);
                 tmem_ld_wait();
-                if (row < plan.rows) {
+                if (row_ok) {
                     uint32_t w[16];
 #pragma unroll
                     for (int c = 0; c < 16; ++c) {
-                        const float a = row_ok ? __uint_as_float(o[2 * c]) * inv : 0.f;
-                        const float bb = row_ok ? __uint_as_float(o[2 * c + 1]) * inv : 0.f;
-                        __nv_bfloat162 hh = __floats2bfloat162_rn(a, bb);
+                        __nv_bfloat162 hh = __floats2bfloat162_rn(__uint_as_float(o[2 * c]) * inv, __uint_as_float(o[2 * c + 1]) * inv);
                         w[c] = *reinterpret_cast<uint32_t*>(&hh);
                     }
                     uint4* dst = reinterpret_cast<uint4*>(out + orow * kD + cc * 32);
@@ -470,7 +481,7 @@ attn_umma_kernel(const __grid_constant__ AttnLayers<NL> layers, const sd_batch b
                     for (int c = 0; c < 4; ++c) dst[c] = make_uint4(w[4 * c], w[4 * c + 1], w[4 * c + 2], w[4 * c + 3]);
                 }
             }
-            if (row < plan.rows && lse) lse[orow] = row_ok ? (m_used + log2f(l)) * 0.6931471805599453f : 0.f;
+            if (row_ok && lse) lse[orow] = (m_used + log2f(l)) * 0.6931471805599453f;
         } else if (ok) {
             rows_ready = true;         // several chunks: the rows leave for their finishing CTAs below
         } else if (!ok && lane == 0) {
@@ -496,10 +507,8 @@ attn_umma_kernel(const __grid_constant__ AttnLayers<NL> layers, const sd_batch b
             const int slot = chunk * rows_per + rr % rows_per;
             const uint32_t xo_remote = map_dsmem(smem_u32(k_smem), (uint32_t)(rr / rows_per));
             const uint32_t xs_remote = xo_remote + kRowTile * kD * 4;
-            // rows beyond the tile's last query row and rows of unused nodes are not exchanged: the merge
-            // writes zeros for the latter without reading anything
-            const int push_row = rt * kRowTile + rr;
-            const bool mine = rows_ready && row_in_tile >= 0 && push_row < plan.rows && push_row / G < n;
+            // rows beyond the sequence's last query row are not exchanged
+            const bool mine = rows_ready && row_in_tile >= 0 && rt * kRowTile + rr < rows;
             tc_fence_after_sync();
 #pragma unroll
             for (int cc = 0; cc < 4; ++cc) {
@@ -525,7 +534,7 @@ attn_umma_kernel(const __grid_constant__ AttnLayers<NL> layers, const sd_batch b
         if (warp < 4) {
             const uint32_t xo_addr = smem_u32(k_smem);
             const MergeCtx mc{bt, plan, out, lse, xo_addr, xo_addr + kRowTile * kD * 4,
-                              chunk, rt, b, kvh, n, tpc, tiles_total, warp, lane};
+                              chunk, rt, b, kvh, rows, tpc, tiles_total, warp, lane};
             if (plan.n_chunks == 2) merge_rows<2>(mc);
             else if (plan.n_chunks == 4) merge_rows<4>(mc);
             else merge_rows<8>(mc);

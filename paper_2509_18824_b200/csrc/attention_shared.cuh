@@ -62,7 +62,7 @@ struct AttnLayers { AttnLayer l[NL]; };
 struct MergeCtx {
     const sd_batch& bt; const AttnPlan& plan; __nv_bfloat16* out; float* lse;
     uint32_t xo_addr, xs_addr;          // this CTA's exchange area: rows, then maxima [128] and sums [128]
-    int chunk, rt, b, kvh, n, tpc, tiles_total, warp, lane;
+    int chunk, rt, b, kvh, rows, tpc, tiles_total, warp, lane;
 };
 
 template <int NCH>
@@ -82,7 +82,7 @@ __device__ __forceinline__ void merge_rows(const MergeCtx& x) {
     for (int i = 0; i < kPerWarp; i += 4) {
         const int rl = x.warp * kPerWarp + i + sub;             // row among this CTA's rows
         const int row = first + i;
-        const bool has_data = row < x.plan.rows && node < x.n;  // only such rows were pushed
+        const bool has_data = row < x.rows;                     // only such rows were pushed
         float mc[NCH];
         float M = -INFINITY;
 #pragma unroll
@@ -108,27 +108,21 @@ __device__ __forceinline__ void merge_rows(const MergeCtx& x) {
                 acc[p].z = fmaf(w, v.z, acc[p].z); acc[p].w = fmaf(w, v.w, acc[p].w);
             }
         }
-        if (row < x.plan.rows) {
+        if (has_data) {
             const size_t orow = ((size_t)x.b * x.bt.T_max + node) * x.bt.Hq + x.kvh * G + g;
             uint4* dst = reinterpret_cast<uint4*>(x.out + orow * kD + ql * 16);
-            if (node >= x.n) {                                   // unused node: zero row
-                dst[0] = make_uint4(0, 0, 0, 0);
-                dst[1] = make_uint4(0, 0, 0, 0);
-                if (x.lse && ql == 0) x.lse[orow] = 0.f;
-            } else {
-                const float inv = __frcp_rn(den);
-                uint32_t w[8];
+            const float inv = __frcp_rn(den);
+            uint32_t w[8];
 #pragma unroll
-                for (int p = 0; p < 4; ++p) {
-                    __nv_bfloat162 h0 = __floats2bfloat162_rn(acc[p].x * inv, acc[p].y * inv);
-                    __nv_bfloat162 h1 = __floats2bfloat162_rn(acc[p].z * inv, acc[p].w * inv);
-                    w[2 * p] = *reinterpret_cast<uint32_t*>(&h0);
-                    w[2 * p + 1] = *reinterpret_cast<uint32_t*>(&h1);
-                }
-                dst[0] = make_uint4(w[0], w[1], w[2], w[3]);
-                dst[1] = make_uint4(w[4], w[5], w[6], w[7]);
-                if (x.lse && ql == 0) x.lse[orow] = (M + __log2f(den)) * 0.6931471805599453f;
+            for (int p = 0; p < 4; ++p) {
+                __nv_bfloat162 h0 = __floats2bfloat162_rn(acc[p].x * inv, acc[p].y * inv);
+                __nv_bfloat162 h1 = __floats2bfloat162_rn(acc[p].z * inv, acc[p].w * inv);
+                w[2 * p] = *reinterpret_cast<uint32_t*>(&h0);
+                w[2 * p + 1] = *reinterpret_cast<uint32_t*>(&h1);
             }
+            dst[0] = make_uint4(w[0], w[1], w[2], w[3]);
+            dst[1] = make_uint4(w[4], w[5], w[6], w[7]);
+            if (x.lse && ql == 0) x.lse[orow] = (M + __log2f(den)) * 0.6931471805599453f;
         }
         g += 4;                                                  // the next group's row: four further on
         while (g >= G) { g -= G; ++node; }
