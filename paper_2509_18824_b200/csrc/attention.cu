@@ -11,9 +11,9 @@
 // 64-token cache blocks of the chunk (TMA, 128-byte swizzle, located through the
 // block table) and, for the last chunk, one extra tile holding the tree's own
 // keys, masked per row by the node's ancestor bitmask.  Softmax runs one thread
-// per row straight out of TMEM (no cross-thread reductions); the running maximum
-// is only raised when it grows by more than 2^8, so the accumulator in TMEM is
-// rescaled rarely.  P goes back into TMEM and feeds the second MMA from there.
+// per row straight out of TMEM (no cross-thread reductions); the row's reference is
+// the maximum of its first tile and is raised only when a tile's sum leaves the
+// safe range, so the accumulator in TMEM is practically never rescaled.  P goes back into TMEM and feeds the second MMA from there.
 // With one chunk the CTA writes the output itself; otherwise the chunks of a row
 // tile form a thread-block cluster: every CTA pushes its (max, sum, unnormalised
 // O) rows into the shared memory of the CTA that finishes them (remote stores),
@@ -329,6 +329,8 @@ attn_umma_kernel(const __grid_constant__ AttnLayers<NL> layers, const sd_batch b
         }
         const uint64_t amask = row_ok ? bt.anc_mask[(size_t)b * T + node] : ~0ull;
         const uint32_t lane_field = (uint32_t)(warp * 32) << 16;
+        const uint64_t scale2 = pack_f32x2(scale_log2, scale_log2);
+        uint64_t neg_m2 = 0ull;                                // -(reference of this row), twice
         bool ok = true;
         for (int j = 0; j < nt && ok; ++j) {
             const int s = j & 1;
@@ -369,50 +371,41 @@ attn_umma_kernel(const __grid_constant__ AttnLayers<NL> layers, const sd_batch b
             const uint32_t mask_hi = tree ? (uint32_t)(amask >> 32)
                                           : (valid >= 64 ? ~0u : (valid <= 32 ? 0u : ((1u << (valid - 32)) - 1u)));
             const bool masked = tree || valid < kKeyTile;
-            if (masked) {
-#pragma unroll
-                for (int c = 0; c < 32; ++c)
-                    r0[c] = ((mask_lo >> c) & 1u) ? r0[c] : 0xff800000u;      // -inf
-            }
-            // The exponentials are taken against the current reference maximum right away, while the
-            // tile's own maximum is found alongside (independent instruction streams); only when that
-            // maximum turns out to exceed the reference by more than the threshold (rare after the
-            // first tiles) is the reference raised and the tile's exponentials redone.
+            if (masked) mask_scores(r0, mask_lo);
+            // The exponentials are taken against the row's reference straight away.  The reference is the
+            // maximum of the first tile and need not follow later ones: P (bf16) and the sums (fp32) have
+            // fp32's exponent range, so their relative precision does not depend on how far a score lies
+            // above the reference.  Only when the tile's sum leaves the safe range (> 2^40: some score more
+            // than about 34 powers of two above the reference) is the reference raised and the tile redone.
+            // The sum is needed anyway, so the usual tile tracks no maximum at all, and scaling and sums run
+            // two elements per instruction: 160 instead of 256 arithmetic instructions per thread and tile.
+            // (Two warps share a scheduler partition: 1024 of the 1550 cycles a pair of tiles took were
+            // the exponential unit's, about 1100 were issue slots.)
             uint32_t pk[32];
-            float ps[4] = {0.f, 0.f, 0.f, 0.f};
-            float mx[4] = {-INFINITY, -INFINITY, -INFINITY, -INFINITY};
-            const float neg_m = -m_used;
-#pragma unroll
-            for (int c = 0; c < 16; ++c) {
-                const float a = __uint_as_float(r0[2 * c]), bq = __uint_as_float(r0[2 * c + 1]);
-                mx[c & 3] = max3(mx[c & 3], a, bq);
-                const float p0 = ex2_approx(fmaf(a, scale_log2, neg_m));
-                const float p1 = ex2_approx(fmaf(bq, scale_log2, neg_m));
-                ps[c & 3] += p0 + p1;
-                __nv_bfloat162 h = __floats2bfloat162_rn(p0, p1);
-                pk[c] = *reinterpret_cast<uint32_t*>(&h);
+            float psum = 0.f;
+            bool raise = row_in_tile >= 0;
+            if (j > 0) {
+                uint64_t ps[2] = {0ull, 0ull};
+                exp_pack_half(r0, scale2, neg_m2, pk, ps);
+                tmem_ld_wait();
+                if (masked) mask_scores(r1, mask_hi);
+                exp_pack_half(r1, scale2, neg_m2, pk + 16, ps);
+                psum = sum_f32x2(add_f32x2(ps[0], ps[1]));
+                // (padding rows have zero scores; NaN scores of a real row end up here as well and stay NaN)
+                raise = row_ok && !(psum <= kSumLimit);
+            } else {
+                tmem_ld_wait();
+                if (masked) mask_scores(r1, mask_hi);
             }
-            tmem_ld_wait();
-            if (masked) {
-#pragma unroll
-                for (int c = 0; c < 32; ++c)
-                    r1[c] = ((mask_hi >> c) & 1u) ? r1[c] : 0xff800000u;
-            }
-#pragma unroll
-            for (int c = 0; c < 16; ++c) {
-                const float a = __uint_as_float(r1[2 * c]), bq = __uint_as_float(r1[2 * c + 1]);
-                mx[c & 3] = max3(mx[c & 3], a, bq);
-                const float p0 = ex2_approx(fmaf(a, scale_log2, neg_m));
-                const float p1 = ex2_approx(fmaf(bq, scale_log2, neg_m));
-                ps[c & 3] += p0 + p1;
-                __nv_bfloat162 h = __floats2bfloat162_rn(p0, p1);
-                pk[16 + c] = *reinterpret_cast<uint32_t*>(&h);
-            }
-            const float mt = fmaxf(fmaxf(mx[0], mx[1]), fmaxf(mx[2], mx[3])) * scale_log2;   // scale > 0
-            // raise the reference maximum only when it would grow by more than the threshold
-            // true on the first tile (m_used = -inf); lanes without a row hold stale scores and never ask
-            const bool raise = (row_in_tile >= 0) && (mt > m_used + kRescaleThreshold);
             if (__any_sync(0xffffffffu, raise)) {
+                float mx[4] = {-INFINITY, -INFINITY, -INFINITY, -INFINITY};
+#pragma unroll
+                for (int c = 0; c < 16; ++c) {
+                    mx[c & 3] = max3(mx[c & 3], __uint_as_float(r0[2 * c]), __uint_as_float(r0[2 * c + 1]));
+                    mx[(c + 2) & 3] = max3(mx[(c + 2) & 3], __uint_as_float(r1[2 * c]), __uint_as_float(r1[2 * c + 1]));
+                }
+                const float mt = fmaxf(fmaxf(mx[0], mx[1]), fmaxf(mx[2], mx[3])) * scale_log2;   // scale > 0
+                raise = raise && mt > m_used;
                 if (j > 0) {
                     if (!mbar_wait(pv_done, (uint32_t)(j - 1) & 1u, abort_flag, plan.wait_cycles)) { ok = false; break; }
                     tc_fence_after_sync();
@@ -430,23 +423,13 @@ attn_umma_kernel(const __grid_constant__ AttnLayers<NL> layers, const sd_batch b
                     l *= alpha;
                 }
                 if (raise) m_used = mt;
-                // redo the tile against the new reference (same values for rows that did not raise)
-                const float neg_m2 = -m_used;
-                ps[0] = ps[1] = ps[2] = ps[3] = 0.f;
-#pragma unroll
-                for (int c = 0; c < 16; ++c) {
-                    const float p0 = ex2_approx(fmaf(__uint_as_float(r0[2 * c]), scale_log2, neg_m2));
-                    const float p1 = ex2_approx(fmaf(__uint_as_float(r0[2 * c + 1]), scale_log2, neg_m2));
-                    const float p2 = ex2_approx(fmaf(__uint_as_float(r1[2 * c]), scale_log2, neg_m2));
-                    const float p3 = ex2_approx(fmaf(__uint_as_float(r1[2 * c + 1]), scale_log2, neg_m2));
-                    ps[c & 3] += (p0 + p1) + (p2 + p3);
-                    __nv_bfloat162 h0 = __floats2bfloat162_rn(p0, p1);
-                    __nv_bfloat162 h1 = __floats2bfloat162_rn(p2, p3);
-                    pk[c] = *reinterpret_cast<uint32_t*>(&h0);
-                    pk[16 + c] = *reinterpret_cast<uint32_t*>(&h1);
-                }
+                neg_m2 = pack_f32x2(-m_used, -m_used);
+                // (again) against the new reference: the same values for rows that did not raise
+                uint64_t ps[2] = {0ull, 0ull};
+                exp_pack_half(r0, scale2, neg_m2, pk, ps);
+                exp_pack_half(r1, scale2, neg_m2, pk + 16, ps);
+                psum = sum_f32x2(add_f32x2(ps[0], ps[1]));
             }
-            const float psum = (ps[0] + ps[1]) + (ps[2] + ps[3]);
             l += psum;
             // P replaces the S columns this thread has just consumed (its own TMEM lane)
             tmem_st32(tmem_s + lane_field + s * kKeyTile, pk);

@@ -10,7 +10,7 @@ using namespace sm100;
 
 constexpr int kRowTile = 128;                  // query rows per row tile (MMA M)
 constexpr float kLog2e = 1.4426950408889634f;
-constexpr float kRescaleThreshold = 8.0f;      // log2 units
+constexpr float kSumLimit = 1.0995e12f;        // 2^40: a tile's sum above this raises the row's reference
 constexpr int kMaxChunks = 8;                  // = portable cluster size
 constexpr int kSplitRounds = 8;                // launches of fewer whole rounds get their remainder as a chunked launch
 
@@ -23,6 +23,49 @@ __device__ __forceinline__ float ex2_approx(float x) {
     float y;
     asm("ex2.approx.ftz.f32 %0, %1;" : "=f"(y) : "f"(x));
     return y;
+}
+
+// two fp32 values per 64-bit register: one instruction scales, or adds, both (round to nearest even, each)
+__device__ __forceinline__ uint64_t pack_f32x2(float lo, float hi) {
+    uint64_t d;
+    asm("mov.b64 %0, {%1, %2};" : "=l"(d) : "f"(lo), "f"(hi));
+    return d;
+}
+__device__ __forceinline__ uint64_t fma_f32x2(uint64_t a, uint64_t b, uint64_t c) {
+    uint64_t d;
+    asm("fma.rn.f32x2 %0, %1, %2, %3;" : "=l"(d) : "l"(a), "l"(b), "l"(c));
+    return d;
+}
+__device__ __forceinline__ uint64_t add_f32x2(uint64_t a, uint64_t b) {
+    uint64_t d;
+    asm("add.rn.f32x2 %0, %1, %2;" : "=l"(d) : "l"(a), "l"(b));
+    return d;
+}
+__device__ __forceinline__ float sum_f32x2(uint64_t a) {
+    float lo, hi;
+    asm("mov.b64 {%0, %1}, %2;" : "=f"(lo), "=f"(hi) : "l"(a));
+    return lo + hi;
+}
+
+// keys outside the mask get the score -inf
+__device__ __forceinline__ void mask_scores(uint32_t (&r)[32], uint32_t mask) {
+#pragma unroll
+    for (int c = 0; c < 32; ++c) r[c] = ((mask >> c) & 1u) ? r[c] : 0xff800000u;
+}
+
+// 32 raw scores of a row -> 2^(score * scale - reference), packed to bf16 in pairs, and added to the sums
+__device__ __forceinline__ void exp_pack_half(const uint32_t (&r)[32], uint64_t scale2, uint64_t neg_m2, uint32_t* pk,
+                                              uint64_t (&ps)[2]) {
+#pragma unroll
+    for (int c = 0; c < 16; ++c) {
+        const uint64_t x = fma_f32x2(pack_f32x2(__uint_as_float(r[2 * c]), __uint_as_float(r[2 * c + 1])), scale2, neg_m2);
+        float x0, x1;
+        asm("mov.b64 {%0, %1}, %2;" : "=f"(x0), "=f"(x1) : "l"(x));
+        const float p0 = ex2_approx(x0), p1 = ex2_approx(x1);
+        ps[c & 1] = add_f32x2(ps[c & 1], pack_f32x2(p0, p1));
+        const __nv_bfloat162 h = __floats2bfloat162_rn(p0, p1);
+        pk[c] = *reinterpret_cast<const uint32_t*>(&h);
+    }
 }
 
 struct AttnPlan {
