@@ -56,7 +56,8 @@ attn_umma_kernel(const __grid_constant__ AttnLayers<NL> layers, const sd_batch b
                                          //     cannot complete the previous tile's phase
     uint64_t* pv_done = bars + 14;       // MMA -> softmax   (O updated by tile j; phase j)
     uint64_t* o_full = bars + 15;        // MMA -> softmax   (single use: every MMA of the CTA has completed)
-    uint64_t* q_full = bars + 16;        // softmax -> MMA   (Q staged)
+    uint64_t* q_full = bars + 16;        // TMA -> MMA       (Q tile)
+    uint64_t* x_full = bars + 20;        // clustered launches: the other chunks' rows have arrived (single use)
     uint32_t* tmem_slot = reinterpret_cast<uint32_t*>(bars + 17);
     int* abort_flag = reinterpret_cast<int*>(bars + 18);
 
@@ -76,6 +77,7 @@ attn_umma_kernel(const __grid_constant__ AttnLayers<NL> layers, const sd_batch b
     const int lb = zz / bt.Hkv;
     const int rank_b = lb / plan.n_layers;
     const AttnLayer& ly = layers.l[lb % plan.n_layers];
+    const CUtensorMap* const map_q = &ly.q;
     const CUtensorMap* const map_kc = &ly.k_cache;
     const CUtensorMap* const map_vc = &ly.v_cache;
     const CUtensorMap* const map_kt = &ly.k_tree;
@@ -94,7 +96,7 @@ attn_umma_kernel(const __grid_constant__ AttnLayers<NL> layers, const sd_batch b
             for (int i = 0; i < kKStages; ++i) { mbar_init(&k_full[i], 1); mbar_init(&k_empty[i], 1); }
             for (int i = 0; i < kVStages; ++i) { mbar_init(&v_full[i], 1); mbar_init(&v_empty[i], 1); }
             for (int i = 0; i < 2; ++i) { mbar_init(&s_full[i], 1); mbar_init(&p_full[i], 4); }
-            mbar_init(pv_done, 1); mbar_init(q_full, 4); mbar_init(o_full, 1);
+            mbar_init(pv_done, 1); mbar_init(q_full, 1); mbar_init(o_full, 1); mbar_init(x_full, 1);
             fence_barrier_init();
         }
         if (warp == kTmaWarp) {                            // a full warp (the MMA warp is a single thread)
@@ -102,7 +104,7 @@ attn_umma_kernel(const __grid_constant__ AttnLayers<NL> layers, const sd_batch b
             tmem_relinquish();
         }
         if (warp == kTmaWarp && lane == 0) {
-            prefetch_tensormap(map_kc); prefetch_tensormap(map_vc);
+            prefetch_tensormap(map_q); prefetch_tensormap(map_kc); prefetch_tensormap(map_vc);
             prefetch_tensormap(map_kt); prefetch_tensormap(map_vt);
         }
     } else if (threadIdx.x == 0) {
@@ -128,12 +130,22 @@ attn_umma_kernel(const __grid_constant__ AttnLayers<NL> layers, const sd_batch b
         __syncthreads();
         b = s_seq;
     }
-    const uint16_t* __restrict__ q = ly.q;
     __nv_bfloat16* __restrict__ out = ly.out;
     float* __restrict__ lse = ly.lse;
     const int num_blocks = ly.num_blocks;
     const int G = bt.Hq / bt.Hkv;
     const int T = bt.T_max;
+    // The Q tile depends on nothing but b, so it is requested before the lengths are known: one copy of
+    // whole nodes (tile_rows = the largest multiple of G up to 128; rows of unused nodes are loaded too and
+    // reach no output, the smem rows behind tile_rows hold whatever they held).  (Staged through registers
+    // by the softmax threads it took two more dependent memory latencies before the first scores.)
+    const int tile_rows = plan.tile_rows;
+    if (aligned && warp == kTmaWarp && lane == 0) {
+        const uint64_t pol = policy_evict_first();
+        mbar_arrive_expect_tx(q_full, (uint32_t)tile_rows * kD * 2);
+        tma_load_3d(q_smem, map_q, 0, kvh * G, b * T + rt * plan.tile_nodes, q_full, pol);
+        tma_load_3d(q_smem + kRowTile * 128, map_q, 64, kvh * G, b * T + rt * plan.tile_nodes, q_full, pol);
+    }
     const int n = min(max(__ldg(bt.n_nodes + b), 0), T);
     const int len = max(__ldg(bt.len + b), 0);
     // Rows of this sequence: its own nodes only (rows are node-major, so they are the first n * G).  A tree
@@ -143,18 +155,7 @@ attn_umma_kernel(const __grid_constant__ AttnLayers<NL> layers, const sd_batch b
     // A last row tile of at most 64 rows (420 rows = 3 x 128 + 36) runs its MMAs with M = 64: the
     // accumulator rows then sit in lanes 0..15 of each 32-lane TMEM quadrant (row = 16 * quadrant + lane),
     // the tensor cores work at half width and only 64 rows of Q are staged and re-read per key tile.
-    const bool m64 = (rows - rt * kRowTile) <= 64;
-    const int q_tid = warp * 32 + lane;
-    const int q_row_in_tile = (warp >= 4) ? -1 : (m64 ? (lane < 16 ? warp * 16 + lane : -1) : q_tid);   // -1: no row
-    const int q_row = (q_row_in_tile >= 0) ? rt * kRowTile + q_row_in_tile : rows;
-    uint4 q_regs[16];
-    if (q_row < rows) {
-        const int node = q_row / G;
-        const uint4* src = reinterpret_cast<const uint4*>(
-            q + (((size_t)b * T + node) * bt.Hq + kvh * G + (q_row - node * G)) * kD);
-#pragma unroll
-        for (int c = 0; c < 16; ++c) q_regs[c] = __ldg(src + c);
-    }
+    const bool m64 = (rows - rt * tile_rows) <= 64;
 
     // key tiles of this CTA: cache blocks [t0, t1) and, for the last chunk, the tree tile
     int tiles_total = (len + kKeyTile - 1) / kKeyTile;
@@ -169,12 +170,12 @@ attn_umma_kernel(const __grid_constant__ AttnLayers<NL> layers, const sd_batch b
     const int nt = (t1 - t0) + (has_tree ? 1 : 0);
     // A CTA without key tiles has nothing to compute, but it still takes part in the cluster barriers; a
     // row tile without rows is skipped by every CTA of its cluster.
-    const bool has_rows = rt * kRowTile < rows;
+    const bool has_rows = rt * tile_rows < rows;
     const bool active = (nt > 0) && aligned && has_rows;
     const bool clustered = (plan.n_chunks > 1) && has_rows;   // cluster = the chunks of one (b, kvh, row tile)
     // rows of unused nodes are zeroed by the first chunk's CTA, 16 bytes per lane
     if (chunk == 0) {
-        const int z0 = max(rows, rt * kRowTile), z1 = min(plan.rows, (rt + 1) * kRowTile);
+        const int z0 = max(rows, rt * tile_rows), z1 = min(plan.rows, (rt + 1) * tile_rows);
         for (int i = z0 * 16 + (int)threadIdx.x; i < z1 * 16; i += kAttThreads) {
             const int row = i >> 4, node = row / G;
             const size_t orow = ((size_t)b * T + node) * bt.Hq + kvh * G + (row - node * G);
@@ -312,21 +313,11 @@ attn_umma_kernel(const __grid_constant__ AttnLayers<NL> layers, const sd_batch b
         // ------------------------------------------------------------ softmax: one thread per row
         const int tid = warp * 32 + lane;
         const int row_in_tile = m64 ? (lane < 16 ? warp * 16 + lane : -1) : tid;   // -1: a TMEM lane without a row
-        const int row = (row_in_tile >= 0) ? rt * kRowTile + row_in_tile : rows;
+        const int row = (row_in_tile >= 0 && row_in_tile < tile_rows) ? rt * tile_rows + row_in_tile : rows;
         const int node = row / G;
         const int g = row - node * G;
         const bool row_ok = row < rows;
-        {   // stage this row of Q (zeros for padding rows) in the swizzled K-major layout
-#pragma unroll
-            for (int c = 0; c < 16; ++c) {
-                uint4 u = row_ok ? q_regs[c] : make_uint4(0, 0, 0, 0);
-                uint8_t* dst = q_smem + (c >> 3) * (kRowTile * 128) + row_in_tile * 128 + (((c & 7) ^ (row_in_tile & 7)) << 4);
-                if (row_in_tile >= 0) *reinterpret_cast<uint4*>(dst) = u;
-            }
-            fence_proxy_async_smem();
-            __syncwarp();
-            if (lane == 0) mbar_arrive(q_full);
-        }
+        if (!row_ok) m_used = 0.f;                             // (finite exponentials for rows that nobody reads)
         const uint64_t amask = row_ok ? bt.anc_mask[(size_t)b * T + node] : ~0ull;
         const uint32_t lane_field = (uint32_t)(warp * 32) << 16;
         const uint64_t scale2 = pack_f32x2(scale_log2, scale_log2);
@@ -383,7 +374,7 @@ attn_umma_kernel(const __grid_constant__ AttnLayers<NL> layers, const sd_batch b
             // the exponential unit's, about 1100 were issue slots.)
             uint32_t pk[32];
             float psum = 0.f;
-            bool raise = row_in_tile >= 0;
+            bool raise = row_ok;
             if (j > 0) {
                 uint64_t ps[2] = {0ull, 0ull};
                 exp_pack_half(r0, scale2, neg_m2, pk, ps);
@@ -473,55 +464,84 @@ attn_umma_kernel(const __grid_constant__ AttnLayers<NL> layers, const sd_batch b
     }
     }   // active
 
+    if (!active && aligned && warp == kTmaWarp && lane == 0)       // nobody else waits for the Q copy
+        mbar_wait(q_full, 0, abort_flag, plan.wait_cycles);
+
     if (clustered) {
+        // Row r of the tile is finished by the CTA of chunk r / (128 / n_chunks): every other chunk's CTA
+        // sends it that row's maximum, sum and unnormalised O straight from tensor memory, with stores that
+        // report their bytes to the receiver's barrier (so the receiver waits for exactly what it gets, and
+        // no second cluster-wide barrier and release stand between the last row and the merge).
+        const int rows_per = kRowTile / plan.n_chunks;
+        const uint32_t xo_addr = smem_u32(k_smem), xs_addr = xo_addr + kRowTile * kD * 4;
+        if (threadIdx.x == 0) {
+            const int mine = min(max(min(rows - rt * tile_rows, tile_rows) - chunk * rows_per, 0), rows_per);
+            int others = 0;                                // chunks with key tiles, this one aside
+            for (int c = 0; c < plan.n_chunks; ++c)
+                others += (c != chunk && (c == plan.n_chunks - 1 || c * tpc < tiles_total)) ? 1 : 0;
+            mbar_arrive_expect_tx(x_full, (uint32_t)(others * mine * (kD * 4 + 8)));
+        }
         // every thread of every CTA of the cluster: all MMAs and copies of the cluster have completed, so
         // every CTA's K/V rings are free to receive rows
         __syncwarp();
         cluster_arrive_release();
         cluster_wait_acquire();
         if (active && warp < 4) {
-            // Each row (maximum, sum, unnormalised O) goes straight from tensor memory into the shared
-            // memory of the CTA that finishes it: remote stores stream, remote loads would each cost a
-            // round trip.  Row r of the tile is finished by the CTA of chunk r / (128 / n_chunks).
-            const int rows_per = kRowTile / plan.n_chunks;
-            const int tid = warp * 32 + lane;
-            const int row_in_tile = m64 ? (lane < 16 ? warp * 16 + lane : -1) : tid;
+            const int row_in_tile = m64 ? (lane < 16 ? warp * 16 + lane : -1) : warp * 32 + lane;
             const int rr = max(row_in_tile, 0);
-            const int slot = chunk * rows_per + rr % rows_per;
-            const uint32_t xo_remote = map_dsmem(smem_u32(k_smem), (uint32_t)(rr / rows_per));
-            const uint32_t xs_remote = xo_remote + kRowTile * kD * 4;
+            const int dest = rr / rows_per, rl = rr % rows_per;
             // rows beyond the sequence's last query row are not exchanged
-            const bool mine = rows_ready && row_in_tile >= 0 && rt * kRowTile + rr < rows;
+            const bool mine = rows_ready && row_in_tile >= 0 && rr < tile_rows && rt * tile_rows + rr < rows;
+            // Exchange area: [chunk][16-byte piece of the row][row of the finisher], so that a warp's store
+            // (32 rows, one piece each) fills 512 consecutive bytes: remote stores travel in packets of
+            // consecutive bytes (measured with 256 CTAs in pairs: 24.5 B/clk per CTA against 12.5 for one
+            // 512-byte line per row).
+            const uint32_t off = (uint32_t)(((chunk * 32) * rows_per + rl) * 16);
+            const uint32_t xo_remote = map_dsmem(xo_addr, (uint32_t)dest) + off;
+            const uint32_t xs_remote = map_dsmem(xs_addr, (uint32_t)dest) + (uint32_t)(chunk * rows_per + rl) * 4;
+            const uint32_t bar_remote = map_dsmem(smem_u32(x_full), (uint32_t)dest);
             tc_fence_after_sync();
 #pragma unroll
             for (int cc = 0; cc < 4; ++cc) {
                 uint32_t o[32];
                 tmem_ld32(tmem_base + ((uint32_t)(warp * 32) << 16) + cc * 32, o);
                 tmem_ld_wait();
-                if (mine) {
+                if (mine && dest != chunk) {
 #pragma unroll
                     for (int k = 0; k < 8; ++k)
-                        st_dsmem_v4(xo_remote + (uint32_t)(slot * kD + (((cc * 8 + k) ^ (slot & 31)) << 2)) * 4,
-                                    o[4 * k], o[4 * k + 1], o[4 * k + 2], o[4 * k + 3]);
+                        st_async_v4(xo_remote + (uint32_t)((cc * 8 + k) * rows_per * 16), o[4 * k], o[4 * k + 1], o[4 * k + 2],
+                                    o[4 * k + 3], bar_remote);
+                } else if (mine) {
+#pragma unroll
+                    for (int k = 0; k < 8; ++k)
+                        st_smem_v4(xo_addr + off + (uint32_t)((cc * 8 + k) * rows_per * 16), o[4 * k], o[4 * k + 1], o[4 * k + 2],
+                                   o[4 * k + 3]);
                 }
             }
-            if (mine) {
-                st_dsmem_f32(xs_remote + slot * 4, m_used);
-                st_dsmem_f32(xs_remote + (kRowTile + slot) * 4, l);
+            if (mine && dest != chunk) {
+                st_async_b32(xs_remote, __float_as_uint(m_used), bar_remote);
+                st_async_b32(xs_remote + kRowTile * 4, __float_as_uint(l), bar_remote);
+            } else if (mine) {
+                st_smem_f32(xs_addr + (uint32_t)(chunk * rows_per + rl) * 4, m_used);
+                st_smem_f32(xs_addr + (uint32_t)(kRowTile + chunk * rows_per + rl) * 4, l);
             }
         }
-        // all rows have landed where they are finished
         __syncwarp();
-        cluster_arrive_release();
-        cluster_wait_acquire();
+        cluster_arrive_relaxed();                          // (waited for at the end: nobody leaves before its peers have sent)
         if (warp < 4) {
-            const uint32_t xo_addr = smem_u32(k_smem);
-            const MergeCtx mc{bt, plan, out, lse, xo_addr, xo_addr + kRowTile * kD * 4,
-                              chunk, rt, b, kvh, rows, tpc, tiles_total, warp, lane};
-            if (plan.n_chunks == 2) merge_rows<2>(mc);
-            else if (plan.n_chunks == 4) merge_rows<4>(mc);
-            else merge_rows<8>(mc);
+            asm volatile("bar.sync 1, 128;" ::: "memory"); // this CTA's own rows
+            if (mbar_wait_cluster(x_full, 0, abort_flag, plan.wait_cycles)) {
+                const MergeCtx mc{bt, plan, out, lse, xo_addr, xs_addr, chunk, rt, b, kvh, rows, tpc, tiles_total, (int)threadIdx.x};
+                if (plan.n_chunks == 2) merge_rows<2>(mc);
+                else if (plan.n_chunks == 4) merge_rows<4>(mc);
+                else merge_rows<8>(mc);
+            } else if (lane == 0) {
+                set_status(status, SD_ERR_TIMEOUT);
+                for (int i = 0; i < 1000; ++i) __nanosleep(1000);      // let rows in flight land
+            }
         }
+        __syncwarp();
+        cluster_wait_acquire();
     }
     if (!aligned) return;
     tc_fence_before_sync();
@@ -534,6 +554,11 @@ attn_umma_kernel(const __grid_constant__ AttnLayers<NL> layers, const sd_batch b
 
 static bool fill_layer(AttnLayer* ly, const sd_batch& bt, const sd_kv_layer& cache, const void* q,
                        const void* kt, const void* vt, void* out, float* lse) {
+    const int G = bt.Hq / bt.Hkv;
+    const uint64_t q_dims[3] = {(uint64_t)kD, (uint64_t)bt.Hq, (uint64_t)bt.B * bt.T_max};
+    const uint64_t q_strides[2] = {(uint64_t)kD * 2, (uint64_t)bt.Hq * kD * 2};
+    const uint32_t q_box[3] = {64, (uint32_t)G, (uint32_t)(kRowTile / G)};
+    if (!encode_tmap_bf16_3d(&ly->q, q, q_dims, q_strides, q_box, 128)) return false;
     const uint64_t cache_rows = (uint64_t)cache.num_blocks * bt.Hkv * kKeyTile;
     if (!encode_tmap_bf16_2d(&ly->k_cache, cache.k, cache_rows, kD, kD * 2, 64, kKeyTile, 128) ||
         !encode_tmap_bf16_2d(&ly->v_cache, cache.v, cache_rows, kD, kD * 2, 64, kKeyTile, 128))
@@ -544,7 +569,6 @@ static bool fill_layer(AttnLayer* ly, const sd_batch& bt, const sd_kv_layer& cac
     if (!encode_tmap_bf16_3d(&ly->k_tree, kt, dims, strides, box, 128) ||
         !encode_tmap_bf16_3d(&ly->v_tree, vt, dims, strides, box, 128))
         return false;
-    ly->q = static_cast<const uint16_t*>(q);
     ly->out = static_cast<__nv_bfloat16*>(out);
     ly->lse = lse;
     ly->num_blocks = cache.num_blocks;
@@ -558,7 +582,7 @@ sd_status launch_rows1(const AttnLayers<NL>& layers, const sd_batch& bt, float s
     if (cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, kAttSmem) != cudaSuccess)
         return SD_ERR_CUDA;
     cudaLaunchConfig_t cfg = {};
-    cfg.gridDim = dim3(plan.n_chunks, plan.ctas_per_group, z_count);
+    cfg.gridDim = dim3(plan.n_chunks, plan.row_tiles, z_count);
     cfg.blockDim = dim3(kAttThreads);
     cfg.dynamicSmemBytes = kAttSmem;
     cfg.stream = st;
@@ -604,8 +628,9 @@ static AttnPlan make_plan(const sd_batch& bt, int n_layers, int sms) {
     AttnPlan p;
     const int G = bt.Hq / bt.Hkv;
     p.rows = bt.T_max * G;
-    p.row_tiles = (p.rows + kRowTile - 1) / kRowTile;
-    p.ctas_per_group = p.row_tiles;
+    p.tile_nodes = kRowTile / G;
+    p.tile_rows = p.tile_nodes * G;
+    p.row_tiles = (p.rows + p.tile_rows - 1) / p.tile_rows;
     // Pick the chunk count that minimises (waves of CTAs) x (key tiles per CTA + fixed cost),
     // two CTAs being resident per SM.  Few waves are counted whole; many waves balance out.
     const int max_tiles = bt.max_blocks_per_seq;

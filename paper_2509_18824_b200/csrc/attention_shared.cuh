@@ -71,8 +71,9 @@ __device__ __forceinline__ void exp_pack_half(const uint32_t (&r)[32], uint64_t 
 struct AttnPlan {
     int n_chunks;      // key chunks per sequence (the last one also takes the tree tile)
     int rows;          // T_max * G
+    int tile_nodes;    // tree nodes of a row tile: its rows are whole nodes, the query heads of one KV head each
+    int tile_rows;     // tile_nodes * G <= 128
     int row_tiles;
-    int ctas_per_group;// CTAs along blockIdx.y per (layer, sequence, KV head): row tiles, or pairs of row tiles
     int n_layers;      // layers of this launch
     int ranked;        // dispatch the sequences longest first (only matters when the grid runs in several waves)
     int z0;            // first (sequence rank, layer, KV head) index of this launch: blockIdx.z counts from here
@@ -83,9 +84,9 @@ struct AttnPlan {
 // Everything the CTAs of one layer need.  A launch covers up to kMaxLayersPerLaunch layers (the
 // descriptors travel as kernel parameters); blockIdx.z enumerates (sequence, layer, KV head).
 struct AttnLayer {
+    CUtensorMap q;                  // 3-D (128, Hq, B*T_max), box 64 x G x tile_nodes
     CUtensorMap k_cache, v_cache;   // 2-D [num_blocks*Hkv*64][128], box 64 x 64
     CUtensorMap k_tree, v_tree;     // 3-D (128, Hkv, B*T_max), box 64 x 1 x 64
-    const uint16_t* q;              // bf16 [B][T_max][Hq][D]
     __nv_bfloat16* out;             // bf16 [B][T_max][Hq][D]
     float* lse;                     // f32  [B][T_max][Hq] or null
     int32_t num_blocks;
@@ -94,81 +95,70 @@ constexpr int kMaxLayersPerLaunch = 32;
 template <int NL>
 struct AttnLayers { AttnLayer l[NL]; };
 
-// Final step of a clustered launch.  Chunk c's CTA has PUSHED its unnormalised rows (and their
-// maximum and sum) into the shared memory of the CTA that finishes them: the CTA of chunk o owns rows
-// o * 128 / NCH .. of the tile and holds, for each of its rows, one slot per chunk (slot = c * rows
-// per CTA + local row).  Every read here is local.  A warp takes a few rows at a time, every lane
-// four output columns, and adds up the chunks in chunk order (so the result does not depend on
-// timing).  A slot is one contiguous 512-byte line whose 16-byte pieces are XOR-swizzled by the slot
-// index (the pushing threads write one row each: without the swizzle a warp's stores would meet in
-// one bank group).
+// Final step of a clustered launch.  The CTA of chunk o finishes rows o * 128 / NCH .. of the tile and
+// holds, in its exchange area, those rows' unnormalised O of every chunk ([chunk][16-byte piece][row], its
+// own rows stored locally, the others' by the CTAs that computed them) and their references and sums
+// ([chunk][row] each).  One thread takes one row and 16 output columns at a time: consecutive lanes read
+// consecutive rows of a piece (no bank conflicts) and each writes a whole 32-byte sector; chunks are
+// added in chunk order, so the result does not depend on timing.
 struct MergeCtx {
     const sd_batch& bt; const AttnPlan& plan; __nv_bfloat16* out; float* lse;
-    uint32_t xo_addr, xs_addr;          // this CTA's exchange area: rows, then maxima [128] and sums [128]
-    int chunk, rt, b, kvh, rows, tpc, tiles_total, warp, lane;
+    uint32_t xo_addr, xs_addr;          // this CTA's exchange area: rows, then references [128] and sums [128]
+    int chunk, rt, b, kvh, rows, tpc, tiles_total, tid;
 };
 
 template <int NCH>
 __device__ __forceinline__ void merge_rows(const MergeCtx& x) {
-    // Eight lanes per row (16 output columns each), four rows per warp at a time; the warp's rows are
-    // consecutive, so node and head within the group are counted up instead of divided out.
     constexpr int kRowsPer = kRowTile / NCH;        // rows this CTA finishes
-    constexpr int kPerWarp = kRowsPer / 4;          // ... and each of its four warps (a multiple of 4)
     const int G = x.bt.Hq / x.bt.Hkv;
-    const int sub = x.lane >> 3, ql = x.lane & 7;
-    const int first = x.rt * kRowTile + x.chunk * kRowsPer + x.warp * kPerWarp + sub;   // this lane's first row
-    int node = first / G;
-    int g = first - node * G;
-    // (unrolled: the groups are independent, and one warp per scheduler partition has nothing else to
-    //  hide the latency of a group's dependent loads, exponentials and stores behind)
+    const int rl = x.tid % kRowsPer;
+    const int in_tile = x.chunk * kRowsPer + rl, row = x.rt * x.plan.tile_rows + in_tile;
+    if (in_tile >= x.plan.tile_rows || row >= x.rows) return;      // only rows of the sequence were sent
+    float w[NCH];
+    float M = -INFINITY;
 #pragma unroll
-    for (int i = 0; i < kPerWarp; i += 4) {
-        const int rl = x.warp * kPerWarp + i + sub;             // row among this CTA's rows
-        const int row = first + i;
-        const bool has_data = row < x.rows;                     // only such rows were pushed
-        float mc[NCH];
-        float M = -INFINITY;
+    for (int c = 0; c < NCH; ++c) {
+        const bool live = (c == NCH - 1) || (c * x.tpc < x.tiles_total);       // that chunk had key tiles
+        w[c] = live ? ld_smem_f32(x.xs_addr + (c * kRowsPer + rl) * 4) : -INFINITY;
+        M = fmaxf(M, w[c]);
+    }
+    float den = 0.f;
 #pragma unroll
-        for (int c = 0; c < NCH; ++c) {
-            const bool live = has_data && ((c == NCH - 1) || (c * x.tpc < x.tiles_total));   // that chunk had key tiles
-            mc[c] = live ? ld_smem_f32(x.xs_addr + (c * kRowsPer + rl) * 4) : -INFINITY;
-            M = fmaxf(M, mc[c]);
-        }
-        float den = 0.f;
+    for (int c = 0; c < NCH; ++c) {
+        if (w[c] == -INFINITY) { w[c] = 0.f; continue; }
+        w[c] = ex2_approx(w[c] - M);
+        den = fmaf(w[c], ld_smem_f32(x.xs_addr + (kRowTile + c * kRowsPer + rl) * 4), den);
+    }
+    const float inv = __frcp_rn(den);
+    const int node = row / G, g = row - node * G;
+    const size_t orow = ((size_t)x.b * x.bt.T_max + node) * x.bt.Hq + x.kvh * G + g;
+    if (x.lse && x.tid < kRowsPer) x.lse[orow] = (M + __log2f(den)) * 0.6931471805599453f;
+#pragma unroll
+    for (int cg = x.tid / kRowsPer; cg < 8; cg += kRowTile / kRowsPer) {       // 16 columns: pieces 4 cg .. + 3
         float4 acc[4];
 #pragma unroll
         for (int p = 0; p < 4; ++p) acc[p] = make_float4(0.f, 0.f, 0.f, 0.f);
 #pragma unroll
         for (int c = 0; c < NCH; ++c) {
-            if (mc[c] == -INFINITY) continue;                    // a chunk without tiles
-            const int slot = c * kRowsPer + rl;
-            const float w = ex2_approx(mc[c] - M);
-            den = fmaf(w, ld_smem_f32(x.xs_addr + (kRowTile + slot) * 4), den);
+            if (!((c == NCH - 1) || (c * x.tpc < x.tiles_total))) continue;    // (nothing was written there)
 #pragma unroll
             for (int p = 0; p < 4; ++p) {
-                const float4 v = ld_smem_v4(x.xo_addr + (uint32_t)(slot * kD + (((ql * 4 + p) ^ (slot & 31)) << 2)) * 4);
-                acc[p].x = fmaf(w, v.x, acc[p].x); acc[p].y = fmaf(w, v.y, acc[p].y);
-                acc[p].z = fmaf(w, v.z, acc[p].z); acc[p].w = fmaf(w, v.w, acc[p].w);
+                const float4 v = ld_smem_v4(x.xo_addr + (uint32_t)(((c * 32 + cg * 4 + p) * kRowsPer + rl) * 16));
+                acc[p].x = fmaf(w[c], v.x, acc[p].x); acc[p].y = fmaf(w[c], v.y, acc[p].y);
+                acc[p].z = fmaf(w[c], v.z, acc[p].z); acc[p].w = fmaf(w[c], v.w, acc[p].w);
             }
         }
-        if (has_data) {
-            const size_t orow = ((size_t)x.b * x.bt.T_max + node) * x.bt.Hq + x.kvh * G + g;
-            uint4* dst = reinterpret_cast<uint4*>(x.out + orow * kD + ql * 16);
-            const float inv = __frcp_rn(den);
-            uint32_t w[8];
+        uint32_t o[8];
 #pragma unroll
-            for (int p = 0; p < 4; ++p) {
-                __nv_bfloat162 h0 = __floats2bfloat162_rn(acc[p].x * inv, acc[p].y * inv);
-                __nv_bfloat162 h1 = __floats2bfloat162_rn(acc[p].z * inv, acc[p].w * inv);
-                w[2 * p] = *reinterpret_cast<uint32_t*>(&h0);
-                w[2 * p + 1] = *reinterpret_cast<uint32_t*>(&h1);
-            }
-            dst[0] = make_uint4(w[0], w[1], w[2], w[3]);
-            dst[1] = make_uint4(w[4], w[5], w[6], w[7]);
-            if (x.lse && ql == 0) x.lse[orow] = (M + __log2f(den)) * 0.6931471805599453f;
+        for (int p = 0; p < 4; ++p) {
+            const __nv_bfloat162 h0 = __floats2bfloat162_rn(acc[p].x * inv, acc[p].y * inv);
+            const __nv_bfloat162 h1 = __floats2bfloat162_rn(acc[p].z * inv, acc[p].w * inv);
+            o[2 * p] = *reinterpret_cast<const uint32_t*>(&h0);
+            o[2 * p + 1] = *reinterpret_cast<const uint32_t*>(&h1);
         }
-        g += 4;                                                  // the next group's row: four further on
-        while (g >= G) { g -= G; ++node; }
+        uint4* dst = reinterpret_cast<uint4*>(x.out + orow * kD + cg * 16);
+        dst[0] = make_uint4(o[0], o[1], o[2], o[3]);
+        dst[1] = make_uint4(o[4], o[5], o[6], o[7]);
     }
 }
 
