@@ -91,21 +91,21 @@ attn_umma_kernel(const __grid_constant__ AttnLayers<NL> layers, const sd_batch b
     const bool aligned = (smem_u32(smem) & 1023u) == 0;    // swizzled tiles need 1 KiB alignment
     uint32_t tmem_base = 0;
     if (aligned) {
-        if (warp == kMmaWarp) {                            // (a thread with nothing else to do at this point)
-            *abort_flag = 0;
-            for (int i = 0; i < kKStages; ++i) { mbar_init(&k_full[i], 1); mbar_init(&k_empty[i], 1); }
-            for (int i = 0; i < kVStages; ++i) { mbar_init(&v_full[i], 1); mbar_init(&v_empty[i], 1); }
-            for (int i = 0; i < 2; ++i) { mbar_init(&s_full[i], 1); mbar_init(&p_full[i], 4); }
-            mbar_init(pv_done, 1); mbar_init(q_full, 1); mbar_init(o_full, 1); mbar_init(x_full, 1);
-            fence_barrier_init();
-        }
         if (warp == kTmaWarp) {                            // a full warp (the MMA warp is a single thread)
+            if (lane == 0) {                               // (this thread uses some of them before the block meets)
+                *abort_flag = 0;
+                for (int i = 0; i < kKStages; ++i) { mbar_init(&k_full[i], 1); mbar_init(&k_empty[i], 1); }
+                for (int i = 0; i < kVStages; ++i) { mbar_init(&v_full[i], 1); mbar_init(&v_empty[i], 1); }
+                for (int i = 0; i < 2; ++i) { mbar_init(&s_full[i], 1); mbar_init(&p_full[i], 4); }
+                mbar_init(pv_done, 1); mbar_init(q_full, 1); mbar_init(o_full, 1); mbar_init(x_full, 1);
+                fence_barrier_init();
+                fence_proxy_async_smem();
+                prefetch_tensormap(map_q); prefetch_tensormap(map_kc); prefetch_tensormap(map_vc);
+                prefetch_tensormap(map_kt); prefetch_tensormap(map_vt);
+            }
+            __syncwarp();
             tmem_alloc(tmem_slot, kTmemCols);
             tmem_relinquish();
-        }
-        if (warp == kTmaWarp && lane == 0) {
-            prefetch_tensormap(map_q); prefetch_tensormap(map_kc); prefetch_tensormap(map_vc);
-            prefetch_tensormap(map_kt); prefetch_tensormap(map_vt);
         }
     } else if (threadIdx.x == 0) {
         set_status(status, SD_ERR_UNSUPPORTED);
@@ -140,8 +140,8 @@ attn_umma_kernel(const __grid_constant__ AttnLayers<NL> layers, const sd_batch b
     // reach no output, the smem rows behind tile_rows hold whatever they held).  (Staged through registers
     // by the softmax threads it took two more dependent memory latencies before the first scores.)
     const int tile_rows = plan.tile_rows;
+    const uint64_t pol = policy_evict_first();
     if (aligned && warp == kTmaWarp && lane == 0) {
-        const uint64_t pol = policy_evict_first();
         mbar_arrive_expect_tx(q_full, (uint32_t)tile_rows * kD * 2);
         tma_load_3d(q_smem, map_q, 0, kvh * G, b * T + rt * plan.tile_nodes, q_full, pol);
         tma_load_3d(q_smem + kRowTile * 128, map_q, 64, kvh * G, b * T + rt * plan.tile_nodes, q_full, pol);
@@ -158,14 +158,10 @@ attn_umma_kernel(const __grid_constant__ AttnLayers<NL> layers, const sd_batch b
     const bool m64 = (rows - rt * tile_rows) <= 64;
 
     // key tiles of this CTA: cache blocks [t0, t1) and, for the last chunk, the tree tile
-    int tiles_total = (len + kKeyTile - 1) / kKeyTile;
-    if (tiles_total > bt.max_blocks_per_seq) {             // the block table does not cover this length
-        if (threadIdx.x == 0) set_status(status, SD_ERR_BOUNDS);
-        tiles_total = bt.max_blocks_per_seq;
-    }
-    const int tpc = (tiles_total + plan.n_chunks - 1) / plan.n_chunks;
-    const int t0 = min(chunk * tpc, tiles_total);
-    const int t1 = min(t0 + tpc, tiles_total);
+    if ((len + kKeyTile - 1) / kKeyTile > bt.max_blocks_per_seq && threadIdx.x == 0)
+        set_status(status, SD_ERR_BOUNDS);                 // the block table does not cover this length
+    const ChunkRange cr = chunk_range(len, bt.max_blocks_per_seq, plan.n_chunks, chunk);
+    const int tiles_total = cr.tiles_total, tpc = cr.tpc, t0 = cr.t0, t1 = cr.t1;
     const bool has_tree = (chunk == plan.n_chunks - 1);
     const int nt = (t1 - t0) + (has_tree ? 1 : 0);
     // A CTA without key tiles has nothing to compute, but it still takes part in the cluster barriers; a
@@ -173,6 +169,43 @@ attn_umma_kernel(const __grid_constant__ AttnLayers<NL> layers, const sd_batch b
     const bool has_rows = rt * tile_rows < rows;
     const bool active = (nt > 0) && aligned && has_rows;
     const bool clustered = (plan.n_chunks > 1) && has_rows;   // cluster = the chunks of one (b, kvh, row tile)
+    // The producer thread fills the rings before the block meets: K and V tiles travel through separate
+    // rings and are issued independently, whichever slot frees first: the next K tile (needed early, for
+    // the score MMA issued one tile ahead) must not queue behind a V slot that is only released when P.V
+    // has finished.  The block table is looked up ahead of its use (the first entries all at once).
+    const int32_t* table = bt.block_table + (size_t)b * bt.max_blocks_per_seq;
+    const int n_pref = t1 - t0;
+    int jk = 0, jv = 0, blk_k = 0, blk_v = 0;
+    auto issue = [&](int j, int blk, bool is_v) {
+        const int stages = is_v ? kVStages : kKStages;
+        const int s = j % stages;
+        uint64_t* full = (is_v ? v_full : k_full) + s;
+        uint8_t* dst = (is_v ? v_smem : k_smem) + s * kKVStage;
+        mbar_arrive_expect_tx(full, kKVStage);
+        if (j >= n_pref) {
+            const CUtensorMap* m = is_v ? map_vt : map_kt;
+            tma_load_3d(dst, m, 0, kvh, b * T, full, pol);
+            tma_load_3d(dst + kSubTile, m, 64, kvh, b * T, full, pol);
+        } else {
+            if (blk < 0 || blk >= num_blocks) { set_status(status, SD_ERR_BOUNDS); blk = 0; }
+            const CUtensorMap* m = is_v ? map_vc : map_kc;
+            const int y = (blk * bt.Hkv + kvh) * kKeyTile;
+            tma_load_2d(dst, m, 0, y, full, pol);
+            tma_load_2d(dst + kSubTile, m, 64, y, full, pol);
+        }
+    };
+    if (active && warp == kTmaWarp && lane == 0) {
+        int first[kKStages + 1];
+#pragma unroll
+        for (int i = 0; i <= kKStages; ++i) first[i] = i < n_pref ? __ldg(table + t0 + i) : 0;
+        blk_k = kKStages < n_pref ? first[kKStages] : 0;
+        blk_v = kVStages < n_pref ? first[kVStages] : 0;
+#pragma unroll
+        for (int i = 0; i < kKStages; ++i) {
+            if (i < nt) { issue(i, first[i], false); jk = i + 1; }
+            if (i < kVStages && i < nt) { issue(i, first[i], true); jv = i + 1; }
+        }
+    }
     // rows of unused nodes are zeroed by the first chunk's CTA, 16 bytes per lane
     if (chunk == 0) {
         const int z0 = max(rows, rt * tile_rows), z1 = min(plan.rows, (rt + 1) * tile_rows);
@@ -197,45 +230,18 @@ attn_umma_kernel(const __grid_constant__ AttnLayers<NL> layers, const sd_batch b
     if (active) {
     if (warp == kTmaWarp) {
         // ------------------------------------------------------------ TMA producer (one thread)
-        // K and V tiles travel through separate rings and are issued independently, whichever slot
-        // frees first: the next K tile (needed early, for the score MMA issued one tile ahead) must
-        // not queue behind a V slot that is only released when P.V has finished.
         if (lane == 0) {
-            const uint64_t pol = policy_evict_first();
-            const int32_t* table = bt.block_table + (size_t)b * bt.max_blocks_per_seq;
-            const int n_pref = t1 - t0;
-            int jk = 0, jv = 0;
-            int blk_k = (n_pref > 0) ? __ldg(table + t0) : 0;      // looked up one tile ahead
-            int blk_v = blk_k;
             bool ok = true;
             long long t_last = clock64();
-            auto issue = [&](int j, int blk, bool is_v) {
-                const int stages = is_v ? kVStages : kKStages;
-                const int s = j % stages;
-                uint64_t* full = (is_v ? v_full : k_full) + s;
-                uint8_t* dst = (is_v ? v_smem : k_smem) + s * kKVStage;
-                mbar_arrive_expect_tx(full, kKVStage);
-                if (j >= n_pref) {
-                    const CUtensorMap* m = is_v ? map_vt : map_kt;
-                    tma_load_3d(dst, m, 0, kvh, b * T, full, pol);
-                    tma_load_3d(dst + kSubTile, m, 64, kvh, b * T, full, pol);
-                } else {
-                    if (blk < 0 || blk >= num_blocks) { set_status(status, SD_ERR_BOUNDS); blk = 0; }
-                    const CUtensorMap* m = is_v ? map_vc : map_kc;
-                    const int y = (blk * bt.Hkv + kvh) * kKeyTile;
-                    tma_load_2d(dst, m, 0, y, full, pol);
-                    tma_load_2d(dst + kSubTile, m, 64, y, full, pol);
-                }
-            };
             while ((jk < nt || jv < nt) && ok) {
                 bool progress = false;
-                if (jk < nt && mbar_try_wait(&k_empty[jk % kKStages], ((uint32_t)(jk / kKStages) & 1u) ^ 1u)) {
+                if (jk < nt && mbar_test_wait(&k_empty[jk % kKStages], ((uint32_t)(jk / kKStages) & 1u) ^ 1u)) {
                     issue(jk, blk_k, false);
                     ++jk;
                     if (jk < n_pref) blk_k = __ldg(table + t0 + jk);
                     progress = true;
                 }
-                if (jv < nt && mbar_try_wait(&v_empty[jv % kVStages], ((uint32_t)(jv / kVStages) & 1u) ^ 1u)) {
+                if (jv < nt && mbar_test_wait(&v_empty[jv % kVStages], ((uint32_t)(jv / kVStages) & 1u) ^ 1u)) {
                     issue(jv, blk_v, true);
                     ++jv;
                     if (jv < n_pref) blk_v = __ldg(table + t0 + jv);
@@ -323,9 +329,44 @@ attn_umma_kernel(const __grid_constant__ AttnLayers<NL> layers, const sd_batch b
         const uint64_t scale2 = pack_f32x2(scale_log2, scale_log2);
         uint64_t neg_m2 = 0ull;                                // -(reference of this row), twice
         bool ok = true;
+        const int n_full = max(min(len / kKeyTile - t0, n_pref), 0);    // leading tiles whose 64 keys are all inside the prefix
         for (int j = 0; j < nt && ok; ++j) {
             const int s = j & 1;
             const uint32_t ph = (uint32_t)(j >> 1) & 1u;
+            // The usual tile (all keys visible, reference known): nothing but loads, exponentials and stores.
+            // Masks, a new reference and clearing V rows live in the other body below; as branches inside
+            // one body they cost every tile 370 of 1600 cycles (predicated masks, scores kept alive).
+            // The exponentials are taken against the row's reference straight away.  The reference is the
+            // maximum of the first tile and need not follow later ones: P (bf16) and the sums (fp32) have
+            // fp32's exponent range, so their relative precision does not depend on how far a score lies
+            // above the reference.  Only when the tile's sum leaves the safe range (> 2^40: some score more
+            // than about 34 powers of two above the reference) is the reference raised and the tile redone
+            // (its scores are still in tensor memory).  The sum is needed anyway, so no maximum is tracked,
+            // and scaling and sums run two elements per instruction.
+            if (j > 0 && j < n_full) {
+                if (!mbar_wait(&s_full[s], ph, abort_flag, plan.wait_cycles)) { ok = false; break; }
+                tc_fence_after_sync();
+                uint32_t r0[32], r1[32], pk[32];
+                uint64_t ps[2] = {0ull, 0ull};
+                tmem_ld32(tmem_s + lane_field + s * kKeyTile, r0);
+                tmem_ld_wait();
+                tmem_ld32(tmem_s + lane_field + s * kKeyTile + 32, r1);   // in flight while the first half is processed
+                exp_pack_half(r0, scale2, neg_m2, pk, ps);
+                tmem_ld_wait();
+                exp_pack_half(r1, scale2, neg_m2, pk + 16, ps);
+                const float psum = sum_f32x2(add_f32x2(ps[0], ps[1]));
+                // (padding rows have harmless scores; NaN scores of a real row take the other body and stay NaN)
+                if (!__any_sync(0xffffffffu, row_ok && !(psum <= kSumLimit))) {
+                    l += psum;
+                    // P replaces the S columns this thread has just consumed (its own TMEM lane)
+                    tmem_st32(tmem_s + lane_field + s * kKeyTile, pk);
+                    tmem_st_wait();
+                    tc_fence_before_sync();
+                    __syncwarp();
+                    if (lane == 0) mbar_arrive(&p_full[s]);
+                    continue;
+                }
+            }
             const bool tree = (j >= t1 - t0);
             const int valid = tree ? kKeyTile : len - (t0 + j) * kKeyTile;   // keys of this block inside the prefix
             if (!mbar_wait(&s_full[s], ph, abort_flag, plan.wait_cycles)) { ok = false; break; }
@@ -352,42 +393,22 @@ attn_umma_kernel(const __grid_constant__ AttnLayers<NL> layers, const sd_batch b
                     fence_proxy_async_smem();
                 }
             }
-            // The scores arrive in two halves; the second half is in flight while the first is
-            // processed.  Raw scores stay unscaled: scale * log2(e) is folded into the exponent's FMA.
-            uint32_t r0[32], r1[32];
+            uint32_t r0[32], r1[32], pk[32];
             tmem_ld32(tmem_s + lane_field + s * kKeyTile, r0);
-            tmem_ld_wait();
             tmem_ld32(tmem_s + lane_field + s * kKeyTile + 32, r1);
-            const uint32_t mask_lo = tree ? (uint32_t)amask : (valid >= 32 ? ~0u : ((1u << max(valid, 0)) - 1u));
-            const uint32_t mask_hi = tree ? (uint32_t)(amask >> 32)
-                                          : (valid >= 64 ? ~0u : (valid <= 32 ? 0u : ((1u << (valid - 32)) - 1u)));
-            const bool masked = tree || valid < kKeyTile;
-            if (masked) mask_scores(r0, mask_lo);
-            // The exponentials are taken against the row's reference straight away.  The reference is the
-            // maximum of the first tile and need not follow later ones: P (bf16) and the sums (fp32) have
-            // fp32's exponent range, so their relative precision does not depend on how far a score lies
-            // above the reference.  Only when the tile's sum leaves the safe range (> 2^40: some score more
-            // than about 34 powers of two above the reference) is the reference raised and the tile redone.
-            // The sum is needed anyway, so the usual tile tracks no maximum at all, and scaling and sums run
-            // two elements per instruction: 160 instead of 256 arithmetic instructions per thread and tile.
-            // (Two warps share a scheduler partition: 1024 of the 1550 cycles a pair of tiles took were
-            // the exponential unit's, about 1100 were issue slots.)
-            uint32_t pk[32];
-            float psum = 0.f;
-            bool raise = row_ok;
-            if (j > 0) {
-                uint64_t ps[2] = {0ull, 0ull};
-                exp_pack_half(r0, scale2, neg_m2, pk, ps);
-                tmem_ld_wait();
-                if (masked) mask_scores(r1, mask_hi);
-                exp_pack_half(r1, scale2, neg_m2, pk + 16, ps);
-                psum = sum_f32x2(add_f32x2(ps[0], ps[1]));
-                // (padding rows have zero scores; NaN scores of a real row end up here as well and stay NaN)
-                raise = row_ok && !(psum <= kSumLimit);
-            } else {
-                tmem_ld_wait();
-                if (masked) mask_scores(r1, mask_hi);
+            tmem_ld_wait();
+            if (tree || valid < kKeyTile) {
+                mask_scores(r0, tree ? (uint32_t)amask : (valid >= 32 ? ~0u : ((1u << max(valid, 0)) - 1u)));
+                mask_scores(r1, tree ? (uint32_t)(amask >> 32)
+                                     : (valid >= 64 ? ~0u : (valid <= 32 ? 0u : ((1u << (valid - 32)) - 1u))));
             }
+            uint64_t ps[2] = {0ull, 0ull};
+            if (j > 0) {
+                exp_pack_half(r0, scale2, neg_m2, pk, ps);
+                exp_pack_half(r1, scale2, neg_m2, pk + 16, ps);
+            }
+            float psum = sum_f32x2(add_f32x2(ps[0], ps[1]));
+            bool raise = row_ok && (j == 0 || !(psum <= kSumLimit));
             if (__any_sync(0xffffffffu, raise)) {
                 float mx[4] = {-INFINITY, -INFINITY, -INFINITY, -INFINITY};
 #pragma unroll
@@ -416,7 +437,7 @@ attn_umma_kernel(const __grid_constant__ AttnLayers<NL> layers, const sd_batch b
                 if (raise) m_used = mt;
                 neg_m2 = pack_f32x2(-m_used, -m_used);
                 // (again) against the new reference: the same values for rows that did not raise
-                uint64_t ps[2] = {0ull, 0ull};
+                ps[0] = ps[1] = 0ull;
                 exp_pack_half(r0, scale2, neg_m2, pk, ps);
                 exp_pack_half(r1, scale2, neg_m2, pk + 16, ps);
                 psum = sum_f32x2(add_f32x2(ps[0], ps[1]));

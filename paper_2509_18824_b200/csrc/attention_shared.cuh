@@ -81,6 +81,17 @@ struct AttnPlan {
     int withhold;      // test hook: the softmax warps never report their first tile, so that a wait runs out
 };
 
+// cache blocks [t0, t1) of one key chunk of a sequence
+struct ChunkRange { int tiles_total, tpc, t0, t1; };
+__device__ __forceinline__ ChunkRange chunk_range(int len, int max_blocks, int n_chunks, int chunk) {
+    ChunkRange r;
+    r.tiles_total = min((len + kBlock - 1) / kBlock, max_blocks);
+    r.tpc = (r.tiles_total + n_chunks - 1) / n_chunks;
+    r.t0 = min(chunk * r.tpc, r.tiles_total);
+    r.t1 = min(r.t0 + r.tpc, r.tiles_total);
+    return r;
+}
+
 // Everything the CTAs of one layer need.  A launch covers up to kMaxLayersPerLaunch layers (the
 // descriptors travel as kernel parameters); blockIdx.z enumerates (sequence, layer, KV head).
 struct AttnLayer {
