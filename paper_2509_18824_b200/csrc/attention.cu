@@ -67,11 +67,7 @@ attn_umma_kernel(const __grid_constant__ AttnLayers<NL> layers, const sd_batch b
     const int lane = threadIdx.x & 31;
     const int chunk = blockIdx.x;
     const int rt = blockIdx.y;
-    // blockIdx.z enumerates (sequence rank, layer, KV head): the CTAs of the longest sequences are
-    // dispatched first, in every layer, so that a ragged batch does not end on a few long stragglers.
-    // The rank -> sequence lookup is done here (up to 64 sequences: each of the first B threads ranks
-    // one sequence by cached length, ties by index); larger batches, and launches that fit the GPU in
-    // one wave, run in index order.
+    // blockIdx.z enumerates (sequence rank, layer, KV head), see sequence_of_rank
     const int zz = (int)blockIdx.z + plan.z0;
     const int kvh = zz % bt.Hkv;
     const int lb = zz / bt.Hkv;
@@ -113,23 +109,10 @@ attn_umma_kernel(const __grid_constant__ AttnLayers<NL> layers, const sd_batch b
     // everything below reads (or writes) global memory that the kernel ahead may still be working on
     griddep_wait();
 
+    // (the slot lives in the dynamic shared-memory block: a static variable would push that block's
+    //  1 KiB-aligned start and cost the second resident CTA)
     int b = rank_b;
-    if (plan.ranked) {
-        // (the slot lives in the dynamic shared-memory block: a static variable would push that block's
-        //  1 KiB-aligned start and cost the second resident CTA)
-        int& s_seq = *reinterpret_cast<int*>(bars + 19);
-        if ((int)threadIdx.x < bt.B) {
-            const int mine = __ldg(bt.len + threadIdx.x);
-            int r = 0;
-            for (int j = 0; j < bt.B; ++j) {
-                const int other = __ldg(bt.len + j);
-                r += (other > mine || (other == mine && j < (int)threadIdx.x)) ? 1 : 0;
-            }
-            if (r == rank_b) s_seq = threadIdx.x;
-        }
-        __syncthreads();
-        b = s_seq;
-    }
+    if (plan.ranked) b = sequence_of_rank(bt, rank_b, *reinterpret_cast<int*>(bars + 19));
     __nv_bfloat16* __restrict__ out = ly.out;
     float* __restrict__ lse = ly.lse;
     const int num_blocks = ly.num_blocks;
@@ -160,15 +143,16 @@ attn_umma_kernel(const __grid_constant__ AttnLayers<NL> layers, const sd_batch b
     // key tiles of this CTA: cache blocks [t0, t1) and, for the last chunk, the tree tile
     if ((len + kKeyTile - 1) / kKeyTile > bt.max_blocks_per_seq && threadIdx.x == 0)
         set_status(status, SD_ERR_BOUNDS);                 // the block table does not cover this length
-    const ChunkRange cr = chunk_range(len, bt.max_blocks_per_seq, plan.n_chunks, chunk);
+    const int n_chunks = chunks_of(min((len + kKeyTile - 1) / kKeyTile, bt.max_blocks_per_seq), plan.n_chunks, plan.chunk_blocks);   // of this sequence; CTAs beyond have nothing to do
+    const ChunkRange cr = chunk_range(len, bt.max_blocks_per_seq, n_chunks, chunk);
     const int tiles_total = cr.tiles_total, tpc = cr.tpc, t0 = cr.t0, t1 = cr.t1;
-    const bool has_tree = (chunk == plan.n_chunks - 1);
+    const bool has_tree = (chunk == n_chunks - 1);
     const int nt = (t1 - t0) + (has_tree ? 1 : 0);
     // A CTA without key tiles has nothing to compute, but it still takes part in the cluster barriers; a
     // row tile without rows is skipped by every CTA of its cluster.
-    const bool has_rows = rt * tile_rows < rows;
+    const bool has_rows = rt * tile_rows < rows && chunk < n_chunks;
     const bool active = (nt > 0) && aligned && has_rows;
-    const bool clustered = (plan.n_chunks > 1) && has_rows;   // cluster = the chunks of one (b, kvh, row tile)
+    const bool clustered = (n_chunks > 1) && has_rows;   // cluster = the chunks of one (b, kvh, row tile)
     // The producer thread fills the rings before the block meets: K and V tiles travel through separate
     // rings and are issued independently, whichever slot frees first: the next K tile (needed early, for
     // the score MMA issued one tile ahead) must not queue behind a V slot that is only released when P.V
@@ -206,16 +190,7 @@ attn_umma_kernel(const __grid_constant__ AttnLayers<NL> layers, const sd_batch b
             if (i < kVStages && i < nt) { issue(i, first[i], true); jv = i + 1; }
         }
     }
-    // rows of unused nodes are zeroed by the first chunk's CTA, 16 bytes per lane
-    if (chunk == 0) {
-        const int z0 = max(rows, rt * tile_rows), z1 = min(plan.rows, (rt + 1) * tile_rows);
-        for (int i = z0 * 16 + (int)threadIdx.x; i < z1 * 16; i += kAttThreads) {
-            const int row = i >> 4, node = row / G;
-            const size_t orow = ((size_t)b * T + node) * bt.Hq + kvh * G + (row - node * G);
-            reinterpret_cast<uint4*>(out + orow * kD)[i & 15] = make_uint4(0, 0, 0, 0);
-            if (lse && (i & 15) == 0) lse[orow] = 0.f;
-        }
-    }
+    if (chunk == 0) zero_unused_rows(bt, plan, ly, b, rt, kvh, rows, (int)threadIdx.x, kAttThreads);
     float m_used = -INFINITY, l = 0.f;                     // softmax state of this thread's row (warps 0-3)
     bool rows_ready = false;                               // ... and whether it completed (clustered launches)
 
@@ -489,73 +464,23 @@ attn_umma_kernel(const __grid_constant__ AttnLayers<NL> layers, const sd_batch b
         mbar_wait(q_full, 0, abort_flag, plan.wait_cycles);
 
     if (clustered) {
-        // Row r of the tile is finished by the CTA of chunk r / (128 / n_chunks): every other chunk's CTA
-        // sends it that row's maximum, sum and unnormalised O straight from tensor memory, with stores that
-        // report their bytes to the receiver's barrier (so the receiver waits for exactly what it gets, and
-        // no second cluster-wide barrier and release stand between the last row and the merge).
-        const int rows_per = kRowTile / plan.n_chunks;
-        const uint32_t xo_addr = smem_u32(k_smem), xs_addr = xo_addr + kRowTile * kD * 4;
-        if (threadIdx.x == 0) {
-            const int mine = min(max(min(rows - rt * tile_rows, tile_rows) - chunk * rows_per, 0), rows_per);
-            int others = 0;                                // chunks with key tiles, this one aside
-            for (int c = 0; c < plan.n_chunks; ++c)
-                others += (c != chunk && (c == plan.n_chunks - 1 || c * tpc < tiles_total)) ? 1 : 0;
-            mbar_arrive_expect_tx(x_full, (uint32_t)(others * mine * (kD * 4 + 8)));
-        }
-        // every thread of every CTA of the cluster: all MMAs and copies of the cluster have completed, so
-        // every CTA's K/V rings are free to receive rows
+        // The chunks' rows meet as described at exchange_rows; the rings are free by now.
+        const RowExchange x{bt, plan, ly, smem_u32(k_smem), smem_u32(x_full), chunk, n_chunks, rt, b, kvh, rows, tpc, tiles_total};
+        if (threadIdx.x == 0) exchange_expect(x, x_full);
         __syncwarp();
-        cluster_arrive_release();
+        cluster_arrive_release();                          // every CTA's MMAs and copies are complete
         cluster_wait_acquire();
-        if (active && warp < 4) {
-            const int row_in_tile = m64 ? (lane < 16 ? warp * 16 + lane : -1) : warp * 32 + lane;
-            const int rr = max(row_in_tile, 0);
-            const int dest = rr / rows_per, rl = rr % rows_per;
-            // rows beyond the sequence's last query row are not exchanged
-            const bool mine = rows_ready && row_in_tile >= 0 && rr < tile_rows && rt * tile_rows + rr < rows;
-            // Exchange area: [chunk][16-byte piece of the row][row of the finisher], so that a warp's store
-            // (32 rows, one piece each) fills 512 consecutive bytes: remote stores travel in packets of
-            // consecutive bytes (measured with 256 CTAs in pairs: 24.5 B/clk per CTA against 12.5 for one
-            // 512-byte line per row).
-            const uint32_t off = (uint32_t)(((chunk * 32) * rows_per + rl) * 16);
-            const uint32_t xo_remote = map_dsmem(xo_addr, (uint32_t)dest) + off;
-            const uint32_t xs_remote = map_dsmem(xs_addr, (uint32_t)dest) + (uint32_t)(chunk * rows_per + rl) * 4;
-            const uint32_t bar_remote = map_dsmem(smem_u32(x_full), (uint32_t)dest);
-            tc_fence_after_sync();
-#pragma unroll
-            for (int cc = 0; cc < 4; ++cc) {
-                uint32_t o[32];
-                tmem_ld32(tmem_base + ((uint32_t)(warp * 32) << 16) + cc * 32, o);
-                tmem_ld_wait();
-                if (mine && dest != chunk) {
-#pragma unroll
-                    for (int k = 0; k < 8; ++k)
-                        st_async_v4(xo_remote + (uint32_t)((cc * 8 + k) * rows_per * 16), o[4 * k], o[4 * k + 1], o[4 * k + 2],
-                                    o[4 * k + 3], bar_remote);
-                } else if (mine) {
-#pragma unroll
-                    for (int k = 0; k < 8; ++k)
-                        st_smem_v4(xo_addr + off + (uint32_t)((cc * 8 + k) * rows_per * 16), o[4 * k], o[4 * k + 1], o[4 * k + 2],
-                                   o[4 * k + 3]);
-                }
-            }
-            if (mine && dest != chunk) {
-                st_async_b32(xs_remote, __float_as_uint(m_used), bar_remote);
-                st_async_b32(xs_remote + kRowTile * 4, __float_as_uint(l), bar_remote);
-            } else if (mine) {
-                st_smem_f32(xs_addr + (uint32_t)(chunk * rows_per + rl) * 4, m_used);
-                st_smem_f32(xs_addr + (uint32_t)(kRowTile + chunk * rows_per + rl) * 4, l);
-            }
-        }
+        if (active && warp < 4)
+            exchange_push<4>(x, tmem_base + ((uint32_t)(warp * 32) << 16), 0, rows_ready,
+                             m64 ? (lane < 16 ? warp * 16 + lane : -1) : (int)threadIdx.x, m_used, l);
         __syncwarp();
         cluster_arrive_relaxed();                          // (waited for at the end: nobody leaves before its peers have sent)
         if (warp < 4) {
             asm volatile("bar.sync 1, 128;" ::: "memory"); // this CTA's own rows
             if (mbar_wait_cluster(x_full, 0, abort_flag, plan.wait_cycles)) {
-                const MergeCtx mc{bt, plan, out, lse, xo_addr, xs_addr, chunk, rt, b, kvh, rows, tpc, tiles_total, (int)threadIdx.x};
-                if (plan.n_chunks == 2) merge_rows<2>(mc);
-                else if (plan.n_chunks == 4) merge_rows<4>(mc);
-                else merge_rows<8>(mc);
+                if (n_chunks == 2) merge_rows<2, 128>(x, (int)threadIdx.x);
+                else if (n_chunks == 4) merge_rows<4, 128>(x, (int)threadIdx.x);
+                else merge_rows<8, 128>(x, (int)threadIdx.x);
             } else if (lane == 0) {
                 set_status(status, SD_ERR_TIMEOUT);
                 for (int i = 0; i < 1000; ++i) __nanosleep(1000);      // let rows in flight land
@@ -599,29 +524,7 @@ static bool fill_layer(AttnLayer* ly, const sd_batch& bt, const sd_kv_layer& cac
 template <int NL>
 sd_status launch_rows1(const AttnLayers<NL>& layers, const sd_batch& bt, float scale, const AttnPlan& plan,
                        int z_count, int32_t* dev_status, cudaStream_t st) {
-    auto kern = attn_umma_kernel<NL>;
-    if (cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, kAttSmem) != cudaSuccess)
-        return SD_ERR_CUDA;
-    cudaLaunchConfig_t cfg = {};
-    cfg.gridDim = dim3(plan.n_chunks, plan.row_tiles, z_count);
-    cfg.blockDim = dim3(kAttThreads);
-    cfg.dynamicSmemBytes = kAttSmem;
-    cfg.stream = st;
-    cudaLaunchAttribute attr[2];
-    attr[0].id = cudaLaunchAttributeClusterDimension;      // the chunks of one row tile form a cluster
-    attr[0].val.clusterDim.x = plan.n_chunks;
-    attr[0].val.clusterDim.y = 1;
-    attr[0].val.clusterDim.z = 1;
-    // The launch may begin while the kernel before it in the stream is still running (its CTAs take the
-    // SM slots that one frees and do their set-up); the kernel waits for that kernel's completion before
-    // it touches global memory.  Consecutive attention calls - one per layer - overlap their ends this way.
-    attr[1].id = cudaLaunchAttributeProgrammaticStreamSerialization;
-    attr[1].val.programmaticStreamSerializationAllowed = 1;
-    cfg.attrs = attr;
-    cfg.numAttrs = 2;
-    if (cudaLaunchKernelEx(&cfg, kern, layers, bt, scale * kLog2e, plan, dev_status) != cudaSuccess)
-        return SD_ERR_CUDA;
-    return SD_OK;
+    return launch_attn(attn_umma_kernel<NL>, kAttThreads, kAttSmem, layers, bt, scale, plan, z_count, dev_status, st);
 }
 template sd_status launch_rows1<1>(const AttnLayers<1>&, const sd_batch&, float, const AttnPlan&, int, int32_t*,
                                    cudaStream_t);
@@ -644,14 +547,58 @@ static int sm_count() {
 // attention needs no global scratch (a nominal size keeps the argument checks uniform).
 size_t attention_workspace_bytes(const sd_batch&) { return 256; }
 
-// How many key chunks per sequence.
-static AttnPlan make_plan(const sd_batch& bt, int n_layers, int sms) {
+static AttnPlan common_plan(const sd_batch& bt, int n_layers, const TestKnobs& knobs) {
     AttnPlan p;
     const int G = bt.Hq / bt.Hkv;
     p.rows = bt.T_max * G;
     p.tile_nodes = kRowTile / G;
     p.tile_rows = p.tile_nodes * G;
+    p.g_magic = (65536 + G - 1) / G;
     p.row_tiles = (p.rows + p.tile_rows - 1) / p.tile_rows;
+    p.n_layers = n_layers;
+    p.z0 = 0;
+    p.wait_cycles = knobs.wait_cycles;
+    p.withhold = knobs.withhold;
+    return p;
+}
+
+// The 128-key kernel (attention_wide.cu) runs one CTA per SM.  A round of it takes about 0.36 us per cache block
+// of its longest chunk, plus 8 us for launch, first copies and output (11 when CTAs of another round follow:
+// nothing overlaps them), plus the merge of the chunks.  Measured per call in us, chunks 1 / 2 / 4 / 8: one
+// sequence of 2048 tokens and 60 nodes 17.2 / 13.5 / 10.9 / 17.9 (16 clusters of eight are more than fit at a
+// time), four of 8192 52 / 32 / 41, eight of 4096 32 / 40, eight chains of 11 nodes 29.6 / 20.8 / 17.8.
+// The 64-key kernel's two CTAs per SM overlap each other's ends: a round of twice as many CTAs takes about
+// 0.9 us per block plus 13 us.  It is left for launches of several rounds in which those ends weigh more
+// (256 CTAs of 1000 tokens: 28.7 against 33.9 us; of 4096: 71.4 against 69.9).
+static bool wide_plan(AttnPlan* p, const sd_batch& bt, int dev, int sms, const TestKnobs& knobs) {
+    const long long base = (long long)p->n_layers * bt.B * bt.Hkv * p->row_tiles;
+    const int blocks = bt.max_blocks_per_seq;
+    const double merge[4] = {0.0, 2.0, 2.3, 3.0};
+    int n = 1;
+    long long n_rounds = 1;
+    double best = 1e30;
+    for (int c = 1, i = 0; c <= kMaxChunks && c <= blocks; c *= 2, ++i) {
+        const int resident = wide_resident_clusters(dev, sms, c);
+        const long long rounds = (base + resident - 1) / resident;
+        const double us = rounds * ((rounds > 1 ? 11.0 : 8.0) + merge[i] + 0.36 * ((blocks + c - 1) / c));
+        if (knobs.chunks > 0 && knobs.chunks <= blocks ? c == knobs.chunks : us < best - 1e-9) { best = us; n = c; n_rounds = rounds; }
+    }
+    if (n_rounds > 1) {
+        const double rounds = base <= 2 * sms ? 1.0 : (double)base / (2 * sms) + 0.25;     // a partial round, cut into chunks
+        if (best > 0.95 * rounds * (13.0 + 0.9 * blocks)) return false;
+    }
+    p->n_chunks = n;
+    // Shorter sequences are cut into fewer chunks where all clusters run at once; in several rounds the CTAs that
+    // leave would still hold back the next cluster (half-empty pairs halved the machine).
+    p->chunk_blocks = n_rounds == 1 ? (blocks + n - 1) / n : 0;
+    p->ranked = (bt.B > 1 && bt.B <= 64 && base * n > sms) ? 1 : 0;
+    return true;
+}
+
+// The others run the 64-key kernel, two CTAs per SM, whose set-up and output overlap the other CTA's tiles.
+static void narrow_plan(AttnPlan* plan, const sd_batch& bt, int sms, const TestKnobs& knobs) {
+    AttnPlan& p = *plan;
+    const int n_layers = p.n_layers;
     // Pick the chunk count that minimises (waves of CTAs) x (key tiles per CTA + fixed cost),
     // two CTAs being resident per SM.  Few waves are counted whole; many waves balance out.
     const int max_tiles = bt.max_blocks_per_seq;
@@ -678,30 +625,31 @@ static AttnPlan make_plan(const sd_batch& bt, int n_layers, int sms) {
         const double cost = waves * ((max_tiles + c - 1) / c + 3 + merge);
         if (cost < best - 1e-9) { best = cost; n = c; }
     }
-    const TestKnobs knobs = test_knobs();
     if (knobs.chunks > 0 && knobs.chunks <= max_tiles) n = knobs.chunks;     // test hook
     p.n_chunks = n;
-    p.n_layers = n_layers;
+    p.chunk_blocks = 0;
     p.ranked = (bt.B > 1 && bt.B <= 64 && (long long)base * n > slots) ? 1 : 0;
-    p.z0 = 0;
-    p.wait_cycles = knobs.wait_cycles;
-    p.withhold = knobs.withhold;
-    return p;
 }
 
 template <int NL>
 static sd_status launch_group(const AttnLayers<NL>& layers, int n_layers, const sd_batch& bt, float scale,
                               int32_t* dev_status, cudaStream_t st) {
-    AttnPlan plan = make_plan(bt, n_layers, sm_count());
+    int dev = 0;
+    if (cudaGetDevice(&dev) != cudaSuccess) return SD_ERR_CUDA;
+    const int sms = sm_count();
+    const TestKnobs knobs = test_knobs();
+    AttnPlan plan = common_plan(bt, n_layers, knobs);
     const int Z = n_layers * bt.B * bt.Hkv;
+    if (wide_plan(&plan, bt, dev, sms, knobs)) return launch_wide<NL>(layers, bt, scale, plan, Z, dev_status, st);
+    narrow_plan(&plan, bt, sms, knobs);
     // A launch of whole-sequence CTAs that runs for more than one round ends on a partial round, in which
     // the CTAs left over would each work through a whole sequence while most of the GPU idles.  They go
     // into a second launch of the same kernel with the keys split into chunks (a cluster per row tile),
     // so that the remainder also spreads over the SMs and takes a fraction of a round.  (In a ranked
     // launch these are the shortest sequences.)
-    const int slots = 2 * sm_count();
+    const int slots = 2 * sms;
     const long long ctas = (long long)Z * plan.row_tiles;
-    if (plan.n_chunks == 1 && ctas > slots && ctas / slots < kSplitRounds && test_knobs().chunks == 0) {
+    if (plan.n_chunks == 1 && ctas > slots && ctas / slots < kSplitRounds && knobs.chunks == 0) {
         const int z_main = (int)((ctas / slots) * slots / plan.row_tiles);
         const int z_rest = Z - z_main;
         int c = 1;

@@ -11,6 +11,7 @@ using namespace sm100;
 constexpr int kRowTile = 128;                  // query rows per row tile (MMA M)
 constexpr float kLog2e = 1.4426950408889634f;
 constexpr float kSumLimit = 1.0995e12f;        // 2^40: a tile's sum above this raises the row's reference
+constexpr float kRaiseAbove = 32.f;            // log2 units: ... where the maximum itself is looked at (128 x 2^32 < 2^40)
 constexpr int kMaxChunks = 8;                  // = portable cluster size
 constexpr int kSplitRounds = 8;                // launches of fewer whole rounds get their remainder as a chunked launch
 
@@ -68,18 +69,47 @@ __device__ __forceinline__ void exp_pack_half(const uint32_t (&r)[32], uint64_t 
     }
 }
 
+// key chunks of a sequence (the last one also takes the tree's keys): the smallest power of two, up to
+// n_chunks, whose chunks have at most chunk_blocks cache blocks
+__device__ __forceinline__ int chunks_of(int blocks, int n_chunks, int chunk_blocks) {
+    int c = 1;
+    while (c < n_chunks && blocks > c * chunk_blocks) c *= 2;
+    return c;
+}
+
 struct AttnPlan {
-    int n_chunks;      // key chunks per sequence (the last one also takes the tree tile)
+    int n_chunks;      // CTAs per row tile along the keys (a cluster): key chunks of the longest sequences
+    int chunk_blocks;  // cache blocks of such a chunk; a shorter sequence is cut into fewer chunks
     int rows;          // T_max * G
     int tile_nodes;    // tree nodes of a row tile: its rows are whole nodes, the query heads of one KV head each
     int tile_rows;     // tile_nodes * G <= 128
     int row_tiles;
+    int g_magic;       // ceil(65536 / G): row / G for rows below 64 * 8
+    __host__ __device__ __forceinline__ int node_of(int row) const { return (row * g_magic) >> 16; }
     int n_layers;      // layers of this launch
     int ranked;        // dispatch the sequences longest first (only matters when the grid runs in several waves)
     int z0;            // first (sequence rank, layer, KV head) index of this launch: blockIdx.z counts from here
     long long wait_cycles;   // bound of every barrier wait, in SM cycles
     int withhold;      // test hook: the softmax warps never report their first tile, so that a wait runs out
 };
+
+// blockIdx.z enumerates (sequence rank, layer, KV head): the CTAs of the longest sequences are dispatched
+// first, in every layer, so that a ragged batch does not end on a few long stragglers.  The rank -> sequence
+// lookup is done here (up to 64 sequences: each of the first B threads ranks one sequence by cached length,
+// ties by index); larger batches, and launches that fit the GPU in one round, run in index order.
+__device__ __forceinline__ int sequence_of_rank(const sd_batch& bt, int rank, int& s_seq) {
+    if ((int)threadIdx.x < bt.B) {
+        const int mine = __ldg(bt.len + threadIdx.x);
+        int r = 0;
+        for (int j = 0; j < bt.B; ++j) {
+            const int other = __ldg(bt.len + j);
+            r += (other > mine || (other == mine && j < (int)threadIdx.x)) ? 1 : 0;
+        }
+        if (r == rank) s_seq = threadIdx.x;
+    }
+    __syncthreads();
+    return s_seq;
+}
 
 // cache blocks [t0, t1) of one key chunk of a sequence
 struct ChunkRange { int tiles_total, tpc, t0, t1; };
@@ -106,31 +136,101 @@ constexpr int kMaxLayersPerLaunch = 32;
 template <int NL>
 struct AttnLayers { AttnLayer l[NL]; };
 
-// Final step of a clustered launch.  The CTA of chunk o finishes rows o * 128 / NCH .. of the tile and
-// holds, in its exchange area, those rows' unnormalised O of every chunk ([chunk][16-byte piece][row], its
-// own rows stored locally, the others' by the CTAs that computed them) and their references and sums
-// ([chunk][row] each).  One thread takes one row and 16 output columns at a time: consecutive lanes read
-// consecutive rows of a piece (no bank conflicts) and each writes a whole 32-byte sector; chunks are
-// added in chunk order, so the result does not depend on timing.
-struct MergeCtx {
-    const sd_batch& bt; const AttnPlan& plan; __nv_bfloat16* out; float* lse;
-    uint32_t xo_addr, xs_addr;          // this CTA's exchange area: rows, then references [128] and sums [128]
-    int chunk, rt, b, kvh, rows, tpc, tiles_total, tid;
+// rows of unused nodes become zeros, 16 bytes per thread (by the CTA of the first chunk)
+__device__ __forceinline__ void zero_unused_rows(const sd_batch& bt, const AttnPlan& plan, const AttnLayer& ly, int b, int rt, int kvh,
+                                                 int rows, int tid, int threads) {
+    const int G = bt.Hq / bt.Hkv;
+    const int z0 = max(rows, rt * plan.tile_rows), z1 = min(plan.rows, (rt + 1) * plan.tile_rows);
+    for (int i = z0 * 16 + tid; i < z1 * 16; i += threads) {
+        const int row = i >> 4, node = plan.node_of(row);
+        const size_t orow = ((size_t)b * bt.T_max + node) * bt.Hq + kvh * G + (row - node * G);
+        reinterpret_cast<uint4*>(ly.out + orow * kD)[i & 15] = make_uint4(0, 0, 0, 0);
+        if (ly.lse && (i & 15) == 0) ly.lse[orow] = 0.f;
+    }
+}
+
+// Final step of a clustered launch.  Row r of the tile is finished by the CTA of chunk r / (128 / n_chunks).
+// Every other chunk's CTA sends it that row's reference, sum and unnormalised O straight from tensor memory,
+// with stores that report their bytes to the receiver's barrier (so the receiver waits for exactly what it
+// gets, and no second cluster-wide barrier and release stand between the last row and the merge); its own
+// rows it stores locally.
+// Exchange area (over the K ring): [chunk][16-byte piece of the row][row of the finisher], so that a warp's
+// store (32 rows, one piece each) fills 512 consecutive bytes: remote stores travel in packets of
+// consecutive bytes (measured with 256 CTAs in pairs: 24.5 B/clk per CTA against 12.5 for one 512-byte
+// line per row); behind it references and sums, [chunk][row] each.
+struct RowExchange {
+    const sd_batch& bt; const AttnPlan& plan; const AttnLayer& ly;
+    uint32_t xo_addr;                   // this CTA's exchange area
+    uint32_t bar_addr;                  // its barrier for the rows of the other chunks
+    int chunk, n_chunks, rt, b, kvh, rows, tpc, tiles_total;
+    __device__ __forceinline__ uint32_t xs_addr() const { return xo_addr + kRowTile * kD * 4; }
+    // rows beyond the sequence's last one are not exchanged
+    __device__ __forceinline__ bool has(int in_tile) const { return in_tile < plan.tile_rows && rt * plan.tile_rows + in_tile < rows; }
+    // does that chunk have key tiles (the last one has the tree's)
+    __device__ __forceinline__ bool live(int c) const { return c == n_chunks - 1 || c * tpc < tiles_total; }
 };
 
-template <int NCH>
-__device__ __forceinline__ void merge_rows(const MergeCtx& x) {
+// bytes this CTA will receive (one thread, before the cluster barrier)
+__device__ __forceinline__ void exchange_expect(const RowExchange& x, uint64_t* bar) {
+    const int per = kRowTile / x.n_chunks;
+    const int mine = min(max(min(x.rows - x.rt * x.plan.tile_rows, x.plan.tile_rows) - x.chunk * per, 0), per);
+    int others = 0;
+    for (int c = 0; c < x.n_chunks; ++c) others += (c != x.chunk && x.live(c)) ? 1 : 0;
+    mbar_arrive_expect_tx(bar, (uint32_t)(others * mine * (kD * 4 + 8)));
+}
+
+// NC 32-column pieces of this thread's row from column 32 * cc0 on; tmem: O at this warp's lanes
+template <int NC>
+__device__ __forceinline__ void exchange_push(const RowExchange& x, uint32_t tmem, int cc0, bool ready, int row_in_tile, float ref,
+                                              float sum) {
+    const int per = kRowTile / x.n_chunks;
+    const int rr = max(row_in_tile, 0), dest = rr / per, rl = rr % per;
+    const bool mine = ready && row_in_tile >= 0 && x.has(rr), remote = dest != x.chunk;
+    const uint32_t off = (uint32_t)((x.chunk * 32 * per + rl) * 16);
+    const uint32_t xo = (remote ? map_dsmem(x.xo_addr, (uint32_t)dest) : x.xo_addr) + off;
+    const uint32_t bar = map_dsmem(x.bar_addr, (uint32_t)dest);
+    tc_fence_after_sync();
+#pragma unroll
+    for (int cc = cc0; cc < cc0 + NC; ++cc) {
+        uint32_t o[32];
+        tmem_ld32(tmem + cc * 32, o);
+        tmem_ld_wait();
+#pragma unroll
+        for (int k = 0; k < 8; ++k) {
+            const uint32_t at = xo + (uint32_t)((cc * 8 + k) * per * 16);
+            if (mine && remote) st_async_v4(at, o[4 * k], o[4 * k + 1], o[4 * k + 2], o[4 * k + 3], bar);
+            else if (mine) st_smem_v4(at, o[4 * k], o[4 * k + 1], o[4 * k + 2], o[4 * k + 3]);
+        }
+    }
+    if (mine && cc0 == 0) {
+        const uint32_t at = x.xs_addr() + (uint32_t)(x.chunk * per + rl) * 4;
+        if (remote) {
+            const uint32_t to = map_dsmem(at, (uint32_t)dest);
+            st_async_b32(to, __float_as_uint(ref), bar);
+            st_async_b32(to + kRowTile * 4, __float_as_uint(sum), bar);
+        } else {
+            st_smem_f32(at, ref);
+            st_smem_f32(at + kRowTile * 4, sum);
+        }
+    }
+}
+
+// The finisher adds up the chunks in chunk order (so the result does not depend on timing).  One thread takes
+// one row and 16 output columns at a time: consecutive lanes read consecutive rows of a piece (no bank
+// conflicts) and each writes a whole 32-byte sector.
+template <int NCH, int THREADS>
+__device__ __forceinline__ void merge_rows(const RowExchange& x, int tid) {
     constexpr int kRowsPer = kRowTile / NCH;        // rows this CTA finishes
     const int G = x.bt.Hq / x.bt.Hkv;
-    const int rl = x.tid % kRowsPer;
+    const int rl = tid % kRowsPer;
     const int in_tile = x.chunk * kRowsPer + rl, row = x.rt * x.plan.tile_rows + in_tile;
-    if (in_tile >= x.plan.tile_rows || row >= x.rows) return;      // only rows of the sequence were sent
+    if (!x.has(in_tile)) return;
+    const uint32_t xs = x.xs_addr();
     float w[NCH];
     float M = -INFINITY;
 #pragma unroll
     for (int c = 0; c < NCH; ++c) {
-        const bool live = (c == NCH - 1) || (c * x.tpc < x.tiles_total);       // that chunk had key tiles
-        w[c] = live ? ld_smem_f32(x.xs_addr + (c * kRowsPer + rl) * 4) : -INFINITY;
+        w[c] = x.live(c) ? ld_smem_f32(xs + (c * kRowsPer + rl) * 4) : -INFINITY;
         M = fmaxf(M, w[c]);
     }
     float den = 0.f;
@@ -138,20 +238,20 @@ __device__ __forceinline__ void merge_rows(const MergeCtx& x) {
     for (int c = 0; c < NCH; ++c) {
         if (w[c] == -INFINITY) { w[c] = 0.f; continue; }
         w[c] = ex2_approx(w[c] - M);
-        den = fmaf(w[c], ld_smem_f32(x.xs_addr + (kRowTile + c * kRowsPer + rl) * 4), den);
+        den = fmaf(w[c], ld_smem_f32(xs + (kRowTile + c * kRowsPer + rl) * 4), den);
     }
     const float inv = __frcp_rn(den);
-    const int node = row / G, g = row - node * G;
+    const int node = x.plan.node_of(row), g = row - node * G;
     const size_t orow = ((size_t)x.b * x.bt.T_max + node) * x.bt.Hq + x.kvh * G + g;
-    if (x.lse && x.tid < kRowsPer) x.lse[orow] = (M + __log2f(den)) * 0.6931471805599453f;
+    if (x.ly.lse && tid < kRowsPer) x.ly.lse[orow] = (M + __log2f(den)) * 0.6931471805599453f;
 #pragma unroll
-    for (int cg = x.tid / kRowsPer; cg < 8; cg += kRowTile / kRowsPer) {       // 16 columns: pieces 4 cg .. + 3
+    for (int cg = tid / kRowsPer; cg < 8; cg += THREADS / kRowsPer) {       // 16 columns: pieces 4 cg .. + 3
         float4 acc[4];
 #pragma unroll
         for (int p = 0; p < 4; ++p) acc[p] = make_float4(0.f, 0.f, 0.f, 0.f);
 #pragma unroll
         for (int c = 0; c < NCH; ++c) {
-            if (!((c == NCH - 1) || (c * x.tpc < x.tiles_total))) continue;    // (nothing was written there)
+            if (!x.live(c)) continue;                                  // (nothing was written there)
 #pragma unroll
             for (int p = 0; p < 4; ++p) {
                 const float4 v = ld_smem_v4(x.xo_addr + (uint32_t)(((c * 32 + cg * 4 + p) * kRowsPer + rl) * 16));
@@ -167,15 +267,42 @@ __device__ __forceinline__ void merge_rows(const MergeCtx& x) {
             o[2 * p] = *reinterpret_cast<const uint32_t*>(&h0);
             o[2 * p + 1] = *reinterpret_cast<const uint32_t*>(&h1);
         }
-        uint4* dst = reinterpret_cast<uint4*>(x.out + orow * kD + cg * 16);
+        uint4* dst = reinterpret_cast<uint4*>(x.ly.out + orow * kD + cg * 16);
         dst[0] = make_uint4(o[0], o[1], o[2], o[3]);
         dst[1] = make_uint4(o[4], o[5], o[6], o[7]);
     }
 }
 
 // one launch of `z_count` (sequence rank, layer, KV head) groups starting at plan.z0
+template <typename Kernel, typename Layers>
+sd_status launch_attn(Kernel kern, int threads, int smem, const Layers& layers, const sd_batch& bt, float scale,
+                      const AttnPlan& plan, int z_count, int32_t* dev_status, cudaStream_t st) {
+    if (!allow_dynamic_smem(kern, smem)) return SD_ERR_CUDA;
+    cudaLaunchConfig_t cfg = {};
+    cfg.gridDim = dim3(plan.n_chunks, plan.row_tiles, z_count);
+    cfg.blockDim = dim3(threads);
+    cfg.dynamicSmemBytes = smem;
+    cfg.stream = st;
+    cudaLaunchAttribute attr[2];
+    attr[0].id = cudaLaunchAttributeClusterDimension;      // the chunks of one row tile form a cluster
+    attr[0].val.clusterDim.x = plan.n_chunks;
+    attr[0].val.clusterDim.y = 1;
+    attr[0].val.clusterDim.z = 1;
+    // The launch may begin while the kernel before it in the stream is still running (its CTAs take the
+    // SM slots that one frees and do their set-up); the kernel waits for that kernel's completion before
+    // it touches global memory.  Consecutive attention calls - one per layer - overlap their ends this way.
+    attr[1].id = cudaLaunchAttributeProgrammaticStreamSerialization;
+    attr[1].val.programmaticStreamSerializationAllowed = 1;
+    cfg.attrs = attr;
+    cfg.numAttrs = 2;
+    return cuda_ok(cudaLaunchKernelEx(&cfg, kern, layers, bt, scale * kLog2e, plan, dev_status));
+}
 template <int NL>
 sd_status launch_rows1(const AttnLayers<NL>& layers, const sd_batch& bt, float scale, const AttnPlan& plan,
-                       int z_count, int32_t* dev_status, cudaStream_t st);     // one row tile per CTA, 64-key tiles
+                       int z_count, int32_t* dev_status, cudaStream_t st);     // 64-key tiles, two CTAs per SM
+template <int NL>
+sd_status launch_wide(const AttnLayers<NL>& layers, const sd_batch& bt, float scale, const AttnPlan& plan,
+                      int z_count, int32_t* dev_status, cudaStream_t st);      // 128-key tiles, one CTA per SM
+int wide_resident_clusters(int dev, int sms, int n_chunks);
 
 }  // namespace sdv

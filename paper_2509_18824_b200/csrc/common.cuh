@@ -26,6 +26,21 @@ inline bool aligned16(const void* p) { return (reinterpret_cast<uintptr_t>(p) & 
 
 inline sd_status cuda_ok(cudaError_t e) { return e == cudaSuccess ? SD_OK : SD_ERR_CUDA; }
 
+// Opts a kernel into `bytes` of dynamic shared memory, once per kernel and device (the attribute stays set)
+template <typename Kernel>
+inline bool allow_dynamic_smem(Kernel* kern, int bytes) {
+    struct Done { const void* kern; int dev, bytes; };
+    static thread_local Done done[16];                     // (a thread's own, so that no lock is needed)
+    static thread_local int next = 0;
+    int dev = 0;
+    if (cudaGetDevice(&dev) != cudaSuccess) return false;
+    for (const Done& d : done)
+        if (d.kern == reinterpret_cast<const void*>(kern) && d.dev == dev && d.bytes >= bytes) return true;
+    if (cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, bytes) != cudaSuccess) return false;
+    done[next++ % 16] = Done{reinterpret_cast<const void*>(kern), dev, bytes};
+    return true;
+}
+
 // Test hooks, read from the environment at every launch (unset in normal use):
 //   SDV_TEST_WAIT_CYCLES  bound of the kernels' barrier waits in SM cycles (default: about a second)
 //   SDV_TEST_WITHHOLD     1: one role of the tensor-core kernels withholds its first arrival, so that

@@ -85,6 +85,19 @@ __device__ __forceinline__ bool mbar_wait_plain(uint64_t* bar, uint32_t parity, 
     return true;
 }
 
+// The wait for a whole warp in uniform control flow: every lane has seen the phase complete when it returns true.
+__device__ __forceinline__ bool mbar_wait_warp(uint64_t* bar, uint32_t parity, volatile int* abort_flag, long long limit) {
+    if (__all_sync(0xffffffffu, mbar_try_wait(bar, parity))) return true;
+    const long long t0 = clock64();
+    while (true) {
+        if (__all_sync(0xffffffffu, mbar_try_wait(bar, parity))) return true;
+        if (__any_sync(0xffffffffu, *abort_flag != 0 || clock64() - t0 > limit)) {
+            *abort_flag = 1;
+            return false;
+        }
+    }
+}
+
 // ---------------------------------------------------------------- programmatic dependent launch
 // A kernel launched with the programmatic-stream-serialization attribute may start while the kernel
 // before it in the stream still runs: griddep_wait() blocks until that kernel has completed and its

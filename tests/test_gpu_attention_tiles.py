@@ -1,0 +1,78 @@
+"""GPU: attention at the edges of the 128-key tiles and key chunks (odd and even block counts, half tiles,
+sequences of one batch cut into different numbers of chunks), and scores that rise so far above the first
+tile's that the rows' reference has to be raised, through both kernels."""
+import numpy as np
+import pytest
+import torch
+
+import oracle
+from paper_2509_18824_b200 import binding as sd
+from paper_2509_18824_b200 import workloads as wl
+from paper_2509_18824_b200.step import to_device
+from helpers import Tiny
+from gpu_util import gpu_attention, check_attention
+
+pytestmark = pytest.mark.gpu
+
+
+def problem(seed, lens, T=19, Hq=14, Hkv=2, gain=3.0):
+    g = np.random.default_rng(seed)
+    B = len(lens)
+    par = np.stack([np.array([-1] + [int(g.integers(0, i)) for i in range(1, T)]) for _ in range(B)])
+    return Tiny(seed, B=B, T=T, Hq=Hq, Hkv=Hkv, D=128, lens=lens, parents=par, gain=gain)
+
+
+@pytest.mark.parametrize("chunks", [0, 1, 2, 4, 8])
+@pytest.mark.parametrize("lens", [(0, 64, 129), (128, 127, 385), (640, 511, 1), (1023, 257, 130), (1409, 1024, 66)])
+def test_tile_and_chunk_edges(monkeypatch, lens, chunks):
+    """19 nodes x 7 heads = a row tile of 126 rows and one of 7."""
+    monkeypatch.setenv("SDV_TEST_CHUNKS", str(chunks))
+    p = problem(sum(lens), lens)
+    p.n_nodes = np.array([19, 18, 5], dtype=np.int32)
+    out, lse, status = gpu_attention(p)
+    assert status == 0
+    ref, rlse = oracle.attention(oracle.Geometry.of(p), p.k_cache, p.v_cache, p.q, p.k_tree, p.v_tree, p.scale)
+    ok = np.isfinite(rlse)
+    check_attention(out[ok], ref[ok], f"lens={lens} chunks={chunks}")
+    np.testing.assert_allclose(lse[ok], rlse[ok], rtol=2e-3, atol=2e-3)
+    for b in range(3):
+        assert (out[b, p.n_nodes[b]:] == 0).all() and (lse[b, p.n_nodes[b]:] == 0).all()
+
+
+def rising(seed):
+    """Keys that grow from block to block: the scores of later tiles lie hundreds of powers of two above the
+    first tile's."""
+    p = problem(seed, (900, 333, 1000), T=12, Hq=8, Hkv=2, gain=1.0)
+    for b in range(p.B):
+        for j in range(int(p.len[b]) // 64 + 1):
+            blk = p.block_table[b, j]
+            x = wl.bf16_bits_to_f32(p.k_cache[blk]) * np.float32(1.0 + 60.0 * ((j * 5) % 8))
+            p.k_cache[blk] = wl.f32_to_bf16_bits(x)
+    return p
+
+
+@pytest.mark.parametrize("layers", [1, 40])
+def test_reference_is_raised(layers):
+    """One layer runs the 128-key kernel, forty layers of this size the 64-key kernel."""
+    p = rising(77)
+    ref, rlse = oracle.attention(oracle.Geometry.of(p), p.k_cache, p.v_cache, p.q, p.k_tree, p.v_tree, p.scale)
+    if layers == 1:
+        out, lse, status = gpu_attention(p)
+        outs, lses = [out], [lse]
+    else:
+        bt, st = sd.Batch.of(p), sd.new_status()
+        sd.sd_tree_prepare(bt, st)
+        kc, vc, q, kt, vt = (to_device(x) for x in (p.k_cache, p.v_cache, p.q, p.k_tree, p.v_tree))
+        o = [torch.full((p.B, p.T_max, p.Hq, p.D), 7.0, dtype=torch.bfloat16, device="cuda") for _ in range(layers)]
+        ls = [torch.zeros((p.B, p.T_max, p.Hq), dtype=torch.float32, device="cuda") for _ in range(layers)]
+        ws = torch.empty(sd.sd_workspace_bytes(bt), dtype=torch.uint8, device="cuda")
+        sd.sd_verify_attention_layers(bt, sd.AttentionLayerSet([kc] * layers, [vc] * layers, [q] * layers, [kt] * layers,
+                                                               [vt] * layers, o, ls), float(p.scale), ws, st)
+        torch.cuda.synchronize()
+        status = int(st.item())
+        outs, lses = [x.float().cpu().numpy() for x in (o[0], o[-1])], [x.cpu().numpy() for x in (ls[0], ls[-1])]
+    assert status == 0
+    for out, lse in zip(outs, lses):
+        rel = np.linalg.norm(out - ref) / np.linalg.norm(ref)
+        assert rel <= 2e-2, rel
+        np.testing.assert_allclose(lse, rlse, rtol=2e-3, atol=2e-3)
