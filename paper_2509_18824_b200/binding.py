@@ -1,8 +1,9 @@
-"""ctypes binding of libsdverify.so: same names as the C header, argument
-marshalling only.  Tensors are torch CUDA tensors (device memory and streams
-are all torch is used for); every step of the computation runs in the
-library's kernels.  There is no CPU fallback: if the shared library cannot be
-loaded, importing this module raises.
+"""Binding of libsdverify.so: same names as the C header, argument
+marshalling only (in native code, csrc/native_calls.cpp; the plain ctypes
+handle of the library is `lib`).  Tensors are torch CUDA tensors (device memory
+and streams are all torch is used for); every step of the computation runs in
+the library's kernels.  There is no CPU fallback: if the shared libraries
+cannot be loaded, importing this module raises.
 """
 from __future__ import annotations
 
@@ -14,6 +15,7 @@ import torch
 
 _HERE = os.path.dirname(os.path.abspath(__file__))
 LIB_PATH = os.path.join(_HERE, "libsdverify.so")
+NATIVE_PATH = os.path.join(_HERE, "_sdnative.so")
 
 SD_OK = 0
 SD_ERR_INVALID_ARG = -1
@@ -49,7 +51,7 @@ class sd_batch(C.Structure):
 
 
 def _load(path: str = LIB_PATH) -> C.CDLL:
-    if path == LIB_PATH and not os.path.exists(LIB_PATH):
+    if path == LIB_PATH and not (os.path.exists(LIB_PATH) and os.path.exists(NATIVE_PATH)):
         from . import build as _build          # needs nvcc; raises if it fails
         _build.build()
     lib = C.CDLL(path)
@@ -119,6 +121,7 @@ def _load(path: str = LIB_PATH) -> C.CDLL:
 
 
 lib = _load()
+from . import _sdnative as _n      # noqa: E402  (linked to the library loaded above)
 
 
 class SdError(RuntimeError):
@@ -149,12 +152,7 @@ def _ptr(t) -> Optional[int]:
     return t.data_ptr()
 
 
-def _stream(stream) -> int:
-    if stream is None:
-        return torch.cuda.current_stream().cuda_stream
-    if isinstance(stream, int):
-        return stream
-    return stream.cuda_stream
+_at = C.addressof          # address of a host structure or array
 
 
 class Batch:
@@ -200,16 +198,20 @@ def sd_workspace_bytes(batch: Optional[Batch], M: int = 0, V: int = 0) -> int:
     return int(lib.sd_workspace_bytes(batch.ref() if batch is not None else None, int(M), int(V)))
 
 
+def _lm_sizes(hidden, W):
+    M, Hd = hidden.size(0), hidden.size(1)
+    assert hidden.dim() == 2 and W.size(1) == Hd
+    return M, Hd, W.size(0)
+
+
 def sd_tree_prepare(batch: Batch, status: torch.Tensor, stream=None) -> None:
-    _check(lib.sd_tree_prepare(batch.ref(), _ptr(status), _stream(stream)))
+    _check(_n.sd_tree_prepare(_at(batch.c), status, stream))
 
 
 def sd_verify_attention(batch: Batch, cache: sd_kv_layer, q, k_tree, v_tree, scale: float,
                         out, lse, workspace, status, stream=None) -> None:
-    _check(lib.sd_verify_attention(batch.ref(), C.byref(cache), _ptr(q), _ptr(k_tree), _ptr(v_tree),
-                                   C.c_float(scale), _ptr(out), _ptr(lse), _ptr(workspace),
-                                   workspace.numel() * workspace.element_size(), _ptr(status),
-                                   _stream(stream)))
+    _check(_n.sd_verify_attention(_at(batch.c), _at(cache), q, k_tree, v_tree, scale, out, lse, workspace, workspace,
+                                  status, stream))
 
 
 class AttentionLayerSet:
@@ -230,35 +232,26 @@ class AttentionLayerSet:
 
 def sd_verify_attention_layers(batch: Batch, layers: AttentionLayerSet, scale: float, workspace, status,
                                stream=None) -> None:
-    _check(lib.sd_verify_attention_layers(batch.ref(), layers.caches, layers.L, layers.q, layers.kt, layers.vt,
-                                          C.c_float(scale), layers.out, layers.lse, _ptr(workspace),
-                                          workspace.numel() * workspace.element_size(), _ptr(status),
-                                          _stream(stream)))
+    _check(_n.sd_verify_attention_layers(_at(batch.c), _at(layers.caches), layers.L, _at(layers.q), _at(layers.kt),
+                                         _at(layers.vt), scale, _at(layers.out), None if layers.lse is None else _at(layers.lse),
+                                         workspace, workspace, status, stream))
 
 
 def sd_lmhead_argmax(hidden, W, argmax, maxlogit, workspace, status, stream=None) -> None:
-    M, Hd = hidden.shape
-    V = W.shape[0]
-    assert W.shape[1] == Hd
-    _check(lib.sd_lmhead_argmax(_ptr(hidden), _ptr(W), int(M), int(Hd), int(V), _ptr(argmax),
-                                _ptr(maxlogit), _ptr(workspace),
-                                workspace.numel() * workspace.element_size(), _ptr(status), _stream(stream)))
+    M, Hd, V = _lm_sizes(hidden, W)
+    _check(_n.sd_lmhead_argmax(hidden, W, M, Hd, V, argmax, maxlogit, workspace, workspace, status, stream))
 
 
 def sd_lmhead_argmax_static(hidden, W, argmax, maxlogit, status, stream=None) -> None:
     """LM-head arg-max using the scratch table built into the library: for callers
     that may not allocate device memory.  At most 512 rows per call."""
-    M, Hd = hidden.shape
-    V = W.shape[0]
-    assert W.shape[1] == Hd
-    _check(lib.sd_lmhead_argmax_static(_ptr(hidden), _ptr(W), int(M), int(Hd), int(V), _ptr(argmax),
-                                       _ptr(maxlogit), _ptr(status), _stream(stream)))
+    M, Hd, V = _lm_sizes(hidden, W)
+    _check(_n.sd_lmhead_argmax_static(hidden, W, M, Hd, V, argmax, maxlogit, status, stream))
 
 
 def sd_accept_tree(batch: Batch, draft_tok, target_argmax, n_acc, path, out_tok, new_len,
                    status, stream=None) -> None:
-    _check(lib.sd_accept_tree(batch.ref(), _ptr(draft_tok), _ptr(target_argmax), _ptr(n_acc), _ptr(path),
-                              _ptr(out_tok), _ptr(new_len), _ptr(status), _stream(stream)))
+    _check(_n.sd_accept_tree(_at(batch.c), draft_tok, target_argmax, n_acc, path, out_tok, new_len, status, stream))
 
 
 class LayerSet:
@@ -275,21 +268,19 @@ class LayerSet:
 
 
 def sd_compact_kv(batch: Batch, layers: LayerSet, n_acc, path, status, stream=None) -> None:
-    _check(lib.sd_compact_kv(batch.ref(), layers.layers, layers.L, layers.kt, layers.vt,
-                             _ptr(n_acc), _ptr(path), _ptr(status), _stream(stream)))
+    _check(_n.sd_compact_kv(_at(batch.c), _at(layers.layers), layers.L, _at(layers.kt), _at(layers.vt), n_acc, path,
+                            status, stream))
 
 
 def sd_lmhead_accept_compact(batch: Batch, hidden, W, draft_tok, layers: LayerSet, argmax, maxlogit,
                              n_acc, path, out_tok, new_len, workspace, status, stream=None) -> None:
     """LM-head arg-max over the B * T_max rows of `hidden`, greedy acceptance and KV compaction in all
     layers; the three steps share one tail kernel."""
-    M, Hd = hidden.shape
-    V = W.shape[0]
-    assert W.shape[1] == Hd and M == batch.B * batch.T_max
-    _check(lib.sd_lmhead_accept_compact(batch.ref(), _ptr(hidden), _ptr(W), int(Hd), int(V), _ptr(draft_tok),
-                                        layers.layers, layers.L, layers.kt, layers.vt, _ptr(argmax), _ptr(maxlogit),
-                                        _ptr(n_acc), _ptr(path), _ptr(out_tok), _ptr(new_len), _ptr(workspace),
-                                        workspace.numel() * workspace.element_size(), _ptr(status), _stream(stream)))
+    M, Hd, V = _lm_sizes(hidden, W)
+    assert M == batch.B * batch.T_max
+    _check(_n.sd_lmhead_accept_compact(_at(batch.c), hidden, W, Hd, V, draft_tok, _at(layers.layers), layers.L,
+                                       _at(layers.kt), _at(layers.vt), argmax, maxlogit, n_acc, path, out_tok,
+                                       new_len, workspace, workspace, status, stream))
 
 
 def group_stats_shape(M: int, V: int):
@@ -301,24 +292,18 @@ def sd_lmhead_stats(hidden, W, inv_temp: float, argmax, maxlogit, lse, workspace
                     group_stats=None) -> None:
     """LM-head arg-max plus lse[r] = log sum_v exp(logit[r][v] * inv_temp); optionally the per-group
     (maximum, sum) table that lets sd_accept_tree_sampled skip its second pass over W."""
-    M, Hd = hidden.shape
-    V = W.shape[0]
-    assert W.shape[1] == Hd
-    _check(lib.sd_lmhead_stats(_ptr(hidden), _ptr(W), int(M), int(Hd), int(V), C.c_float(inv_temp), _ptr(argmax),
-                               _ptr(maxlogit), _ptr(lse), _ptr(group_stats), _ptr(workspace),
-                               workspace.numel() * workspace.element_size(), _ptr(status), _stream(stream)))
+    M, Hd, V = _lm_sizes(hidden, W)
+    _check(_n.sd_lmhead_stats(hidden, W, M, Hd, V, inv_temp, argmax, maxlogit, lse, group_stats, workspace, workspace,
+                              status, stream))
 
 
 def sd_accept_tree_sampled(batch: Batch, hidden, W, inv_temp: float, lse, draft_tok, u, w,
                            n_acc, path, out_tok, new_len, workspace, status, stream=None, group_stats=None) -> None:
     """Acceptance at a sampling temperature (uniforms u [B,T] and w [B] are inputs)."""
-    M, Hd = hidden.shape
-    V = W.shape[0]
-    assert W.shape[1] == Hd and M == batch.B * batch.T_max
-    _check(lib.sd_accept_tree_sampled(batch.ref(), _ptr(hidden), _ptr(W), int(Hd), int(V), C.c_float(inv_temp),
-                                      _ptr(lse), _ptr(group_stats), _ptr(draft_tok), _ptr(u), _ptr(w), _ptr(n_acc), _ptr(path),
-                                      _ptr(out_tok), _ptr(new_len), _ptr(workspace),
-                                      workspace.numel() * workspace.element_size(), _ptr(status), _stream(stream)))
+    M, Hd, V = _lm_sizes(hidden, W)
+    assert M == batch.B * batch.T_max
+    _check(_n.sd_accept_tree_sampled(_at(batch.c), hidden, W, Hd, V, inv_temp, lse, group_stats, draft_tok, u, w,
+                                     n_acc, path, out_tok, new_len, workspace, workspace, status, stream))
 
 
 def sd_lmhead_stats_logits(hidden, W, inv_temp: float, argmax, maxlogit, lse, logits, workspace, status,
@@ -327,9 +312,8 @@ def sd_lmhead_stats_logits(hidden, W, inv_temp: float, argmax, maxlogit, lse, lo
     M, Hd = hidden.shape
     V = W.shape[0]
     assert W.shape[1] == Hd and tuple(logits.shape) == (M, V) and logits.dtype == torch.float32 and logits.is_contiguous()
-    _check(lib.sd_lmhead_stats_logits(_ptr(hidden), _ptr(W), int(M), int(Hd), int(V), C.c_float(inv_temp), _ptr(argmax),
-                                      _ptr(maxlogit), _ptr(lse), _ptr(logits), _ptr(workspace),
-                                      workspace.numel() * workspace.element_size(), _ptr(status), _stream(stream)))
+    _check(_n.sd_lmhead_stats_logits(hidden, W, M, Hd, V, inv_temp, argmax, maxlogit, lse, logits, workspace,
+                                     workspace, status, stream))
 
 
 def sd_accept_tree_sampled_q(batch: Batch, inv_temp: float, lse, logits, draft_tok, q_rows, u, w,
@@ -339,9 +323,8 @@ def sd_accept_tree_sampled_q(batch: Batch, inv_temp: float, lse, logits, draft_t
     M, V = logits.shape
     assert M == batch.B * batch.T_max and tuple(q_rows.shape) == (batch.B, batch.T_max, V)
     assert logits.dtype == torch.float32 and q_rows.dtype == torch.float32 and logits.is_contiguous() and q_rows.is_contiguous()
-    _check(lib.sd_accept_tree_sampled_q(batch.ref(), int(V), C.c_float(inv_temp), _ptr(lse), _ptr(logits), _ptr(draft_tok),
-                                        _ptr(q_rows), _ptr(u), _ptr(w), _ptr(n_acc), _ptr(path), _ptr(out_tok),
-                                        _ptr(new_len), _ptr(status), _stream(stream)))
+    _check(_n.sd_accept_tree_sampled_q(_at(batch.c), V, inv_temp, lse, logits, draft_tok, q_rows, u, w, n_acc, path,
+                                       out_tok, new_len, status, stream))
 
 
 def sd_accept_chain_sampled(batch: Batch, hidden, W, inv_temp: float, lse, draft_tok, q_tok, q_rows, u, w,
@@ -349,14 +332,11 @@ def sd_accept_chain_sampled(batch: Batch, hidden, W, inv_temp: float, lse, draft
     """Acceptance at a sampling temperature for chains drafted by sampling: q_tok [B,T] the draft's
     probability of every drafted token, q_rows [B,T,V] its distributions (device f32); logits: what
     sd_lmhead_stats_logits kept, or None (the stop rows then go through the LM head once more)."""
-    M, Hd = hidden.shape
-    V = W.shape[0]
-    assert W.shape[1] == Hd and M == batch.B * batch.T_max
+    M, Hd, V = _lm_sizes(hidden, W)
+    assert M == batch.B * batch.T_max
     assert tuple(q_rows.shape) == (batch.B, batch.T_max, V) and q_rows.dtype == torch.float32 and q_rows.is_contiguous()
-    _check(lib.sd_accept_chain_sampled(batch.ref(), _ptr(hidden), _ptr(W), int(Hd), int(V), C.c_float(inv_temp),
-                                       _ptr(lse), _ptr(logits), _ptr(draft_tok), _ptr(q_tok), _ptr(q_rows), _ptr(u), _ptr(w),
-                                       _ptr(n_acc), _ptr(path), _ptr(out_tok), _ptr(new_len), _ptr(workspace),
-                                       workspace.numel() * workspace.element_size(), _ptr(status), _stream(stream)))
+    _check(_n.sd_accept_chain_sampled(_at(batch.c), hidden, W, Hd, V, inv_temp, lse, logits, draft_tok, q_tok, q_rows,
+                                      u, w, n_acc, path, out_tok, new_len, workspace, workspace, status, stream))
 
 
 def sd_lmhead_accept_sampled_compact(batch: Batch, hidden, W, inv_temp: float, draft_tok, u, w, layers: LayerSet,
@@ -364,20 +344,16 @@ def sd_lmhead_accept_sampled_compact(batch: Batch, hidden, W, inv_temp: float, d
                                      stream=None) -> None:
     """LM-head statistics, acceptance at a sampling temperature and KV compaction in all layers: the
     LM-head tiles and one tail kernel."""
-    M, Hd = hidden.shape
-    V = W.shape[0]
-    assert W.shape[1] == Hd and M == batch.B * batch.T_max
-    _check(lib.sd_lmhead_accept_sampled_compact(batch.ref(), _ptr(hidden), _ptr(W), int(Hd), int(V), C.c_float(inv_temp),
-                                                _ptr(draft_tok), _ptr(u), _ptr(w), layers.layers, layers.L, layers.kt,
-                                                layers.vt, _ptr(lse), _ptr(group_stats), _ptr(n_acc), _ptr(path),
-                                                _ptr(out_tok), _ptr(new_len), _ptr(workspace),
-                                                workspace.numel() * workspace.element_size(), _ptr(status),
-                                                _stream(stream)))
+    M, Hd, V = _lm_sizes(hidden, W)
+    assert M == batch.B * batch.T_max
+    _check(_n.sd_lmhead_accept_sampled_compact(_at(batch.c), hidden, W, Hd, V, inv_temp, draft_tok, u, w,
+                                               _at(layers.layers), layers.L, _at(layers.kt), _at(layers.vt), lse,
+                                               group_stats, n_acc, path, out_tok, new_len, workspace, workspace,
+                                               status, stream))
 
 
 def sd_draft_feature_attention(qp, k, v, H: int, scale: float, out, stream=None) -> None:
     """Meta-query cross-attention core: qp [Q,D], k and v [S,L,D], out [S,Q,D]; D = H * 128."""
     Q, D = qp.shape
     S, L, _ = k.shape
-    _check(lib.sd_draft_feature_attention(_ptr(qp), _ptr(k), _ptr(v), int(S), int(L), int(Q), int(H), int(D),
-                                          C.c_float(scale), _ptr(out), _stream(stream)))
+    _check(_n.sd_draft_feature_attention(qp, k, v, S, L, Q, H, D, scale, out, stream))

@@ -1,4 +1,4 @@
-"""Builds libsdverify.so (sm_100a) next to this file with nvcc."""
+"""Builds libsdverify.so (sm_100a, nvcc) and its Python entry points _sdnative.so (g++) next to this file."""
 from __future__ import annotations
 
 import os
@@ -11,6 +11,7 @@ CSRC = os.path.join(HERE, "csrc")
 INCLUDE = os.path.join(os.path.dirname(HERE), "include")
 OBJ = os.path.join(HERE, "_build")
 LIB = os.path.join(HERE, "libsdverify.so")
+NATIVE = os.path.join(HERE, "_sdnative.so")
 SOURCES = ["api.cu", "tree.cu", "compact.cu", "attention.cu", "attention_wide.cu", "lmhead.cu", "sampled.cu", "draft.cu", "tmap.cu"]
 NVCC_FLAGS = ["-gencode", "arch=compute_100a,code=sm_100a", "-lineinfo", "-O3", "-std=c++17",
               "-Xcompiler", "-fPIC", "-I", INCLUDE, "-I", CSRC]
@@ -53,7 +54,33 @@ def build(force: bool = False, verbose: bool = False) -> str:
         tmp = LIB + f".{os.getpid()}.tmp"
         subprocess.check_call([_nvcc(), "-shared", "-o", tmp] + objs + ["-gencode", "arch=compute_100a,code=sm_100a"])
         os.replace(tmp, LIB)
+    build_native(force)
     return LIB
+
+
+def build_native(force: bool = False) -> str:
+    """The Python entry points, compiled against torch's headers and linked to LIB."""
+    src = os.path.join(CSRC, "native_calls.cpp")
+    header = os.path.join(INCLUDE, "sdverify.h")
+    if not force and not _stale(NATIVE, [src, header]):
+        return NATIVE
+    import sysconfig
+
+    import torch
+    troot = os.path.dirname(torch.__file__)
+    cuda = os.path.dirname(os.path.dirname(_nvcc())) if os.sep in _nvcc() else "/usr/local/cuda"
+    tmp = NATIVE + f".{os.getpid()}.tmp"
+    cmd = ["g++", "-O2", "-std=c++17", "-shared", "-fPIC", f"-D_GLIBCXX_USE_CXX11_ABI={int(torch._C._GLIBCXX_USE_CXX11_ABI)}",
+           "-I", INCLUDE, "-I", sysconfig.get_paths()["include"], "-I", os.path.join(cuda, "include"),
+           "-I", os.path.join(troot, "include"), "-I", os.path.join(troot, "include", "torch", "csrc", "api", "include"),
+           src, "-o", tmp, "-L", os.path.join(troot, "lib"), "-lc10", "-lc10_cuda", "-ltorch_cpu", "-ltorch_python",
+           "-L", HERE, "-l:libsdverify.so", "-Wl,-rpath,$ORIGIN"]
+    r = subprocess.run(cmd, capture_output=True, text=True)
+    if r.returncode != 0:
+        sys.stderr.write(r.stdout + r.stderr)
+        raise RuntimeError("g++ failed: " + " ".join(cmd))
+    os.replace(tmp, NATIVE)
+    return NATIVE
 
 
 if __name__ == "__main__":

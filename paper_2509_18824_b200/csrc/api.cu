@@ -1,11 +1,24 @@
 // C-ABI entry points: argument validation, then the kernel launchers.
 #include "common.cuh"
 
+#include <atomic>
 #include <stdlib.h>
 
 using namespace sdv;
 
 namespace sdv {
+int sm_count(int dev) {
+    constexpr int kDevs = 64;
+    static std::atomic<int> cache[kDevs];
+    const bool cached = dev >= 0 && dev < kDevs;
+    if (cached)
+        if (const int v = cache[dev].load(std::memory_order_relaxed)) return v;
+    int sms = 0;
+    if (cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, dev) != cudaSuccess || sms <= 0) return 148;
+    if (cached) cache[dev].store(sms, std::memory_order_relaxed);
+    return sms;
+}
+
 TestKnobs test_knobs() {
     TestKnobs k{1ll << 31, 0, 0};
     if (const char* e = getenv("SDV_TEST_WAIT_CYCLES")) { const long long v = atoll(e); if (v >= 1000) k.wait_cycles = v; }

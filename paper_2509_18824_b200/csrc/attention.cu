@@ -129,8 +129,10 @@ attn_umma_kernel(const __grid_constant__ AttnLayers<NL> layers, const sd_batch b
         tma_load_3d(q_smem, map_q, 0, kvh * G, b * T + rt * plan.tile_nodes, q_full, pol);
         tma_load_3d(q_smem + kRowTile * 128, map_q, 64, kvh * G, b * T + rt * plan.tile_nodes, q_full, pol);
     }
-    const int n = min(max(__ldg(bt.n_nodes + b), 0), T);
-    const int len = max(__ldg(bt.len + b), 0);
+    const int32_t *n_nodes = bt.n_nodes, *lens = bt.len, *tables = bt.block_table;
+    settle(n_nodes); settle(lens); settle(tables);         // (no load of theirs in front of the wait)
+    const int n = min(max(__ldg(n_nodes + b), 0), T);
+    const int len = max(__ldg(lens + b), 0);
     // Rows of this sequence: its own nodes only (rows are node-major, so they are the first n * G).  A tree
     // smaller than T_max pays for the row tiles it fills: the rows behind them only get their zeros.  (A
     // batch of 16 trees of 30 to 60 nodes, T_max = 60: 2.9 of 4 row tiles run.)
@@ -157,7 +159,7 @@ attn_umma_kernel(const __grid_constant__ AttnLayers<NL> layers, const sd_batch b
     // rings and are issued independently, whichever slot frees first: the next K tile (needed early, for
     // the score MMA issued one tile ahead) must not queue behind a V slot that is only released when P.V
     // has finished.  The block table is looked up ahead of its use (the first entries all at once).
-    const int32_t* table = bt.block_table + (size_t)b * bt.max_blocks_per_seq;
+    const int32_t* table = tables + (size_t)b * bt.max_blocks_per_seq;
     const int n_pref = t1 - t0;
     int jk = 0, jv = 0, blk_k = 0, blk_v = 0;
     auto issue = [&](int j, int blk, bool is_v) {
@@ -531,18 +533,6 @@ template sd_status launch_rows1<1>(const AttnLayers<1>&, const sd_batch&, float,
 template sd_status launch_rows1<kMaxLayersPerLaunch>(const AttnLayers<kMaxLayersPerLaunch>&, const sd_batch&, float,
                                                      const AttnPlan&, int, int32_t*, cudaStream_t);
 
-// SM count of the current device (cached per device ordinal)
-static int sm_count() {
-    constexpr int kDevs = 64;
-    static int cache[kDevs];
-    int dev = 0, sms = 0;
-    if (cudaGetDevice(&dev) != cudaSuccess || dev < 0) return 148;
-    if (dev < kDevs && cache[dev] > 0) return cache[dev];
-    if (cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, dev) != cudaSuccess || sms <= 0) sms = 148;
-    if (dev < kDevs) cache[dev] = sms;
-    return sms;
-}
-
 // The chunks of a row tile are merged inside a thread-block cluster, through shared memory:
 // attention needs no global scratch (a nominal size keeps the argument checks uniform).
 size_t attention_workspace_bytes(const sd_batch&) { return 256; }
@@ -636,7 +626,7 @@ static sd_status launch_group(const AttnLayers<NL>& layers, int n_layers, const 
                               int32_t* dev_status, cudaStream_t st) {
     int dev = 0;
     if (cudaGetDevice(&dev) != cudaSuccess) return SD_ERR_CUDA;
-    const int sms = sm_count();
+    const int sms = sm_count(dev);
     const TestKnobs knobs = test_knobs();
     AttnPlan plan = common_plan(bt, n_layers, knobs);
     const int Z = n_layers * bt.B * bt.Hkv;

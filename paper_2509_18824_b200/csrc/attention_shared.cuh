@@ -98,11 +98,13 @@ struct AttnPlan {
 // lookup is done here (up to 64 sequences: each of the first B threads ranks one sequence by cached length,
 // ties by index); larger batches, and launches that fit the GPU in one round, run in index order.
 __device__ __forceinline__ int sequence_of_rank(const sd_batch& bt, int rank, int& s_seq) {
+    const int32_t* lens = bt.len;
+    settle(lens);
     if ((int)threadIdx.x < bt.B) {
-        const int mine = __ldg(bt.len + threadIdx.x);
+        const int mine = __ldg(lens + threadIdx.x);
         int r = 0;
         for (int j = 0; j < bt.B; ++j) {
-            const int other = __ldg(bt.len + j);
+            const int other = __ldg(lens + j);
             r += (other > mine || (other == mine && j < (int)threadIdx.x)) ? 1 : 0;
         }
         if (r == rank) s_seq = threadIdx.x;

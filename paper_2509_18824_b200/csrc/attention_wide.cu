@@ -105,10 +105,12 @@ attn_wide_kernel(const __grid_constant__ AttnLayers<NL> layers, const sd_batch b
         tma_load_3d(q_smem, &ly.q, 0, kvh * G, b * T + rt * plan.tile_nodes, q_full, pol);
         tma_load_3d(q_smem + kRowTile * 128, &ly.q, 64, kvh * G, b * T + rt * plan.tile_nodes, q_full, pol);
     }
-    const int n = min(max(__ldg(bt.n_nodes + b), 0), T);
-    const int len = max(__ldg(bt.len + b), 0);
+    const int32_t *n_nodes = bt.n_nodes, *lens = bt.len, *tables = bt.block_table;
+    settle(n_nodes); settle(lens); settle(tables);         // (no load of theirs in front of the wait)
+    const int n = min(max(__ldg(n_nodes + b), 0), T);
+    const int len = max(__ldg(lens + b), 0);
     const int t0_guess = chunk_range(len_guess, bt.max_blocks_per_seq, chunks_of(min((len_guess + kBlock - 1) / kBlock, bt.max_blocks_per_seq), plan.n_chunks, plan.chunk_blocks), chunk).t0;
-    const int32_t* const seq_table = bt.block_table + (size_t)b * bt.max_blocks_per_seq;
+    const int32_t* const seq_table = tables + (size_t)b * bt.max_blocks_per_seq;
     int even = 0, odd = 0;                                 // block table of this chunk (producer warp)
     if (warp == kWTmaWarp) {
         if (t0_guess + lane < bt.max_blocks_per_seq) even = __ldg(seq_table + t0_guess + lane);

@@ -26,6 +26,9 @@ inline bool aligned16(const void* p) { return (reinterpret_cast<uintptr_t>(p) & 
 
 inline sd_status cuda_ok(cudaError_t e) { return e == cudaSuccess ? SD_OK : SD_ERR_CUDA; }
 
+// SM count of device `dev` (asked once per device)
+int sm_count(int dev);
+
 // Opts a kernel into `bytes` of dynamic shared memory, once per kernel and device (the attribute stays set)
 template <typename Kernel>
 inline bool allow_dynamic_smem(Kernel* kern, int bytes) {
@@ -39,6 +42,43 @@ inline bool allow_dynamic_smem(Kernel* kern, int bytes) {
     if (cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, bytes) != cudaSuccess) return false;
     done[next++ % 16] = Done{reinterpret_cast<const void*>(kern), dev, bytes};
     return true;
+}
+
+// Launch that may start while the kernel before it in the stream still runs (programmatic dependent launch):
+// the kernel does its set-up and then waits (griddep_wait) for that kernel's completion before it reads or
+// writes global memory; every kernel of the library does, so an order of three launches stays an order.
+// cluster: CTAs per cluster along x.
+template <typename... P, typename... A>
+inline sd_status launch_dependent(void (*kern)(P...), dim3 grid, int threads, size_t smem, int cluster, cudaStream_t st, A... args) {
+    cudaLaunchConfig_t cfg = {};
+    cfg.gridDim = grid;
+    cfg.blockDim = dim3(threads);
+    cfg.dynamicSmemBytes = smem;
+    cfg.stream = st;
+    cudaLaunchAttribute attr[2];
+    attr[0].id = cudaLaunchAttributeProgrammaticStreamSerialization;
+    attr[0].val.programmaticStreamSerializationAllowed = 1;
+    attr[1].id = cudaLaunchAttributeClusterDimension;
+    attr[1].val.clusterDim.x = cluster;
+    attr[1].val.clusterDim.y = 1;
+    attr[1].val.clusterDim.z = 1;
+    cfg.attrs = attr;
+    cfg.numAttrs = cluster > 1 ? 2 : 1;
+    return cuda_ok(cudaLaunchKernelEx(&cfg, kern, static_cast<P>(args)...));
+}
+
+// Start of such a kernel's work on global memory.  The pointers pass through the asm so that no load from
+// them, read-only ones included, can be moved in front of the wait.
+template <typename Ptr>
+__device__ __forceinline__ void settle(Ptr& p) { asm volatile("" : "+l"(p)); }
+__device__ __forceinline__ void settle(sd_batch& bt) {
+    settle(bt.block_table); settle(bt.len); settle(bt.n_nodes); settle(bt.parents); settle(bt.anc_mask);
+}
+template <typename... T>
+__device__ __forceinline__ void begin_dependent(T&... p) {
+    asm volatile("griddepcontrol.launch_dependents;" ::: "memory");
+    asm volatile("griddepcontrol.wait;" ::: "memory");
+    (settle(p), ...);
 }
 
 // Test hooks, read from the environment at every launch (unset in normal use):

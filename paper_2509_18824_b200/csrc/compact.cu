@@ -10,6 +10,7 @@ __global__ void __launch_bounds__(256)
 compact_kernel(sd_batch bt, const __grid_constant__ CompactLayers ly,
                const int32_t* __restrict__ n_acc, const int32_t* __restrict__ path,
                int32_t* status) {
+    begin_dependent(bt, n_acc, path);
     const int b = blockIdx.x;
     const int na = min(n_acc[b], bt.T_max);
     compact_sequence(bt, ly, blockIdx.y, 1, b, na, path + (size_t)b * bt.T_max, threadIdx.x, blockDim.x, status);
@@ -33,9 +34,7 @@ sd_status launch_compact(const sd_batch& bt, const sd_kv_layer* layers, int L,
         const int nl = (L - l0 < kLayersPerLaunch) ? (L - l0) : kLayersPerLaunch;
         CompactLayers ly;
         fill_compact_layers(&ly, layers, kt, vt, l0, nl);
-        dim3 grid(bt.B, nl);
-        compact_kernel<<<grid, 256, 0, st>>>(bt, ly, n_acc, path, dev_status);
-        sd_status s = cuda_ok(cudaGetLastError());
+        const sd_status s = launch_dependent(compact_kernel, dim3(bt.B, nl), 256, 0, 1, st, bt, ly, n_acc, path, dev_status);
         if (s != SD_OK) return s;
     }
     return SD_OK;

@@ -33,6 +33,7 @@ draft_feature_attention_kernel(const uint16_t* __restrict__ qp, const uint16_t* 
                                const uint16_t* __restrict__ v, int S, int L, int Q, int H, float scale,
                                uint16_t* __restrict__ out) {
     extern __shared__ __align__(16) uint8_t dsm[];
+    begin_dependent(qp, k, v, out);
     const int D = H * kDh;
     uint16_t* qs = reinterpret_cast<uint16_t*>(dsm);                                // [Q][D] meta queries
     const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
@@ -157,21 +158,16 @@ sd_status launch_draft_feature_attention(const void* qp, const void* k, const vo
     const int D = H * kDh;
     const size_t smem = (((size_t)Q * D * 2 + 15) & ~(size_t)15) + (size_t)kDraftWarps * kVTile;
     if (smem > 200 * 1024) return SD_ERR_UNSUPPORTED;
-    int dev = 0, sms = 0;
-    if (cudaGetDevice(&dev) != cudaSuccess ||
-        cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, dev) != cudaSuccess)
-        return SD_ERR_CUDA;
+    int dev = 0;
+    if (cudaGetDevice(&dev) != cudaSuccess) return SD_ERR_CUDA;
+    const int sms = sm_count(dev);
     const long long tasks = (long long)S * H;
     const long long want = (tasks + kDraftWarps - 1) / kDraftWarps;
     const long long cap = (long long)sms * 6;                        // resident CTAs, grid-stride beyond
     const int grid = (int)(want < cap ? want : cap);
     auto kern = (k == v) ? draft_feature_attention_kernel<true> : draft_feature_attention_kernel<false>;
-    if (cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem) != cudaSuccess)
-        return SD_ERR_CUDA;
-    kern<<<grid, kDraftWarps * 32, smem, st>>>(
-        static_cast<const uint16_t*>(qp), static_cast<const uint16_t*>(k), static_cast<const uint16_t*>(v), S, L, Q, H, scale,
-        static_cast<uint16_t*>(out));
-    return cuda_ok(cudaGetLastError());
+    if (!allow_dynamic_smem(kern, (int)smem)) return SD_ERR_CUDA;
+    return launch_dependent(kern, dim3(grid), kDraftWarps * 32, smem, 1, st, qp, k, v, S, L, Q, H, scale, out);
 }
 
 }  // namespace sdv

@@ -317,6 +317,7 @@ lmhead_umma_kernel(const __grid_constant__ CUtensorMap tmW, const __grid_constan
     __syncthreads();
     tc_fence_after_sync();
     const uint32_t tmem_base = tmem_base_slot;
+    griddep_wait();                    // set-up done: global memory from here on
 
     if (warp == kTmaWarpLm) {
         // ------------------------------------------------ TMA producer
@@ -461,6 +462,7 @@ lmhead_umma_pair_kernel(const __grid_constant__ CUtensorMap tmW, const __grid_co
     cluster_wait_acquire();
     tc_fence_after_sync();
     const uint32_t tmem_base = tmem_base_slot;
+    griddep_wait();                    // set-up done: global memory from here on
 
     if (warp == kTmaWarpLm) {
         // ------------------------------------------------ TMA producer (one per CTA)
@@ -557,19 +559,19 @@ lmhead_umma_pair_kernel(const __grid_constant__ CUtensorMap tmW, const __grid_co
     }
 }
 
-// one thread per hidden row: merge the per-CTA candidates (lowest index on ties)
-__global__ void lmhead_merge_kernel(const int32_t* __restrict__ part_key, const int32_t* __restrict__ part_idx,
+// merge of the per-CTA candidates (lowest index on ties), eight threads per hidden row
+__global__ void __launch_bounds__(256)
+lmhead_merge_kernel(const int32_t* __restrict__ part_key, const int32_t* __restrict__ part_idx,
                                     int n_ctas, int rows, int row0, int32_t* __restrict__ argmax,
                                     float* __restrict__ maxlogit) {
-    const int col = blockIdx.x * blockDim.x + threadIdx.x;
-    if (col >= rows) return;
-    int32_t k = INT32_MIN, i = 0x7fffffff;
-    for (int c = 0; c < n_ctas; ++c) {
-        const int32_t k2 = part_key[(size_t)c * kMaxCols + col], i2 = part_idx[(size_t)c * kMaxCols + col];
-        if (k2 > k || (k2 == k && i2 < i)) { k = k2; i = i2; }
+    begin_dependent(part_key, part_idx);
+    const int col = blockIdx.x * 32 + (threadIdx.x >> 3), sub = threadIdx.x & 7;
+    int32_t k, i;
+    merge_row_argmax(part_key, part_idx, n_ctas, kMaxCols, col, col < rows, sub, k, i);
+    if (col < rows && sub == 0) {
+        argmax[row0 + col] = i;
+        if (maxlogit) maxlogit[row0 + col] = key_to_float(k);
     }
-    argmax[row0 + col] = i;
-    if (maxlogit) maxlogit[row0 + col] = key_to_float(k);
 }
 
 // the same merge plus log sum exp(logit / temperature) of every hidden row (natural log);
@@ -579,6 +581,7 @@ lmhead_merge_stats_kernel(const int32_t* __restrict__ part_key, const int32_t* _
                           const float* __restrict__ part_ref, const float* __restrict__ part_sum,
                           int n_ctas, int rows, int row0, float c2, int32_t* __restrict__ argmax,
                           float* __restrict__ maxlogit, float* __restrict__ lse) {
+    begin_dependent(part_key, part_idx, part_ref, part_sum);
     const int col = blockIdx.x * 32 + (threadIdx.x >> 3), sub = threadIdx.x & 7;
     int32_t k, i;
     const float row_lse = merge_row_stats(part_key, part_idx, part_ref, part_sum, n_ctas, kMaxCols, col, col < rows, sub, c2, k, i);
@@ -601,10 +604,9 @@ static sd_status launch_lmhead_impl(const void* hidden, const void* W, int M, in
                                     float* group_stats = nullptr, float* logit_out = nullptr) {
     if (ws_bytes < (lse ? stats_workspace_bytes(M, V) : lmhead_workspace_bytes(M, V))) return SD_ERR_WORKSPACE;
     if (tiles_only_ctas && M > kMaxCols) return SD_ERR_UNSUPPORTED;
-    int dev = 0, sms = 0;
-    if (cudaGetDevice(&dev) != cudaSuccess ||
-        cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, dev) != cudaSuccess)
-        return SD_ERR_CUDA;
+    int dev = 0;
+    if (cudaGetDevice(&dev) != cudaSuccess) return SD_ERR_CUDA;
+    const int sms = sm_count(dev);
 
     const int n_blocks = (M + kMaxCols - 1) / kMaxCols;
     const int rows_per_block = round_up((M + n_blocks - 1) / n_blocks, 16);
@@ -671,41 +673,27 @@ static sd_status launch_lmhead_impl(const void* hidden, const void* W, int M, in
             }
             auto kern = (bk == 64) ? (p.n_parts == 2 ? lmhead_umma_pair_kernel<64, 2> : lmhead_umma_pair_kernel<64, 1>)
                                    : (p.n_parts == 2 ? lmhead_umma_pair_kernel<32, 2> : lmhead_umma_pair_kernel<32, 1>);
-            if (cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)dyn) != cudaSuccess)
-                return SD_ERR_CUDA;
-            cudaLaunchConfig_t cfg = {};
-            cfg.gridDim = dim3(grid);
-            cfg.blockDim = dim3(kLmThreads);
-            cfg.dynamicSmemBytes = dyn;
-            cfg.stream = st;
-            cudaLaunchAttribute attr[1];
-            attr[0].id = cudaLaunchAttributeClusterDimension;
-            attr[0].val.clusterDim.x = 2;
-            attr[0].val.clusterDim.y = 1;
-            attr[0].val.clusterDim.z = 1;
-            cfg.attrs = attr;
-            cfg.numAttrs = 1;
-            if (cudaLaunchKernelEx(&cfg, kern, tmW, tmH, p, dev_status) != cudaSuccess) return SD_ERR_CUDA;
+            if (!allow_dynamic_smem(kern, (int)dyn)) return SD_ERR_CUDA;
+            const sd_status ls = launch_dependent(kern, dim3(grid), kLmThreads, dyn, 2, st, tmW, tmH, p, dev_status);
+            if (ls != SD_OK) return ls;
         } else {
             if (grid > p.n_tiles) grid = p.n_tiles;
             auto kern = (bk == 64) ? lmhead_umma_kernel<64> : lmhead_umma_kernel<32>;
-            if (cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)dyn) != cudaSuccess)
-                return SD_ERR_CUDA;
-            kern<<<grid, kLmThreads, dyn, st>>>(tmW, tmH, p, dev_status);
-            if (cudaGetLastError() != cudaSuccess) return SD_ERR_CUDA;
+            if (!allow_dynamic_smem(kern, (int)dyn)) return SD_ERR_CUDA;
+            const sd_status ls = launch_dependent(kern, dim3(grid), kLmThreads, dyn, 1, st, tmW, tmH, p, dev_status);
+            if (ls != SD_OK) return ls;
         }
         if (tiles_only_ctas) {
             *tiles_only_ctas = grid;
             return SD_OK;
         }
         if (mass_out) continue;                      // nothing to merge: the epilogue stored the probabilities
-        if (lse)
-            lmhead_merge_stats_kernel<<<(p.rows + 31) / 32, 256, 0, st>>>(p.part_key, p.part_idx, p.part_ref, p.part_sum,
-                                                                           grid, p.rows, p.row0, p.c2, argmax, maxlogit, lse);
-        else
-            lmhead_merge_kernel<<<(p.rows + 127) / 128, 128, 0, st>>>(p.part_key, p.part_idx, grid, p.rows, p.row0,
-                                                                     argmax, maxlogit);
-        if (cudaGetLastError() != cudaSuccess) return SD_ERR_CUDA;
+        const dim3 mgrid((p.rows + 31) / 32);
+        const sd_status ms = lse ? launch_dependent(lmhead_merge_stats_kernel, mgrid, 256, 0, 1, st, p.part_key, p.part_idx, p.part_ref,
+                                                    p.part_sum, grid, p.rows, p.row0, p.c2, argmax, maxlogit, lse)
+                                 : launch_dependent(lmhead_merge_kernel, mgrid, 256, 0, 1, st, p.part_key, p.part_idx, grid, p.rows,
+                                                    p.row0, argmax, maxlogit);
+        if (ms != SD_OK) return ms;
     }
     return SD_OK;
 }
@@ -764,6 +752,7 @@ tail_kernel(sd_batch bt, const __grid_constant__ CompactLayers ly,
     __shared__ int32_t s_target[kMaxT];
     __shared__ int32_t s_path[kMaxT];
     __shared__ int s_na;
+    begin_dependent(bt, part_key, part_idx, draft);
     const int b = blockIdx.x;
     const int layer = blockIdx.y;
     const int T = bt.T_max;
@@ -771,18 +760,8 @@ tail_kernel(sd_batch bt, const __grid_constant__ CompactLayers ly,
     // 1. arg-max of this sequence's rows: eight threads per row, each an eighth of the CTAs' candidates
     for (int row0 = 0; row0 < T; row0 += 32) {
         const int row = row0 + (threadIdx.x >> 3), sub = threadIdx.x & 7;
-        int32_t k = INT32_MIN, i = 0x7fffffff;
-        if (row < T) {
-            const int col = b * T + row;
-#pragma unroll 4
-            for (int c = sub; c < n_ctas; c += 8)
-                take_better(k, i, __ldg(part_key + (size_t)c * kMaxCols + col), __ldg(part_idx + (size_t)c * kMaxCols + col));
-        }
-#pragma unroll
-        for (int d = 1; d <= 4; d <<= 1) {
-            const int32_t k2 = __shfl_xor_sync(0xffffffffu, k, d), i2 = __shfl_xor_sync(0xffffffffu, i, d);
-            take_better(k, i, k2, i2);
-        }
+        int32_t k, i;
+        merge_row_argmax(part_key, part_idx, n_ctas, kMaxCols, b * T + row, row < T, sub, k, i);
         if (row < T && sub == 0) {
             if (writer) {
                 argmax[b * T + row] = i;
@@ -835,9 +814,8 @@ sd_status launch_lmhead_accept_compact(const sd_batch& bt, const void* hidden, c
     const int32_t* part_idx = part_key + (size_t)kMaxCtas * kMaxCols;
     // scratch for the non-writing CTAs' acceptance outputs: behind the candidate tables
     int32_t* scratch = static_cast<int32_t*>(ws) + (size_t)kMaxCtas * kMaxCols * 2;
-    tail_kernel<<<dim3(bt.B, L), 256, 0, st>>>(bt, ly, part_key, part_idx, n_ctas, draft, argmax, maxlogit,
-                                               n_acc, path, out_tok, new_len, dev_status, scratch);
-    return cuda_ok(cudaGetLastError());
+    return launch_dependent(tail_kernel, dim3(bt.B, L), 256, 0, 1, st, bt, ly, part_key, part_idx, n_ctas, draft, argmax, maxlogit,
+                            n_acc, path, out_tok, new_len, dev_status, scratch);
 }
 
 

@@ -131,6 +131,7 @@ __global__ void __launch_bounds__(128)
 child_prob_kernel(sd_batch bt, const uint16_t* __restrict__ hidden, const uint16_t* __restrict__ W, int Hd, int V,
                   float inv_temp, const float* __restrict__ lse, const int32_t* __restrict__ draft,
                   float* __restrict__ p_child, int32_t* status) {
+    begin_dependent(bt, hidden, W, lse, draft);
     const int warp = (blockIdx.x * blockDim.x + threadIdx.x) >> 5, lane = threadIdx.x & 31;
     const int T = bt.T_max;
     if (warp >= bt.B * T) return;
@@ -210,6 +211,7 @@ __global__ void sampled_walk_kernel(sd_batch bt, const int32_t* __restrict__ dra
                                     const float* __restrict__ u, int32_t* n_acc, int32_t* path, int32_t* out_tok,
                                     int32_t* new_len, float* resid, int32_t* stop_row, int32_t* n_excl, int32_t* excl,
                                     float* excl_p, int32_t* status) {
+    begin_dependent(bt, draft, p_child, u);
     const int b = blockIdx.x, lane = threadIdx.x;
     const int T = bt.T_max;
     const WalkOut o{path + (size_t)b * T, out_tok + (size_t)b * T, excl + (size_t)b * 64, excl_p + (size_t)b * 64};
@@ -227,6 +229,7 @@ __global__ void sampled_walk_kernel(sd_batch bt, const int32_t* __restrict__ dra
 __global__ void gather_stop_rows_kernel(const uint16_t* __restrict__ hidden, int Hd, const float* __restrict__ lse,
                                         const int32_t* __restrict__ stop_row, uint16_t* __restrict__ stop_hidden,
                                         float* __restrict__ stop_lse) {
+    begin_dependent(hidden, lse, stop_row);
     const int b = blockIdx.x;
     const int row = stop_row[b];
     const uint4* src = reinterpret_cast<const uint4*>(hidden + (size_t)row * Hd);
@@ -248,6 +251,7 @@ residual_blocksum_kernel(int V, const int32_t* __restrict__ n_excl, const int32_
                          const float* __restrict__ logits, const float* __restrict__ lse, float inv_temp,
                          float* __restrict__ mass, float* __restrict__ block_sum, int n_blocks) {
     __shared__ float s_v[kResBlock];
+    begin_dependent(n_excl, excl, q_rows, stop_row, logits, lse, mass);
     const int b = blockIdx.y;
     const int t = blockIdx.x * kResBlock + threadIdx.x;
     float m = 0.f;
@@ -338,6 +342,7 @@ residual_pick_kernel(sd_batch bt, int V, const float* __restrict__ w, const floa
     __shared__ float s_m[kResBlock];
     __shared__ float s_acc, s_target;
     __shared__ int s_k, s_pick, s_last;
+    begin_dependent(bt, w, mass, block_sum, n_acc);
     const int b = blockIdx.x;
     const int na = n_acc[b];
     if (na < 1 || na > bt.T_max) return;                               // bad tree: already reported
@@ -534,6 +539,7 @@ residual_pick_groups_kernel(sd_batch bt, const uint16_t* __restrict__ hidden, co
                             const float* __restrict__ w, const int32_t* __restrict__ stop_row, const int32_t* __restrict__ n_excl,
                             const int32_t* __restrict__ excl, const float* __restrict__ excl_p, const int32_t* __restrict__ n_acc,
                             int32_t* out_tok, int32_t* status) {
+    begin_dependent(bt, hidden, W, lse, group_stats, w, stop_row, n_excl, excl, excl_p, n_acc);
     const int b = blockIdx.x;
     const int na = n_acc[b];
     if (na < 1 || na > bt.T_max) return;                               // bad tree: already reported
@@ -550,6 +556,7 @@ __global__ void chain_walk_q_kernel(sd_batch bt, const int32_t* __restrict__ dra
                                     const float* __restrict__ q_tok, const float* __restrict__ u, int32_t* n_acc,
                                     int32_t* path, int32_t* out_tok, int32_t* new_len, int32_t* stop_row, int32_t* rejected,
                                     int32_t* status) {
+    begin_dependent(bt, draft, p_child, q_tok, u);
     const int b = blockIdx.x, lane = threadIdx.x;
     const int T = bt.T_max;
     const int n = bt.n_nodes[b];
@@ -607,22 +614,26 @@ sd_status launch_accept_chain_sampled(const sd_batch& bt, const void* hidden, co
     const uint16_t* h = static_cast<const uint16_t*>(hidden);
     const uint16_t* Wp = static_cast<const uint16_t*>(W);
     const int n_blocks = (V + kResBlock - 1) / kResBlock;
-    child_prob_kernel<<<(B * T * 32 + 127) / 128, 128, 0, st>>>(bt, h, Wp, Hd, V, inv_temp, lse, draft, s.p_child, dev_status);
-    chain_walk_q_kernel<<<B, 32, 0, st>>>(bt, draft, s.p_child, q_tok, u, n_acc, path, out_tok, new_len, s.stop_row, s.n_excl,
-                                         dev_status);
+    sd_status r = SD_OK;
+    auto go = [&](sd_status x) { if (r == SD_OK) r = x; };
+    go(launch_dependent(child_prob_kernel, dim3((B * T * 32 + 127) / 128), 128, 0, 1, st, bt, h, Wp, Hd, V, inv_temp, lse, draft,
+                        s.p_child, dev_status));
+    go(launch_dependent(chain_walk_q_kernel, dim3(B), 32, 0, 1, st, bt, draft, s.p_child, q_tok, u, n_acc, path, out_tok, new_len,
+                        s.stop_row, s.n_excl, dev_status));
     if (!logits) {
         // the stop rows' probabilities over the vocabulary: the LM-head kernel once more, in its store mode
-        gather_stop_rows_kernel<<<B, 128, 0, st>>>(h, Hd, lse, s.stop_row, s.stop_hidden, s.stop_lse);
+        go(launch_dependent(gather_stop_rows_kernel, dim3(B), 128, 0, 1, st, h, Hd, lse, s.stop_row, s.stop_hidden, s.stop_lse));
         const sd_status ls = launch_lmhead_mass(s.stop_hidden, W, B, Hd, V, inv_temp, s.stop_lse, s.mass, s.lm_ws,
                                                 stats_workspace_bytes(B, V), dev_status, st);
         if (ls != SD_OK) return ls;
     }
     // ... turned into the residual max(p - q, 0) where a draft was rejected (with the kept logits of the
     // LM-head pass the probabilities themselves are formed here as well)
-    residual_blocksum_kernel<<<dim3(n_blocks, B), kResBlock, 0, st>>>(V, s.n_excl, s.excl, q_rows, s.stop_row, logits, lse,
-                                                                      inv_temp, s.mass, s.block_sum, n_blocks);
-    residual_pick_kernel<<<B, kResBlock, 0, st>>>(bt, V, w, s.mass, s.block_sum, n_blocks, n_acc, out_tok, dev_status);
-    return cuda_ok(cudaGetLastError());
+    go(launch_dependent(residual_blocksum_kernel, dim3(n_blocks, B), kResBlock, 0, 1, st, V, s.n_excl, s.excl, q_rows, s.stop_row,
+                        logits, lse, inv_temp, s.mass, s.block_sum, n_blocks));
+    go(launch_dependent(residual_pick_kernel, dim3(B), kResBlock, 0, 1, st, bt, V, w, s.mass, s.block_sum, n_blocks, n_acc,
+                        out_tok, dev_status));
+    return r;
 }
 
 // ---------------------------------------------------------------------------
@@ -655,6 +666,7 @@ tree_walk_q_kernel(sd_batch bt, int V, float inv_temp, const float* __restrict__
     __shared__ int32_t s_path[kMaxT];
     __shared__ float s_px, s_qx;
     __shared__ int s_bad;
+    begin_dependent(bt, lse, logits, draft, q_rows, u, w);
     const int b = blockIdx.x / kTreeQCluster;
     const int rank = (int)sm100::cluster_ctarank();
     const int T = bt.T_max, tid = threadIdx.x, lane = tid & 31;
@@ -804,24 +816,9 @@ sd_status launch_accept_tree_sampled_q(const sd_batch& bt, int V, float inv_temp
     const int slice = (V + kTreeQCluster - 1) / kTreeQCluster;
     if (slice > kTreeQMaxSlice) return SD_ERR_UNSUPPORTED;
     const size_t dyn = (size_t)slice * 2 * sizeof(float);
-    if (cudaFuncSetAttribute(tree_walk_q_kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)dyn) != cudaSuccess)
-        return SD_ERR_CUDA;
-    cudaLaunchConfig_t cfg = {};
-    cfg.gridDim = dim3(bt.B * kTreeQCluster);
-    cfg.blockDim = dim3(kTreeQThreads);
-    cfg.dynamicSmemBytes = dyn;
-    cfg.stream = st;
-    cudaLaunchAttribute attr[1];
-    attr[0].id = cudaLaunchAttributeClusterDimension;
-    attr[0].val.clusterDim.x = kTreeQCluster;
-    attr[0].val.clusterDim.y = 1;
-    attr[0].val.clusterDim.z = 1;
-    cfg.attrs = attr;
-    cfg.numAttrs = 1;
-    if (cudaLaunchKernelEx(&cfg, tree_walk_q_kernel, bt, V, inv_temp, lse, logits, draft, q_rows, u, w, n_acc, path, out_tok,
-                           new_len, dev_status) != cudaSuccess)
-        return SD_ERR_CUDA;
-    return SD_OK;
+    if (!allow_dynamic_smem(tree_walk_q_kernel, (int)dyn)) return SD_ERR_CUDA;
+    return launch_dependent(tree_walk_q_kernel, dim3(bt.B * kTreeQCluster), kTreeQThreads, dyn, kTreeQCluster, st, bt, V, inv_temp, lse,
+                            logits, draft, q_rows, u, w, n_acc, path, out_tok, new_len, dev_status);
 }
 
 // ---------------------------------------------------------------------------
@@ -845,6 +842,7 @@ sampled_tail_kernel(sd_batch bt, const __grid_constant__ CompactLayers ly, int L
     __shared__ int32_t s_path[kMaxT], s_tok[kMaxT], s_excl[64];
     __shared__ float s_excl_p[64];
     __shared__ WalkEnd s_end;
+    begin_dependent(bt, tb.part_key, tb.part_idx, tb.part_ref, tb.part_sum, hidden, W, group_stats, draft, u, w, lse, p_child);
     const int b = blockIdx.x / kTailCluster;
     const int rank = (int)sm100::cluster_ctarank();
     const int T = bt.T_max, warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
@@ -925,24 +923,11 @@ sd_status launch_lmhead_accept_sampled_compact(const sd_batch& bt, const void* h
     if (r != SD_OK) return r;
     CompactLayers ly;
     fill_compact_layers(&ly, layers, kt, vt, 0, L);
-    cudaLaunchConfig_t cfg = {};
-    cfg.gridDim = dim3(B * kTailCluster);
-    cfg.blockDim = dim3(256);
-    cfg.stream = st;
-    cudaLaunchAttribute attr[1];
-    attr[0].id = cudaLaunchAttributeClusterDimension;
-    attr[0].val.clusterDim.x = kTailCluster;
-    attr[0].val.clusterDim.y = 1;
-    attr[0].val.clusterDim.z = 1;
-    cfg.attrs = attr;
-    cfg.numAttrs = 1;
     const float c2 = inv_temp * 1.4426950408889634f;
     const int n_groups = (V + 31) / 32;
-    if (cudaLaunchKernelEx(&cfg, sampled_tail_kernel, bt, ly, L, tb, c2, static_cast<const uint16_t*>(hidden),
-                           static_cast<const uint16_t*>(W), Hd, V, inv_temp, reinterpret_cast<const float2*>(group_stats),
-                           n_groups, draft, u, w, lse, s.p_child, n_acc, path, out_tok, new_len, dev_status) != cudaSuccess)
-        return SD_ERR_CUDA;
-    return SD_OK;
+    return launch_dependent(sampled_tail_kernel, dim3(B * kTailCluster), 256, 0, kTailCluster, st, bt, ly, L, tb, c2, hidden, W, Hd, V,
+                            inv_temp, reinterpret_cast<const float2*>(group_stats), n_groups, draft, u, w, lse, s.p_child, n_acc, path,
+                            out_tok, new_len, dev_status);
 }
 
 sd_status launch_accept_sampled(const sd_batch& bt, const void* hidden, const void* W, int Hd, int V, float inv_temp,
@@ -959,26 +944,31 @@ sd_status launch_accept_sampled(const sd_batch& bt, const void* hidden, const vo
     const uint16_t* h = static_cast<const uint16_t*>(hidden);
     const uint16_t* Wp = static_cast<const uint16_t*>(W);
     const int n_blocks = (V + kResBlock - 1) / kResBlock;
-    child_prob_kernel<<<(B * T * 32 + 127) / 128, 128, 0, st>>>(bt, h, Wp, Hd, V, inv_temp, lse, draft, s.p_child, dev_status);
-    sampled_walk_kernel<<<B, 32, 0, st>>>(bt, draft, s.p_child, u, n_acc, path, out_tok, new_len, s.resid, s.stop_row,
-                                         s.n_excl, s.excl, s.excl_p, dev_status);
+    sd_status r = SD_OK;
+    auto go = [&](sd_status x) { if (r == SD_OK) r = x; };
+    go(launch_dependent(child_prob_kernel, dim3((B * T * 32 + 127) / 128), 128, 0, 1, st, bt, h, Wp, Hd, V, inv_temp, lse, draft,
+                        s.p_child, dev_status));
+    go(launch_dependent(sampled_walk_kernel, dim3(B), 32, 0, 1, st, bt, draft, s.p_child, u, n_acc, path, out_tok, new_len,
+                        s.resid, s.stop_row, s.n_excl, s.excl, s.excl_p, dev_status));
     if (group_stats) {
         // the LM-head pass left (maximum, sum) of every 32 vocabulary rows: no second pass over W
         const int n_groups = (V + 31) / 32;
-        residual_pick_groups_kernel<<<B, 256, 0, st>>>(bt, h, Wp, Hd, V, inv_temp, lse, reinterpret_cast<const float2*>(group_stats),
-                                                      n_groups, w, s.stop_row, s.n_excl, s.excl, s.excl_p, n_acc, out_tok, dev_status);
-        return cuda_ok(cudaGetLastError());
+        go(launch_dependent(residual_pick_groups_kernel, dim3(B), 256, 0, 1, st, bt, h, Wp, Hd, V, inv_temp, lse,
+                            reinterpret_cast<const float2*>(group_stats), n_groups, w, s.stop_row, s.n_excl, s.excl, s.excl_p,
+                            n_acc, out_tok, dev_status));
+        return r;
     }
-    gather_stop_rows_kernel<<<B, 128, 0, st>>>(h, Hd, lse, s.stop_row, s.stop_hidden, s.stop_lse);
+    go(launch_dependent(gather_stop_rows_kernel, dim3(B), 128, 0, 1, st, h, Hd, lse, s.stop_row, s.stop_hidden, s.stop_lse));
     // probabilities of the stop rows over the vocabulary: one more pass of the tensor-core LM-head kernel,
     // its epilogue storing instead of reducing (W is streamed once for all sequences)
     sd_status ls = launch_lmhead_mass(s.stop_hidden, W, B, Hd, V, inv_temp, s.stop_lse, s.mass, s.lm_ws,
                                       stats_workspace_bytes(B, V), dev_status, st);
     if (ls != SD_OK) return ls;
-    residual_blocksum_kernel<<<dim3(n_blocks, B), kResBlock, 0, st>>>(V, s.n_excl, s.excl, nullptr, nullptr, nullptr, nullptr, 0.f,
-                                                                      s.mass, s.block_sum, n_blocks);
-    residual_pick_kernel<<<B, kResBlock, 0, st>>>(bt, V, w, s.mass, s.block_sum, n_blocks, n_acc, out_tok, dev_status);
-    return cuda_ok(cudaGetLastError());
+    go(launch_dependent(residual_blocksum_kernel, dim3(n_blocks, B), kResBlock, 0, 1, st, V, s.n_excl, s.excl, nullptr, nullptr,
+                        nullptr, nullptr, 0.f, s.mass, s.block_sum, n_blocks));
+    go(launch_dependent(residual_pick_kernel, dim3(B), kResBlock, 0, 1, st, bt, V, w, s.mass, s.block_sum, n_blocks, n_acc,
+                        out_tok, dev_status));
+    return r;
 }
 
 }  // namespace sdv

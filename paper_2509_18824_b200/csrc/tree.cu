@@ -6,6 +6,7 @@ namespace sdv {
 
 // anc_mask[b][i] = bit i | anc_mask[b][parent(i)], computed by walking up.
 __global__ void tree_prepare_kernel(sd_batch bt, int32_t* status) {
+    begin_dependent(bt);
     const int b = blockIdx.x;
     const int lane = threadIdx.x;
     const int T = bt.T_max;
@@ -45,6 +46,7 @@ __global__ void accept_kernel(sd_batch bt, const int32_t* __restrict__ draft,
                               const int32_t* __restrict__ target,
                               int32_t* n_acc, int32_t* path, int32_t* out_tok, int32_t* new_len,
                               int32_t* status) {
+    begin_dependent(bt, draft, target);
     const int b = blockIdx.x;
     const int T = bt.T_max;
     accept_sequence(bt, b, threadIdx.x, bt.parents + (size_t)b * T, draft + (size_t)b * T, target + (size_t)b * T,
@@ -52,15 +54,13 @@ __global__ void accept_kernel(sd_batch bt, const int32_t* __restrict__ draft,
 }
 
 sd_status launch_tree_prepare(const sd_batch& bt, int32_t* dev_status, cudaStream_t st) {
-    tree_prepare_kernel<<<bt.B, 32, 0, st>>>(bt, dev_status);
-    return cuda_ok(cudaGetLastError());
+    return launch_dependent(tree_prepare_kernel, dim3(bt.B), 32, 0, 1, st, bt, dev_status);
 }
 
 sd_status launch_accept(const sd_batch& bt, const int32_t* draft, const int32_t* target,
                         int32_t* n_acc, int32_t* path, int32_t* out_tok, int32_t* new_len,
                         int32_t* dev_status, cudaStream_t st) {
-    accept_kernel<<<bt.B, 32, 0, st>>>(bt, draft, target, n_acc, path, out_tok, new_len, dev_status);
-    return cuda_ok(cudaGetLastError());
+    return launch_dependent(accept_kernel, dim3(bt.B), 32, 0, 1, st, bt, draft, target, n_acc, path, out_tok, new_len, dev_status);
 }
 
 }  // namespace sdv

@@ -43,6 +43,36 @@ __device__ __forceinline__ void merge_sumexp(float& ref, float& sum, float ref2,
     else            { sum += sum2 * ex2_lm((ref2 - ref) * c2); }
 }
 
+// Arg-max candidate of one hidden row (column `col` of the per-CTA tables), merged by the eight consecutive
+// lanes that share the row; all of them return the result.  Every lane of the warp must call this.
+__device__ __forceinline__ void merge_row_argmax(const int32_t* part_key, const int32_t* part_idx, int n_ctas, int row_stride,
+                                                 int col, bool active, int sub, int32_t& k, int32_t& i) {
+    k = INT32_MIN; i = 0x7fffffff;
+    if (active) {
+        // (the loads of a batch are issued together: one memory latency instead of a chain of them)
+        constexpr int kAhead = 20;                  // 148 CTAs: 19 per lane
+        for (int c0 = sub; c0 < n_ctas; c0 += 8 * kAhead) {
+            int32_t pk[kAhead], pi[kAhead];
+#pragma unroll
+            for (int a = 0; a < kAhead; ++a) {
+                const int c = c0 + 8 * a;
+                if (c < n_ctas) {
+                    pk[a] = part_key[(size_t)c * row_stride + col];
+                    pi[a] = part_idx[(size_t)c * row_stride + col];
+                }
+            }
+#pragma unroll
+            for (int a = 0; a < kAhead; ++a)
+                if (c0 + 8 * a < n_ctas) take_better(k, i, pk[a], pi[a]);
+        }
+    }
+#pragma unroll
+    for (int d = 1; d <= 4; d <<= 1) {
+        const int32_t k2 = __shfl_xor_sync(0xffffffffu, k, d), i2 = __shfl_xor_sync(0xffffffffu, i, d);
+        take_better(k, i, k2, i2);
+    }
+}
+
 // Candidates and soft-max partials of one hidden row (column `col` of the per-CTA tables), merged by the
 // eight consecutive lanes that share the row: lane `sub` takes the CTAs sub, sub + 8, ..., then three
 // exchange steps combine the eight (always lower lane first, so all eight end with the same bits).
