@@ -12,7 +12,7 @@ INCLUDE = os.path.join(os.path.dirname(HERE), "include")
 OBJ = os.path.join(HERE, "_build")
 LIB = os.path.join(HERE, "libsdverify.so")
 NATIVE = os.path.join(HERE, "_sdnative.so")
-SOURCES = ["api.cu", "tree.cu", "compact.cu", "attention.cu", "attention_wide.cu", "lmhead.cu", "sampled.cu", "draft.cu", "tmap.cu"]
+SOURCES = ["api.cu", "tree.cu", "compact.cu", "attention.cu", "attention_wide.cu", "lmhead.cu", "sampled.cu", "sampled_q.cu", "draft.cu", "tmap.cu"]
 NVCC_FLAGS = ["-gencode", "arch=compute_100a,code=sm_100a", "-lineinfo", "-O3", "-std=c++17",
               "-Xcompiler", "-fPIC", "-I", INCLUDE, "-I", CSRC]
 

@@ -143,6 +143,11 @@ sd_status launch_accept_chain_sampled(const sd_batch& bt, const void* hidden, co
                                       const float* q_rows, const float* u, const float* w, int32_t* n_acc, int32_t* path,
                                       int32_t* out_tok, int32_t* new_len, void* ws, size_t ws_bytes, int32_t* dev_status,
                                       cudaStream_t st);
+bool q_kernels_hold(int V);      // whether a cluster of the kernels for sampled drafts holds a row of V entries
+sd_status launch_accept_chain_logits(const sd_batch& bt, int V, float inv_temp, const float* lse, const float* logits,
+                                     const int32_t* draft, const float* q_tok, const float* q_rows, const float* u, const float* w,
+                                     int32_t* n_acc, int32_t* path, int32_t* out_tok, int32_t* new_len, int32_t* dev_status,
+                                     cudaStream_t st);
 sd_status launch_accept_tree_sampled_q(const sd_batch& bt, int V, float inv_temp, const float* lse, const float* logits,
                                        const int32_t* draft, const float* q_rows, const float* u, const float* w,
                                        int32_t* n_acc, int32_t* path, int32_t* out_tok, int32_t* new_len,

@@ -121,6 +121,53 @@ __device__ __forceinline__ float merge_row_stats(const int32_t* __restrict__ par
     return (rf * c2 + log2f(sm)) * 0.6931471805599453f;
 }
 
+// Where the running sum *acc_io + v[0] + v[1] + ... first reaches `target`, among the elements with
+// v > 0 (all v >= 0), found by one warp in a few rounds: the range is cut into 32 consecutive pieces,
+// every lane sums one, an inclusive scan over the lanes gives each piece's end value, and the search
+// goes on inside the first piece that has mass and whose end value reaches the target, until the
+// pieces are single elements.  Every addition happens in a fixed order, so the answer is the same in
+// every run.  Returns the index, or -1 when the whole sum stays short; *acc_io then holds the running
+// sum in front of the returned element (all of it for -1); *last_pos the last index with v > 0, if any.
+// One level down the same elements are added in smaller pieces: where that leaves the refined search
+// a rounding short of the target, the piece's last element with mass is the answer.
+__device__ __forceinline__ int warp_find_crossing(const float* v, int n, float target, float* acc_io, int* last_pos, int lane) {
+    int lo = 0, hi = n;
+    float base = *acc_io;
+    for (bool top = true;; top = false) {
+        const int chunk = (hi - lo + 31) / 32;
+        const int i0 = min(hi, lo + lane * chunk), i1 = min(hi, i0 + chunk);
+        float sum = 0.f;
+        int lastp = -1;
+        for (int i = i0; i < i1; ++i) {
+            const float x = v[i];
+            sum += x;
+            if (x > 0.f) lastp = i;
+        }
+        float incl = sum;
+#pragma unroll
+        for (int d = 1; d < 32; d <<= 1) {
+            const float y = __shfl_up_sync(0xffffffffu, incl, d);
+            if (lane >= d) incl += y;
+        }
+        float excl = __shfl_up_sync(0xffffffffu, incl, 1);
+        if (lane == 0) excl = 0.f;
+        const int lp = __reduce_max_sync(0xffffffffu, lastp);
+        if (top && last_pos && lp >= 0) *last_pos = lp;
+        const uint32_t cand = __ballot_sync(0xffffffffu, sum > 0.f && base + incl >= target);
+        if (!cand) {
+            const float all = base + __shfl_sync(0xffffffffu, incl, 31);
+            if (top) { *acc_io = all; return -1; }
+            *acc_io = all - v[lp];                                   // (lp >= 0: the piece was chosen for having mass)
+            return lp;
+        }
+        const int L0 = __ffs(cand) - 1;
+        base += __shfl_sync(0xffffffffu, excl, L0);
+        lo = __shfl_sync(0xffffffffu, i0, L0);
+        hi = __shfl_sync(0xffffffffu, i1, L0);
+        if (chunk == 1) { *acc_io = base; return lo; }
+    }
+}
+
 // Greedy acceptance for one sequence, executed by one warp.  par/dt/tg point at the sequence's
 // parents, draft tokens and target arg-max (tg may be shared memory).  Returns the number of
 // accepted nodes (0 for a bad tree, which is reported through *status) and, in lane 0, has written
