@@ -328,9 +328,9 @@ attn_umma_kernel(const __grid_constant__ AttnLayers<NL> layers, const sd_batch b
                 tmem_ld32(tmem_s + lane_field + s * kKeyTile, r0);
                 tmem_ld_wait();
                 tmem_ld32(tmem_s + lane_field + s * kKeyTile + 32, r1);   // in flight while the first half is processed
-                exp_pack_half(r0, scale2, neg_m2, pk, ps);
+                exp_pack(r0, scale2, neg_m2, pk, ps);
                 tmem_ld_wait();
-                exp_pack_half(r1, scale2, neg_m2, pk + 16, ps);
+                exp_pack(r1, scale2, neg_m2, pk + 16, ps);
                 const float psum = sum_f32x2(add_f32x2(ps[0], ps[1]));
                 // (padding rows have harmless scores; NaN scores of a real row take the other body and stay NaN)
                 if (!__any_sync(0xffffffffu, row_ok && !(psum <= kSumLimit))) {
@@ -381,8 +381,8 @@ attn_umma_kernel(const __grid_constant__ AttnLayers<NL> layers, const sd_batch b
             }
             uint64_t ps[2] = {0ull, 0ull};
             if (j > 0) {
-                exp_pack_half(r0, scale2, neg_m2, pk, ps);
-                exp_pack_half(r1, scale2, neg_m2, pk + 16, ps);
+                exp_pack(r0, scale2, neg_m2, pk, ps);
+                exp_pack(r1, scale2, neg_m2, pk + 16, ps);
             }
             float psum = sum_f32x2(add_f32x2(ps[0], ps[1]));
             bool raise = row_ok && (j == 0 || !(psum <= kSumLimit));
@@ -415,8 +415,8 @@ attn_umma_kernel(const __grid_constant__ AttnLayers<NL> layers, const sd_batch b
                 neg_m2 = pack_f32x2(-m_used, -m_used);
                 // (again) against the new reference: the same values for rows that did not raise
                 ps[0] = ps[1] = 0ull;
-                exp_pack_half(r0, scale2, neg_m2, pk, ps);
-                exp_pack_half(r1, scale2, neg_m2, pk + 16, ps);
+                exp_pack(r0, scale2, neg_m2, pk, ps);
+                exp_pack(r1, scale2, neg_m2, pk + 16, ps);
                 psum = sum_f32x2(add_f32x2(ps[0], ps[1]));
             }
             l += psum;

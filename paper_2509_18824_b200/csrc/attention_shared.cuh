@@ -54,11 +54,12 @@ __device__ __forceinline__ void mask_scores(uint32_t (&r)[32], uint32_t mask) {
     for (int c = 0; c < 32; ++c) r[c] = ((mask >> c) & 1u) ? r[c] : 0xff800000u;
 }
 
-// 32 raw scores of a row -> 2^(score * scale - reference), packed to bf16 in pairs, and added to the sums
-__device__ __forceinline__ void exp_pack_half(const uint32_t (&r)[32], uint64_t scale2, uint64_t neg_m2, uint32_t* pk,
+// N raw scores of a row -> 2^(score * scale - reference), packed to bf16 in pairs, and added to the sums
+template <int N>
+__device__ __forceinline__ void exp_pack(const uint32_t (&r)[N], uint64_t scale2, uint64_t neg_m2, uint32_t* pk,
                                               uint64_t (&ps)[2]) {
 #pragma unroll
-    for (int c = 0; c < 16; ++c) {
+    for (int c = 0; c < N / 2; ++c) {
         const uint64_t x = fma_f32x2(pack_f32x2(__uint_as_float(r[2 * c]), __uint_as_float(r[2 * c + 1])), scale2, neg_m2);
         float x0, x1;
         asm("mov.b64 {%0, %1}, %2;" : "=f"(x0), "=f"(x1) : "l"(x));

@@ -298,7 +298,7 @@ attn_wide_kernel(const __grid_constant__ AttnLayers<NL> layers, const sd_batch b
                 m_used = *my_ref;
                 neg_m2 = pack_f32x2(-m_used, -m_used);
             }
-            // The usual tile: all keys visible, reference known.  (See exp_pack_half and kSumLimit: nothing
+            // The usual tile: all keys visible, reference known.  (See exp_pack and kSumLimit: nothing
             // but loads, exponentials and stores; masks, a new reference and clearing V rows are below.)
             if (j < n_full) {
                 if (!mbar_wait(&s_full[s], ph, abort_flag, plan.wait_cycles)) { ok = false; break; }
@@ -327,20 +327,19 @@ attn_wide_kernel(const __grid_constant__ AttnLayers<NL> layers, const sd_batch b
                     __syncwarp();
                     if (lane == 0) mbar_arrive(&ref_full[quad]);   // (the other group need not wait for the tile)
                 }
-                uint32_t r0[32], r1[32], pk0[32], pk1[32];
+                uint32_t ra[16], rb[16], pk0[32], pk1[32];
                 uint64_t ps[2] = {0ull, 0ull};
-                tmem_ld32(ts, r0);                         // every quarter but the first arrives while one is processed
-                tmem_ld_wait();
-                tmem_ld32(ts + 32, r1);
-                exp_pack_half(r0, scale2, neg_m2, pk0, ps);
-                tmem_ld_wait();
-                tmem_ld32(ts + 64, r0);
-                exp_pack_half(r1, scale2, neg_m2, pk0 + 16, ps);
-                tmem_ld_wait();
-                tmem_ld32(ts + 96, r1);
-                exp_pack_half(r0, scale2, neg_m2, pk1, ps);
-                tmem_ld_wait();
-                exp_pack_half(r1, scale2, neg_m2, pk1 + 16, ps);
+                tmem_ld16(ts, ra);                         // sixteen scores at a time, the next ones on their way
+#pragma unroll
+                for (int c = 0; c < 8; c += 2) {           // (thirty-two at a time left too few registers: spills)
+                    uint32_t* pk = (c < 4 ? pk0 : pk1) + (c & 2) * 8;
+                    tmem_ld_wait();
+                    tmem_ld16(ts + (c + 1) * 16, rb);
+                    exp_pack(ra, scale2, neg_m2, pk, ps);
+                    tmem_ld_wait();
+                    if (c < 6) tmem_ld16(ts + (c + 2) * 16, ra);
+                    exp_pack(rb, scale2, neg_m2, pk + 8, ps);
+                }
                 const float psum = sum_f32x2(add_f32x2(ps[0], ps[1]));
                 // the tile before is final, and its reference still the one used here
                 if (j > 0 && !mbar_wait(&commit[quad], (uint32_t)(j - 1) & 1u, abort_flag, plan.wait_cycles)) { ok = false; break; }
@@ -438,7 +437,7 @@ attn_wide_kernel(const __grid_constant__ AttnLayers<NL> layers, const sd_batch b
                 tmem_ld32(ts + c * 32, r);
                 tmem_ld_wait();
                 mask_scores(r, c < 2 ? (c ? mask[1] : mask[0]) : (c == 3 ? mask[3] : mask[2]));
-                exp_pack_half(r, scale2, neg_m2, pk, ps);
+                exp_pack(r, scale2, neg_m2, pk, ps);
                 tmem_st16(ts + c * 16, pk);
                 tmem_st_wait();
             }
