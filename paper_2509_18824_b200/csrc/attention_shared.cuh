@@ -49,9 +49,10 @@ __device__ __forceinline__ float sum_f32x2(uint64_t a) {
 }
 
 // keys outside the mask get the score -inf
-__device__ __forceinline__ void mask_scores(uint32_t (&r)[32], uint32_t mask) {
+template <int N>
+__device__ __forceinline__ void mask_scores(uint32_t (&r)[N], uint32_t mask) {
 #pragma unroll
-    for (int c = 0; c < 32; ++c) r[c] = ((mask >> c) & 1u) ? r[c] : 0xff800000u;
+    for (int c = 0; c < N; ++c) r[c] = ((mask >> c) & 1u) ? r[c] : 0xff800000u;
 }
 
 // N raw scores of a row -> 2^(score * scale - reference), packed to bf16 in pairs, and added to the sums

@@ -11,44 +11,22 @@
 // the one O, which works because a row's reference stays at the first tile's maximum (see kSumLimit): the
 // rare tile that raises it is serialised through a per-warp commit barrier that every tile passes anyway.
 #include <atomic>
-#include "attention_shared.cuh"
+#include "attention_wide.cuh"
 
 namespace sdv {
-
-constexpr int kWTile = 128;                     // keys per tile: two cache blocks
-constexpr int kWThreads = 289;                  // warps 0-3, 4-7 softmax groups, warp 8 TMA, warp 9 = ONE thread: MMA issuer
-constexpr int kWTmaWarp = 8, kWMmaWarp = 9;
-constexpr int kWStages = 3;                     // K and V ring slots, score buffers
-constexpr int kWHalf = kWTile * 128;            // bytes of one D-half of a tile: [128 keys][64] bf16, swizzled (16 KiB)
-constexpr int kWStage = 2 * kWHalf;             // 32 KiB
-constexpr int kWQBytes = 2 * kRowTile * 128;    // 32 KiB
-constexpr int kWBars = 256;                     // barriers and two words
-constexpr int kWSmem = kWQBytes + 2 * kWStages * kWStage + kWBars + 3 * kRowTile * 4;   // + references, two groups' sums
 
 template <int NL>
 __global__ void __launch_bounds__(kWThreads, 1)
 attn_wide_kernel(const __grid_constant__ AttnLayers<NL> layers, const sd_batch bt,
                  const float scale_log2, const AttnPlan plan, int32_t* status) {
     extern __shared__ __align__(1024) uint8_t smem[];
-    uint8_t* q_smem = smem;
-    uint8_t* k_smem = smem + kWQBytes;
-    uint8_t* v_smem = k_smem + kWStages * kWStage;
-    uint64_t* bars = reinterpret_cast<uint64_t*>(v_smem + kWStages * kWStage);
-    uint64_t* k_full = bars;             // [3] TMA -> MMA
-    uint64_t* v_full = bars + 3;         // [3] TMA -> MMA (and whoever clears V rows)
-    uint64_t* s_full = bars + 6;         // [3] MMA -> softmax, TMA: scores of tile j in buffer j % 3, K slot j % 3 read
-    uint64_t* v_empty = bars + 9;        // [3] MMA -> TMA: O updated by tile j, V slot j % 3 read
-    uint64_t* p_full = bars + 12;        // [3] softmax -> MMA: P of tile j written over its scores
-    uint64_t* commit = bars + 15;        // [4] per TMEM quadrant: tile j's softmax is final (phase j)
-    uint64_t* o_full = bars + 19;        // MMA -> softmax (single use)
-    uint64_t* q_full = bars + 20;        // TMA -> MMA
-    uint64_t* x_full = bars + 21;        // clustered launches: the other chunks' rows have arrived
-    uint64_t* ref_full = bars + 22;      // [4] per TMEM quadrant: the first tile's reference is known (single use)
-    uint32_t* tmem_slot = reinterpret_cast<uint32_t*>(bars + 26);
-    int* abort_flag = reinterpret_cast<int*>(bars + 27);
-    int& s_seq = *reinterpret_cast<int*>(bars + 28);
-    float* ref_smem = reinterpret_cast<float*>(reinterpret_cast<uint8_t*>(bars) + kWBars);   // [128] by TMEM lane
-    float* sum_smem = ref_smem + kRowTile;                                                   // [2][128]
+    const WideShared sh(smem);
+    uint8_t *const q_smem = sh.q_smem, *const k_smem = sh.k_smem, *const v_smem = sh.v_smem;
+    uint64_t *const k_full = sh.k_full, *const v_full = sh.v_full, *const s_full = sh.s_full, *const v_empty = sh.v_empty;
+    uint64_t *const p_full = sh.p_full, *const o_full = sh.o_full, *const q_full = sh.q_full, *const x_full = sh.x_full;
+    uint32_t* const tmem_slot = sh.tmem_slot;
+    int* const abort_flag = sh.abort_flag;
+    float *const ref_smem = sh.ref_smem, *const sum_smem = sh.sum_smem;
 
     const int warp = __shfl_sync(0xffffffffu, (int)(threadIdx.x >> 5), 0);
     const int lane = threadIdx.x & 31;
@@ -65,13 +43,7 @@ attn_wide_kernel(const __grid_constant__ AttnLayers<NL> layers, const sd_batch b
     if (aligned) {
         if (warp == kWTmaWarp) {
             if (lane == 0) {
-                *abort_flag = 0;
-                for (int i = 0; i < kWStages; ++i) {
-                    mbar_init(&k_full[i], 1); mbar_init(&v_full[i], 1); mbar_init(&s_full[i], 1);
-                    mbar_init(&v_empty[i], 1); mbar_init(&p_full[i], 4);
-                }
-                for (int i = 0; i < 4; ++i) { mbar_init(&commit[i], 1); mbar_init(&ref_full[i], 1); }
-                mbar_init(o_full, 1); mbar_init(q_full, 1); mbar_init(x_full, 1);
+                sh.init_barriers();
                 fence_barrier_init();
                 fence_proxy_async_smem();
                 prefetch_tensormap(&ly.q); prefetch_tensormap(&ly.k_cache); prefetch_tensormap(&ly.v_cache);
@@ -95,7 +67,7 @@ attn_wide_kernel(const __grid_constant__ AttnLayers<NL> layers, const sd_batch b
     griddep_wait();                                        // global memory from here on
 
     int b = rank_b;
-    if (plan.ranked) b = sequence_of_rank(bt, rank_b, s_seq);
+    if (plan.ranked) b = sequence_of_rank(bt, rank_b, *sh.seq);
     const int G = bt.Hq / bt.Hkv;
     const int T = bt.T_max;
     const int tile_rows = plan.tile_rows;
@@ -225,26 +197,31 @@ attn_wide_kernel(const __grid_constant__ AttnLayers<NL> layers, const sd_batch b
             for (int i = 0; i < 1000; ++i) __nanosleep(1000);      // let copies in flight land
         }
     } else if (warp == kWMmaWarp) {
-        // ------------------------------------------------------------ MMA issuer (this warp is one thread)
+        // ------------------------------------------------------------ MMA issuer
         const int M = m64 ? 64 : kRowTile;
         const uint32_t idesc_s = make_idesc_bf16(M, kWTile, false, false), idesc_s_half = make_idesc_bf16(M, kWTile / 2, false, false);
         const uint32_t idesc_o = make_idesc_bf16(M, kD, false, true);
+        // (A whole warp in uniform control flow, one lane elected around the instructions, as in the producer: eight
+        //  MMAs take 375 to 440 cycles to issue; a warp of one thread needed 470 to 480.)
         const uint64_t qdesc = make_smem_desc(smem_u32(q_smem), 16, 1024, 128);
         const uint64_t kdesc0 = make_smem_desc(smem_u32(k_smem), 16, 1024, 128);
         const uint64_t vdesc0 = make_smem_desc(smem_u32(v_smem), kWHalf, 1024, 128);   // [key][d]: N (= d) contiguous
-        bool ok = mbar_wait(q_full, 0, abort_flag, plan.wait_cycles);
+        bool ok = mbar_wait_warp(q_full, 0, abort_flag, plan.wait_cycles);
         auto issue_s = [&](int j) -> bool {
             const int s = j % kWStages;
-            if (!mbar_wait(&k_full[s], (uint32_t)(j / kWStages) & 1u, abort_flag, plan.wait_cycles)) return false;
+            if (!mbar_wait_warp(&k_full[s], (uint32_t)(j / kWStages) & 1u, abort_flag, plan.wait_cycles)) return false;
             tc_fence_after_sync();
             const uint64_t kd = kdesc0 + (uint64_t)(s * (kWStage >> 4));
             const uint32_t d = tmem_s + s * kWTile;
             const uint32_t idesc = 2 * j + 1 < nb ? idesc_s : idesc_s_half;
+            if (elect_one()) {
 #pragma unroll
-            for (int k = 0; k < kD / 16; ++k)
-                mma_ss(d, qdesc + (uint64_t)((k >> 2) * ((kRowTile * 128) >> 4) + (k & 3) * 2),
-                       kd + (uint64_t)((k >> 2) * (kWHalf >> 4) + (k & 3) * 2), idesc, k != 0 ? 1u : 0u);
-            mma_commit(&s_full[s]);
+                for (int k = 0; k < kD / 16; ++k)
+                    mma_ss(d, qdesc + (uint64_t)((k >> 2) * ((kRowTile * 128) >> 4) + (k & 3) * 2),
+                           kd + (uint64_t)((k >> 2) * (kWHalf >> 4) + (k & 3) * 2), idesc, k != 0 ? 1u : 0u);
+                mma_commit(&s_full[s]);
+            }
+            __syncwarp();
             return true;
         };
         for (int j = 0; j < kWStages - 1 && j < nt && ok; ++j) ok = issue_s(j);
@@ -254,25 +231,29 @@ attn_wide_kernel(const __grid_constant__ AttnLayers<NL> layers, const sd_batch b
             if (!ok) break;
             const int s = j % kWStages;
             const uint32_t ph = (uint32_t)(j / kWStages) & 1u;
-            if (!mbar_wait(&p_full[s], ph, abort_flag, plan.wait_cycles)) { ok = false; break; }
-            if (!mbar_wait(&v_full[s], ph, abort_flag, plan.wait_cycles)) { ok = false; break; }
+            if (!mbar_wait_warp(&p_full[s], ph, abort_flag, plan.wait_cycles)) { ok = false; break; }
+            if (!mbar_wait_warp(&v_full[s], ph, abort_flag, plan.wait_cycles)) { ok = false; break; }
             tc_fence_after_sync();
             const uint64_t vd = vdesc0 + (uint64_t)(s * (kWStage >> 4));
             const uint32_t pa = tmem_s + s * kWTile;       // P from tensor memory: 16 keys = 8 columns
             const uint32_t first = (j != 0) ? 1u : 0u;
+            if (elect_one()) {
 #pragma unroll
-            for (int k = 0; k < 4; ++k)
-                mma_ts(tmem_o, pa + k * 8, vd + (uint64_t)(k * (2048 >> 4)), idesc_o, k != 0 ? 1u : first);
-            if (2 * j + 1 < nb) {
+                for (int k = 0; k < 4; ++k)
+                    mma_ts(tmem_o, pa + k * 8, vd + (uint64_t)(k * (2048 >> 4)), idesc_o, k != 0 ? 1u : first);
+                if (2 * j + 1 < nb) {
 #pragma unroll
-                for (int k = 4; k < 8; ++k) mma_ts(tmem_o, pa + k * 8, vd + (uint64_t)(k * (2048 >> 4)), idesc_o, 1u);
+                    for (int k = 4; k < 8; ++k) mma_ts(tmem_o, pa + k * 8, vd + (uint64_t)(k * (2048 >> 4)), idesc_o, 1u);
+                }
+                mma_commit(&v_empty[s]);
             }
-            mma_commit(&v_empty[s]);
+            __syncwarp();
         }
-        mma_commit(o_full);
+        if (elect_one()) mma_commit(o_full);
+        __syncwarp();
         if (!ok) {
             // unwinding: nothing may give tensor memory back while an MMA issued above still runs
-            set_status(status, SD_ERR_TIMEOUT);
+            if (lane == 0) set_status(status, SD_ERR_TIMEOUT);
             mbar_wait_plain(o_full, 0, plan.wait_cycles);
         }
     } else {
@@ -284,168 +265,9 @@ attn_wide_kernel(const __grid_constant__ AttnLayers<NL> layers, const sd_batch b
         const bool row_ok = row < rows;
         const uint64_t amask = row_ok ? bt.anc_mask[(size_t)b * T + plan.node_of(row)] : ~0ull;
         const uint32_t lane_field = (uint32_t)(quad * 32) << 16;
-        const uint64_t scale2 = pack_f32x2(scale_log2, scale_log2);
-        uint64_t neg_m2 = 0ull;                            // -(reference of this row), twice
+        bool ok = wide_softmax(plan, sh, WideTiles{nt, nb, n_pref, cr.t0, len, n, 0, 0}, tmem_o, tmem_s, group, quad, lane, row_ok, amask,
+                               scale_log2, m_used, l);
         volatile float* my_ref = ref_smem + gt;
-        bool ok = true;
-        const int n_full = max(min(len / kBlock - cr.t0, n_pref), 0) / 2;   // leading tiles with all 128 keys inside the prefix
-        for (int j = group; j < nt && ok; j += 2) {
-            const int s = j % kWStages;
-            const uint32_t ph = (uint32_t)(j / kWStages) & 1u;
-            const uint32_t ts = tmem_s + lane_field + s * kWTile;
-            if (j == 1) {                                  // the reference that the other group found in tile 0
-                if (!mbar_wait(&ref_full[quad], 0, abort_flag, plan.wait_cycles)) { ok = false; break; }
-                m_used = *my_ref;
-                neg_m2 = pack_f32x2(-m_used, -m_used);
-            }
-            // The usual tile: all keys visible, reference known.  (See exp_pack and kSumLimit: nothing
-            // but loads, exponentials and stores; masks, a new reference and clearing V rows are below.)
-            if (j < n_full) {
-                if (!mbar_wait(&s_full[s], ph, abort_flag, plan.wait_cycles)) { ok = false; break; }
-                tc_fence_after_sync();
-                if (j == 0) {                              // its maximum becomes the reference
-                    float mt = -INFINITY;
-#pragma unroll 1
-                    for (int c = 0; c < kWTile; c += 64) {
-                        uint32_t a[32], d[32];
-                        tmem_ld32(ts + c, a);
-                        tmem_ld32(ts + c + 32, d);
-                        tmem_ld_wait();
-                        float m0 = -INFINITY, m1 = -INFINITY, m2 = -INFINITY, m3 = -INFINITY;
-#pragma unroll
-                        for (int k = 0; k < 32; k += 4) {
-                            m0 = max3(m0, __uint_as_float(a[k]), __uint_as_float(a[k + 1]));
-                            m1 = max3(m1, __uint_as_float(a[k + 2]), __uint_as_float(a[k + 3]));
-                            m2 = max3(m2, __uint_as_float(d[k]), __uint_as_float(d[k + 1]));
-                            m3 = max3(m3, __uint_as_float(d[k + 2]), __uint_as_float(d[k + 3]));
-                        }
-                        mt = max3(mt, fmaxf(m0, m1), fmaxf(m2, m3));
-                    }
-                    m_used = row_ok ? mt * scale_log2 : 0.f;       // scale > 0; finite for rows that nobody reads
-                    *my_ref = m_used;
-                    neg_m2 = pack_f32x2(-m_used, -m_used);
-                    __syncwarp();
-                    if (lane == 0) mbar_arrive(&ref_full[quad]);   // (the other group need not wait for the tile)
-                }
-                uint32_t ra[16], rb[16], pk0[32], pk1[32];
-                uint64_t ps[2] = {0ull, 0ull};
-                tmem_ld16(ts, ra);                         // sixteen scores at a time, the next ones on their way
-#pragma unroll
-                for (int c = 0; c < 8; c += 2) {           // (thirty-two at a time left too few registers: spills)
-                    uint32_t* pk = (c < 4 ? pk0 : pk1) + (c & 2) * 8;
-                    tmem_ld_wait();
-                    tmem_ld16(ts + (c + 1) * 16, rb);
-                    exp_pack(ra, scale2, neg_m2, pk, ps);
-                    tmem_ld_wait();
-                    if (c < 6) tmem_ld16(ts + (c + 2) * 16, ra);
-                    exp_pack(rb, scale2, neg_m2, pk + 8, ps);
-                }
-                const float psum = sum_f32x2(add_f32x2(ps[0], ps[1]));
-                // the tile before is final, and its reference still the one used here
-                if (j > 0 && !mbar_wait(&commit[quad], (uint32_t)(j - 1) & 1u, abort_flag, plan.wait_cycles)) { ok = false; break; }
-                const float ref = *my_ref;
-                if (!__any_sync(0xffffffffu, row_ok && (!(psum <= kSumLimit) || ref != m_used))) {
-                    l += psum;
-                    tmem_st32(ts, pk0);                    // P over the scores this thread has just consumed
-                    tmem_st32(ts + 32, pk1);
-                    tmem_st_wait();
-                    tc_fence_before_sync();
-                    __syncwarp();
-                    if (lane == 0 && !(plan.withhold && j == 0)) { mbar_arrive(&p_full[s]); mbar_arrive(&commit[quad]); }
-                    continue;
-                }
-            }
-            // Any tile.  First the V rows of keys that no row may see (cache slots at and beyond len, rows of
-            // unused tree nodes): they carry weight 0, but 0 x NaN or 0 x Inf would still poison the
-            // accumulator, so they are cleared in shared memory before P.V reads them (the arrival on p_full
-            // orders the two).  This comes after the wait for the scores of tile j: they were issued behind
-            // P.V of tile j - 3, which read the V tile that used this ring slot before, so the slot's
-            // barrier is by now in the phase of tile j.
-            if (!mbar_wait(&s_full[s], ph, abort_flag, plan.wait_cycles)) { ok = false; break; }
-            tc_fence_after_sync();
-            uint32_t mask[4];                              // visible keys of the four 32-key quarters
-            int v_rows[2];
-#pragma unroll
-            for (int h = 0; h < 2; ++h) {
-                const int i = 2 * j + h;
-                const bool tree = i >= n_pref;
-                const int valid = i >= nb ? 0 : (tree ? kBlock : max(min(len - (cr.t0 + i) * kBlock, kBlock), 0));
-                v_rows[h] = i >= nb ? kBlock : (tree ? n : valid);
-                const uint64_t m = (tree && i < nb) ? amask : (valid >= 64 ? ~0ull : ((1ull << valid) - 1ull));
-                mask[2 * h] = (uint32_t)m; mask[2 * h + 1] = (uint32_t)(m >> 32);
-            }
-            if (v_rows[0] < kBlock || v_rows[1] < kBlock) {
-                if (!mbar_wait(&v_full[s], ph, abort_flag, plan.wait_cycles)) { ok = false; break; }
-                const int h = gt >> 6, key = gt & 63;
-                if (key >= v_rows[h]) {
-                    uint4* z = reinterpret_cast<uint4*>(v_smem + s * kWStage + gt * 128);
-#pragma unroll
-                    for (int c = 0; c < 8; ++c) {
-                        z[c] = make_uint4(0, 0, 0, 0);
-                        z[c + kWHalf / 16] = make_uint4(0, 0, 0, 0);
-                    }
-                    fence_proxy_async_smem();
-                }
-            }
-            if (j > 0) {
-                if (!mbar_wait(&commit[quad], (uint32_t)(j - 1) & 1u, abort_flag, plan.wait_cycles)) { ok = false; break; }
-                const float ref = *my_ref;                 // raised by the other group since?
-                if (ref != m_used) { l *= exp2f(m_used - ref); m_used = ref; }
-            }
-            const int n_quarters = 2 * j + 1 < nb ? 4 : 2;
-            float mt = -INFINITY;
-#pragma unroll 1
-            for (int c = 0; c < n_quarters; ++c) {
-                uint32_t r[32];
-                tmem_ld32(ts + c * 32, r);
-                tmem_ld_wait();
-                mask_scores(r, c < 2 ? (c ? mask[1] : mask[0]) : (c == 3 ? mask[3] : mask[2]));
-#pragma unroll
-                for (int k = 0; k < 32; k += 2) mt = max3(mt, __uint_as_float(r[k]), __uint_as_float(r[k + 1]));
-            }
-            mt *= scale_log2;                              // scale > 0
-            // first tile: its maximum becomes the reference; later: only a score far above it changes it
-            const bool raise = row_ok && (m_used == -INFINITY || mt > m_used + kRaiseAbove) && mt > m_used;
-            if (__any_sync(0xffffffffu, raise) && j > 0) {
-                if (!mbar_wait(&v_empty[(j - 1) % kWStages], (uint32_t)((j - 1) / kWStages) & 1u, abort_flag, plan.wait_cycles)) { ok = false; break; }
-                tc_fence_after_sync();
-                const float alpha = raise ? exp2f(m_used - mt) : 1.f;
-#pragma unroll 1
-                for (int cc = 0; cc < 4; ++cc) {
-                    uint32_t o[32];
-                    tmem_ld32(tmem_o + lane_field + cc * 32, o);
-                    tmem_ld_wait();
-#pragma unroll
-                    for (int c = 0; c < 32; ++c) o[c] = __float_as_uint(__uint_as_float(o[c]) * alpha);
-                    tmem_st32(tmem_o + lane_field + cc * 32, o);
-                }
-                tmem_st_wait();
-                l *= alpha;
-            }
-            if (raise) m_used = mt;
-            if (!row_ok) m_used = 0.f;                     // (finite exponentials for rows that nobody reads)
-            *my_ref = m_used;
-            neg_m2 = pack_f32x2(-m_used, -m_used);
-            if (j == 0 && n_full == 0) {
-                __syncwarp();
-                if (lane == 0) mbar_arrive(&ref_full[quad]);
-            }
-            uint64_t ps[2] = {0ull, 0ull};
-#pragma unroll 1
-            for (int c = 0; c < n_quarters; ++c) {         // P of a quarter lands on scores that have been read
-                uint32_t r[32], pk[16];
-                tmem_ld32(ts + c * 32, r);
-                tmem_ld_wait();
-                mask_scores(r, c < 2 ? (c ? mask[1] : mask[0]) : (c == 3 ? mask[3] : mask[2]));
-                exp_pack(r, scale2, neg_m2, pk, ps);
-                tmem_st16(ts + c * 16, pk);
-                tmem_st_wait();
-            }
-            l += sum_f32x2(add_f32x2(ps[0], ps[1]));
-            tc_fence_before_sync();
-            __syncwarp();
-            if (lane == 0 && !(plan.withhold && j == 0)) { mbar_arrive(&p_full[s]); mbar_arrive(&commit[quad]); }
-        }
         // ------------------------------------------------------------ epilogue
         if (ok) ok = mbar_wait(o_full, 0, abort_flag, plan.wait_cycles);
         if (ok) {
