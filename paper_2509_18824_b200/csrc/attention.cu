@@ -559,7 +559,8 @@ static AttnPlan common_plan(const sd_batch& bt, int n_layers, const TestKnobs& k
 // time), four of 8192 52 / 32 / 41, eight of 4096 32 / 40, eight chains of 11 nodes 29.6 / 20.8 / 17.8.
 // The 64-key kernel's two CTAs per SM overlap each other's ends: a round of twice as many CTAs takes about
 // 0.9 us per block plus 13 us.  It is left for launches of several rounds in which those ends weigh more
-// (256 CTAs of 1000 tokens: 28.7 against 33.9 us; of 4096: 71.4 against 69.9).
+// (256 CTAs of 1000 tokens: 28.7 against 33.9 us; of 4096: 71.4 against 69.9; 1792 CTAs of 4096 tokens under the
+// power cap, where 64-key tiles cost more energy: 569 against 544).
 static bool wide_plan(AttnPlan* p, const sd_batch& bt, int dev, int sms, const TestKnobs& knobs) {
     const long long base = (long long)p->n_layers * bt.B * bt.Hkv * p->row_tiles;
     const int blocks = bt.max_blocks_per_seq;
@@ -575,7 +576,7 @@ static bool wide_plan(AttnPlan* p, const sd_batch& bt, int dev, int sms, const T
     }
     if (n_rounds > 1) {
         const double rounds = base <= 2 * sms ? 1.0 : (double)base / (2 * sms) + 0.25;     // a partial round, cut into chunks
-        if (best > 0.95 * rounds * (13.0 + 0.9 * blocks)) return false;
+        if (best > 1.05 * rounds * (13.0 + 0.9 * blocks)) return false;
     }
     p->n_chunks = n;
     // Shorter sequences are cut into fewer chunks where all clusters run at once; in several rounds the CTAs that

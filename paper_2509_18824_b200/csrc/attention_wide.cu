@@ -8,7 +8,7 @@
 // commits, the softmax warps' waits, loads, votes and stores - is paid once per 128 keys.  Two groups of
 // four softmax warps take the tiles in turn, so that one group's latencies hide behind the other's
 // exponentials; three score buffers keep the tensor pipe fed while they do.  Both groups accumulate into
-// the one O, which works because a row's reference stays at the first tile's maximum (see kSumLimit): the
+// the one O, which works because a row's reference stays where its first scores put it (see kSumLimit): the
 // rare tile that raises it is serialised through a per-warp commit barrier that every tile passes anyway.
 #include <atomic>
 #include "attention_wide.cuh"

@@ -73,7 +73,7 @@ __device__ __forceinline__ bool wide_softmax(const AttnPlan& plan, const WideSha
     const uint64_t scale2 = pack_f32x2(scale_log2, scale_log2);
     uint64_t neg_m2 = 0ull;                            // -(reference of this row), twice
     const int n_full = max(min(w.len / kBlock - w.t0, w.n_pref), 0) / 2;   // leading tiles with all 128 keys inside the prefix
-    // Loads, exponentials and stores of one tile against the row's reference (tile 0 sets it to its maximum), see
+    // Loads, exponentials and stores of one tile against the row's reference (tile 0 sets it), see
     // exp_pack and kSumLimit.  0: done, 1: the reference has to be raised first (nothing stored yet), -1: a wait ran
     // out.  The usual tile has all keys visible; masked ones (the last: cache slots behind len, the tree's keys)
     // take the same body with the scores of hidden keys replaced.  (As a body of their own that looked for the
@@ -84,23 +84,25 @@ __device__ __forceinline__ bool wide_softmax(const AttnPlan& plan, const WideSha
         const int s = jj % kWStages;
         const uint32_t ts = tmem_s + lane_field + s * kWTile;
         if (j == 0) {
-            float mt = -INFINITY;
-#pragma unroll 1
-            for (int c = 0; c < (half ? kWTile / 2 : kWTile); c += 64) {
-                uint32_t a[32], d[32];
-                tmem_ld32(ts + c, a);
-                tmem_ld32(ts + c + 32, d);
-                tmem_ld_wait();
-                if (kMasked) { mask_scores(a, c ? mask[2] : mask[0]); mask_scores(d, c ? mask[3] : mask[1]); }
-                float m0 = -INFINITY, m1 = -INFINITY, m2 = -INFINITY, m3 = -INFINITY;
+            // The reference: the largest of the first sixteen scores (any score of the row will do, see kSumLimit; a
+            // maximum over all of them took 800 cycles in front of every call's first exponentials), or, where some
+            // row sees none of those keys, of all.
+            uint32_t a[16];
+            tmem_ld16(ts, a);
+            tmem_ld_wait();
+            if (kMasked) mask_scores(a, mask[0]);
+            float mt = fmaxf(__uint_as_float(a[0]), __uint_as_float(a[1]));
 #pragma unroll
-                for (int k = 0; k < 32; k += 4) {
-                    m0 = max3(m0, __uint_as_float(a[k]), __uint_as_float(a[k + 1]));
-                    m1 = max3(m1, __uint_as_float(a[k + 2]), __uint_as_float(a[k + 3]));
-                    m2 = max3(m2, __uint_as_float(d[k]), __uint_as_float(d[k + 1]));
-                    m3 = max3(m3, __uint_as_float(d[k + 2]), __uint_as_float(d[k + 3]));
+            for (int k = 2; k < 16; k += 2) mt = max3(mt, __uint_as_float(a[k]), __uint_as_float(a[k + 1]));
+            if (kMasked && __any_sync(0xffffffffu, row_ok && mt == -INFINITY)) {
+#pragma unroll 1
+                for (int c = 0; c < (half ? 4 : 8); ++c) {
+                    tmem_ld16(ts + c * 16, a);
+                    tmem_ld_wait();
+                    mask_scores(a, (c < 4 ? (c < 2 ? mask[0] : mask[1]) : (c < 6 ? mask[2] : mask[3])) >> ((c & 1) * 16));
+#pragma unroll
+                    for (int k = 0; k < 16; k += 2) mt = max3(mt, __uint_as_float(a[k]), __uint_as_float(a[k + 1]));
                 }
-                mt = max3(mt, fmaxf(m0, m1), fmaxf(m2, m3));
             }
             m_used = row_ok ? mt * scale_log2 : 0.f;       // scale > 0; finite for rows that nobody reads
             *my_ref = m_used;
@@ -206,7 +208,7 @@ __device__ __forceinline__ bool wide_softmax(const AttnPlan& plan, const WideSha
         }
         mt *= scale_log2;                                  // scale > 0
         const bool raise = row_ok && mt > m_used + kRaiseAbove;
-        if (__any_sync(0xffffffffu, raise)) {              // (never in tile 0)
+        if (__any_sync(0xffffffffu, raise) && j > 0) {     // (nothing has been accumulated before tile 0)
             if (!mbar_wait(&sh.v_empty[(jj - 1) % kWStages], (uint32_t)((jj - 1) / kWStages) & 1u, sh.abort_flag, plan.wait_cycles)) return false;
             tc_fence_after_sync();
             const float alpha = raise ? exp2f(m_used - mt) : 1.f;
