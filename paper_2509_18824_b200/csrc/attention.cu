@@ -466,7 +466,7 @@ attn_umma_kernel(const __grid_constant__ AttnLayers<NL> layers, const sd_batch b
         mbar_wait(q_full, 0, abort_flag, plan.wait_cycles);
 
     if (clustered) {
-        // The chunks' rows meet as described at exchange_rows; the rings are free by now.
+        // The chunks' rows meet as described at RowExchange; the rings are free by now.
         const RowExchange x{bt, plan, ly, smem_u32(k_smem), smem_u32(x_full), chunk, n_chunks, rt, b, kvh, rows, tpc, tiles_total};
         if (threadIdx.x == 0) exchange_expect(x, x_full);
         __syncwarp();
@@ -554,9 +554,12 @@ static AttnPlan common_plan(const sd_batch& bt, int n_layers, const TestKnobs& k
 
 // The 128-key kernel (attention_wide.cu) runs one CTA per SM.  A round of it takes about 0.36 us per cache block
 // of its longest chunk, plus 8 us for launch, first copies and output (11 when CTAs of another round follow:
-// nothing overlaps them), plus the merge of the chunks.  Measured per call in us, chunks 1 / 2 / 4 / 8: one
-// sequence of 2048 tokens and 60 nodes 17.2 / 13.5 / 10.9 / 17.9 (16 clusters of eight are more than fit at a
-// time), four of 8192 52 / 32 / 41, eight of 4096 32 / 40, eight chains of 11 nodes 29.6 / 20.8 / 17.8.
+// nothing overlaps them), plus the merge of the chunks, plus about 1 us where the next call's CTAs find no
+// free SMs to set up on while this one runs.  Measured per call in us for 1 to 8 chunks: one sequence of 2048
+// tokens and 60 nodes 16.4 13.0 11.4 10.6 10.7 10.7 17.3 17.5 (16 clusters of seven or eight are more than fit
+// at a time), of 8192 50.6 30.3 23.0 19.2 17.6 16.7 26.8 26.0, one chain of 11 nodes over 4096 27.3 18.5 14.6
+// 12.9 12.0 11.2 10.9 10.9.  Chunk counts that are no powers of two fill SMs that those leave idle: ten such
+// chains 19.6 us with three chunks (22.2 with two), five sequences of 2000 tokens with 16 heads 13.5 (15.1).
 // The 64-key kernel's two CTAs per SM overlap each other's ends: a round of twice as many CTAs takes about
 // 0.9 us per block plus 13 us.  It is left for launches of several rounds in which those ends weigh more
 // (256 CTAs of 1000 tokens: 28.7 against 33.9 us; of 4096: 71.4 against 69.9; 1792 CTAs of 4096 tokens under the
@@ -564,14 +567,14 @@ static AttnPlan common_plan(const sd_batch& bt, int n_layers, const TestKnobs& k
 static bool wide_plan(AttnPlan* p, const sd_batch& bt, int dev, int sms, const TestKnobs& knobs) {
     const long long base = (long long)p->n_layers * bt.B * bt.Hkv * p->row_tiles;
     const int blocks = bt.max_blocks_per_seq;
-    const double merge[4] = {0.0, 2.0, 2.3, 3.0};
+    const double merge[kMaxChunks] = {0.0, 2.8, 3.2, 3.2, 3.3, 3.4, 3.6, 3.8};
     int n = 1;
     long long n_rounds = 1;
     double best = 1e30;
-    for (int c = 1, i = 0; c <= kMaxChunks && c <= blocks; c *= 2, ++i) {
+    for (int c = 1; c <= kMaxChunks && c <= blocks; ++c) {
         const int resident = wide_resident_clusters(dev, sms, c);
         const long long rounds = (base + resident - 1) / resident;
-        const double us = rounds * ((rounds > 1 ? 11.0 : 8.0) + merge[i] + 0.36 * ((blocks + c - 1) / c));
+        const double us = rounds * ((rounds > 1 ? 11.0 : (2 * base * c > sms ? 9.1 : 8.0)) + merge[c - 1] + 0.36 * ((blocks + c - 1) / c));
         if (knobs.chunks > 0 && knobs.chunks <= blocks ? c == knobs.chunks : us < best - 1e-9) { best = us; n = c; n_rounds = rounds; }
     }
     if (n_rounds > 1) {
@@ -616,7 +619,7 @@ static void narrow_plan(AttnPlan* plan, const sd_batch& bt, int sms, const TestK
         const double cost = waves * ((max_tiles + c - 1) / c + 3 + merge);
         if (cost < best - 1e-9) { best = cost; n = c; }
     }
-    if (knobs.chunks > 0 && knobs.chunks <= max_tiles) n = knobs.chunks;     // test hook
+    if (knobs.chunks > 0 && knobs.chunks <= max_tiles && (knobs.chunks & (knobs.chunks - 1)) == 0) n = knobs.chunks;     // test hook
     p.n_chunks = n;
     p.chunk_blocks = 0;
     p.ranked = (bt.B > 1 && bt.B <= 64 && (long long)base * n > slots) ? 1 : 0;

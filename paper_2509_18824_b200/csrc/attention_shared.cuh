@@ -71,13 +71,16 @@ __device__ __forceinline__ void exp_pack(const uint32_t (&r)[N], uint64_t scale2
     }
 }
 
-// key chunks of a sequence (the last one also takes the tree's keys): the smallest power of two, up to
+// key chunks of a sequence (the last one also takes the tree's keys): the smallest number, up to
 // n_chunks, whose chunks have at most chunk_blocks cache blocks
 __device__ __forceinline__ int chunks_of(int blocks, int n_chunks, int chunk_blocks) {
     int c = 1;
-    while (c < n_chunks && blocks > c * chunk_blocks) c *= 2;
+    while (c < n_chunks && blocks > c * chunk_blocks) ++c;
     return c;
 }
+// rows of a row tile that each of its chunks' CTAs finishes: in eights, so that what a warp sends to one CTA
+// are whole 128-byte lines (the last CTAs may have fewer, or none)
+__host__ __device__ constexpr int rows_per_chunk(int n_chunks) { return ((kRowTile + n_chunks - 1) / n_chunks + 7) & ~7; }
 
 struct AttnPlan {
     int n_chunks;      // CTAs per row tile along the keys (a cluster): key chunks of the longest sequences
@@ -153,7 +156,7 @@ __device__ __forceinline__ void zero_unused_rows(const sd_batch& bt, const AttnP
     }
 }
 
-// Final step of a clustered launch.  Row r of the tile is finished by the CTA of chunk r / (128 / n_chunks).
+// Final step of a clustered launch.  Row r of the tile is finished by the CTA of chunk r / rows_per_chunk.
 // Every other chunk's CTA sends it that row's reference, sum and unnormalised O straight from tensor memory,
 // with stores that report their bytes to the receiver's barrier (so the receiver waits for exactly what it
 // gets, and no second cluster-wide barrier and release stand between the last row and the merge); its own
@@ -167,7 +170,8 @@ struct RowExchange {
     uint32_t xo_addr;                   // this CTA's exchange area
     uint32_t bar_addr;                  // its barrier for the rows of the other chunks
     int chunk, n_chunks, rt, b, kvh, rows, tpc, tiles_total;
-    __device__ __forceinline__ uint32_t xs_addr() const { return xo_addr + kRowTile * kD * 4; }
+    __device__ __forceinline__ uint32_t sum_off() const { return (uint32_t)(n_chunks * rows_per_chunk(n_chunks)) * 4; }
+    __device__ __forceinline__ uint32_t xs_addr() const { return xo_addr + sum_off() * kD; }
     // rows beyond the sequence's last one are not exchanged
     __device__ __forceinline__ bool has(int in_tile) const { return in_tile < plan.tile_rows && rt * plan.tile_rows + in_tile < rows; }
     // does that chunk have key tiles (the last one has the tree's)
@@ -176,7 +180,7 @@ struct RowExchange {
 
 // bytes this CTA will receive (one thread, before the cluster barrier)
 __device__ __forceinline__ void exchange_expect(const RowExchange& x, uint64_t* bar) {
-    const int per = kRowTile / x.n_chunks;
+    const int per = rows_per_chunk(x.n_chunks);
     const int mine = min(max(min(x.rows - x.rt * x.plan.tile_rows, x.plan.tile_rows) - x.chunk * per, 0), per);
     int others = 0;
     for (int c = 0; c < x.n_chunks; ++c) others += (c != x.chunk && x.live(c)) ? 1 : 0;
@@ -187,8 +191,8 @@ __device__ __forceinline__ void exchange_expect(const RowExchange& x, uint64_t* 
 template <int NC>
 __device__ __forceinline__ void exchange_push(const RowExchange& x, uint32_t tmem, int cc0, bool ready, int row_in_tile, float ref,
                                               float sum) {
-    const int per = kRowTile / x.n_chunks;
-    const int rr = max(row_in_tile, 0), dest = rr / per, rl = rr % per;
+    const int per = rows_per_chunk(x.n_chunks);
+    const int rr = max(row_in_tile, 0), dest = rr / per, rl = rr - dest * per;
     const bool mine = ready && row_in_tile >= 0 && x.has(rr), remote = dest != x.chunk;
     const uint32_t off = (uint32_t)((x.chunk * 32 * per + rl) * 16);
     const uint32_t xo = (remote ? map_dsmem(x.xo_addr, (uint32_t)dest) : x.xo_addr) + off;
@@ -211,10 +215,10 @@ __device__ __forceinline__ void exchange_push(const RowExchange& x, uint32_t tme
         if (remote) {
             const uint32_t to = map_dsmem(at, (uint32_t)dest);
             st_async_b32(to, __float_as_uint(ref), bar);
-            st_async_b32(to + kRowTile * 4, __float_as_uint(sum), bar);
+            st_async_b32(to + x.sum_off(), __float_as_uint(sum), bar);
         } else {
             st_smem_f32(at, ref);
-            st_smem_f32(at + kRowTile * 4, sum);
+            st_smem_f32(at + x.sum_off(), sum);
         }
     }
 }
@@ -224,12 +228,13 @@ __device__ __forceinline__ void exchange_push(const RowExchange& x, uint32_t tme
 // conflicts) and each writes a whole 32-byte sector.
 template <int NCH, int THREADS>
 __device__ __forceinline__ void merge_rows(const RowExchange& x, int tid) {
-    constexpr int kRowsPer = kRowTile / NCH;        // rows this CTA finishes
+    constexpr int kRowsPer = rows_per_chunk(NCH);   // rows this CTA finishes
+    constexpr int kGroups = THREADS / kRowsPer;     // threads that share a row (those beyond the last whole group rest)
     const int G = x.bt.Hq / x.bt.Hkv;
     const int rl = tid % kRowsPer;
     const int in_tile = x.chunk * kRowsPer + rl, row = x.rt * x.plan.tile_rows + in_tile;
-    if (!x.has(in_tile)) return;
-    const uint32_t xs = x.xs_addr();
+    if (tid >= kGroups * kRowsPer || !x.has(in_tile)) return;
+    const uint32_t xs = x.xo_addr + NCH * kRowsPer * kD * 4;
     float w[NCH];
     float M = -INFINITY;
 #pragma unroll
@@ -242,14 +247,14 @@ __device__ __forceinline__ void merge_rows(const RowExchange& x, int tid) {
     for (int c = 0; c < NCH; ++c) {
         if (w[c] == -INFINITY) { w[c] = 0.f; continue; }
         w[c] = ex2_approx(w[c] - M);
-        den = fmaf(w[c], ld_smem_f32(xs + (kRowTile + c * kRowsPer + rl) * 4), den);
+        den = fmaf(w[c], ld_smem_f32(xs + (NCH * kRowsPer + c * kRowsPer + rl) * 4), den);
     }
     const float inv = __frcp_rn(den);
     const int node = x.plan.node_of(row), g = row - node * G;
     const size_t orow = ((size_t)x.b * x.bt.T_max + node) * x.bt.Hq + x.kvh * G + g;
     if (x.ly.lse && tid < kRowsPer) x.ly.lse[orow] = (M + __log2f(den)) * 0.6931471805599453f;
 #pragma unroll
-    for (int cg = tid / kRowsPer; cg < 8; cg += THREADS / kRowsPer) {       // 16 columns: pieces 4 cg .. + 3
+    for (int cg = tid / kRowsPer; cg < 8; cg += kGroups) {       // 16 columns: pieces 4 cg .. + 3
         float4 acc[4];
 #pragma unroll
         for (int p = 0; p < 4; ++p) acc[p] = make_float4(0.f, 0.f, 0.f, 0.f);

@@ -327,7 +327,7 @@ attn_wide_kernel(const __grid_constant__ AttnLayers<NL> layers, const sd_batch b
         mbar_wait(q_full, 0, abort_flag, plan.wait_cycles);
 
     if (clustered) {
-        // The chunks' rows meet as described at exchange_rows; the rings are free by now.
+        // The chunks' rows meet as described at RowExchange; the rings are free by now.
         const int gt = (int)threadIdx.x & 127;
         const int row_in_tile = m64 ? (lane < 16 ? (warp & 3) * 16 + lane : -1) : gt;
         const RowExchange x{bt, plan, ly, smem_u32(k_smem), smem_u32(x_full), chunk, n_chunks, rt, b, kvh, rows, cr.tpc, cr.tiles_total};
@@ -342,9 +342,15 @@ attn_wide_kernel(const __grid_constant__ AttnLayers<NL> layers, const sd_batch b
         if (warp < 8) {
             asm volatile("bar.sync 1, 256;" ::: "memory"); // this CTA's own rows
             if (mbar_wait_cluster(x_full, 0, abort_flag, plan.wait_cycles)) {
-                if (n_chunks == 2) merge_rows<2, 256>(x, (int)threadIdx.x);
-                else if (n_chunks == 4) merge_rows<4, 256>(x, (int)threadIdx.x);
-                else merge_rows<8, 256>(x, (int)threadIdx.x);
+                switch (n_chunks) {
+                    case 2: merge_rows<2, 256>(x, (int)threadIdx.x); break;
+                    case 3: merge_rows<3, 256>(x, (int)threadIdx.x); break;
+                    case 4: merge_rows<4, 256>(x, (int)threadIdx.x); break;
+                    case 5: merge_rows<5, 256>(x, (int)threadIdx.x); break;
+                    case 6: merge_rows<6, 256>(x, (int)threadIdx.x); break;
+                    case 7: merge_rows<7, 256>(x, (int)threadIdx.x); break;
+                    default: merge_rows<8, 256>(x, (int)threadIdx.x); break;
+                }
             } else if (lane == 0) {
                 set_status(status, SD_ERR_TIMEOUT);
                 for (int i = 0; i < 1000; ++i) __nanosleep(1000);      // let rows in flight land
@@ -375,11 +381,10 @@ template sd_status launch_wide<kMaxLayersPerLaunch>(const AttnLayers<kMaxLayersP
 // CTA per SM it depends on how many SMs each GPC has; 8 x 16 of the 148 do not all fit, for instance).
 int wide_resident_clusters(int dev, int sms, int n_chunks) {
     constexpr int kDevs = 64;
-    static std::atomic<int> cache[kDevs][4];
+    static std::atomic<int> cache[kDevs][kMaxChunks + 1];
     if (n_chunks <= 1) return sms;
-    const int slot = n_chunks == 2 ? 1 : (n_chunks == 4 ? 2 : 3);
     if (dev >= 0 && dev < kDevs)
-        if (const int v = cache[dev][slot].load(std::memory_order_relaxed)) return v;
+        if (const int v = cache[dev][n_chunks].load(std::memory_order_relaxed)) return v;
     cudaLaunchConfig_t cfg = {};
     cfg.gridDim = dim3(n_chunks, 1, sms);
     cfg.blockDim = dim3(kWThreads);
@@ -396,7 +401,7 @@ int wide_resident_clusters(int dev, int sms, int n_chunks) {
         cudaOccupancyMaxActiveClusters(&n, attn_wide_kernel<1>, &cfg) != cudaSuccess || n < 1)
         n = max(1, sms / n_chunks - n_chunks);             // (no answer: a cautious guess, and ask again next time)
     else if (dev >= 0 && dev < kDevs)
-        cache[dev][slot].store(n, std::memory_order_relaxed);
+        cache[dev][n_chunks].store(n, std::memory_order_relaxed);
     return n;
 }
 

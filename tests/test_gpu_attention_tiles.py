@@ -22,7 +22,7 @@ def problem(seed, lens, T=19, Hq=14, Hkv=2, gain=3.0):
     return Tiny(seed, B=B, T=T, Hq=Hq, Hkv=Hkv, D=128, lens=lens, parents=par, gain=gain)
 
 
-@pytest.mark.parametrize("chunks", [0, 1, 2, 4, 8])
+@pytest.mark.parametrize("chunks", [0, 1, 2, 3, 4, 5, 6, 7, 8])
 @pytest.mark.parametrize("lens", [(0, 64, 129), (128, 127, 385), (640, 511, 1), (1023, 257, 130), (1409, 1024, 66)])
 def test_tile_and_chunk_edges(monkeypatch, lens, chunks):
     """19 nodes x 7 heads = a row tile of 126 rows and one of 7."""
