@@ -61,46 +61,53 @@ attn_wide_kernel(const __grid_constant__ AttnLayers<NL> layers, const sd_batch b
     tc_fence_after_sync();
     const uint32_t tmem_base = aligned ? *tmem_slot : 0;
     const uint32_t tmem_o = tmem_base, tmem_s = tmem_base + 128;   // O, then three score buffers of 128 columns
-    // A guess at the sequence's length, read while the kernel ahead may still change it: only used to fetch
-    // the block table together with the real length instead of after it.
-    const int len_guess = plan.ranked ? 0 : max(__ldcg(bt.len + rank_b), 0);
-    griddep_wait();                                        // global memory from here on
-
-    int b = rank_b;
-    if (plan.ranked) b = sequence_of_rank(bt, rank_b, *sh.seq);
     const int G = bt.Hq / bt.Hkv;
     const int T = bt.T_max;
     const int tile_rows = plan.tile_rows;
     const uint64_t pol = policy_evict_first();
-    if (aligned && warp == kWTmaWarp && lane == 0) {       // depends on nothing but b
-        mbar_arrive_expect_tx(q_full, (uint32_t)tile_rows * kD * 2);
-        tma_load_3d(q_smem, &ly.q, 0, kvh * G, b * T + rt * plan.tile_nodes, q_full, pol);
-        tma_load_3d(q_smem + kRowTile * 128, &ly.q, 64, kvh * G, b * T + rt * plan.tile_nodes, q_full, pol);
-    }
+    // The work of this CTA is worked out before the wait for the kernel ahead, from the length and node count
+    // that stand there now, although that kernel may still change them: behind the wait they are read again,
+    // and where they differ it is worked out anew.  (Layers of one step find them unchanged.  With all of it
+    // behind the wait 2400 cycles passed from there to the first K copy, 700 of them for the reads.  With this and the
+    // early report below a call for one sequence of 2048 tokens takes 9.7 instead of 10.5 us, eight chains of
+    // 11 nodes over 4096 tokens 16.4 instead of 17.1.)
+    int n = 0, len = 0;
+    if (!plan.ranked) { n = __ldcg(bt.n_nodes + rank_b); len = __ldcg(bt.len + rank_b); }
+    WideWork wk = wide_work(bt, plan, n, len, chunk);
+    wk.settle();
+    griddep_wait();                                        // global memory from here on
+
+    int b = rank_b;
+    if (plan.ranked) b = sequence_of_rank(bt, rank_b, *sh.seq);
     const int32_t *n_nodes = bt.n_nodes, *lens = bt.len, *tables = bt.block_table;
     settle(n_nodes); settle(lens); settle(tables);         // (no load of theirs in front of the wait)
-    const int n = min(max(__ldg(n_nodes + b), 0), T);
-    const int len = max(__ldg(lens + b), 0);
-    const int t0_guess = chunk_range(len_guess, bt.max_blocks_per_seq, chunks_of(min((len_guess + kBlock - 1) / kBlock, bt.max_blocks_per_seq), plan.n_chunks, plan.chunk_blocks), chunk).t0;
     const int32_t* const seq_table = tables + (size_t)b * bt.max_blocks_per_seq;
+    const int n_now = __ldg(n_nodes + b), len_now = __ldg(lens + b);
     int even = 0, odd = 0;                                 // block table of this chunk (producer warp)
     if (warp == kWTmaWarp) {
-        if (t0_guess + lane < bt.max_blocks_per_seq) even = __ldg(seq_table + t0_guess + lane);
-        if (t0_guess + 32 + lane < bt.max_blocks_per_seq) odd = __ldg(seq_table + t0_guess + 32 + lane);
+        const int i = wk.t0 + lane;                        // (within the table whatever the length)
+        if (i < bt.max_blocks_per_seq) even = __ldg(seq_table + i);
+        if (i + 32 < bt.max_blocks_per_seq) odd = __ldg(seq_table + i + 32);
+        if (aligned && lane == 0) {                        // Q depends on nothing but b
+            mbar_arrive_expect_tx(q_full, (uint32_t)tile_rows * kD * 2);
+            tma_load_3d(q_smem, &ly.q, 0, kvh * G, b * T + rt * plan.tile_nodes, q_full, pol);
+            tma_load_3d(q_smem + kRowTile * 128, &ly.q, 64, kvh * G, b * T + rt * plan.tile_nodes, q_full, pol);
+        }
+        __syncwarp();
     }
+    const bool as_guessed = n_now == n && len_now == len;
+    const int t0_read = wk.t0;                             // where `even` and `odd` were read
+    if (!as_guessed) wk = wide_work(bt, plan, n_now, len_now, chunk);
+    n = wk.n; len = wk.len;
     const int rows = n * G;                                // rows of this sequence's own nodes
     const bool m64 = (rows - rt * tile_rows) <= 64;        // last row tile of at most 64 rows: M = 64 (lanes 0..15 of a quadrant)
     if ((len + kBlock - 1) / kBlock > bt.max_blocks_per_seq && threadIdx.x == 0) set_status(status, SD_ERR_BOUNDS);
-    // key chunks of this sequence; CTAs beyond have nothing to do
-    const int n_chunks = chunks_of(min((len + kBlock - 1) / kBlock, bt.max_blocks_per_seq), plan.n_chunks, plan.chunk_blocks);
-    const ChunkRange cr = chunk_range(len, bt.max_blocks_per_seq, n_chunks, chunk);
-    const int n_pref = cr.t1 - cr.t0;                      // cache blocks of this chunk ...
-    const int nb = n_pref + (chunk == n_chunks - 1 ? 1 : 0);           // ... and the tree's keys as one more
+    const int n_chunks = wk.n_chunks, n_pref = wk.n_pref, nb = wk.nb, t0 = wk.t0;
     const int nt = (nb + 1) / 2;
-    const bool has_rows = rt * tile_rows < rows && chunk < n_chunks;
+    const bool has_rows = rt * tile_rows < rows && chunk < n_chunks;   // (CTAs beyond have nothing to do)
     const bool active = (nt > 0) && aligned && has_rows;
     const bool clustered = (n_chunks > 1) && has_rows;     // (a CTA without work leaves; cluster barriers do not wait for it)
-    const int32_t* table = seq_table + cr.t0;
+    const int32_t* table = seq_table + t0;
     // The producer is a whole warp in uniform control flow with one lane elected around the copies (32 cycles
     // per copy; 70 from a lane-0 branch, where every operand has to be moved to uniform registers under
     // divergence, and eight copies a tile made the producer the kernel's bound).  Its lanes hold the
@@ -150,11 +157,20 @@ attn_wide_kernel(const __grid_constant__ AttnLayers<NL> layers, const sd_batch b
     if (chunk == 0) zero_unused_rows(bt, plan, ly, b, rt, kvh, rows, (int)threadIdx.x, kWThreads);
     float m_used = -INFINITY, l = 0.f;                     // this thread's row: reference, sum over its group's tiles
     bool rows_ready = false;
+    const RowExchange x{bt, plan, ly, smem_u32(k_smem), smem_u32(x_full), chunk, n_chunks, rt, b, kvh, rows, wk.tpc, wk.tiles_total};
+    // The chunks' rows meet in the K ring as described at RowExchange.  A CTA's K ring is free when its last scores
+    // are there, which is where its warps report it to the cluster: the barrier then hides behind the last
+    // tile's exponentials and P.V (reported behind them it took another 850 cycles).
+    if (clustered && warp == kWMmaWarp && lane == 0) exchange_expect(x, x_full);
+    auto ring_is_free = [&] {
+        __syncwarp();
+        if (clustered) cluster_arrive_release();
+    };
 
     if (active) {
     if (warp == kWTmaWarp) {
         // ------------------------------------------------------------ TMA producer
-        if (cr.t0 != t0_guess) {
+        if (t0 != t0_read) {
             even = window(0);
             odd = window(32);
         }
@@ -196,6 +212,7 @@ attn_wide_kernel(const __grid_constant__ AttnLayers<NL> layers, const sd_batch b
             if (lane == 0) set_status(status, SD_ERR_TIMEOUT);
             for (int i = 0; i < 1000; ++i) __nanosleep(1000);      // let copies in flight land
         }
+        ring_is_free();
     } else if (warp == kWMmaWarp) {
         // ------------------------------------------------------------ MMA issuer
         const int M = m64 ? 64 : kRowTile;
@@ -256,6 +273,7 @@ attn_wide_kernel(const __grid_constant__ AttnLayers<NL> layers, const sd_batch b
             if (lane == 0) set_status(status, SD_ERR_TIMEOUT);
             mbar_wait_plain(o_full, 0, plan.wait_cycles);
         }
+        ring_is_free();
     } else {
         // ------------------------------------------------------------ softmax: one thread per row and group
         const int group = warp >> 2, quad = warp & 3;
@@ -265,8 +283,9 @@ attn_wide_kernel(const __grid_constant__ AttnLayers<NL> layers, const sd_batch b
         const bool row_ok = row < rows;
         const uint64_t amask = row_ok ? bt.anc_mask[(size_t)b * T + plan.node_of(row)] : ~0ull;
         const uint32_t lane_field = (uint32_t)(quad * 32) << 16;
-        bool ok = wide_softmax(plan, sh, WideTiles{nt, nb, n_pref, cr.t0, len, n, 0, 0}, tmem_o, tmem_s, group, quad, lane, row_ok, amask,
+        bool ok = wide_softmax(plan, sh, WideTiles{nt, nb, n_pref, t0, len, n, 0, 0}, tmem_o, tmem_s, group, quad, lane, row_ok, amask,
                                scale_log2, m_used, l);
+        ring_is_free();
         volatile float* my_ref = ref_smem + gt;
         // ------------------------------------------------------------ epilogue
         if (ok) ok = mbar_wait(o_full, 0, abort_flag, plan.wait_cycles);
@@ -321,20 +340,18 @@ attn_wide_kernel(const __grid_constant__ AttnLayers<NL> layers, const sd_batch b
             set_status(status, SD_ERR_TIMEOUT);
         }
     }
-    }   // active
+    } else {
+        ring_is_free();
+    }
 
     if (!active && aligned && warp == kWTmaWarp && lane == 0)      // nobody else waits for the Q copy
         mbar_wait(q_full, 0, abort_flag, plan.wait_cycles);
 
     if (clustered) {
-        // The chunks' rows meet as described at RowExchange; the rings are free by now.
         const int gt = (int)threadIdx.x & 127;
         const int row_in_tile = m64 ? (lane < 16 ? (warp & 3) * 16 + lane : -1) : gt;
-        const RowExchange x{bt, plan, ly, smem_u32(k_smem), smem_u32(x_full), chunk, n_chunks, rt, b, kvh, rows, cr.tpc, cr.tiles_total};
-        if (threadIdx.x == 0) exchange_expect(x, x_full);
         __syncwarp();
-        cluster_arrive_release();                          // every CTA's MMAs and copies are complete
-        cluster_wait_acquire();
+        cluster_wait_acquire();                            // every chunk's K ring is free
         if (active && warp < 8)
             exchange_push<2>(x, tmem_base + ((uint32_t)((warp & 3) * 32) << 16), (warp >> 2) * 2, rows_ready, row_in_tile, m_used, l);
         __syncwarp();

@@ -59,6 +59,32 @@ struct WideShared {
     }
 };
 
+// What a CTA has to do for a sequence of len cached tokens and n nodes: its share of the key chunks.
+struct WideWork {
+    int n, len;
+    int n_chunks;                   // key chunks of this sequence
+    int tiles_total, tpc;           // cache blocks of the sequence and of a chunk, see chunk_range
+    int t0, n_pref;                 // this chunk's first cache block, and how many
+    int nb;                         // blocks of keys: those, and the tree's in the last chunk
+    // (what has been worked out stays in front of the code that follows)
+    __device__ __forceinline__ void settle() {
+        asm volatile("" : "+r"(n), "+r"(len), "+r"(n_chunks), "+r"(tiles_total), "+r"(tpc), "+r"(t0), "+r"(n_pref), "+r"(nb));
+    }
+};
+__device__ __forceinline__ WideWork wide_work(const sd_batch& bt, const AttnPlan& plan, int n, int len, int chunk) {
+    WideWork w;
+    w.n = min(max(n, 0), bt.T_max);
+    w.len = min(max(len, 0), 0x7fffffff - kBlock);         // (any number may stand there before the kernel ahead is done)
+    w.n_chunks = chunks_of(min((w.len + kBlock - 1) / kBlock, bt.max_blocks_per_seq), plan.n_chunks, plan.chunk_blocks);
+    const ChunkRange cr = chunk_range(w.len, bt.max_blocks_per_seq, w.n_chunks, chunk);
+    w.tiles_total = cr.tiles_total;
+    w.tpc = cr.tpc;
+    w.t0 = cr.t0;
+    w.n_pref = cr.t1 - cr.t0;
+    w.nb = w.n_pref + (chunk == w.n_chunks - 1 ? 1 : 0);
+    return w;
+}
+
 // The key tiles of one row tile: nt tiles over nb blocks, of which n_pref are cache blocks t0 .. of the sequence
 // (len cached tokens, n nodes), the one behind them the tree's.  base: tiles this CTA has worked on before.
 struct WideTiles { int nt, nb, n_pref, t0, len, n, base; uint32_t ref_phase; };

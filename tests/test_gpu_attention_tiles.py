@@ -76,3 +76,31 @@ def test_reference_is_raised(layers):
         rel = np.linalg.norm(out - ref) / np.linalg.norm(ref)
         assert rel <= 2e-2, rel
         np.testing.assert_allclose(lse, rlse, rtol=2e-3, atol=2e-3)
+
+
+@pytest.mark.parametrize("stale", [0, -7, 333, 5000, 2**31 - 1])
+def test_lengths_written_by_the_kernel_ahead(stale):
+    """An attention call may begin while the kernel ahead still runs, and looks at the lengths then: whatever
+    stands there must not matter once that kernel (here acceptance, which writes them) has finished."""
+    p = problem(5, (900, 333, 1000))
+    ref, ref_lse, status = gpu_attention(p)
+    assert status == 0
+    bt, src = sd.Batch.of(p), sd.Batch.of(p)
+    src.len -= 1                                          # one node accepted: the length of p
+    st = sd.new_status()
+    sd.sd_tree_prepare(bt, st)
+    i32 = lambda *shape: torch.zeros(shape, dtype=torch.int32, device="cuda")
+    draft, argmax, n_acc, path, tok = i32(p.B, p.T_max) + 1, i32(p.B * p.T_max), i32(p.B), i32(p.B, p.T_max), i32(p.B, p.T_max)
+    cache = sd.kv_layer(to_device(p.k_cache), to_device(p.v_cache))
+    q, kt, vt = to_device(p.q), to_device(p.k_tree), to_device(p.v_tree)
+    ws = torch.empty(sd.sd_workspace_bytes(bt), dtype=torch.uint8, device="cuda")
+    for _ in range(8):
+        out = torch.full((p.B, p.T_max, p.Hq, p.D), 7.0, dtype=torch.bfloat16, device="cuda")
+        lse = torch.zeros((p.B, p.T_max, p.Hq), dtype=torch.float32, device="cuda")
+        bt.len.fill_(stale)
+        sd.sd_accept_tree(src, draft, argmax, n_acc, path, tok, bt.len, st)
+        sd.sd_verify_attention(bt, cache, q, kt, vt, float(p.scale), out, lse, ws, st)
+        torch.cuda.synchronize()
+        assert int(st.item()) == 0 and (n_acc == 1).all()
+        np.testing.assert_array_equal(out.float().cpu().numpy(), ref)
+        np.testing.assert_array_equal(lse.cpu().numpy(), ref_lse)
