@@ -15,11 +15,16 @@ namespace sdv {
 using namespace sm100;
 
 constexpr int kBM = 128;            // vocabulary rows per tile (MMA M)
-constexpr int kEpiWarps = 8;        // two epilogue warps per TMEM lane quadrant: even and odd 32-column chunks
-constexpr int kTmaWarpLm = kEpiWarps, kMmaWarpLm = kEpiWarps + 1;
-constexpr int kLmThreads = kEpiWarps * 32 + 32 + 1;   // epilogue warps, TMA producer warp, ONE thread: MMA issuer
-                                    // (a one-thread warp keeps the issue loop in uniform control flow, so
-                                    //  the MMA descriptors stay in uniform registers)
+// Warps: PAR epilogue warps per TMEM lane quadrant, the 32-column chunks dealt out among them, then the TMA
+// producer warp, then ONE thread: MMA issuer (a one-thread warp keeps the issue loop in uniform control flow, so
+// the MMA descriptors stay in uniform registers).  Up to 256 hidden rows PAR = 2: the accumulator is
+// double-buffered and the epilogue hides behind the next tile's MMAs.  Above, the one buffer is drained while
+// the tensor cores wait, and the redux and vote latencies of two warps per scheduler left half of the issue
+// slots empty: PAR = 4 takes 480 rows from 434 to 419 us, with statistics and logits from 528 to 493 (below
+// 256 rows it gains nothing and costs 1 % in power).
+constexpr int kEpiChunks = 4;       // chunks of 32 columns per epilogue warp, at most
+__host__ __device__ constexpr int epi_threads(int par) { return par * 128; }
+__host__ __device__ constexpr int lm_threads(int par) { return epi_threads(par) + 32 + 1; }
 constexpr int kMaxCols = kLmMaxCols; // hidden rows per launch (TMEM columns)
 constexpr int kMaxCtas = 256;
 constexpr int kMaxStages = 8;
@@ -169,31 +174,32 @@ __device__ __forceinline__ void column_argmax_stats32(const uint32_t (&r)[32], b
 }
 
 // ---------------------------------------------------------------------------
-// Epilogue shared by the one-CTA and the two-CTA kernel.  Warp w of the eight epilogue warps works on
+// Epilogue shared by the one-CTA and the two-CTA kernel.  Warp w of the 4 PAR epilogue warps works on
 // TMEM lanes 32 * (w & 3) .. +31 (the only ones it may read) and on the 32-column chunks of parity
 // w >> 2; per (warp, column) it keeps a running best (value, vocabulary row) and, for the soft-max
 // statistics, a running (reference, sum).
 // ---------------------------------------------------------------------------
 struct EpiState {
-    float best_val[kMaxCols / 64];
-    int32_t best_idx[kMaxCols / 64];
-    float run_ref[kMaxCols / 64], run_sum[kMaxCols / 64];
+    float best_val[kEpiChunks];
+    int32_t best_idx[kEpiChunks];
+    float run_ref[kEpiChunks], run_sum[kEpiChunks];
 };
 
 __device__ __forceinline__ void epi_init(EpiState& e) {
 #pragma unroll
-    for (int c = 0; c < kMaxCols / 64; ++c) {
+    for (int c = 0; c < kEpiChunks; ++c) {
         e.best_val[c] = -INFINITY; e.best_idx[c] = 0x7fffffff; e.run_ref[c] = -INFINITY; e.run_sum[c] = 0.f;
     }
 }
 
 // one accumulator tile (128 vocabulary rows from v_base - 32 * quad on; this warp's 32 of them start at v_base)
+template <int PAR>
 __device__ __forceinline__ void epi_tile(const LmParams& p, EpiState& e, uint32_t taddr, int v_base, int lane, int par) {
     const bool stats = p.c2 > 0.f;
     const bool v_ok = (v_base + lane) < p.V;
 #pragma unroll
-    for (int h = 0; h < kMaxCols / 64; ++h) {
-        const int c = 2 * h + par;                 // this warp's chunk of the pair (2h, 2h + 1)
+    for (int h = 0; h < kEpiChunks; ++h) {
+        const int c = PAR * h + par;               // this warp's chunk of each PAR
         if (c * 32 < p.n_pad) {
             uint32_t r[32];
             tmem_ld32(taddr + c * 32, r);
@@ -239,25 +245,27 @@ __device__ __forceinline__ void epi_tile(const LmParams& p, EpiState& e, uint32_
 // After the last tile: the four lane quadrants' results are merged through shared memory (the pipeline
 // stages are idle by now: the last accumulator was complete, so every copy has landed and every MMA has
 // read it) and this CTA's row of the candidate tables is written.
+template <int PAR>
 __device__ __forceinline__ void epi_finish(const LmParams& p, const EpiState& e, uint8_t* smem, int quad, int par,
                                            int lane, bool ok, int32_t* status) {
+    constexpr int cols = kEpiChunks * PAR * 32;            // (the others have no hidden row)
     const bool stats = p.c2 > 0.f;
-    asm volatile("bar.sync 1, %0;" ::"n"(kEpiWarps * 32) : "memory");
+    asm volatile("bar.sync 1, %0;" ::"n"(epi_threads(PAR)) : "memory");
     int32_t* red_key = reinterpret_cast<int32_t*>(smem);
     int32_t* red_idx = red_key + 4 * kMaxCols;
     float* red_ref = reinterpret_cast<float*>(red_idx + 4 * kMaxCols);
     float* red_sum = red_ref + 4 * kMaxCols;
 #pragma unroll
-    for (int h = 0; h < kMaxCols / 64; ++h) {
-        red_key[quad * kMaxCols + (2 * h + par) * 32 + lane] = ordered_key(__float_as_uint(e.best_val[h]));
-        red_idx[quad * kMaxCols + (2 * h + par) * 32 + lane] = e.best_idx[h];
+    for (int h = 0; h < kEpiChunks; ++h) {
+        red_key[quad * kMaxCols + (PAR * h + par) * 32 + lane] = ordered_key(__float_as_uint(e.best_val[h]));
+        red_idx[quad * kMaxCols + (PAR * h + par) * 32 + lane] = e.best_idx[h];
         if (stats) {
-            red_ref[quad * kMaxCols + (2 * h + par) * 32 + lane] = e.run_ref[h];
-            red_sum[quad * kMaxCols + (2 * h + par) * 32 + lane] = e.run_sum[h];
+            red_ref[quad * kMaxCols + (PAR * h + par) * 32 + lane] = e.run_ref[h];
+            red_sum[quad * kMaxCols + (PAR * h + par) * 32 + lane] = e.run_sum[h];
         }
     }
-    asm volatile("bar.sync 1, %0;" ::"n"(kEpiWarps * 32) : "memory");
-    for (int col = threadIdx.x; col < kMaxCols; col += kEpiWarps * 32) {
+    asm volatile("bar.sync 1, %0;" ::"n"(epi_threads(PAR)) : "memory");
+    for (int col = threadIdx.x; col < cols; col += epi_threads(PAR)) {
         int32_t k = red_key[col], i = red_idx[col];
 #pragma unroll
         for (int w = 1; w < 4; ++w) {
@@ -278,9 +286,10 @@ __device__ __forceinline__ void epi_finish(const LmParams& p, const EpiState& e,
 }
 
 template <int BK>
-__global__ void __launch_bounds__(kLmThreads, 1)
+__global__ void __launch_bounds__(lm_threads(4), 1)
 lmhead_umma_kernel(const __grid_constant__ CUtensorMap tmW, const __grid_constant__ CUtensorMap tmH,
                    const LmParams p, int32_t* status) {
+    constexpr int kPar = 4, kTmaWarpLm = 4 * kPar, kMmaWarpLm = kTmaWarpLm + 1;
     constexpr int kSwz = BK * 2;                 // bytes per smem row = swizzle span
     constexpr int kGroup = 8 * kSwz;             // 8-row swizzle group
     extern __shared__ uint8_t smem_raw[];
@@ -304,7 +313,7 @@ lmhead_umma_kernel(const __grid_constant__ CUtensorMap tmW, const __grid_constan
     if (threadIdx.x == 0) {
         abort_flag = 0;
         for (int s = 0; s < p.stages; ++s) { mbar_init(&full_bar[s], 1); mbar_init(&empty_bar[s], 1); }
-        for (int b = 0; b < 2; ++b) { mbar_init(&tmem_full[b], 1); mbar_init(&tmem_empty[b], kEpiWarps); }
+        for (int b = 0; b < 2; ++b) { mbar_init(&tmem_full[b], 1); mbar_init(&tmem_empty[b], 4 * kPar); }
         mbar_init(&mma_idle, 1);
         fence_barrier_init();
     }
@@ -385,7 +394,7 @@ lmhead_umma_kernel(const __grid_constant__ CUtensorMap tmW, const __grid_constan
             }
         }
     } else {
-        // ------------------------------------------------ epilogue warps 0..7
+        // ------------------------------------------------ epilogue warps
         const int quad = warp & 3, par = warp >> 2;
         EpiState e;
         epi_init(e);
@@ -396,12 +405,12 @@ lmhead_umma_kernel(const __grid_constant__ CUtensorMap tmW, const __grid_constan
             if (!mbar_wait(&tmem_full[buf], use & 1u, &abort_flag, p.wait_cycles)) { ok = false; break; }
             tc_fence_after_sync();
             const int v_base = ((int)blockIdx.x + t * (int)gridDim.x) * kBM + quad * 32;
-            epi_tile(p, e, tmem_base + ((uint32_t)(quad * 32) << 16) + (uint32_t)(buf * p.buf_stride), v_base, lane, par);
+            epi_tile<kPar>(p, e, tmem_base + ((uint32_t)(quad * 32) << 16) + (uint32_t)(buf * p.buf_stride), v_base, lane, par);
             tc_fence_before_sync();
             __syncwarp();
             if (lane == 0) mbar_arrive(&tmem_empty[buf]);
         }
-        epi_finish(p, e, smem, quad, par, lane, ok, status);
+        epi_finish<kPar>(p, e, smem, quad, par, lane, ok, status);
     }
     tc_fence_before_sync();
     __syncthreads();
@@ -419,9 +428,10 @@ lmhead_umma_kernel(const __grid_constant__ CUtensorMap tmW, const __grid_constan
 // The hidden matrix is therefore re-read from L2 half as often per W byte.
 // ---------------------------------------------------------------------------
 template <int BK, int NPARTS>
-__global__ void __launch_bounds__(kLmThreads, 1)
+__global__ void __launch_bounds__(lm_threads(2 * NPARTS), 1)
 lmhead_umma_pair_kernel(const __grid_constant__ CUtensorMap tmW, const __grid_constant__ CUtensorMap tmH,
                         const LmParams p, int32_t* status) {
+    constexpr int kPar = 2 * NPARTS, kTmaWarpLm = 4 * kPar, kMmaWarpLm = kTmaWarpLm + 1;
     constexpr int kSwz = BK * 2;
     constexpr int kGroup = 8 * kSwz;
     extern __shared__ uint8_t smem_raw[];
@@ -433,7 +443,7 @@ lmhead_umma_pair_kernel(const __grid_constant__ CUtensorMap tmW, const __grid_co
     __shared__ __align__(8) uint64_t full_bar[kMaxStages];   // used in the leader: both CTAs' loads
     __shared__ __align__(8) uint64_t empty_bar[kMaxStages];  // in each CTA: stage consumed
     __shared__ __align__(8) uint64_t tmem_full[2];           // in each CTA: accumulator complete
-    __shared__ __align__(8) uint64_t tmem_empty[2];          // used in the leader: 8 epilogue warps done
+    __shared__ __align__(8) uint64_t tmem_empty[2];          // used in the leader: both CTAs' epilogue warps done
     __shared__ uint32_t tmem_base_slot;
     __shared__ int abort_flag;
 
@@ -448,7 +458,7 @@ lmhead_umma_pair_kernel(const __grid_constant__ CUtensorMap tmW, const __grid_co
     if (threadIdx.x == 0) {
         abort_flag = 0;
         for (int s = 0; s < p.stages; ++s) { mbar_init(&full_bar[s], 1); mbar_init(&empty_bar[s], 1); }
-        for (int b = 0; b < 2; ++b) { mbar_init(&tmem_full[b], 1); mbar_init(&tmem_empty[b], 2 * kEpiWarps); }
+        for (int b = 0; b < 2; ++b) { mbar_init(&tmem_full[b], 1); mbar_init(&tmem_empty[b], 8 * kPar); }
         fence_barrier_init();
     }
     if (warp == kTmaWarpLm) {          // a full warp
@@ -529,7 +539,7 @@ lmhead_umma_pair_kernel(const __grid_constant__ CUtensorMap tmW, const __grid_co
             if (!ok) set_status(status, SD_ERR_TIMEOUT);
         }
     } else {
-        // ------------------------------------------------ epilogue warps 0..7
+        // ------------------------------------------------ epilogue warps
         const int quad = warp & 3, par = warp >> 2;
         EpiState e;
         epi_init(e);
@@ -540,14 +550,14 @@ lmhead_umma_pair_kernel(const __grid_constant__ CUtensorMap tmW, const __grid_co
             if (!mbar_wait(&tmem_full[buf], use & 1u, &abort_flag, p.wait_cycles)) { ok = false; break; }
             tc_fence_after_sync();
             const int v_base = ((pair + t * n_pairs) * 2 + (int)rank) * kBM + quad * 32;
-            epi_tile(p, e, tmem_base + ((uint32_t)(quad * 32) << 16) + (uint32_t)(buf * p.buf_stride), v_base, lane, par);
+            epi_tile<kPar>(p, e, tmem_base + ((uint32_t)(quad * 32) << 16) + (uint32_t)(buf * p.buf_stride), v_base, lane, par);
             tc_fence_before_sync();
             __syncwarp();
             // (the accumulator reads above have completed: tcgen05.wait::ld; a CTA-scope release is enough,
             //  and a cluster-scope one costs on the order of a thousand cycles per arrival)
             if (lane == 0) mbar_arrive_remote_light(map_dsmem(smem_u32(&tmem_empty[buf]), 0));
         }
-        epi_finish(p, e, smem, quad, par, lane, ok, status);
+        epi_finish<kPar>(p, e, smem, quad, par, lane, ok, status);
     }
     tc_fence_before_sync();
     __syncthreads();
@@ -674,13 +684,13 @@ static sd_status launch_lmhead_impl(const void* hidden, const void* W, int M, in
             auto kern = (bk == 64) ? (p.n_parts == 2 ? lmhead_umma_pair_kernel<64, 2> : lmhead_umma_pair_kernel<64, 1>)
                                    : (p.n_parts == 2 ? lmhead_umma_pair_kernel<32, 2> : lmhead_umma_pair_kernel<32, 1>);
             if (!allow_dynamic_smem(kern, (int)dyn)) return SD_ERR_CUDA;
-            const sd_status ls = launch_dependent(kern, dim3(grid), kLmThreads, dyn, 2, st, tmW, tmH, p, dev_status);
+            const sd_status ls = launch_dependent(kern, dim3(grid), lm_threads(2 * p.n_parts), dyn, 2, st, tmW, tmH, p, dev_status);
             if (ls != SD_OK) return ls;
         } else {
             if (grid > p.n_tiles) grid = p.n_tiles;
             auto kern = (bk == 64) ? lmhead_umma_kernel<64> : lmhead_umma_kernel<32>;
             if (!allow_dynamic_smem(kern, (int)dyn)) return SD_ERR_CUDA;
-            const sd_status ls = launch_dependent(kern, dim3(grid), kLmThreads, dyn, 1, st, tmW, tmH, p, dev_status);
+            const sd_status ls = launch_dependent(kern, dim3(grid), lm_threads(4), dyn, 1, st, tmW, tmH, p, dev_status);
             if (ls != SD_OK) return ls;
         }
         if (tiles_only_ctas) {
