@@ -41,6 +41,10 @@ struct LmParams {
     int acc_bufs;      // 1 or 2 accumulator buffers
     int tmem_cols;     // allocation (power of two >= 32)
     int n_tiles;       // vocabulary tiles
+    // Pair kernel: the tiles left over after whole rounds of all pairs, cut along the hidden rows (see plan_slices)
+    int rounds;        // whole rounds, if the rest is cut (slices > 0)
+    int slices;        // pieces of such a tile, 0: none is cut
+    int slice_chunks;  // 32-row chunks of a piece
     int stages;
     int32_t* part_key; // [gridDim.x][kMaxCols] order-preserving integer image of the max logit
     int32_t* part_idx; // [gridDim.x][kMaxCols]
@@ -192,15 +196,16 @@ __device__ __forceinline__ void epi_init(EpiState& e) {
     }
 }
 
-// one accumulator tile (128 vocabulary rows from v_base - 32 * quad on; this warp's 32 of them start at v_base)
+// chunks c_lo .. c_hi - 1 of one accumulator tile (128 vocabulary rows from v_base - 32 * quad on; this warp's 32 of them start at v_base)
 template <int PAR>
-__device__ __forceinline__ void epi_tile(const LmParams& p, EpiState& e, uint32_t taddr, int v_base, int lane, int par) {
+__device__ __forceinline__ void epi_tile(const LmParams& p, EpiState& e, uint32_t taddr, int v_base, int lane, int par,
+                                         int c_lo = 0, int c_hi = kMaxCols / 32) {
     const bool stats = p.c2 > 0.f;
     const bool v_ok = (v_base + lane) < p.V;
 #pragma unroll
     for (int h = 0; h < kEpiChunks; ++h) {
         const int c = PAR * h + par;               // this warp's chunk of each PAR
-        if (c * 32 < p.n_pad) {
+        if (c * 32 < p.n_pad && c >= c_lo && c < c_hi) {
             uint32_t r[32];
             tmem_ld32(taddr + c * 32, r);
             tmem_ld_wait();
@@ -427,10 +432,28 @@ lmhead_umma_kernel(const __grid_constant__ CUtensorMap tmW, const __grid_constan
 // halves against both W slabs and fills the accumulators in both CTAs' TMEM.
 // The hidden matrix is therefore re-read from L2 half as often per W byte.
 // ---------------------------------------------------------------------------
+// What a pair works on: whole tiles first, then (CUT: if there are any) pieces of those left over.
+template <bool CUT>
+struct LmItems {
+    int pair, n_pairs, whole, count, n_chunks;
+    struct Item { int tile, c_lo, c_n; };          // vocabulary tile, and its first 32-row chunk and how many of them
+    __device__ __forceinline__ LmItems(const LmParams& p, int pair_, int n_pairs_) : pair(pair_), n_pairs(n_pairs_) {
+        n_chunks = (p.n_pad + 31) / 32;
+        whole = CUT && p.slices ? p.rounds : (p.n_tiles - pair + n_pairs - 1) / n_pairs;
+        count = whole;
+        if (CUT && p.slices) count += ((p.n_tiles - p.rounds * n_pairs) * p.slices - pair + n_pairs - 1) / n_pairs;
+    }
+    __device__ __forceinline__ Item get(const LmParams& p, int t) const {
+        if (!CUT || t < whole) return {pair + t * n_pairs, 0, n_chunks};
+        const int u = pair + (t - whole) * n_pairs, tile = u / p.slices, c_lo = (u - tile * p.slices) * p.slice_chunks;
+        return {p.rounds * n_pairs + tile, c_lo, min(p.slice_chunks, n_chunks - c_lo)};
+    }
+};
+
 template <int BK, int NPARTS>
 __global__ void __launch_bounds__(lm_threads(2 * NPARTS), 1)
 lmhead_umma_pair_kernel(const __grid_constant__ CUtensorMap tmW, const __grid_constant__ CUtensorMap tmH,
-                        const LmParams p, int32_t* status) {
+                        const __grid_constant__ CUtensorMap tmS, const LmParams p, int32_t* status) {
     constexpr int kPar = 2 * NPARTS, kTmaWarpLm = 4 * kPar, kMmaWarpLm = kTmaWarpLm + 1;
     constexpr int kSwz = BK * 2;
     constexpr int kGroup = 8 * kSwz;
@@ -453,7 +476,8 @@ lmhead_umma_pair_kernel(const __grid_constant__ CUtensorMap tmW, const __grid_co
     const int pair = blockIdx.x >> 1;
     const int n_pairs = gridDim.x >> 1;
     const int kblocks = p.Hd / BK;
-    const int my_tiles = (p.n_tiles - pair + n_pairs - 1) / n_pairs;   // tiles of 256 vocabulary rows
+    constexpr bool kCut = NPARTS == 2;
+    const LmItems<kCut> items(p, pair, n_pairs);                    // tiles of 256 vocabulary rows
 
     if (threadIdx.x == 0) {
         abort_flag = 0;
@@ -481,17 +505,23 @@ lmhead_umma_pair_kernel(const __grid_constant__ CUtensorMap tmW, const __grid_co
             const uint64_t pol_h = policy_evict_last();
             int it = 0;
             bool ok = true;
-            for (int t = 0; t < my_tiles && ok; ++t) {
-                const int v0 = ((pair + t * n_pairs) * 2 + (int)rank) * kBM;
+            for (int t = 0; t < items.count && ok; ++t) {
+                const typename LmItems<kCut>::Item item = items.get(p, t);
+                const bool cut = kCut && t >= items.whole;
+                const int v0 = (item.tile * 2 + (int)rank) * kBM;
+                // a piece: one box of half its hidden rows (of the last piece, which may be smaller, some unused)
+                const int h0 = p.row0 + item.c_lo * 32 + (int)rank * item.c_n * 16;
+                const uint32_t bytes = cut ? (uint32_t)(a_bytes + p.slice_chunks * 16 * kSwz) : (uint32_t)stage_bytes;
                 for (int kb = 0; kb < kblocks; ++kb, ++it) {
                     const int s = it % p.stages;
                     const uint32_t ph = (uint32_t)(it / p.stages) & 1u;
                     if (!mbar_wait(&empty_bar[s], ph ^ 1u, &abort_flag, p.wait_cycles)) { ok = false; break; }
                     uint8_t* a = smem + (size_t)s * stage_bytes;
-                    if (rank == 0) mbar_arrive_expect_tx(&full_bar[s], 2u * (uint32_t)stage_bytes);
+                    if (rank == 0) mbar_arrive_expect_tx(&full_bar[s], 2u * bytes);
                     const uint32_t bar = map_dsmem(smem_u32(&full_bar[s]), 0);     // the leader's barrier
                     tma_load_2d_pair(a, &tmW, kb * BK, v0, bar, pol_w);
-                    for (int part = 0; part < p.n_parts; ++part)
+                    if (cut) tma_load_2d_pair(a + a_bytes, &tmS, kb * BK, h0, bar, pol_h);
+                    else for (int part = 0; part < p.n_parts; ++part)
                         tma_load_2d_pair(a + a_bytes + (size_t)part * half_n * kSwz, &tmH, kb * BK,
                                          p.row0 + part * p.part_n + (int)rank * half_n, bar, pol_h);
                 }
@@ -508,12 +538,33 @@ lmhead_umma_pair_kernel(const __grid_constant__ CUtensorMap tmW, const __grid_co
             const uint32_t part_step = (uint32_t)(half_n * kSwz) >> 4;   // next part's B rows, in descriptor units
             int it = 0;
             bool ok = true;
-            for (int t = 0; t < my_tiles && ok; ++t) {
+            for (int t = 0; t < items.count && ok; ++t) {
                 const int buf = t % p.acc_bufs;
                 const uint32_t use = (uint32_t)(t / p.acc_bufs);
                 if (!mbar_wait(&tmem_empty[buf], (use & 1u) ^ 1u, &abort_flag, p.wait_cycles)) { ok = false; break; }
                 tc_fence_after_sync();
                 const uint32_t d0 = tmem_base + (uint32_t)(buf * p.buf_stride);
+                if (kCut && t >= items.whole) {               // a piece of a tile: one MMA over its hidden rows
+                    const typename LmItems<kCut>::Item item = items.get(p, t);
+                    const uint32_t idesc_cut = make_idesc_bf16(2 * kBM, item.c_n * 32, false, false);
+                    const uint32_t d = d0 + (uint32_t)(item.c_lo * 32);
+                    for (int kb = 0; kb < kblocks; ++kb, ++it) {
+                        const int s = it % p.stages;
+                        const uint32_t ph = (uint32_t)(it / p.stages) & 1u;
+                        if (!mbar_wait(&full_bar[s], ph, &abort_flag, p.wait_cycles)) { ok = false; break; }
+                        tc_fence_after_sync();
+                        const uint32_t a_addr = smem_u32(smem + (size_t)s * stage_bytes);
+                        const uint64_t adesc0 = make_smem_desc(a_addr, 16, kGroup, kSwz);
+                        const uint64_t bdesc0 = make_smem_desc(a_addr + (uint32_t)a_bytes, 16, kGroup, kSwz);
+                        const uint32_t first = (kb != 0) ? 1u : 0u;
+#pragma unroll
+                        for (int k = 0; k < BK / 16; ++k)
+                            mma_ss_pair(d, adesc0 + (uint64_t)(k * 2), bdesc0 + (uint64_t)(k * 2), idesc_cut, k != 0 ? 1u : first);
+                        mma_commit_pair(&empty_bar[s], 3);
+                    }
+                    if (ok) mma_commit_pair(&tmem_full[buf], 3);
+                    continue;
+                }
                 for (int kb = 0; kb < kblocks; ++kb, ++it) {
                     const int s = it % p.stages;
                     const uint32_t ph = (uint32_t)(it / p.stages) & 1u;
@@ -544,13 +595,15 @@ lmhead_umma_pair_kernel(const __grid_constant__ CUtensorMap tmW, const __grid_co
         EpiState e;
         epi_init(e);
         bool ok = true;
-        for (int t = 0; t < my_tiles && ok; ++t) {
+        for (int t = 0; t < items.count && ok; ++t) {
             const int buf = t % p.acc_bufs;
             const uint32_t use = (uint32_t)(t / p.acc_bufs);
             if (!mbar_wait(&tmem_full[buf], use & 1u, &abort_flag, p.wait_cycles)) { ok = false; break; }
             tc_fence_after_sync();
-            const int v_base = ((pair + t * n_pairs) * 2 + (int)rank) * kBM + quad * 32;
-            epi_tile<kPar>(p, e, tmem_base + ((uint32_t)(quad * 32) << 16) + (uint32_t)(buf * p.buf_stride), v_base, lane, par);
+            const typename LmItems<kCut>::Item item = items.get(p, t);
+            const int v_base = (item.tile * 2 + (int)rank) * kBM + quad * 32;
+            epi_tile<kPar>(p, e, tmem_base + ((uint32_t)(quad * 32) << 16) + (uint32_t)(buf * p.buf_stride), v_base, lane, par,
+                           kCut ? item.c_lo : 0, kCut ? item.c_lo + item.c_n : kMaxCols / 32);
             tc_fence_before_sync();
             __syncwarp();
             // (the accumulator reads above have completed: tcgen05.wait::ld; a CTA-scope release is enough,
@@ -603,6 +656,26 @@ lmhead_merge_stats_kernel(const int32_t* __restrict__ part_key, const int32_t* _
 }
 
 static int round_up(int x, int m) { return (x + m - 1) / m * m; }
+
+// More than 256 hidden rows, where the tensor cores bound a tile: if few tiles are left over after whole rounds of
+// all pairs (or there are few tiles at all), they are cut along the hidden rows into pieces that are dealt out to
+// all pairs.  A piece costs its share of a tile and about a quarter more: it streams its tile's W through the
+// pair once again, and fills and drains the pipeline.  480 rows: vocabulary of 4099 18.7 -> 15.2 us, 152064
+// (594 tiles, 74 pairs) 375 -> 370; cutting the 49 tiles left over at 50257 took 82 instead of 78, and up to
+// 256 rows, where streaming W is what takes the time, pieces are as slow as whole tiles.
+static bool plan_slices(LmParams* p, int pairs) {
+    const int n_chunks = (p->n_pad + 31) / 32, rest = p->n_tiles % pairs;
+    p->rounds = p->n_tiles / pairs;
+    p->slices = 0;
+    double best = 0.9;                                 // of a round
+    for (int w = 1; w < n_chunks && w <= 8 && rest > 0; ++w) {      // 32 w <= 256: one MMA
+        const int s = (n_chunks + w - 1) / w;
+        const int each = (rest * s + pairs - 1) / pairs;
+        const double cost = each * ((double)w / n_chunks + 0.25);
+        if (cost < best) { best = cost; p->slices = s; p->slice_chunks = w; }
+    }
+    return p->slices > 0;
+}
 
 // tiles_only_ctas != nullptr (M <= 512 required): launch only the tile kernel and report how many
 // CTAs filled the candidate tables; the caller merges them itself (the fused tail kernel).
@@ -663,7 +736,7 @@ static sd_status launch_lmhead_impl(const void* hidden, const void* W, int M, in
         p.group_stats = reinterpret_cast<float2*>(group_stats); p.M_total = M;
         p.logit_out = logit_out;
 
-        CUtensorMap tmW, tmH;
+        CUtensorMap tmW, tmH, tmS;
         if (!encode_tmap_bf16_2d(&tmW, W, (uint64_t)V, (uint64_t)Hd, (uint64_t)Hd * 2, (uint32_t)bk, kBM, bk * 2))
             return SD_ERR_CUDA;
         if (!encode_tmap_bf16_2d(&tmH, hidden, (uint64_t)M, (uint64_t)Hd, (uint64_t)Hd * 2, (uint32_t)bk,
@@ -673,8 +746,15 @@ static sd_status launch_lmhead_impl(const void* hidden, const void* W, int M, in
         const size_t dyn = (size_t)stages * stage_bytes + 1024;
         if (pair) {
             grid &= ~1;
-            if (grid > 2 * p.n_tiles) grid = 2 * p.n_tiles;
-            if (p.n_pad > 128) {
+            p.rounds = p.slices = p.slice_chunks = 0;
+            tmS = tmH;
+            if (p.n_pad > 256 && plan_slices(&p, grid / 2)) {
+                if (!encode_tmap_bf16_2d(&tmS, hidden, (uint64_t)M, (uint64_t)Hd, (uint64_t)Hd * 2, (uint32_t)bk,
+                                         (uint32_t)(p.slice_chunks * 16), bk * 2))
+                    return SD_ERR_CUDA;
+            } else if (grid > 2 * p.n_tiles) {
+                grid = 2 * p.n_tiles;
+            } else if (p.n_pad > 128) {
                 // Tensor-bound sizes: the slowest pair sets the time (ceil(tiles / pairs) rounds), so use
                 // the fewest pairs that still finish in that many rounds; the SMs left idle cost no time
                 // and leave their share of the power budget to the others.
@@ -684,7 +764,7 @@ static sd_status launch_lmhead_impl(const void* hidden, const void* W, int M, in
             auto kern = (bk == 64) ? (p.n_parts == 2 ? lmhead_umma_pair_kernel<64, 2> : lmhead_umma_pair_kernel<64, 1>)
                                    : (p.n_parts == 2 ? lmhead_umma_pair_kernel<32, 2> : lmhead_umma_pair_kernel<32, 1>);
             if (!allow_dynamic_smem(kern, (int)dyn)) return SD_ERR_CUDA;
-            const sd_status ls = launch_dependent(kern, dim3(grid), lm_threads(2 * p.n_parts), dyn, 2, st, tmW, tmH, p, dev_status);
+            const sd_status ls = launch_dependent(kern, dim3(grid), lm_threads(2 * p.n_parts), dyn, 2, st, tmW, tmH, tmS, p, dev_status);
             if (ls != SD_OK) return ls;
         } else {
             if (grid > p.n_tiles) grid = p.n_tiles;
