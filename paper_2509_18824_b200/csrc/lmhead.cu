@@ -500,43 +500,53 @@ lmhead_umma_pair_kernel(const __grid_constant__ CUtensorMap tmW, const __grid_co
 
     if (warp == kTmaWarpLm) {
         // ------------------------------------------------ TMA producer (one per CTA)
-        if (lane == 0) {
-            const uint64_t pol_w = policy_evict_first();
-            const uint64_t pol_h = policy_evict_last();
-            int it = 0;
-            bool ok = true;
-            for (int t = 0; t < items.count && ok; ++t) {
-                const typename LmItems<kCut>::Item item = items.get(p, t);
-                const bool cut = kCut && t >= items.whole;
-                const int v0 = (item.tile * 2 + (int)rank) * kBM;
-                // a piece: one box of half its hidden rows (of the last piece, which may be smaller, some unused)
-                const int h0 = p.row0 + item.c_lo * 32 + (int)rank * item.c_n * 16;
-                const uint32_t bytes = cut ? (uint32_t)(a_bytes + p.slice_chunks * 16 * kSwz) : (uint32_t)stage_bytes;
-                for (int kb = 0; kb < kblocks; ++kb, ++it) {
-                    const int s = it % p.stages;
-                    const uint32_t ph = (uint32_t)(it / p.stages) & 1u;
-                    if (!mbar_wait(&empty_bar[s], ph ^ 1u, &abort_flag, p.wait_cycles)) { ok = false; break; }
-                    uint8_t* a = smem + (size_t)s * stage_bytes;
+        // (A whole warp in uniform control flow, one lane elected around the copies, as in the attention producer:
+        //  and ring slot and phase counted instead of divided out: with a lane-0 branch and two divisions per k-step the
+        //  producer held up every call.  8 rows 178 -> 171 us, 88 rows 183 -> 174, 240 rows 229 -> 212, 300 rows
+        //  285 -> 268.)
+        const uint64_t pol_w = policy_evict_first();
+        const uint64_t pol_h = policy_evict_last();
+        int s = 0;
+        uint32_t ph = 1;                                  // phase of the stage's previous use
+        bool ok = true;
+        for (int t = 0; t < items.count && ok; ++t) {
+            const typename LmItems<kCut>::Item item = items.get(p, t);
+            const bool cut = kCut && t >= items.whole;
+            const int v0 = (item.tile * 2 + (int)rank) * kBM;
+            // a piece: one box of half its hidden rows (of the last piece, which may be smaller, some unused)
+            const int h0 = p.row0 + item.c_lo * 32 + (int)rank * item.c_n * 16;
+            const uint32_t bytes = cut ? (uint32_t)(a_bytes + p.slice_chunks * 16 * kSwz) : (uint32_t)stage_bytes;
+            for (int kb = 0; kb < kblocks; ++kb) {
+                if (!mbar_wait_warp(&empty_bar[s], ph, &abort_flag, p.wait_cycles)) { ok = false; break; }
+                uint8_t* a = smem + (size_t)s * stage_bytes;
+                const uint32_t bar = map_dsmem(smem_u32(&full_bar[s]), 0);     // the leader's barrier
+                if (elect_one()) {
                     if (rank == 0) mbar_arrive_expect_tx(&full_bar[s], 2u * bytes);
-                    const uint32_t bar = map_dsmem(smem_u32(&full_bar[s]), 0);     // the leader's barrier
                     tma_load_2d_pair(a, &tmW, kb * BK, v0, bar, pol_w);
-                    if (cut) tma_load_2d_pair(a + a_bytes, &tmS, kb * BK, h0, bar, pol_h);
-                    else for (int part = 0; part < p.n_parts; ++part)
-                        tma_load_2d_pair(a + a_bytes + (size_t)part * half_n * kSwz, &tmH, kb * BK,
-                                         p.row0 + part * p.part_n + (int)rank * half_n, bar, pol_h);
+                    if (cut) {
+                        tma_load_2d_pair(a + a_bytes, &tmS, kb * BK, h0, bar, pol_h);
+                    } else {
+#pragma unroll
+                        for (int part = 0; part < NPARTS; ++part)
+                            tma_load_2d_pair(a + a_bytes + (size_t)part * half_n * kSwz, &tmH, kb * BK,
+                                             p.row0 + part * p.part_n + (int)rank * half_n, bar, pol_h);
+                    }
                 }
+                __syncwarp();
+                if (++s == p.stages) { s = 0; ph ^= 1u; }
             }
-            if (!ok) {
-                set_status(status, SD_ERR_TIMEOUT);
-                for (int i = 0; i < 1000; ++i) __nanosleep(1000);   // let copies in flight land
-            }
+        }
+        if (!ok) {
+            if (lane == 0) set_status(status, SD_ERR_TIMEOUT);
+            for (int i = 0; i < 1000; ++i) __nanosleep(1000);   // let copies in flight land
         }
     } else if (warp == kMmaWarpLm) {
         // ------------------------------------------------ MMA issuer (leader CTA only; this warp is one thread)
         if (rank == 0) {
             const uint32_t idesc = make_idesc_bf16(2 * kBM, p.part_n, false, false);
             const uint32_t part_step = (uint32_t)(half_n * kSwz) >> 4;   // next part's B rows, in descriptor units
-            int it = 0;
+            int s = 0;
+            uint32_t ph = 0;
             bool ok = true;
             for (int t = 0; t < items.count && ok; ++t) {
                 const int buf = t % p.acc_bufs;
@@ -548,9 +558,7 @@ lmhead_umma_pair_kernel(const __grid_constant__ CUtensorMap tmW, const __grid_co
                     const typename LmItems<kCut>::Item item = items.get(p, t);
                     const uint32_t idesc_cut = make_idesc_bf16(2 * kBM, item.c_n * 32, false, false);
                     const uint32_t d = d0 + (uint32_t)(item.c_lo * 32);
-                    for (int kb = 0; kb < kblocks; ++kb, ++it) {
-                        const int s = it % p.stages;
-                        const uint32_t ph = (uint32_t)(it / p.stages) & 1u;
+                    for (int kb = 0; kb < kblocks; ++kb) {
                         if (!mbar_wait(&full_bar[s], ph, &abort_flag, p.wait_cycles)) { ok = false; break; }
                         tc_fence_after_sync();
                         const uint32_t a_addr = smem_u32(smem + (size_t)s * stage_bytes);
@@ -561,13 +569,12 @@ lmhead_umma_pair_kernel(const __grid_constant__ CUtensorMap tmW, const __grid_co
                         for (int k = 0; k < BK / 16; ++k)
                             mma_ss_pair(d, adesc0 + (uint64_t)(k * 2), bdesc0 + (uint64_t)(k * 2), idesc_cut, k != 0 ? 1u : first);
                         mma_commit_pair(&empty_bar[s], 3);
+                        if (++s == p.stages) { s = 0; ph ^= 1u; }
                     }
                     if (ok) mma_commit_pair(&tmem_full[buf], 3);
                     continue;
                 }
-                for (int kb = 0; kb < kblocks; ++kb, ++it) {
-                    const int s = it % p.stages;
-                    const uint32_t ph = (uint32_t)(it / p.stages) & 1u;
+                for (int kb = 0; kb < kblocks; ++kb) {
                     if (!mbar_wait(&full_bar[s], ph, &abort_flag, p.wait_cycles)) { ok = false; break; }
                     tc_fence_after_sync();
                     // descriptors of the stage; k-steps and parts only move the 16-byte-granular start address
@@ -584,6 +591,7 @@ lmhead_umma_pair_kernel(const __grid_constant__ CUtensorMap tmW, const __grid_co
                         }
                     }
                     mma_commit_pair(&empty_bar[s], 3);        // both CTAs may refill this stage
+                    if (++s == p.stages) { s = 0; ph ^= 1u; }
                 }
                 if (ok) mma_commit_pair(&tmem_full[buf], 3);  // accumulators complete in both CTAs
             }
