@@ -16,8 +16,9 @@ using namespace sm100;
 
 constexpr int kBM = 128;            // vocabulary rows per tile (MMA M)
 // Warps: PAR epilogue warps per TMEM lane quadrant, the 32-column chunks dealt out among them, then the TMA
-// producer warp, then ONE thread: MMA issuer (a one-thread warp keeps the issue loop in uniform control flow, so
-// the MMA descriptors stay in uniform registers).  Up to 256 hidden rows PAR = 2: the accumulator is
+// producer warp, then the MMA issuer.  Both of the pair kernel's are whole warps in uniform control flow with one
+// lane elected around the instructions, which keeps descriptors in uniform registers (a one-thread MMA warp made
+// 8 rows take 171.5 instead of 165.5 us; the single-CTA kernel has one).  Up to 256 hidden rows PAR = 2: the accumulator is
 // double-buffered and the epilogue hides behind the next tile's MMAs.  Above, the one buffer is drained while
 // the tensor cores wait, and the redux and vote latencies of two warps per scheduler left half of the issue
 // slots empty: PAR = 4 takes 480 rows from 434 to 419 us, with statistics and logits from 528 to 493 (below
@@ -451,7 +452,7 @@ struct LmItems {
 };
 
 template <int BK, int NPARTS>
-__global__ void __launch_bounds__(lm_threads(2 * NPARTS), 1)
+__global__ void __launch_bounds__(lm_threads(2 * NPARTS) + 31, 1)
 lmhead_umma_pair_kernel(const __grid_constant__ CUtensorMap tmW, const __grid_constant__ CUtensorMap tmH,
                         const __grid_constant__ CUtensorMap tmS, const LmParams p, int32_t* status) {
     constexpr int kPar = 2 * NPARTS, kTmaWarpLm = 4 * kPar, kMmaWarpLm = kTmaWarpLm + 1;
@@ -541,7 +542,7 @@ lmhead_umma_pair_kernel(const __grid_constant__ CUtensorMap tmW, const __grid_co
             for (int i = 0; i < 1000; ++i) __nanosleep(1000);   // let copies in flight land
         }
     } else if (warp == kMmaWarpLm) {
-        // ------------------------------------------------ MMA issuer (leader CTA only; this warp is one thread)
+        // ------------------------------------------------ MMA issuer (leader CTA only; a whole warp, one lane elected)
         if (rank == 0) {
             const uint32_t idesc = make_idesc_bf16(2 * kBM, p.part_n, false, false);
             const uint32_t part_step = (uint32_t)(half_n * kSwz) >> 4;   // next part's B rows, in descriptor units
@@ -551,7 +552,7 @@ lmhead_umma_pair_kernel(const __grid_constant__ CUtensorMap tmW, const __grid_co
             for (int t = 0; t < items.count && ok; ++t) {
                 const int buf = t % p.acc_bufs;
                 const uint32_t use = (uint32_t)(t / p.acc_bufs);
-                if (!mbar_wait(&tmem_empty[buf], (use & 1u) ^ 1u, &abort_flag, p.wait_cycles)) { ok = false; break; }
+                if (!mbar_wait_warp(&tmem_empty[buf], (use & 1u) ^ 1u, &abort_flag, p.wait_cycles)) { ok = false; break; }
                 tc_fence_after_sync();
                 const uint32_t d0 = tmem_base + (uint32_t)(buf * p.buf_stride);
                 if (kCut && t >= items.whole) {               // a piece of a tile: one MMA over its hidden rows
@@ -559,43 +560,50 @@ lmhead_umma_pair_kernel(const __grid_constant__ CUtensorMap tmW, const __grid_co
                     const uint32_t idesc_cut = make_idesc_bf16(2 * kBM, item.c_n * 32, false, false);
                     const uint32_t d = d0 + (uint32_t)(item.c_lo * 32);
                     for (int kb = 0; kb < kblocks; ++kb) {
-                        if (!mbar_wait(&full_bar[s], ph, &abort_flag, p.wait_cycles)) { ok = false; break; }
+                        if (!mbar_wait_warp(&full_bar[s], ph, &abort_flag, p.wait_cycles)) { ok = false; break; }
                         tc_fence_after_sync();
                         const uint32_t a_addr = smem_u32(smem + (size_t)s * stage_bytes);
                         const uint64_t adesc0 = make_smem_desc(a_addr, 16, kGroup, kSwz);
                         const uint64_t bdesc0 = make_smem_desc(a_addr + (uint32_t)a_bytes, 16, kGroup, kSwz);
                         const uint32_t first = (kb != 0) ? 1u : 0u;
+                        if (elect_one()) {
 #pragma unroll
-                        for (int k = 0; k < BK / 16; ++k)
-                            mma_ss_pair(d, adesc0 + (uint64_t)(k * 2), bdesc0 + (uint64_t)(k * 2), idesc_cut, k != 0 ? 1u : first);
-                        mma_commit_pair(&empty_bar[s], 3);
+                            for (int k = 0; k < BK / 16; ++k)
+                                mma_ss_pair(d, adesc0 + (uint64_t)(k * 2), bdesc0 + (uint64_t)(k * 2), idesc_cut, k != 0 ? 1u : first);
+                            mma_commit_pair(&empty_bar[s], 3);
+                        }
+                        __syncwarp();
                         if (++s == p.stages) { s = 0; ph ^= 1u; }
                     }
-                    if (ok) mma_commit_pair(&tmem_full[buf], 3);
+                    if (ok && elect_one()) mma_commit_pair(&tmem_full[buf], 3);
+                    __syncwarp();
                     continue;
                 }
                 for (int kb = 0; kb < kblocks; ++kb) {
-                    if (!mbar_wait(&full_bar[s], ph, &abort_flag, p.wait_cycles)) { ok = false; break; }
+                    if (!mbar_wait_warp(&full_bar[s], ph, &abort_flag, p.wait_cycles)) { ok = false; break; }
                     tc_fence_after_sync();
                     // descriptors of the stage; k-steps and parts only move the 16-byte-granular start address
                     const uint32_t a_addr = smem_u32(smem + (size_t)s * stage_bytes);
                     const uint64_t adesc0 = make_smem_desc(a_addr, 16, kGroup, kSwz);
                     const uint64_t bdesc0 = make_smem_desc(a_addr + (uint32_t)a_bytes, 16, kGroup, kSwz);
                     const uint32_t first = (kb != 0) ? 1u : 0u;
+                    if (elect_one()) {
 #pragma unroll
-                    for (int k = 0; k < BK / 16; ++k) {
+                        for (int k = 0; k < BK / 16; ++k) {
 #pragma unroll
-                        for (int part = 0; part < NPARTS; ++part) {
-                            mma_ss_pair(d0 + (uint32_t)(part * p.part_n), adesc0 + (uint64_t)(k * 2),
-                                        bdesc0 + (uint64_t)(part * part_step + k * 2), idesc, k != 0 ? 1u : first);
+                            for (int part = 0; part < NPARTS; ++part)
+                                mma_ss_pair(d0 + (uint32_t)(part * p.part_n), adesc0 + (uint64_t)(k * 2),
+                                            bdesc0 + (uint64_t)(part * part_step + k * 2), idesc, k != 0 ? 1u : first);
                         }
+                        mma_commit_pair(&empty_bar[s], 3);    // both CTAs may refill this stage
                     }
-                    mma_commit_pair(&empty_bar[s], 3);        // both CTAs may refill this stage
+                    __syncwarp();
                     if (++s == p.stages) { s = 0; ph ^= 1u; }
                 }
-                if (ok) mma_commit_pair(&tmem_full[buf], 3);  // accumulators complete in both CTAs
+                if (ok && elect_one()) mma_commit_pair(&tmem_full[buf], 3);  // accumulators complete in both CTAs
             }
-            if (!ok) set_status(status, SD_ERR_TIMEOUT);
+            __syncwarp();
+            if (!ok && lane == 0) set_status(status, SD_ERR_TIMEOUT);
         }
     } else {
         // ------------------------------------------------ epilogue warps
@@ -762,17 +770,19 @@ static sd_status launch_lmhead_impl(const void* hidden, const void* W, int M, in
                     return SD_ERR_CUDA;
             } else if (grid > 2 * p.n_tiles) {
                 grid = 2 * p.n_tiles;
-            } else if (p.n_pad > 128) {
-                // Tensor-bound sizes: the slowest pair sets the time (ceil(tiles / pairs) rounds), so use
-                // the fewest pairs that still finish in that many rounds; the SMs left idle cost no time
-                // and leave their share of the power budget to the others.
-                const int rounds = (p.n_tiles + grid / 2 - 1) / (grid / 2);
-                grid = 2 * ((p.n_tiles + rounds - 1) / rounds);
+            } else {
+                // The slowest pair sets the time (ceil(tiles / pairs) rounds), so use the fewest pairs that still
+                // finish in that many rounds; the SMs left idle cost no time and leave their share of the power
+                // budget to the others.  Up to 128 rows, where W's stream bounds the call, only if otherwise most
+                // pairs would idle through a last round of several: 594 tiles of 256 rows on 66 instead of 74
+                // pairs 166 -> 161 us at 8 rows, 175 -> 169 at 144, but 125 tiles on 63 pairs 43.7 -> 44.4.
+                const int pairs = grid / 2, rounds = (p.n_tiles + pairs - 1) / pairs;
+                if (p.n_pad > 128 || (rounds > 3 && 2 * (p.n_tiles % pairs) <= pairs)) grid = 2 * ((p.n_tiles + rounds - 1) / rounds);
             }
             auto kern = (bk == 64) ? (p.n_parts == 2 ? lmhead_umma_pair_kernel<64, 2> : lmhead_umma_pair_kernel<64, 1>)
                                    : (p.n_parts == 2 ? lmhead_umma_pair_kernel<32, 2> : lmhead_umma_pair_kernel<32, 1>);
             if (!allow_dynamic_smem(kern, (int)dyn)) return SD_ERR_CUDA;
-            const sd_status ls = launch_dependent(kern, dim3(grid), lm_threads(2 * p.n_parts), dyn, 2, st, tmW, tmH, tmS, p, dev_status);
+            const sd_status ls = launch_dependent(kern, dim3(grid), lm_threads(2 * p.n_parts) + 31, dyn, 2, st, tmW, tmH, tmS, p, dev_status);
             if (ls != SD_OK) return ls;
         } else {
             if (grid > p.n_tiles) grid = p.n_tiles;
