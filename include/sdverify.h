@@ -363,7 +363,7 @@ sd_status sd_accept_tree_sampled(const sd_batch *batch, const void *hidden, cons
  *            sequence's walk stops is read, and only if a draft was rejected there
  *   u, w   : dev f32 [B][T_max] and [B], uniform numbers in [0, 1)
  *   workspace : at least sd_workspace_bytes(batch, B * T_max, V)
- * Without `logits` the stop nodes' rows go through the LM head once more (their
+ * With `logits` and V <= 163840 everything is one launch.  Without `logits` the stop nodes' rows go through the LM head once more (their
  * probabilities over the vocabulary, B x V floats in the workspace, are then the only
  * logits-sized data that reach memory).  A tree that branches stores SD_ERR_UNSUPPORTED, a bad tree
  * SD_ERR_INVALID_TREE, a draft token outside [0, V) SD_ERR_BOUNDS (through
@@ -397,7 +397,7 @@ sd_status sd_accept_chain_sampled(const sd_batch *batch, const void *hidden, con
  *   q_rows      : dev f32 [B][T_max][V], row [b][i] = q_i (rows of nodes the walk visits are read)
  *   u, w        : dev f32 [B][T_max] and [B], uniform numbers in [0, 1)
  * Outputs as sd_accept_tree.  One cluster of eight CTAs per sequence keeps p_i and q_i
- * of the current node in shared memory (V <= 163840, else SD_ERR_UNSUPPORTED before
+ * of the current node in registers (V <= 163840, else SD_ERR_UNSUPPORTED before
  * anything is launched); every rejection costs one reduction over the vocabulary.
  * A bad tree stores SD_ERR_INVALID_TREE, a draft token outside [0, V) SD_ERR_BOUNDS
  * (n_acc[b] = 0 in both cases).  Arithmetic: fp32, sums in a fixed order.
