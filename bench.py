@@ -36,7 +36,7 @@ import numpy as np
 ROOT = os.path.dirname(os.path.abspath(__file__))
 sys.path.insert(0, ROOT)
 
-# dram__bytes_read.sum + dram__bytes_write.sum of one single-layer launch of attn_umma_kernel, from the ncu
+# dram__bytes_read.sum + dram__bytes_write.sum of one single-layer launch of attn_wide_kernel, from the ncu
 # capture summarised under profiles/.  Set an entry to None whenever the kernel changes until the counters
 # are retaken.
 ATTENTION_DRAM_BYTES_PER_LAUNCH = {"c5": 75.0e6}
@@ -380,7 +380,7 @@ def main():
         lm_s = per_call_ms["tail"] * 1e-3
         lm_tflops = work["lm_flops"] / lm_s / 1e12
         traffic = ATTENTION_DRAM_BYTES_PER_LAUNCH.get(args.config)
-        roofline = {"kernel": "sd_verify_attention, one layer per launch (attn_umma_kernel<1>)", "bound": "tensor",
+        roofline = {"kernel": "sd_verify_attention, one layer per launch (attn_wide_kernel<1>)", "bound": "tensor",
                     "achieved": att_tflops, "peak": peaks["tensor_sustained"], "unit": "TFLOP/s",
                     "frac": att_tflops / peaks["tensor_sustained"],
                     "frac_of_burst_peak": att_tflops / peaks["tensor_burst"], "burst_peak": peaks["tensor_burst"],
