@@ -145,8 +145,8 @@ attn_umma_kernel(const __grid_constant__ AttnLayers<NL> layers, const sd_batch b
     // key tiles of this CTA: cache blocks [t0, t1) and, for the last chunk, the tree tile
     if ((len + kKeyTile - 1) / kKeyTile > bt.max_blocks_per_seq && threadIdx.x == 0)
         set_status(status, SD_ERR_BOUNDS);                 // the block table does not cover this length
-    const int n_chunks = chunks_of(min((len + kKeyTile - 1) / kKeyTile, bt.max_blocks_per_seq), plan.n_chunks, plan.chunk_blocks);   // of this sequence; CTAs beyond have nothing to do
-    const ChunkRange cr = chunk_range(len, bt.max_blocks_per_seq, n_chunks, chunk);
+    const ChunkRange cr = chunk_range(plan, len, bt.max_blocks_per_seq, chunk);
+    const int n_chunks = cr.n_chunks;                      // of this sequence; CTAs beyond have nothing to do
     const int tiles_total = cr.tiles_total, tpc = cr.tpc, t0 = cr.t0, t1 = cr.t1;
     const bool has_tree = (chunk == n_chunks - 1);
     const int nt = (t1 - t0) + (has_tree ? 1 : 0);
@@ -581,10 +581,17 @@ static bool wide_plan(AttnPlan* p, const sd_batch& bt, int dev, int sms, const T
         const double rounds = base <= 2 * sms ? 1.0 : (double)base / (2 * sms) + 0.25;     // a partial round, cut into chunks
         if (best > 1.05 * rounds * (13.0 + 0.9 * blocks)) return false;
     }
-    p->n_chunks = n;
-    // Shorter sequences are cut into fewer chunks where all clusters run at once; in several rounds the CTAs that
-    // leave would still hold back the next cluster (half-empty pairs halved the machine).
-    p->chunk_blocks = n_rounds == 1 ? (blocks + n - 1) / n : 0;
+    // Where all clusters run at once, a sequence so short that the merge costs more than the split saves stays whole
+    // (us per call uncut, in two, three, four, six chunks, one sequence and 60 nodes: 4 blocks 7.1 7.6 7.6 7.6, 6 blocks
+    // 8.1 8.2 8.1 7.9 7.9, 8 blocks 8.6 8.6 8.0 7.9 7.7, 12 blocks 10.0 9.5 9.0 9.0 8.1); the others are cut as far as the
+    // cluster goes.  This must not follow from the table's width, of which a chunk's size was once a share: then one
+    // sequence of 2048 tokens in a table of 512 blocks ran whole (16.3 us, now 9.8; 10.2 in a table of 33), eight chains
+    // of 4096 took 28.7 (17.0), one of 8192 in 2048 blocks 50.7 (16.0).  The other side: in a batch of very different
+    // lengths the short sequences take memory bandwidth from the longest (eight chains over 200 to 8192 tokens
+    // 20.4 us, 19.8 with chunks as long as the longest's; 100 to 3000 tokens 11.4 against 11.7).
+    // In several rounds every sequence is cut alike: the CTAs that leave would still hold back the next cluster
+    // (half-empty pairs halved the machine).
+    p->set_chunks(n, n_rounds > 1 ? -1 : (knobs.chunks > 0 ? 0 : (n == 2 ? 10 : 5)));
     p->ranked = (bt.B > 1 && bt.B <= 64 && base * n > sms) ? 1 : 0;
     return true;
 }
@@ -620,8 +627,7 @@ static void narrow_plan(AttnPlan* plan, const sd_batch& bt, int sms, const TestK
         if (cost < best - 1e-9) { best = cost; n = c; }
     }
     if (knobs.chunks > 0 && knobs.chunks <= max_tiles && (knobs.chunks & (knobs.chunks - 1)) == 0) n = knobs.chunks;     // test hook
-    p.n_chunks = n;
-    p.chunk_blocks = 0;
+    p.set_chunks(n, -1);
     p.ranked = (bt.B > 1 && bt.B <= 64 && (long long)base * n > slots) ? 1 : 0;
 }
 
@@ -653,7 +659,7 @@ static sd_status launch_group(const AttnLayers<NL>& layers, int n_layers, const 
             const sd_status s = launch_rows1<NL>(layers, bt, scale, plan, z_main, dev_status, st);
             if (s != SD_OK) return s;
             plan.z0 = z_main;
-            plan.n_chunks = c;
+            plan.set_chunks(c, -1);
             return launch_rows1<NL>(layers, bt, scale, plan, z_rest, dev_status, st);
         }
     }

@@ -71,26 +71,21 @@ __device__ __forceinline__ void exp_pack(const uint32_t (&r)[N], uint64_t scale2
     }
 }
 
-// key chunks of a sequence (the last one also takes the tree's keys): the smallest number, up to
-// n_chunks, whose chunks have at most chunk_blocks cache blocks
-__device__ __forceinline__ int chunks_of(int blocks, int n_chunks, int chunk_blocks) {
-    int c = 1;
-    while (c < n_chunks && blocks > c * chunk_blocks) ++c;
-    return c;
-}
 // rows of a row tile that each of its chunks' CTAs finishes: in eights, so that what a warp sends to one CTA
 // are whole 128-byte lines (the last CTAs may have fewer, or none)
 __host__ __device__ constexpr int rows_per_chunk(int n_chunks) { return ((kRowTile + n_chunks - 1) / n_chunks + 7) & ~7; }
 
 struct AttnPlan {
-    int n_chunks;      // CTAs per row tile along the keys (a cluster): key chunks of the longest sequences
-    int chunk_blocks;  // cache blocks of such a chunk; a shorter sequence is cut into fewer chunks
+    int n_chunks;      // CTAs per row tile along the keys (a cluster): the most chunks that a sequence's keys are cut into
+    int whole_blocks;  // sequences of at most so many cache blocks stay whole; -1: every one is cut into n_chunks
+    uint32_t chunk_magic;    // ceil(2^32 / n_chunks): x / n_chunks for x below 2^29 (n_chunks > 1)
     int rows;          // T_max * G
     int tile_nodes;    // tree nodes of a row tile: its rows are whole nodes, the query heads of one KV head each
     int tile_rows;     // tile_nodes * G <= 128
     int row_tiles;
     int g_magic;       // ceil(65536 / G): row / G for rows below 64 * 8
     __host__ __device__ __forceinline__ int node_of(int row) const { return (row * g_magic) >> 16; }
+    void set_chunks(int n, int whole) { n_chunks = n; whole_blocks = whole; chunk_magic = (uint32_t)((0x100000000ull + n - 1) / n); }
     int n_layers;      // layers of this launch
     int ranked;        // dispatch the sequences longest first (only matters when the grid runs in several waves)
     int z0;            // first (sequence rank, layer, KV head) index of this launch: blockIdx.z counts from here
@@ -118,12 +113,21 @@ __device__ __forceinline__ int sequence_of_rank(const sd_batch& bt, int rank, in
     return s_seq;
 }
 
-// cache blocks [t0, t1) of one key chunk of a sequence
-struct ChunkRange { int tiles_total, tpc, t0, t1; };
-__device__ __forceinline__ ChunkRange chunk_range(int len, int max_blocks, int n_chunks, int chunk) {
+// The key chunks of a sequence (the last one also takes the tree's keys), and the cache blocks [t0, t1) of one of them.
+// Where sequences may stay whole, the others are cut into the smallest number of chunks, up to n_chunks, whose longest
+// is as short as n_chunks make it.  All of it follows from the sequence's own length: the block table may be far
+// wider than any sequence of the batch.
+struct ChunkRange { int n_chunks, tiles_total, tpc, t0, t1; };
+__device__ __forceinline__ ChunkRange chunk_range(const AttnPlan& plan, int len, int max_blocks, int chunk) {
     ChunkRange r;
     r.tiles_total = min((len + kBlock - 1) / kBlock, max_blocks);
-    r.tpc = (r.tiles_total + n_chunks - 1) / n_chunks;
+    const bool whole = plan.n_chunks == 1 || r.tiles_total <= max(plan.whole_blocks, 0);
+    r.tpc = whole ? r.tiles_total : (int)__umulhi((uint32_t)(r.tiles_total + plan.n_chunks - 1), plan.chunk_magic);
+    r.n_chunks = whole ? 1 : plan.n_chunks;
+    if (plan.whole_blocks >= 0 && !whole) {
+        r.n_chunks = 2;
+        while (r.n_chunks * r.tpc < r.tiles_total) ++r.n_chunks;
+    }
     r.t0 = min(chunk * r.tpc, r.tiles_total);
     r.t1 = min(r.t0 + r.tpc, r.tiles_total);
     return r;

@@ -75,8 +75,8 @@ __device__ __forceinline__ WideWork wide_work(const sd_batch& bt, const AttnPlan
     WideWork w;
     w.n = min(max(n, 0), bt.T_max);
     w.len = min(max(len, 0), 0x7fffffff - kBlock);         // (any number may stand there before the kernel ahead is done)
-    w.n_chunks = chunks_of(min((w.len + kBlock - 1) / kBlock, bt.max_blocks_per_seq), plan.n_chunks, plan.chunk_blocks);
-    const ChunkRange cr = chunk_range(w.len, bt.max_blocks_per_seq, w.n_chunks, chunk);
+    const ChunkRange cr = chunk_range(plan, w.len, bt.max_blocks_per_seq, chunk);
+    w.n_chunks = cr.n_chunks;
     w.tiles_total = cr.tiles_total;
     w.tpc = cr.tpc;
     w.t0 = cr.t0;

@@ -1,6 +1,8 @@
 """GPU: attention at the edges of the 128-key tiles and key chunks (odd and even block counts, half tiles,
 sequences of one batch cut into different numbers of chunks), and scores that rise so far above the first
 tile's that the rows' reference has to be raised, through both kernels."""
+import copy
+
 import numpy as np
 import pytest
 import torch
@@ -104,3 +106,46 @@ def test_lengths_written_by_the_kernel_ahead(stale):
         assert int(st.item()) == 0 and (n_acc == 1).all()
         np.testing.assert_array_equal(out.float().cpu().numpy(), ref)
         np.testing.assert_array_equal(lse.cpu().numpy(), ref_lse)
+
+
+def in_table_of(p, width):
+    """The same problem in a block table of that width (as a server keeps it); nothing may look behind the sequences."""
+    q = copy.copy(p)
+    q.block_table = np.full((p.B, width), 1 << 20, dtype=np.int32)
+    q.block_table[:, :p.block_table.shape[1]] = p.block_table
+    q.max_blocks = width
+    return q
+
+
+@pytest.mark.parametrize("lens", [(2048,), (700, 2300), (4000, 130, 1000)])
+def test_split_follows_the_length_and_not_the_table(monkeypatch, lens):
+    p = problem(sum(lens), lens)
+    cut = {}
+    for chunks in range(1, 9):
+        monkeypatch.setenv("SDV_TEST_CHUNKS", str(chunks))
+        out, lse, status = gpu_attention(p)
+        assert status == 0
+        for width in (200, 512):                          # the same bits whatever the width
+            wide, wide_lse, status = gpu_attention(in_table_of(p, width))
+            assert status == 0
+            np.testing.assert_array_equal(wide, out)
+            np.testing.assert_array_equal(wide_lse, lse)
+        cut[chunks] = out
+    monkeypatch.delenv("SDV_TEST_CHUNKS")
+    out, _, status = gpu_attention(in_table_of(p, 512))
+    assert status == 0
+    b = int(np.argmax(lens))                              # unforced: the long sequence is cut into as many chunks as pay
+    same = [c for c in cut if np.array_equal(out[b], cut[c][b])]
+    assert same and max(same) >= 4, same
+
+
+@pytest.mark.parametrize("blocks", [0, 1, 5, 6, 10, 11, 12])
+@pytest.mark.parametrize("B", [1, 8, 37])
+def test_short_sequences_in_a_wide_table(blocks, B):
+    """Around the lengths from which a sequence is cut, with one to eight chunks (B = 1, 8), and in several rounds."""
+    p = problem(blocks + B, tuple(max(0, blocks * 64 - (b % 3)) for b in range(B)))
+    out, lse, status = gpu_attention(in_table_of(p, 300))
+    assert status == 0
+    ref, rlse = oracle.attention(oracle.Geometry.of(p), p.k_cache, p.v_cache, p.q, p.k_tree, p.v_tree, p.scale)
+    check_attention(out, ref, f"blocks={blocks} B={B}")
+    np.testing.assert_allclose(lse, rlse, rtol=2e-3, atol=2e-3)
