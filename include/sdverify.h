@@ -26,7 +26,8 @@
  *     is launched.  Problems only visible on the device (bad parent array,
  *     block-table entry out of range, an expired bounded wait) store the first
  *     error code into *dev_status (int32, dev, must be 0 on entry) and the
- *     kernel finishes normally; outputs are unspecified in that case.
+ *     kernel finishes normally; outputs are unspecified in that case.  (The one call
+ *     without a status word, sd_draft_feature_attention, writes NaN instead.)
  *   - Same inputs give bit-identical outputs from run to run.
  *   - All dev pointers must be 16-byte aligned.
  *
@@ -449,7 +450,8 @@ sd_status sd_lmhead_accept_sampled_compact(const sd_batch *batch, const void *hi
  *   k,v : dev bf16 [S][L][D]   the tokens' (projected) layer features; may be the same buffer
  *   out : dev bf16 [S][Q][D]   = [S][Q * D] flattened, as the paper uses it
  * L <= 32, Q <= 8.  fp32 accumulation, bf16 output (round to nearest even).
- * Every K and V row is read once; the call is bound by HBM bandwidth.
+ * Every K and V row is read once; the call is bound by HBM bandwidth.  There is no status
+ * word: should a bounded wait run out, the out rows that were not computed hold NaN (0x7fff).
  */
 sd_status sd_draft_feature_attention(const void *qp, const void *k, const void *v,
                                      int32_t S, int32_t L, int32_t Q, int32_t H, int32_t D,

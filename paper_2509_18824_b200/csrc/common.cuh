@@ -83,8 +83,8 @@ __device__ __forceinline__ void begin_dependent(T&... p) {
 
 // Test hooks, read from the environment at every launch (unset in normal use):
 //   SDV_TEST_WAIT_CYCLES  bound of the kernels' barrier waits in SM cycles (default: about a second)
-//   SDV_TEST_WITHHOLD     1: one role of the tensor-core kernels withholds its first arrival, so that
-//                         a bounded wait runs out and the launch ends with SD_ERR_TIMEOUT
+//   SDV_TEST_WITHHOLD     1: one role of a kernel withholds its first arrival (draft side: some bytes of every copy),
+//                         so that a bounded wait runs out and the launch ends with SD_ERR_TIMEOUT (NaN rows)
 //   SDV_TEST_CHUNKS       1 to 8: key chunks per sequence of single-launch attention calls
 struct TestKnobs { long long wait_cycles; int withhold; int chunks; };
 TestKnobs test_knobs();

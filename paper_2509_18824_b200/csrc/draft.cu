@@ -9,6 +9,7 @@
 // that ldmatrix reads them without bank conflicts) through a ring that keeps the whole shared memory in
 // flight; twelve consumer warps take the tasks in turn.  (A warp that fetched its own task and then worked on
 // it left the memory idle in between: S = 4096, L = 28, 28 heads 325 us.)
+// The call has no status word: a task whose bounded wait runs out gets NaN rows.
 #include "common.cuh"
 #include "sm100.cuh"
 
@@ -42,7 +43,8 @@ __device__ __forceinline__ uint32_t pack_bf16(float lo, float hi) {
 template <bool SAME>
 __global__ void __launch_bounds__(kDraftThreads, 1)
 draft_feature_attention_kernel(const __grid_constant__ CUtensorMap map_k, const __grid_constant__ CUtensorMap map_v,
-                               const uint16_t* qp, long long tasks, int L, int Q, int H, float scale, int stages, uint16_t* out) {
+                               const uint16_t* qp, long long tasks, int L, int Q, int H, float scale, int stages,
+                               int tile_bytes, long long wait_cycles, uint16_t* out) {
     using namespace sm100;
     extern __shared__ uint8_t dsm_raw[];
     uint8_t* ring = reinterpret_cast<uint8_t*>((reinterpret_cast<uintptr_t>(dsm_raw) + 1023) & ~(uintptr_t)1023);
@@ -77,13 +79,10 @@ draft_feature_attention_kernel(const __grid_constant__ CUtensorMap map_k, const 
         int s = (int)(first / H), h = (int)(first - (long long)s * H), slot = 0;
         uint32_t ph = 1;
         for (int i = 0; i < n; ++i) {
-            if (!mbar_wait_warp(&empty[slot], ph, &abort_flag, kWaitCycles)) {
-                for (int z = 0; z < 1000; ++z) __nanosleep(1000);                    // let copies in flight land
-                break;
-            }
+            if (!mbar_wait_warp(&empty[slot], ph, &abort_flag, wait_cycles)) { unwind_pause(&abort_flag); break; }
             uint8_t* dst = ring + slot * kSlot;
             if (elect_one()) {
-                mbar_arrive_expect_tx(&full[slot], (SAME ? 2 : 4) * L * 128);
+                mbar_arrive_expect_tx(&full[slot], tile_bytes);
                 tma_load_3d(dst, &map_k, h * kDh, 0, s, &full[slot], pol);
                 tma_load_3d(dst + kHalf, &map_k, h * kDh + 64, 0, s, &full[slot], pol);
                 if (!SAME) {
@@ -100,7 +99,8 @@ draft_feature_attention_kernel(const __grid_constant__ CUtensorMap map_k, const 
     const int g = lane >> 2, t = lane & 3;                                          // mma fragment coordinates
     const int mi = lane >> 3, r = lane & 7;                                         // ldmatrix: matrix and row of this lane
     const float scale_log2 = scale * 1.4426950408889634f;
-    for (int i = warp; i < n; i += kDraftWarps) {
+    int i = warp;
+    for (; i < n; i += kDraftWarps) {
         const int s = (int)((first + i) / H), h = (int)(first + i - (long long)s * H);
         const int slot = i % stages;
         const uint32_t ks_addr = smem_u32(ring + slot * kSlot), vs_addr = SAME ? ks_addr : ks_addr + kTile;
@@ -112,8 +112,7 @@ draft_feature_attention_kernel(const __grid_constant__ CUtensorMap map_k, const 
             qa[ks][0] = g < Q ? __ldg(qr + ks * 8) : 0u;
             qa[ks][1] = g < Q ? __ldg(qr + ks * 8 + 4) : 0u;
         }
-        if (!mbar_wait(&full[slot], (uint32_t)(i / stages) & 1u, &abort_flag)) break;
-        __syncwarp();
+        if (!mbar_wait_warp(&full[slot], (uint32_t)(i / stages) & 1u, &abort_flag, wait_cycles)) break;
         // ---- K rows as B fragments (layer 8 * nt + r; 16-byte piece c of a row sits at piece c ^ (row & 7)) and scores S[q][l]
         float sc[4][4];
 #pragma unroll
@@ -182,6 +181,14 @@ draft_feature_attention_kernel(const __grid_constant__ CUtensorMap map_k, const 
                 reinterpret_cast<const uint4*>(s_out[warp])[x];
         __syncwarp();                                                                // s_out is reused by the next task
     }
+    if (i >= n) return;
+    for (; i < n; i += kDraftWarps) {                                                // a wait ran out: this warp's rows from there on
+        const int s = (int)((first + i) / H), h = (int)(first + i - (long long)s * H);
+        for (int x = lane; x < Q * 16; x += 32)
+            reinterpret_cast<uint4*>(out + ((size_t)s * Q + (x >> 4)) * D + (size_t)h * kDh)[x & 15] =
+                make_uint4(0x7fff7fffu, 0x7fff7fffu, 0x7fff7fffu, 0x7fff7fffu);
+    }
+    unwind_pause(&abort_flag);
 }
 
 sd_status launch_draft_feature_attention(const void* qp, const void* k, const void* v, int S, int L, int Q, int H,
@@ -205,9 +212,12 @@ sd_status launch_draft_feature_attention(const void* qp, const void* k, const vo
     const long long most = (tasks + grid - 1) / grid;                 // a CTA's tasks: no more slots than that
     if (stages > most) stages = (int)most;
     const int smem = stages * slot + 1024;
+    const TestKnobs knobs = test_knobs();
     auto kern = same ? draft_feature_attention_kernel<true> : draft_feature_attention_kernel<false>;
     if (!allow_dynamic_smem(kern, smem)) return SD_ERR_CUDA;
-    return launch_dependent(kern, dim3(grid), kDraftThreads, smem, 1, st, mk, mv, qp, tasks, L, Q, H, scale, stages, out);
+    const int tile_bytes = (same ? 2 : 4) * L * 128 + (knobs.withhold ? 16 : 0);       // (withheld: bytes that do not come)
+    return launch_dependent(kern, dim3(grid), kDraftThreads, smem, 1, st, mk, mv, qp, tasks, L, Q, H, scale, stages, tile_bytes,
+                            knobs.wait_cycles, out);
 }
 
 }  // namespace sdv

@@ -58,13 +58,10 @@ __device__ __forceinline__ bool mbar_test_wait(uint64_t* bar, uint32_t parity) {
     return ok != 0;
 }
 
-// Bounded wait: gives up after `limit` SM cycles (about a second by default), or as soon as another
+// Bounded wait: gives up after `limit` SM cycles (see TestKnobs), or as soon as another
 // thread of the CTA has raised *abort_flag.  Returns false when it gave up (and raises the flag
 // itself), so that callers can unwind instead of hanging.
-constexpr long long kWaitCycles = 1ll << 31;   // about a second
-
-__device__ __forceinline__ bool mbar_wait(uint64_t* bar, uint32_t parity, volatile int* abort_flag,
-                                          long long limit = kWaitCycles) {
+__device__ __forceinline__ bool mbar_wait(uint64_t* bar, uint32_t parity, volatile int* abort_flag, long long limit) {
     if (mbar_try_wait(bar, parity)) return true;
     const long long t0 = clock64();
     while (true) {
@@ -96,6 +93,13 @@ __device__ __forceinline__ bool mbar_wait_warp(uint64_t* bar, uint32_t parity, v
             return false;
         }
     }
+}
+
+// Before a CTA whose wait ran out leaves: copies and remote stores on their way to its shared memory land first (about
+// a millisecond, which is far longer than they take).
+__device__ __forceinline__ void unwind_pause(volatile int* abort_flag) {
+    if (*abort_flag)
+        for (int i = 0; i < 1000; ++i) __nanosleep(1000);
 }
 
 // ---------------------------------------------------------------- programmatic dependent launch

@@ -5,13 +5,14 @@ The waits are made to run out from the host side only, through the library's tes
 variables read at every launch): SDV_TEST_WAIT_CYCLES shortens the bound of every barrier wait to about a
 tenth of a millisecond, SDV_TEST_WITHHOLD=1 makes one role skip a single arrival (the softmax warps never
 report their first tile / the MMA thread never reports its first accumulator), so that its consumer waits
-for something that does not come.  Nothing faults, traps or spins without a bound; the grids are one CTA.
+for something that does not come.  Nothing faults, traps or spins without a bound.
 """
 import numpy as np
 import pytest
 import torch
 
 import oracle
+from oracle.draft_attention import feature_attention
 from paper_2509_18824_b200 import binding as sd
 from paper_2509_18824_b200 import workloads as wl
 from gpu_util import gpu_attention, check_attention, gpu_lmhead, check_argmax
@@ -56,3 +57,32 @@ def test_lmhead_wait_runs_out_and_the_next_call_is_fine(monkeypatch):
     am2, mx2 = gpu_lmhead(h, W)
     ram, t1, t2 = oracle.lmhead(h, W)
     check_argmax(am2, mx2, ram, t1, t2)
+
+
+# one task, one per CTA, two per CTA, and thirteen: more than a CTA's ring of separate K and V tiles holds
+@pytest.mark.parametrize("S,L,H", [(1, 28, 1), (18, 3, 8), (37, 32, 8), (481, 5, 4)])
+@pytest.mark.parametrize("same", [False, True])
+def test_draft_wait_runs_out_and_the_next_call_is_fine(monkeypatch, S, L, H, same):
+    g = np.random.default_rng(S)
+    Q, D, scale = 4, H * 128, 1.0 / np.sqrt(128)
+    bf = lambda *shape: wl.f32_to_bf16_bits(g.standard_normal(shape).astype(np.float32))
+    qp, k = bf(Q, D), bf(S, L, D)
+    v = k if same else bf(S, L, D)
+    qd, kd = to_device(qp), to_device(k)
+    vd = kd if same else to_device(v)
+    out = torch.full((S, Q, D), 7.0, dtype=torch.bfloat16, device="cuda")
+
+    def rows():
+        sd.sd_draft_feature_attention(qd, kd, vd, H, scale, out)
+        torch.cuda.synchronize()
+        return out.float().cpu().numpy()
+
+    ref = feature_attention(wl.bf16_bits_to_f64(qp), wl.bf16_bits_to_f64(k), wl.bf16_bits_to_f64(v), H, scale)
+    monkeypatch.setenv("SDV_TEST_WAIT_CYCLES", "200000")
+    monkeypatch.setenv("SDV_TEST_WITHHOLD", "1")
+    assert np.isnan(rows()).all()                                # (every copy waits for bytes that do not come)
+    monkeypatch.delenv("SDV_TEST_WITHHOLD")
+    monkeypatch.delenv("SDV_TEST_WAIT_CYCLES")
+    for _ in range(2):
+        got = rows()
+        assert np.linalg.norm(got - ref) <= 5e-3 * np.linalg.norm(ref)
