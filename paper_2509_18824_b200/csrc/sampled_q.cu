@@ -22,7 +22,9 @@ constexpr int kQThreads = 512;
 constexpr int kQWarps = kQThreads / 32;
 constexpr int kQPer = 40;                              // entries per thread
 constexpr int kQMaxSlice = kQThreads * kQPer;          // vocabulary entries per CTA: V <= 163840
-constexpr long long kQWaitCycles = 1ll << 31;          // about a second
+
+// mute: test hook, the CTA of a cluster that keeps its sums to itself (-1: none)
+struct QWaits { long long cycles; int mute; };
 
 struct QShared {
     uint64_t bar[2];                                   // two exchanges in turn: a CTA may start the next while a peer still
@@ -68,7 +70,8 @@ struct VocabSlice {
 
 // Sum of max(p - a q, 0) over the whole vocabulary, the same bits in every CTA of the cluster; n_red counts the
 // exchanges so far.  sh.cta_sum[(n_red - 1) & 1] keeps the eight parts.  false: a peer's part did not arrive.
-__device__ __forceinline__ bool reduce_all(QShared& sh, const VocabSlice& v, float a, int rank, int tid, int& n_red, float& all) {
+__device__ __forceinline__ bool reduce_all(QShared& sh, const VocabSlice& v, float a, int rank, int tid, const QWaits& waits, int& n_red,
+                                           float& all) {
     const int set = n_red & 1;
     const uint32_t phase = (uint32_t)(n_red >> 1) & 1u;
     ++n_red;
@@ -82,12 +85,12 @@ __device__ __forceinline__ bool reduce_all(QShared& sh, const VocabSlice& v, flo
         if (tid == rank) {
             sh.cta_sum[set][rank] = total;
             sm100::mbar_arrive_expect_tx(&sh.bar[set], (kQCluster - 1) * 4);
-        } else {
+        } else if (rank != waits.mute) {
             sm100::st_async_b32(sm100::map_dsmem(sm100::smem_u32(&sh.cta_sum[set][rank]), (uint32_t)tid), __float_as_uint(total),
                                 sm100::map_dsmem(sm100::smem_u32(&sh.bar[set]), (uint32_t)tid));
         }
     }
-    const bool ok = sm100::mbar_wait_cluster(&sh.bar[set], phase, &sh.abort_flag, kQWaitCycles);
+    const bool ok = sm100::mbar_wait_cluster(&sh.bar[set], phase, &sh.abort_flag, waits.cycles);
     __syncthreads();                                   // (warp_sum may be written again; the abort flag is everybody's)
     all = 0.f;
 #pragma unroll
@@ -161,17 +164,18 @@ __device__ __forceinline__ void q_begin(QShared& sh, int tid) {
     sm100::cluster_arrive_release();
     sm100::cluster_wait_acquire();
 }
-// nobody leaves while a peer may still send to it
-__device__ __forceinline__ void q_end() {
+// nobody leaves while a peer may still send to it, or has sent what was not waited for
+__device__ __forceinline__ void q_end(QShared& sh) {
     __syncwarp();
     sm100::cluster_arrive_relaxed();
     sm100::cluster_wait_acquire();
+    sm100::unwind_pause(&sh.abort_flag);
 }
 
 __global__ void __launch_bounds__(kQThreads, 1)
 tree_walk_q_kernel(sd_batch bt, int V, float inv_temp, const float* lse, const float* logits, const int32_t* draft,
                    const float* q_rows, const float* u, const float* w, int32_t* n_acc, int32_t* path, int32_t* out_tok,
-                   int32_t* new_len, int32_t* status) {
+                   int32_t* new_len, int32_t* status, const QWaits waits) {
     __shared__ QShared sh;
     const int tid = threadIdx.x, lane = tid & 31;
     q_begin(sh, tid);
@@ -197,7 +201,7 @@ tree_walk_q_kernel(sd_batch bt, int V, float inv_temp, const float* lse, const f
     const int bad = n_ok ? sh.bad : (int)SD_ERR_INVALID_TREE;
     if (bad != 0) {                                    // (the same in every CTA)
         if (rank == 0 && tid == 0) { set_status(status, bad); n_acc[b] = 0; }
-        q_end();
+        q_end(sh);
         return;
     }
     const int par0 = lane < n ? sh.par[lane] : -2, par1 = lane + 32 < n ? sh.par[lane + 32] : -2;
@@ -225,13 +229,13 @@ tree_walk_q_kernel(sd_batch bt, int V, float inv_temp, const float* lse, const f
             kids &= kids - 1;
             if (sh.u[c] * bsum * sh.qx[c] < fmaxf(sh.px[c] - a * sh.qx[c], 0.f)) { nxt = c; break; }
             a += bsum;
-            ok = reduce_all(sh, v, a, rank, tid, n_red, bsum);
+            ok = reduce_all(sh, v, a, rank, tid, waits, n_red, bsum);
             summed = true;
             if (!ok) break;
         }
         if (!ok) break;
         if (nxt < 0) {
-            if (!summed) ok = reduce_all(sh, v, a, rank, tid, n_red, bsum);   // nothing rejected here: all of p
+            if (!summed) ok = reduce_all(sh, v, a, rank, tid, waits, n_red, bsum);   // nothing rejected here: all of p
             break;
         }
         if (tid == 0) sh.path[na] = nxt;
@@ -251,7 +255,7 @@ tree_walk_q_kernel(sd_batch bt, int V, float inv_temp, const float* lse, const f
         }
         draw_token(sh, v, a, w[b], bsum, n_red, rank, tid, v0, out_tok + (size_t)b * T + na - 1, status);
     }
-    q_end();
+    q_end(sh);
 }
 
 // Chains: node j's token is kept iff u * q(token) < p(token), p and q behind node j - 1; the walk stops at the
@@ -260,7 +264,7 @@ tree_walk_q_kernel(sd_batch bt, int V, float inv_temp, const float* lse, const f
 __global__ void __launch_bounds__(kQThreads, 1)
 chain_walk_q_logits_kernel(sd_batch bt, int V, float inv_temp, const float* lse, const float* logits, const int32_t* draft,
                            const float* q_tok, const float* q_rows, const float* u, const float* w, int32_t* n_acc, int32_t* path,
-                           int32_t* out_tok, int32_t* new_len, int32_t* status) {
+                           int32_t* out_tok, int32_t* new_len, int32_t* status, const QWaits waits) {
     __shared__ QShared sh;
     __shared__ uint32_t s_rejected[2];
     const int tid = threadIdx.x;
@@ -297,7 +301,7 @@ chain_walk_q_logits_kernel(sd_batch bt, int V, float inv_temp, const float* lse,
     const int bad = n_ok ? sh.bad : (int)SD_ERR_INVALID_TREE;
     if (bad != 0) {                                    // (the same in every CTA)
         if (rank == 0 && tid == 0) { set_status(status, bad); n_acc[b] = 0; }
-        q_end();
+        q_end(sh);
         return;
     }
     const uint32_t lo = s_rejected[0], hi = s_rejected[1];
@@ -314,11 +318,16 @@ chain_walk_q_logits_kernel(sd_batch bt, int V, float inv_temp, const float* lse,
     }
     int n_red = 0;
     float total = 0.f;
-    if (reduce_all(sh, v, a, rank, tid, n_red, total))
+    if (reduce_all(sh, v, a, rank, tid, waits, n_red, total))
         draw_token(sh, v, a, w[b], total, n_red, rank, tid, v0, out_tok + (size_t)b * T + na - 1, status);
     else if (tid == 0)
         set_status(status, SD_ERR_TIMEOUT);
-    q_end();
+    q_end(sh);
+}
+
+static QWaits q_waits() {
+    const TestKnobs knobs = test_knobs();
+    return {knobs.wait_cycles, knobs.withhold ? 1 : -1};
 }
 
 bool q_kernels_hold(int V) { return (V + kQCluster - 1) / kQCluster <= kQMaxSlice; }
@@ -329,7 +338,7 @@ sd_status launch_accept_tree_sampled_q(const sd_batch& bt, int V, float inv_temp
                                        int32_t* dev_status, cudaStream_t st) {
     if (!q_kernels_hold(V)) return SD_ERR_UNSUPPORTED;
     return launch_dependent(tree_walk_q_kernel, dim3(bt.B * kQCluster), kQThreads, 0, kQCluster, st, bt, V, inv_temp, lse, logits, draft,
-                            q_rows, u, w, n_acc, path, out_tok, new_len, dev_status);
+                            q_rows, u, w, n_acc, path, out_tok, new_len, dev_status, q_waits());
 }
 
 sd_status launch_accept_chain_logits(const sd_batch& bt, int V, float inv_temp, const float* lse, const float* logits,
@@ -337,7 +346,7 @@ sd_status launch_accept_chain_logits(const sd_batch& bt, int V, float inv_temp, 
                                      int32_t* n_acc, int32_t* path, int32_t* out_tok, int32_t* new_len, int32_t* dev_status,
                                      cudaStream_t st) {
     return launch_dependent(chain_walk_q_logits_kernel, dim3(bt.B * kQCluster), kQThreads, 0, kQCluster, st, bt, V, inv_temp, lse, logits,
-                            draft, q_tok, q_rows, u, w, n_acc, path, out_tok, new_len, dev_status);
+                            draft, q_tok, q_rows, u, w, n_acc, path, out_tok, new_len, dev_status, q_waits());
 }
 
 }  // namespace sdv

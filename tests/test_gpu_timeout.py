@@ -12,11 +12,14 @@ import pytest
 import torch
 
 import oracle
+from oracle import sampling as smp
 from oracle.draft_attention import feature_attention
 from paper_2509_18824_b200 import binding as sd
 from paper_2509_18824_b200 import workloads as wl
 from gpu_util import gpu_attention, check_attention, gpu_lmhead, check_argmax
 from paper_2509_18824_b200.step import to_device
+from test_gpu_sampled import (decisive_chain_inputs, decisive_tree_inputs, drafted_chain, drafted_tree, run_chain_q,
+                              run_tree_q)
 
 pytestmark = pytest.mark.gpu
 
@@ -86,3 +89,45 @@ def test_draft_wait_runs_out_and_the_next_call_is_fine(monkeypatch, S, L, H, sam
     for _ in range(2):
         got = rows()
         assert np.linalg.norm(got - ref) <= 5e-3 * np.linalg.norm(ref)
+
+
+def with_short_waits(monkeypatch, fn):
+    """fn with the hooks set around it only (the calls in front of it are ordinary ones)."""
+    def call(*args, **kw):
+        with monkeypatch.context() as m:
+            m.setenv("SDV_TEST_WAIT_CYCLES", "200000")
+            m.setenv("SDV_TEST_WITHHOLD", "1")
+            fn(*args, **kw)
+    return call
+
+
+@pytest.mark.parametrize("cfg,over", [("c1", dict(V=1000, Hd=64)), ("c4", dict(L=1, V=4099, Hd=64, prefix_range=(40, 300)))])
+def test_sampled_tree_wait_runs_out_and_the_next_call_is_fine(monkeypatch, cfg, over):
+    """One CTA of each cluster keeps its sums to itself: the others' exchange runs out."""
+    w = wl.make(cfg, attention=False, hidden_gain=24.0, **over)
+    lg = oracle.logits(w.hidden, w.W)
+    q, tok = drafted_tree(w, lg, 2.0, 0.8, 3)
+    u, wv, ref_n, ref_path, ref_out, _ = decisive_tree_inputs(w, tok, q, lg, 2.0, np.random.default_rng(4))
+    with monkeypatch.context() as m:
+        m.setattr(sd, "sd_accept_tree_sampled_q", with_short_waits(m, sd.sd_accept_tree_sampled_q))
+        assert run_tree_q(w, tok, q, 2.0, u, wv)[-1] == sd.SD_ERR_TIMEOUT
+    n_acc, path, out_tok, _, status = run_tree_q(w, tok, q, 2.0, u, wv)
+    assert status == 0
+    for got, ref in ((n_acc, ref_n), (path, ref_path), (out_tok, ref_out)):
+        np.testing.assert_array_equal(got, ref)
+
+
+@pytest.mark.parametrize("B", [1, 16])
+def test_sampled_chain_wait_runs_out_and_the_next_call_is_fine(monkeypatch, B):
+    w = wl.make("chain11", attention=False, hidden_gain=24.0, L=1, V=3000, Hd=128, prefix=70, B=B)
+    lg = oracle.logits(w.hidden, w.W)
+    q, tok, q_tok = drafted_chain(w, lg, 2.5, 0.6, 3)
+    p, _ = smp.softmax_rows(lg, 2.5)
+    u, wv, ref_n, ref_out = decisive_chain_inputs(w, tok, q, lambda r: p[r], np.random.default_rng(4))
+    with monkeypatch.context() as m:
+        m.setattr(sd, "sd_accept_chain_sampled", with_short_waits(m, sd.sd_accept_chain_sampled))
+        assert run_chain_q(w, tok, q, q_tok, 2.5, u, wv, keep_logits=True)[-1] == sd.SD_ERR_TIMEOUT
+    n_acc, _, out_tok, _, status = run_chain_q(w, tok, q, q_tok, 2.5, u, wv, keep_logits=True)
+    assert status == 0
+    np.testing.assert_array_equal(n_acc, ref_n)
+    np.testing.assert_array_equal(out_tok, ref_out)
