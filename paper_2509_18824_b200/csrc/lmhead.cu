@@ -64,7 +64,7 @@ struct LmParams {
     const float* col_lse;   // [rows of the call]
     float inv_temp;
     long long wait_cycles;  // bound of every barrier wait, in SM cycles
-    int withhold;           // test hook (single-CTA kernel): the first tile's "accumulator complete" is never signalled
+    int withhold;           // test hook: the first tile's "accumulator complete" is never signalled
 };
 
 size_t lmhead_workspace_bytes(int M, int V) {
@@ -468,6 +468,7 @@ lmhead_umma_pair_kernel(const __grid_constant__ CUtensorMap tmW, const __grid_co
     __shared__ __align__(8) uint64_t empty_bar[kMaxStages];  // in each CTA: stage consumed
     __shared__ __align__(8) uint64_t tmem_full[2];           // in each CTA: accumulator complete
     __shared__ __align__(8) uint64_t tmem_empty[2];          // used in the leader: both CTAs' epilogue warps done
+    __shared__ __align__(8) uint64_t mma_idle;               // unwinding only (leader): every MMA issued so far has completed
     __shared__ uint32_t tmem_base_slot;
     __shared__ int abort_flag;
 
@@ -484,6 +485,7 @@ lmhead_umma_pair_kernel(const __grid_constant__ CUtensorMap tmW, const __grid_co
         abort_flag = 0;
         for (int s = 0; s < p.stages; ++s) { mbar_init(&full_bar[s], 1); mbar_init(&empty_bar[s], 1); }
         for (int b = 0; b < 2; ++b) { mbar_init(&tmem_full[b], 1); mbar_init(&tmem_empty[b], 8 * kPar); }
+        mbar_init(&mma_idle, 1);
         fence_barrier_init();
     }
     if (warp == kTmaWarpLm) {          // a full warp
@@ -575,7 +577,7 @@ lmhead_umma_pair_kernel(const __grid_constant__ CUtensorMap tmW, const __grid_co
                         __syncwarp();
                         if (++s == p.stages) { s = 0; ph ^= 1u; }
                     }
-                    if (ok && elect_one()) mma_commit_pair(&tmem_full[buf], 3);
+                    if (ok && !(p.withhold && t == 0) && elect_one()) mma_commit_pair(&tmem_full[buf], 3);
                     __syncwarp();
                     continue;
                 }
@@ -600,10 +602,16 @@ lmhead_umma_pair_kernel(const __grid_constant__ CUtensorMap tmW, const __grid_co
                     __syncwarp();
                     if (++s == p.stages) { s = 0; ph ^= 1u; }
                 }
-                if (ok && elect_one()) mma_commit_pair(&tmem_full[buf], 3);  // accumulators complete in both CTAs
+                if (ok && !(p.withhold && t == 0) && elect_one()) mma_commit_pair(&tmem_full[buf], 3);  // accumulators complete in both CTAs
             }
             __syncwarp();
-            if (!ok && lane == 0) set_status(status, SD_ERR_TIMEOUT);
+            if (!ok || p.withhold) {
+                // unwinding: neither CTA may give tensor memory back while an MMA issued above still runs
+                if (!ok && lane == 0) set_status(status, SD_ERR_TIMEOUT);
+                if (elect_one()) mma_commit_pair(&mma_idle, 1);
+                __syncwarp();
+                mbar_wait_plain(&mma_idle, 0, p.wait_cycles);
+            }
         }
     } else {
         // ------------------------------------------------ epilogue warps

@@ -62,6 +62,25 @@ def test_lmhead_wait_runs_out_and_the_next_call_is_fine(monkeypatch):
     check_argmax(am2, mx2, ram, t1, t2)
 
 
+# one pair of CTAs, pairs with one and several tiles, two MMAs a step (one accumulator), leftover tiles cut into pieces
+@pytest.mark.parametrize("M,V", [(8, 200), (60, 4099), (60, 60000), (300, 4099), (480, 25000)])
+def test_lmhead_pair_wait_runs_out_and_the_next_call_is_fine(monkeypatch, M, V):
+    g = np.random.default_rng(M)
+    Hd = 128
+    h = wl.f32_to_bf16_bits(g.standard_normal((M, Hd)).astype(np.float32))
+    W = wl.f32_to_bf16_bits((g.standard_normal((V, Hd)) / np.sqrt(Hd)).astype(np.float32))
+    hd, Wd = to_device(h), to_device(W)
+    am = torch.full((M,), -5, dtype=torch.int32, device="cuda")
+    ws = torch.empty(sd.sd_workspace_bytes(None, M, V), dtype=torch.uint8, device="cuda")
+    st = sd.new_status()
+    with_short_waits(monkeypatch, sd.sd_lmhead_argmax)(hd, Wd, am, None, ws, st)
+    torch.cuda.synchronize()
+    assert int(st.item()) == sd.SD_ERR_TIMEOUT
+    am2, mx2 = gpu_lmhead(h, W)
+    ram, t1, t2 = oracle.lmhead(h, W)
+    check_argmax(am2, mx2, ram, t1, t2)
+
+
 # one task, one per CTA, two per CTA, and thirteen: more than a CTA's ring of separate K and V tiles holds
 @pytest.mark.parametrize("S,L,H", [(1, 28, 1), (18, 3, 8), (37, 32, 8), (481, 5, 4)])
 @pytest.mark.parametrize("same", [False, True])
