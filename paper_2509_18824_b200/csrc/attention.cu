@@ -233,7 +233,7 @@ attn_umma_kernel(const __grid_constant__ AttnLayers<NL> layers, const sd_batch b
             }
             if (!ok) {
                 set_status(status, SD_ERR_TIMEOUT);
-                for (int i = 0; i < 1000; ++i) __nanosleep(1000);      // let copies in flight land
+                unwind_pause();
             }
         }
     } else if (warp == kMmaWarp) {
@@ -290,6 +290,7 @@ attn_umma_kernel(const __grid_constant__ AttnLayers<NL> layers, const sd_batch b
                 // unwinding: nothing may give tensor memory back while an MMA issued above still runs
                 set_status(status, SD_ERR_TIMEOUT);
                 mbar_wait_plain(o_full, 0, plan.wait_cycles);
+                unwind_pause();
             }
         }
     } else if (warp < 4) {
@@ -456,14 +457,17 @@ attn_umma_kernel(const __grid_constant__ AttnLayers<NL> layers, const sd_batch b
             if (row_ok && lse) lse[orow] = (m_used + log2f(l)) * 0.6931471805599453f;
         } else if (ok) {
             rows_ready = true;         // several chunks: the rows leave for their finishing CTAs below
-        } else if (!ok && lane == 0) {
-            set_status(status, SD_ERR_TIMEOUT);
+        } else {
+            if (lane == 0) set_status(status, SD_ERR_TIMEOUT);
+            unwind_pause();
         }
     }
     }   // active
 
-    if (!active && aligned && warp == kTmaWarp && lane == 0)       // nobody else waits for the Q copy
-        mbar_wait(q_full, 0, abort_flag, plan.wait_cycles);
+    if (!active && aligned && warp == kTmaWarp && lane == 0 && !mbar_wait(q_full, 0, abort_flag, plan.wait_cycles)) {   // nobody else waits for the Q copy
+        set_status(status, SD_ERR_TIMEOUT);
+        unwind_pause();
+    }
 
     if (clustered) {
         // The chunks' rows meet as described at RowExchange; the rings are free by now.
@@ -477,6 +481,7 @@ attn_umma_kernel(const __grid_constant__ AttnLayers<NL> layers, const sd_batch b
                              m64 ? (lane < 16 ? warp * 16 + lane : -1) : (int)threadIdx.x, m_used, l);
         __syncwarp();
         cluster_arrive_relaxed();                          // (waited for at the end: nobody leaves before its peers have sent)
+        bool late = false;
         if (warp < 4) {
             asm volatile("bar.sync 1, 128;" ::: "memory"); // this CTA's own rows
             if (mbar_wait_cluster(x_full, 0, abort_flag, plan.wait_cycles)) {
@@ -485,11 +490,12 @@ attn_umma_kernel(const __grid_constant__ AttnLayers<NL> layers, const sd_batch b
                 else merge_rows<8, 128>(x, (int)threadIdx.x);
             } else if (lane == 0) {
                 set_status(status, SD_ERR_TIMEOUT);
-                for (int i = 0; i < 1000; ++i) __nanosleep(1000);      // let rows in flight land
+                late = true;
             }
         }
         __syncwarp();
         cluster_wait_acquire();
+        if (late) unwind_pause();                          // (rows sent by now)
     }
     if (!aligned) return;
     tc_fence_before_sync();

@@ -210,7 +210,7 @@ attn_wide_kernel(const __grid_constant__ AttnLayers<NL> layers, const sd_batch b
         }
         if (!ok) {
             if (lane == 0) set_status(status, SD_ERR_TIMEOUT);
-            for (int i = 0; i < 1000; ++i) __nanosleep(1000);      // let copies in flight land
+            unwind_pause();
         }
         ring_is_free();
     } else if (warp == kWMmaWarp) {
@@ -272,6 +272,7 @@ attn_wide_kernel(const __grid_constant__ AttnLayers<NL> layers, const sd_batch b
             // unwinding: nothing may give tensor memory back while an MMA issued above still runs
             if (lane == 0) set_status(status, SD_ERR_TIMEOUT);
             mbar_wait_plain(o_full, 0, plan.wait_cycles);
+            unwind_pause();
         }
         ring_is_free();
     } else {
@@ -336,16 +337,19 @@ attn_wide_kernel(const __grid_constant__ AttnLayers<NL> layers, const sd_batch b
                 }
                 if (row_ok && ly.lse && group == 0) ly.lse[orow] = (m_used + log2f(l)) * 0.6931471805599453f;
             }
-        } else if (lane == 0) {
-            set_status(status, SD_ERR_TIMEOUT);
+        } else {
+            if (lane == 0) set_status(status, SD_ERR_TIMEOUT);
+            unwind_pause();
         }
     }
     } else {
         ring_is_free();
     }
 
-    if (!active && aligned && warp == kWTmaWarp && lane == 0)      // nobody else waits for the Q copy
-        mbar_wait(q_full, 0, abort_flag, plan.wait_cycles);
+    if (!active && aligned && warp == kWTmaWarp && lane == 0 && !mbar_wait(q_full, 0, abort_flag, plan.wait_cycles)) {   // nobody else waits for the Q copy
+        set_status(status, SD_ERR_TIMEOUT);
+        unwind_pause();
+    }
 
     if (clustered) {
         const int gt = (int)threadIdx.x & 127;
@@ -356,6 +360,7 @@ attn_wide_kernel(const __grid_constant__ AttnLayers<NL> layers, const sd_batch b
             exchange_push<2>(x, tmem_base + ((uint32_t)((warp & 3) * 32) << 16), (warp >> 2) * 2, rows_ready, row_in_tile, m_used, l);
         __syncwarp();
         cluster_arrive_relaxed();                          // (waited for at the end: nobody leaves before its peers have sent)
+        bool late = false;
         if (warp < 8) {
             asm volatile("bar.sync 1, 256;" ::: "memory"); // this CTA's own rows
             if (mbar_wait_cluster(x_full, 0, abort_flag, plan.wait_cycles)) {
@@ -370,11 +375,12 @@ attn_wide_kernel(const __grid_constant__ AttnLayers<NL> layers, const sd_batch b
                 }
             } else if (lane == 0) {
                 set_status(status, SD_ERR_TIMEOUT);
-                for (int i = 0; i < 1000; ++i) __nanosleep(1000);      // let rows in flight land
+                late = true;
             }
         }
         __syncwarp();
         cluster_wait_acquire();
+        if (late) unwind_pause();                          // (rows sent by now)
     }
     if (!aligned) return;
     tc_fence_before_sync();

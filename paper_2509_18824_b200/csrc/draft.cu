@@ -79,7 +79,7 @@ draft_feature_attention_kernel(const __grid_constant__ CUtensorMap map_k, const 
         int s = (int)(first / H), h = (int)(first - (long long)s * H), slot = 0;
         uint32_t ph = 1;
         for (int i = 0; i < n; ++i) {
-            if (!mbar_wait_warp(&empty[slot], ph, &abort_flag, wait_cycles)) { unwind_pause(&abort_flag); break; }
+            if (!mbar_wait_warp(&empty[slot], ph, &abort_flag, wait_cycles)) { unwind_pause(); break; }
             uint8_t* dst = ring + slot * kSlot;
             if (elect_one()) {
                 mbar_arrive_expect_tx(&full[slot], tile_bytes);
@@ -188,7 +188,7 @@ draft_feature_attention_kernel(const __grid_constant__ CUtensorMap map_k, const 
             reinterpret_cast<uint4*>(out + ((size_t)s * Q + (x >> 4)) * D + (size_t)h * kDh)[x & 15] =
                 make_uint4(0x7fff7fffu, 0x7fff7fffu, 0x7fff7fffu, 0x7fff7fffu);
     }
-    unwind_pause(&abort_flag);
+    unwind_pause();
 }
 
 sd_status launch_draft_feature_attention(const void* qp, const void* k, const void* v, int S, int L, int Q, int H,

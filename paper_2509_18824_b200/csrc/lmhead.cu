@@ -256,6 +256,7 @@ __device__ __forceinline__ void epi_finish(const LmParams& p, const EpiState& e,
                                            int lane, bool ok, int32_t* status) {
     constexpr int cols = kEpiChunks * PAR * 32;            // (the others have no hidden row)
     const bool stats = p.c2 > 0.f;
+    if (!ok) unwind_pause();
     asm volatile("bar.sync 1, %0;" ::"n"(epi_threads(PAR)) : "memory");
     int32_t* red_key = reinterpret_cast<int32_t*>(smem);
     int32_t* red_idx = red_key + 4 * kMaxCols;
@@ -357,7 +358,7 @@ lmhead_umma_kernel(const __grid_constant__ CUtensorMap tmW, const __grid_constan
             }
             if (!ok) {
                 set_status(status, SD_ERR_TIMEOUT);
-                for (int i = 0; i < 1000; ++i) __nanosleep(1000);   // let copies in flight land
+                unwind_pause();
             }
         }
     } else if (warp == kMmaWarpLm) {
@@ -397,6 +398,7 @@ lmhead_umma_kernel(const __grid_constant__ CUtensorMap tmW, const __grid_constan
                 if (!ok) set_status(status, SD_ERR_TIMEOUT);
                 mma_commit(&mma_idle);
                 mbar_wait_plain(&mma_idle, 0, p.wait_cycles);
+                if (!ok) unwind_pause();
             }
         }
     } else {
@@ -541,7 +543,7 @@ lmhead_umma_pair_kernel(const __grid_constant__ CUtensorMap tmW, const __grid_co
         }
         if (!ok) {
             if (lane == 0) set_status(status, SD_ERR_TIMEOUT);
-            for (int i = 0; i < 1000; ++i) __nanosleep(1000);   // let copies in flight land
+            unwind_pause();
         }
     } else if (warp == kMmaWarpLm) {
         // ------------------------------------------------ MMA issuer (leader CTA only; a whole warp, one lane elected)
@@ -611,6 +613,7 @@ lmhead_umma_pair_kernel(const __grid_constant__ CUtensorMap tmW, const __grid_co
                 if (elect_one()) mma_commit_pair(&mma_idle, 1);
                 __syncwarp();
                 mbar_wait_plain(&mma_idle, 0, p.wait_cycles);
+                if (!ok) unwind_pause();
             }
         }
     } else {

@@ -169,7 +169,7 @@ __device__ __forceinline__ void q_end(QShared& sh) {
     __syncwarp();
     sm100::cluster_arrive_relaxed();
     sm100::cluster_wait_acquire();
-    sm100::unwind_pause(&sh.abort_flag);
+    if (*reinterpret_cast<volatile int*>(&sh.abort_flag)) sm100::unwind_pause();
 }
 
 __global__ void __launch_bounds__(kQThreads, 1)

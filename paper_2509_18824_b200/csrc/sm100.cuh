@@ -95,11 +95,11 @@ __device__ __forceinline__ bool mbar_wait_warp(uint64_t* bar, uint32_t parity, v
     }
 }
 
-// Before a CTA whose wait ran out leaves: copies and remote stores on their way to its shared memory land first (about
-// a millisecond, which is far longer than they take).
-__device__ __forceinline__ void unwind_pause(volatile int* abort_flag) {
-    if (*abort_flag)
-        for (int i = 0; i < 1000; ++i) __nanosleep(1000);
+// What a warp does whose wait ran out: copies and remote stores on their way to this CTA's shared memory land before the
+// CTA leaves (about a millisecond, which is far longer than they take).  Every role that gives up does it, not only
+// the one that issued the copies, which may have left long before.
+__device__ __forceinline__ void unwind_pause() {
+    for (int i = 0; i < 1000; ++i) __nanosleep(1000);
 }
 
 // ---------------------------------------------------------------- programmatic dependent launch
