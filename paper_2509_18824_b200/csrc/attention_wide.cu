@@ -284,7 +284,7 @@ attn_wide_kernel(const __grid_constant__ AttnLayers<NL> layers, const sd_batch b
         const bool row_ok = row < rows;
         const uint64_t amask = row_ok ? bt.anc_mask[(size_t)b * T + plan.node_of(row)] : ~0ull;
         const uint32_t lane_field = (uint32_t)(quad * 32) << 16;
-        bool ok = wide_softmax(plan, sh, WideTiles{nt, nb, n_pref, t0, len, n, 0, 0}, tmem_o, tmem_s, group, quad, lane, row_ok, amask,
+        bool ok = wide_softmax(plan, sh, WideTiles{nt, nb, n_pref, t0, len, n}, tmem_o, tmem_s, group, quad, lane, row_ok, amask,
                                scale_log2, m_used, l);
         ring_is_free();
         volatile float* my_ref = ref_smem + gt;

@@ -86,8 +86,8 @@ __device__ __forceinline__ WideWork wide_work(const sd_batch& bt, const AttnPlan
 }
 
 // The key tiles of one row tile: nt tiles over nb blocks, of which n_pref are cache blocks t0 .. of the sequence
-// (len cached tokens, n nodes), the one behind them the tree's.  base: tiles this CTA has worked on before.
-struct WideTiles { int nt, nb, n_pref, t0, len, n, base; uint32_t ref_phase; };
+// (len cached tokens, n nodes), the one behind them the tree's.
+struct WideTiles { int nt, nb, n_pref, t0, len, n; };
 
 // Softmax of those tiles by the two groups of four warps, one thread per row and group; false: a wait ran out.
 __device__ __forceinline__ bool wide_softmax(const AttnPlan& plan, const WideShared& sh, const WideTiles& w, uint32_t tmem_o, uint32_t tmem_s,
@@ -106,8 +106,7 @@ __device__ __forceinline__ bool wide_softmax(const AttnPlan& plan, const WideSha
     // maximum first they took 4800 instead of 1500 cycles, at the end of every call.)
     auto tile = [&](auto masked, auto only_half, int j, const uint32_t (&mask)[4]) -> int {
         constexpr bool kMasked = decltype(masked)::value, half = decltype(only_half)::value;     // half: 64 keys
-        const int jj = w.base + j;
-        const int s = jj % kWStages;
+        const int s = j % kWStages;
         const uint32_t ts = tmem_s + lane_field + s * kWTile;
         if (j == 0) {
             // The reference: the largest of the first sixteen scores (any score of the row will do, see kSumLimit; a
@@ -154,7 +153,7 @@ __device__ __forceinline__ bool wide_softmax(const AttnPlan& plan, const WideSha
         }
         const float psum = sum_f32x2(add_f32x2(ps[0], ps[1]));
         // the tile before is final, and its reference still the one used here
-        if (j > 0 && !mbar_wait(&sh.commit[quad], (uint32_t)(jj - 1) & 1u, sh.abort_flag, plan.wait_cycles)) return -1;
+        if (j > 0 && !mbar_wait(&sh.commit[quad], (uint32_t)(j - 1) & 1u, sh.abort_flag, plan.wait_cycles)) return -1;
         const float ref = *my_ref;
         if (__any_sync(0xffffffffu, row_ok && (!(psum <= kSumLimit) || ref != m_used))) return 1;
         l += psum;
@@ -167,12 +166,11 @@ __device__ __forceinline__ bool wide_softmax(const AttnPlan& plan, const WideSha
         return 0;
     };
     for (int j = group; j < w.nt; j += 2) {
-        const int jj = w.base + j;                         // tiles of this CTA so far
-        const int s = jj % kWStages;
-        const uint32_t ph = (uint32_t)(jj / kWStages) & 1u;
+        const int s = j % kWStages;
+        const uint32_t ph = (uint32_t)(j / kWStages) & 1u;
         const uint32_t ts = tmem_s + lane_field + s * kWTile;
         if (j == 1) {                                      // the reference that the other group found in tile 0
-            if (!mbar_wait(&sh.ref_full[quad], w.ref_phase, sh.abort_flag, plan.wait_cycles)) return false;
+            if (!mbar_wait(&sh.ref_full[quad], 0, sh.abort_flag, plan.wait_cycles)) return false;
             m_used = *my_ref;
             neg_m2 = pack_f32x2(-m_used, -m_used);
         }
@@ -235,7 +233,7 @@ __device__ __forceinline__ bool wide_softmax(const AttnPlan& plan, const WideSha
         mt *= scale_log2;                                  // scale > 0
         const bool raise = row_ok && mt > m_used + kRaiseAbove;
         if (__any_sync(0xffffffffu, raise) && j > 0) {     // (nothing has been accumulated before tile 0)
-            if (!mbar_wait(&sh.v_empty[(jj - 1) % kWStages], (uint32_t)((jj - 1) / kWStages) & 1u, sh.abort_flag, plan.wait_cycles)) return false;
+            if (!mbar_wait(&sh.v_empty[(j - 1) % kWStages], (uint32_t)((j - 1) / kWStages) & 1u, sh.abort_flag, plan.wait_cycles)) return false;
             tc_fence_after_sync();
             const float alpha = raise ? exp2f(m_used - mt) : 1.f;
 #pragma unroll 1

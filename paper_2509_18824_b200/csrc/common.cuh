@@ -16,9 +16,6 @@ __device__ __forceinline__ void set_status(int32_t* status, int code) {
     if (status) atomicCAS(status, 0, code);
 }
 
-__device__ __forceinline__ float bf16_bits_to_float(uint16_t b) {
-    return __uint_as_float(((uint32_t)b) << 16);
-}
 __device__ __forceinline__ float bf16lo(uint32_t u) { return __uint_as_float(u << 16); }
 __device__ __forceinline__ float bf16hi(uint32_t u) { return __uint_as_float(u & 0xffff0000u); }
 
