@@ -118,11 +118,11 @@ __device__ __forceinline__ int sequence_of_rank(const sd_batch& bt, int rank, in
 // is as short as n_chunks make it.  All of it follows from the sequence's own length: the block table may be far
 // wider than any sequence of the batch.
 struct ChunkRange { int n_chunks, tiles_total, tpc, t0, t1; };
-__device__ __forceinline__ ChunkRange chunk_range(const AttnPlan& plan, int len, int max_blocks, int chunk) {
+__host__ __device__ __forceinline__ ChunkRange chunk_range(const AttnPlan& plan, int len, int max_blocks, int chunk) {
     ChunkRange r;
     r.tiles_total = min((len + kBlock - 1) / kBlock, max_blocks);
     const bool whole = plan.n_chunks == 1 || r.tiles_total <= max(plan.whole_blocks, 0);
-    r.tpc = whole ? r.tiles_total : (int)__umulhi((uint32_t)(r.tiles_total + plan.n_chunks - 1), plan.chunk_magic);
+    r.tpc = whole ? r.tiles_total : (int)(((uint64_t)(uint32_t)(r.tiles_total + plan.n_chunks - 1) * plan.chunk_magic) >> 32);
     r.n_chunks = whole ? 1 : plan.n_chunks;
     if (plan.whole_blocks >= 0 && !whole) {
         r.n_chunks = 2;
