@@ -122,6 +122,9 @@ sd_status sd_tree_prepare(const sd_batch *batch, int32_t *dev_status, void *stre
  *   lse               : dev f32 [B][T_max][Hq] or NULL; natural-log sum of exp of the scaled scores
  *   workspace         : dev scratch of at least sd_workspace_bytes(batch, 0, 0)
  * Arithmetic: bf16 inputs, fp32 accumulation, bf16 output (round to nearest even).
+ * Range: a row's weights are relative to one of its first scores until the division at the end and
+ * may add up to 2^40 per cache block, so that |V| has to stay below 2^78 (for up to 2^16 cached
+ * tokens; half of that for twice as many) where the weighted mean itself would be finite.
  * Needs batch->anc_mask filled.  Errors: SD_ERR_INVALID_ARG, SD_ERR_UNSUPPORTED,
  * SD_ERR_WORKSPACE (workspace_bytes below sd_workspace_bytes) on the host;
  * SD_ERR_BOUNDS (block-table entry outside [0, num_blocks), or len[b] needs
