@@ -562,10 +562,14 @@ static AttnPlan common_plan(const sd_batch& bt, int n_layers, const TestKnobs& k
 // of its longest chunk, plus 8 us for launch, first copies and output (11 when CTAs of another round follow:
 // nothing overlaps them), plus the merge of the chunks, plus about 1 us where the next call's CTAs find no
 // free SMs to set up on while this one runs.  Measured per call in us for 1 to 8 chunks: one sequence of 2048
-// tokens and 60 nodes 16.4 13.0 11.4 10.6 10.7 10.7 17.3 17.5 (16 clusters of seven or eight are more than fit
-// at a time), of 8192 50.6 30.3 23.0 19.2 17.6 16.7 26.8 26.0, one chain of 11 nodes over 4096 27.3 18.5 14.6
-// 12.9 12.0 11.2 10.9 10.9.  Chunk counts that are no powers of two fill SMs that those leave idle: ten such
-// chains 19.6 us with three chunks (22.2 with two), five sequences of 2000 tokens with 16 heads 13.5 (15.1).
+// tokens and 60 nodes 16.6 12.6 11.0 10.2 9.8 9.8 15.6 15.4 (16 clusters of seven or eight are more than fit
+// at a time), of 8192 50.7 29.7 22.2 18.5 16.8 15.9 25.1 24.2, one chain of 11 nodes over 4096 27.9 18.3 14.4
+// 12.6 11.6 11.0 10.4 10.4.  Chunk counts that are no powers of two fill SMs that those leave idle: ten such
+// chains 19.3 us with three chunks (21.4 with two), five sequences of 2000 tokens with 16 heads 13.0 (14.6).
+// The table's width stands for the longest length here, which the host does not know: a table that is far wider
+// makes long launches look longer than they are (in a table of 512 blocks 256 CTAs of 1000 tokens take 26.4 instead
+// of 22.7 us, 160 of 2048 54.6 instead of 35), but what a single round's sequences are cut into follows from
+// their own lengths.
 // The 64-key kernel's two CTAs per SM overlap each other's ends: a round of twice as many CTAs takes about
 // 0.9 us per block plus 13 us.  It is left for launches of several rounds in which those ends weigh more
 // (256 CTAs of 1000 tokens: 28.7 against 33.9 us; of 4096: 71.4 against 69.9; 1792 CTAs of 4096 tokens under the

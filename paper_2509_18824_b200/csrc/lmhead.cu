@@ -21,7 +21,7 @@ constexpr int kBM = 128;            // vocabulary rows per tile (MMA M)
 // 8 rows take 171.5 instead of 165.5 us; the single-CTA kernel has one).  Up to 256 hidden rows PAR = 2: the accumulator is
 // double-buffered and the epilogue hides behind the next tile's MMAs.  Above, the one buffer is drained while
 // the tensor cores wait, and the redux and vote latencies of two warps per scheduler left half of the issue
-// slots empty: PAR = 4 takes 480 rows from 434 to 419 us, with statistics and logits from 528 to 493 (below
+// slots empty: PAR = 4 takes 480 rows from 434 to 419 us, with statistics and logits from 523 to 489 (below
 // 256 rows it gains nothing and costs 1 % in power).
 constexpr int kEpiChunks = 4;       // chunks of 32 columns per epilogue warp, at most
 __host__ __device__ constexpr int epi_threads(int par) { return par * 128; }
@@ -180,8 +180,8 @@ __device__ __forceinline__ void column_argmax_stats32(const uint32_t (&r)[32], b
 
 // ---------------------------------------------------------------------------
 // Epilogue shared by the one-CTA and the two-CTA kernel.  Warp w of the 4 PAR epilogue warps works on
-// TMEM lanes 32 * (w & 3) .. +31 (the only ones it may read) and on the 32-column chunks of parity
-// w >> 2; per (warp, column) it keeps a running best (value, vocabulary row) and, for the soft-max
+// TMEM lanes 32 * (w & 3) .. +31 (the only ones it may read) and on every PAR-th 32-column chunk from
+// w >> 2 on; per (warp, column) it keeps a running best (value, vocabulary row) and, for the soft-max
 // statistics, a running (reference, sum).
 // ---------------------------------------------------------------------------
 struct EpiState {
@@ -687,8 +687,8 @@ static int round_up(int x, int m) { return (x + m - 1) / m * m; }
 // More than 256 hidden rows, where the tensor cores bound a tile: if few tiles are left over after whole rounds of
 // all pairs (or there are few tiles at all), they are cut along the hidden rows into pieces that are dealt out to
 // all pairs.  A piece costs its share of a tile and about a quarter more: it streams its tile's W through the
-// pair once again, and fills and drains the pipeline.  480 rows: vocabulary of 4099 18.7 -> 15.2 us, 152064
-// (594 tiles, 74 pairs) 375 -> 370; cutting the 49 tiles left over at 50257 took 82 instead of 78, and up to
+// pair once again, and fills and drains the pipeline.  480 rows, hidden size 3584: vocabulary of 4099 39.1 -> 24.7 us,
+// 152064 (594 tiles, 74 pairs) 377 -> 368; cutting the 49 tiles left over at 50257 took 82 instead of 78, and up to
 // 256 rows, where streaming W is what takes the time, pieces are as slow as whole tiles.
 static bool plan_slices(LmParams* p, int pairs) {
     const int n_chunks = (p->n_pad + 31) / 32, rest = p->n_tiles % pairs;
