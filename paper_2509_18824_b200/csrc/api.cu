@@ -3,6 +3,8 @@
 
 #include <atomic>
 #include <stdlib.h>
+#include <string.h>
+#include <unistd.h>
 
 using namespace sdv;
 
@@ -19,11 +21,21 @@ int sm_count(int dev) {
     return sms;
 }
 
+// (One pass over the environment: three getenv calls took 0.35 us with 200 variables, a tenth of what the smallest
+// calls take on the host; this 0.15.)
 TestKnobs test_knobs() {
     TestKnobs k{1ll << 31, 0, 0};
-    if (const char* e = getenv("SDV_TEST_WAIT_CYCLES")) { const long long v = atoll(e); if (v >= 1000) k.wait_cycles = v; }
-    if (const char* e = getenv("SDV_TEST_WITHHOLD")) k.withhold = atoi(e) == 1 ? 1 : 0;
-    if (const char* e = getenv("SDV_TEST_CHUNKS")) { const int v = atoi(e); if (v >= 1 && v <= 8) k.chunks = v; }
+    for (char** e = environ; e && *e; ++e) {
+        if ((*e)[0] != 'S' || (*e)[1] != 'D' || strncmp(*e, "SDV_TEST_", 9) != 0) continue;
+        const char* name = *e + 9;
+        const auto value = [&](const char* n) -> const char* {             // behind "n=", if that is the variable
+            const size_t l = strlen(n);
+            return strncmp(name, n, l) == 0 && name[l] == '=' ? name + l + 1 : nullptr;
+        };
+        if (const char* v = value("WAIT_CYCLES")) { if (atoll(v) >= 1000) k.wait_cycles = atoll(v); }
+        else if (const char* v = value("WITHHOLD")) k.withhold = atoi(v) == 1 ? 1 : 0;
+        else if (const char* v = value("CHUNKS")) { if (atoi(v) >= 1 && atoi(v) <= 8) k.chunks = atoi(v); }
+    }
     return k;
 }
 }  // namespace sdv
