@@ -131,8 +131,9 @@ attn_umma_kernel(const __grid_constant__ AttnLayers<NL> layers, const sd_batch b
     }
     const int32_t *n_nodes = bt.n_nodes, *lens = bt.len, *tables = bt.block_table;
     settle(n_nodes); settle(lens); settle(tables);         // (no load of theirs in front of the wait)
-    const int n = min(max(__ldg(n_nodes + b), 0), T);
-    const int len = max(__ldg(lens + b), 0);
+    // (lengths that a kernel of this library wrote while this one was already there: not for the read-only path)
+    const int n = min(max(__ldcg(n_nodes + b), 0), T);
+    const int len = max(__ldcg(lens + b), 0);
     // Rows of this sequence: its own nodes only (rows are node-major, so they are the first n * G).  A tree
     // smaller than T_max pays for the row tiles it fills: the rows behind them only get their zeros.  (A
     // batch of 16 trees of 30 to 60 nodes, T_max = 60: 2.9 of 4 row tiles run.)

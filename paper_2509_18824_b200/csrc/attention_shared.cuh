@@ -101,10 +101,10 @@ __device__ __forceinline__ int sequence_of_rank(const sd_batch& bt, int rank, in
     const int32_t* lens = bt.len;
     settle(lens);
     if ((int)threadIdx.x < bt.B) {
-        const int mine = __ldg(lens + threadIdx.x);
+        const int mine = __ldcg(lens + threadIdx.x);
         int r = 0;
         for (int j = 0; j < bt.B; ++j) {
-            const int other = __ldg(lens + j);
+            const int other = __ldcg(lens + j);
             r += (other > mine || (other == mine && j < (int)threadIdx.x)) ? 1 : 0;
         }
         if (r == rank) s_seq = threadIdx.x;

@@ -81,8 +81,9 @@ attn_wide_kernel(const __grid_constant__ AttnLayers<NL> layers, const sd_batch b
     if (plan.ranked) b = sequence_of_rank(bt, rank_b, *sh.seq);
     const int32_t *n_nodes = bt.n_nodes, *lens = bt.len, *tables = bt.block_table;
     settle(n_nodes); settle(lens); settle(tables);         // (no load of theirs in front of the wait)
+    // (lengths that a kernel of this library wrote while this one was already there: not for the read-only path)
     const int32_t* const seq_table = tables + (size_t)b * bt.max_blocks_per_seq;
-    const int n_now = __ldg(n_nodes + b), len_now = __ldg(lens + b);
+    const int n_now = __ldcg(n_nodes + b), len_now = __ldcg(lens + b);
     int even = 0, odd = 0;                                 // block table of this chunk (producer warp)
     if (warp == kWTmaWarp) {
         const int i = wk.t0 + lane;                        // (within the table whatever the length)

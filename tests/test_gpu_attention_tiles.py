@@ -149,3 +149,35 @@ def test_short_sequences_in_a_wide_table(blocks, B):
     ref, rlse = oracle.attention(oracle.Geometry.of(p), p.k_cache, p.v_cache, p.q, p.k_tree, p.v_tree, p.scale)
     check_attention(out, ref, f"blocks={blocks} B={B}")
     np.testing.assert_allclose(lse, rlse, rtol=2e-3, atol=2e-3)
+
+
+@pytest.mark.parametrize("lens,T", [((900, 333, 1000), 19), ((130, 64), 40), (tuple(range(500, 200, -5)), 40),
+                                    (tuple(range(2600, 2400, -5)), 19)])
+def test_attention_and_acceptance_back_to_back(lens, T):
+    """Attention, acceptance that rewrites the lengths, attention, ...: launches that may all begin while the ones
+    ahead of them still run.  One round of CTAs, and several (dispatched by length) through both kernels."""
+    long = problem(11, lens, T=T)
+    short = copy.copy(long)
+    short.len = (long.len // 3).astype(np.int32)
+    refs = [gpu_attention(x)[:2] for x in (long, short)]
+    bt, srcs, st = sd.Batch.of(long), [sd.Batch.of(x) for x in (long, short)], sd.new_status()
+    for s in srcs:
+        s.len -= 1                                        # one node accepted: the lengths of long and short
+    sd.sd_tree_prepare(bt, st)
+    i32 = lambda *shape: torch.zeros(shape, dtype=torch.int32, device="cuda")
+    draft, argmax, n_acc, path, tok = i32(bt.B, T) + 1, i32(bt.B * T), i32(bt.B), i32(bt.B, T), i32(bt.B, T)
+    cache = sd.kv_layer(to_device(long.k_cache), to_device(long.v_cache))
+    q, kt, vt = to_device(long.q), to_device(long.k_tree), to_device(long.v_tree)
+    ws = torch.empty(sd.sd_workspace_bytes(bt), dtype=torch.uint8, device="cuda")
+    runs = 16
+    outs = torch.full((runs, bt.B, T, bt.Hq, bt.D), 7.0, dtype=torch.bfloat16, device="cuda")
+    lses = torch.zeros((runs, bt.B, T, bt.Hq), dtype=torch.float32, device="cuda")
+    torch.cuda.synchronize()
+    for i in range(runs):
+        sd.sd_accept_tree(srcs[i % 2], draft, argmax, n_acc, path, tok, bt.len, st)
+        sd.sd_verify_attention(bt, cache, q, kt, vt, float(long.scale), outs[i], lses[i], ws, st)
+    torch.cuda.synchronize()
+    assert int(st.item()) == 0
+    for i in range(runs):
+        np.testing.assert_array_equal(outs[i].float().cpu().numpy(), refs[i % 2][0])
+        np.testing.assert_array_equal(lses[i].cpu().numpy(), refs[i % 2][1])
