@@ -65,7 +65,9 @@ inline sd_status launch_dependent(void (*kern)(P...), dim3 grid, int threads, si
 }
 
 // Start of such a kernel's work on global memory.  The pointers pass through the asm so that no load from
-// them, read-only ones included, can be moved in front of the wait.
+// them, read-only ones included, can be moved in front of the wait.  (The read-only path, __ldg, is for what no kernel
+// writes that may still run when this one begins: a caller's inputs, and what the LM-head tiles leave, which let
+// nobody begin early.)
 template <typename Ptr>
 __device__ __forceinline__ void settle(Ptr& p) { asm volatile("" : "+l"(p)); }
 __device__ __forceinline__ void settle(sd_batch& bt) {

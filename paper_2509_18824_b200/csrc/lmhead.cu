@@ -219,7 +219,7 @@ __device__ __forceinline__ void epi_tile(const LmParams& p, EpiState& e, uint32_
                         const int row = c * 32 + j;
                         if (row < p.rows)
                             p.mass_out[(size_t)(p.row0 + row) * p.V + v_base + lane] =
-                                __expf(__uint_as_float(r[j]) * p.inv_temp - __ldg(p.col_lse + p.row0 + row));
+                                __expf(__uint_as_float(r[j]) * p.inv_temp - __ldca(p.col_lse + p.row0 + row));
                     }
                 }
                 continue;

@@ -258,7 +258,7 @@ residual_blocksum_kernel(int V, const int32_t* __restrict__ n_excl, const int32_
     if (t < V) {
         if (logits) {
             const int row = stop_row[b];
-            m = __expf(__ldg(logits + (size_t)row * V + t) * inv_temp - __ldg(lse + row));
+            m = __expf(__ldg(logits + (size_t)row * V + t) * inv_temp - lse[row]);
             if (!q_rows || !n_excl[b]) mass[(size_t)b * V + t] = m;
         } else {
             m = mass[(size_t)b * V + t];
@@ -271,7 +271,7 @@ residual_blocksum_kernel(int V, const int32_t* __restrict__ n_excl, const int32_
             }
         } else {
             bool hit = false;
-            for (int e = 0; e < ne; ++e) hit |= (__ldg(excl + (size_t)b * 64 + e) == t);
+            for (int e = 0; e < ne; ++e) hit |= (excl[(size_t)b * 64 + e] == t);
             if (hit) { m = 0.f; mass[(size_t)b * V + t] = 0.f; }
         }
     }
