@@ -18,10 +18,21 @@ from paper_2509_18824_b200 import binding as sd
 from paper_2509_18824_b200 import workloads as wl
 from gpu_util import gpu_attention, check_attention, gpu_lmhead, check_argmax
 from paper_2509_18824_b200.step import to_device
+from test_gpu_attention_tiles import problem
 from test_gpu_sampled import (decisive_chain_inputs, decisive_tree_inputs, drafted_chain, drafted_tree, run_chain_q,
                               run_tree_q)
 
 pytestmark = pytest.mark.gpu
+
+
+def with_short_waits(monkeypatch, fn):
+    """fn with the hooks set around it only (the calls in front of it are ordinary ones)."""
+    def call(*args, **kw):
+        with monkeypatch.context() as m:
+            m.setenv("SDV_TEST_WAIT_CYCLES", "200000")
+            m.setenv("SDV_TEST_WITHHOLD", "1")
+            fn(*args, **kw)
+    return call
 
 
 def test_attention_wait_runs_out_and_the_next_call_is_fine(monkeypatch):
@@ -39,6 +50,36 @@ def test_attention_wait_runs_out_and_the_next_call_is_fine(monkeypatch):
         out, lse, status = gpu_attention(w, layer=0)
         assert status == 0
         check_attention(out, ref, "after a timed-out call")
+
+
+def all_layers(p, layers):
+    """`layers` times the same layer in one call: (first and last output, status)."""
+    bt, st = sd.Batch.of(p), sd.new_status()
+    sd.sd_tree_prepare(bt, st)
+    kc, vc, q, kt, vt = (to_device(x) for x in (p.k_cache, p.v_cache, p.q, p.k_tree, p.v_tree))
+    o = [torch.full((p.B, p.T_max, p.Hq, p.D), 7.0, dtype=torch.bfloat16, device="cuda") for _ in range(layers)]
+    ws = torch.empty(sd.sd_workspace_bytes(bt), dtype=torch.uint8, device="cuda")
+    same = lambda x: [x] * layers
+    sd.sd_verify_attention_layers(bt, sd.AttentionLayerSet(same(kc), same(vc), same(q), same(kt), same(vt), o), float(p.scale), ws, st)
+    torch.cuda.synchronize()
+    return [x.float().cpu().numpy() for x in (o[0], o[-1])], int(st.item())
+
+
+# key chunks in clusters: the 128-key kernel, and (32 layers of short sequences) the 64-key one, whole and in chunks
+@pytest.mark.parametrize("lens,layers,chunks", [((700, 2300), 1, 2), ((700, 2300), 1, 3), ((700, 2300), 1, 8),
+                                                ((900, 333, 1000), 32, 1), ((900, 333, 1000), 32, 2)])
+def test_attention_in_chunks_wait_runs_out_and_the_next_call_is_fine(monkeypatch, lens, layers, chunks):
+    p = problem(sum(lens), lens, T=12, Hq=8, Hkv=2, gain=1.0)
+    ref, _ = oracle.attention(oracle.Geometry.of(p), p.k_cache, p.v_cache, p.q, p.k_tree, p.v_tree, p.scale)
+    monkeypatch.setenv("SDV_TEST_CHUNKS", str(chunks))
+    with monkeypatch.context() as m:
+        m.setattr(sd, "sd_verify_attention_layers", with_short_waits(m, sd.sd_verify_attention_layers))
+        assert all_layers(p, layers)[1] == sd.SD_ERR_TIMEOUT
+    for _ in range(2):
+        outs, status = all_layers(p, layers)
+        assert status == 0
+        for out in outs:
+            check_attention(out, ref, "after a timed-out call")
 
 
 def test_lmhead_wait_runs_out_and_the_next_call_is_fine(monkeypatch):
@@ -108,16 +149,6 @@ def test_draft_wait_runs_out_and_the_next_call_is_fine(monkeypatch, S, L, H, sam
     for _ in range(2):
         got = rows()
         assert np.linalg.norm(got - ref) <= 5e-3 * np.linalg.norm(ref)
-
-
-def with_short_waits(monkeypatch, fn):
-    """fn with the hooks set around it only (the calls in front of it are ordinary ones)."""
-    def call(*args, **kw):
-        with monkeypatch.context() as m:
-            m.setenv("SDV_TEST_WAIT_CYCLES", "200000")
-            m.setenv("SDV_TEST_WITHHOLD", "1")
-            fn(*args, **kw)
-    return call
 
 
 @pytest.mark.parametrize("cfg,over", [("c1", dict(V=1000, Hd=64)), ("c4", dict(L=1, V=4099, Hd=64, prefix_range=(40, 300)))])
