@@ -603,6 +603,7 @@ static bool wide_plan(AttnPlan* p, const sd_batch& bt, int dev, int sms, const T
     // In several rounds every sequence is cut alike: the CTAs that leave would still hold back the next cluster
     // (half-empty pairs halved the machine).
     p->set_chunks(n, n_rounds > 1 ? -1 : (knobs.chunks > 0 ? 0 : (n == 2 ? 10 : 5)));
+    p->tree_blocks = kTreeBlocks;
     p->ranked = (bt.B > 1 && bt.B <= 64 && base * n > sms) ? 1 : 0;
     return true;
 }

@@ -13,6 +13,8 @@ constexpr float kLog2e = 1.4426950408889634f;
 constexpr float kSumLimit = 1.0995e12f;        // 2^40: a tile's sum above this raises the row's reference
 constexpr float kRaiseAbove = 32.f;            // log2 units: ... where the maximum itself is looked at (128 x 2^32 < 2^40)
 constexpr int kMaxChunks = 8;                  // = portable cluster size
+constexpr int kStartBlocks = 5;                // cache blocks that fit the 128-key kernel's ring at once beside the tree's
+constexpr int kTreeBlocks = 3;                 // blocks that the tree counts for in its longer chunks, see chunk_range
 constexpr int kSplitRounds = 8;                // launches of fewer whole rounds get their remainder as a chunked launch
 
 __device__ __forceinline__ float max3(float a, float b, float c) {
@@ -78,6 +80,7 @@ __host__ __device__ constexpr int rows_per_chunk(int n_chunks) { return ((kRowTi
 struct AttnPlan {
     int n_chunks;      // CTAs per row tile along the keys (a cluster): the most chunks that a sequence's keys are cut into
     int whole_blocks;  // sequences of at most so many cache blocks stay whole; -1: every one is cut into n_chunks
+    int tree_blocks = 0;     // cache blocks that the tree's keys count for in chunks of more than kStartBlocks (chunk_range)
     uint32_t chunk_magic;    // ceil(2^32 / n_chunks): x / n_chunks for x below 2^29 (n_chunks > 1)
     int rows;          // T_max * G
     int tile_nodes;    // tree nodes of a row tile: its rows are whole nodes, the query heads of one KV head each
@@ -117,16 +120,25 @@ __device__ __forceinline__ int sequence_of_rank(const sd_batch& bt, int rank, in
 // Where sequences may stay whole, the others are cut into the smallest number of chunks, up to n_chunks, whose longest
 // is as short as n_chunks make it.  All of it follows from the sequence's own length: the block table may be far
 // wider than any sequence of the batch.
+// The tree's keys, in the last chunk, take as long as about three blocks where their copies cannot start with the first
+// ones (kStartBlocks and the tree fill the ring): they wait for a V slot, the softmax for them, because it clears the
+// rows of unused nodes, and masked scores take longer.  With the blocks alone dealt out evenly the last chunk's
+// softmax ended 1.6 us behind the others' of one sequence of 2048 tokens and 60 nodes, 3 us in eight chains of 4096
+// tokens.  Us per call with the tree counted as 0, 1, 2, 3, 4 blocks: eight chains of 4096 tokens 16.8 16.4 16.4 16.4
+// 16.4, four sequences of 2048 and 60 nodes 13.9 14.3 14.4 14.0 14.0, one chain of 8192 13.1 12.6 12.6 12.6 12.6, 28 layers
+// of one sequence of 2048 (and the LM head) 468 456 456 456 456; in shorter chunks it gains nothing (15 blocks in four
+// chunks: 8.05 8.17 9.01 9.04 8.97: an odd block is half a tile).
 struct ChunkRange { int n_chunks, tiles_total, tpc, t0, t1; };
 __host__ __device__ __forceinline__ ChunkRange chunk_range(const AttnPlan& plan, int len, int max_blocks, int chunk) {
     ChunkRange r;
     r.tiles_total = min((len + kBlock - 1) / kBlock, max_blocks);
     const bool whole = plan.n_chunks == 1 || r.tiles_total <= max(plan.whole_blocks, 0);
-    r.tpc = whole ? r.tiles_total : (int)(((uint64_t)(uint32_t)(r.tiles_total + plan.n_chunks - 1) * plan.chunk_magic) >> 32);
+    const int counted = r.tiles_total + (r.tiles_total > kStartBlocks * plan.n_chunks ? plan.tree_blocks : 0);
+    r.tpc = whole ? r.tiles_total : (int)(((uint64_t)(uint32_t)(counted + plan.n_chunks - 1) * plan.chunk_magic) >> 32);
     r.n_chunks = whole ? 1 : plan.n_chunks;
     if (plan.whole_blocks >= 0 && !whole) {
         r.n_chunks = 2;
-        while (r.n_chunks * r.tpc < r.tiles_total) ++r.n_chunks;
+        while (r.n_chunks * r.tpc < counted) ++r.n_chunks;
     }
     r.t0 = min(chunk * r.tpc, r.tiles_total);
     r.t1 = min(r.t0 + r.tpc, r.tiles_total);
