@@ -559,13 +559,18 @@ static AttnPlan common_plan(const sd_batch& bt, int n_layers, const TestKnobs& k
     return p;
 }
 
-// The 128-key kernel (attention_wide.cu) runs one CTA per SM.  A round of it takes about 0.36 us per cache block
-// of its longest chunk, plus 8 us for launch, first copies and output (11 when CTAs of another round follow:
-// nothing overlaps them), plus the merge of the chunks, plus about 1 us where the next call's CTAs find no
-// free SMs to set up on while this one runs.  Measured per call in us for 1 to 8 chunks: one sequence of 2048
-// tokens and 60 nodes 16.6 12.6 11.0 10.2 9.8 9.8 15.6 15.4 (16 clusters of seven or eight are more than fit
-// at a time), of 8192 50.7 29.7 22.2 18.5 16.8 15.9 25.1 24.2, one chain of 11 nodes over 4096 27.9 18.3 14.4
-// 12.6 11.6 11.0 10.4 10.4.  Chunk counts that are no powers of two fill SMs that those leave idle: ten such
+// The 128-key kernel (attention_wide.cu) runs one CTA per SM.  One round of it takes 5 us, or about 6 with a merge of
+// chunks, plus 0.02 us per CTA (they share the memory that the first copies come from), plus 0.4 us per cache block
+// of its longest chunk, in tiles of two, plus about 0.5 us where the next call's CTAs find no free SMs to set up on
+// while this one runs: fitted to calls of 1 to 16 sequences of 200 to 8192 tokens, trees of 11, 28 and 60 nodes, 1 to 8
+// chunks, of which it picks one within 1.5 % of the fastest on average (12 % at most).  With 8 us and 2.8 to 3.8 us for
+// the merge, which it took before, middling sequences stayed whole or in two for too long: two of 900 tokens and 60 nodes
+// 11.2 us instead of 10.0, four of 1100 13.0 instead of 11.7, eight of 1300 and 28 nodes 14.4 instead of 12.8.  In
+// launches of several rounds, where nothing overlaps a round's ends, each takes 11 us, the merge, and 0.36 us per block.
+// Measured per call in us for 1 to 8 chunks: one sequence of 2048 tokens and 60 nodes 16.4 12.7 10.9 9.9 9.9 10.1 15.6
+// 15.2 (16 clusters of seven or eight are more than fit at a time), of 8192 50.8 29.7 22.1 18.3 17.1 16.0 25.1 23.7, one
+// chain of 11 nodes over 4096 27.8 18.0 14.3 12.2 11.5 11.0 10.5 9.9.  Chunk counts that are no powers of two fill SMs that
+// those leave idle: ten such
 // chains 19.3 us with three chunks (21.4 with two), five sequences of 2000 tokens with 16 heads 13.0 (14.6).
 // The table's width stands for the longest length here, which the host does not know: a table that is far wider
 // makes long launches look longer than they are (in a table of 512 blocks 256 CTAs of 1000 tokens take 26.4 instead
@@ -582,11 +587,21 @@ static bool wide_plan(AttnPlan* p, const sd_batch& bt, int dev, int sms, const T
     int n = 1;
     long long n_rounds = 1;
     double best = 1e30;
+    p->tree_blocks = kTreeBlocks;
+    const bool forced = knobs.chunks > 0 && knobs.chunks <= blocks;
+    auto whole = [&](int c) { return forced ? 0 : (c == 2 ? 10 : 5); };   // blocks of a sequence that is not cut, see below
     for (int c = 1; c <= kMaxChunks && c <= blocks; ++c) {
+        if (c > 1 && blocks <= whole(c)) continue;         // (CTAs without work: eight chains of 200 tokens 7.6 instead of 7.0 us)
         const int resident = wide_resident_clusters(dev, sms, c);
         const long long rounds = (base + resident - 1) / resident;
-        const double us = rounds * ((rounds > 1 ? 11.0 : (2 * base * c > sms ? 9.1 : 8.0)) + merge[c - 1] + 0.36 * ((blocks + c - 1) / c));
-        if (knobs.chunks > 0 && knobs.chunks <= blocks ? c == knobs.chunks : us < best - 1e-9) { best = us; n = c; n_rounds = rounds; }
+        double us = rounds * (11.0 + merge[c - 1] + 0.36 * ((blocks + c - 1) / c));
+        if (rounds == 1) {                                 // blocks of the longest chunk, of a sequence and its tree that fill the table
+            p->set_chunks(c, whole(c));
+            const ChunkRange last = chunk_range(*p, (min(blocks, 1 << 24) - 1) * kBlock, blocks, c - 1);
+            const int per = max(last.tpc, last.t1 - last.t0 + 1);
+            us = (c == 1 ? 5.0 : 5.8 + 0.1 * c) + 0.02 * base * c + (2 * base * c > sms ? 0.52 : 0.0) + 0.28 * per + 0.25 * ((per + 1) / 2);
+        }
+        if (forced ? c == knobs.chunks : us < best - 1e-9) { best = us; n = c; n_rounds = rounds; }
     }
     if (n_rounds > 1) {
         const double rounds = base <= 2 * sms ? 1.0 : (double)base / (2 * sms) + 0.25;     // a partial round, cut into chunks
@@ -602,8 +617,7 @@ static bool wide_plan(AttnPlan* p, const sd_batch& bt, int dev, int sms, const T
     // 20.4 us, 19.8 with chunks as long as the longest's; 100 to 3000 tokens 11.4 against 11.7).
     // In several rounds every sequence is cut alike: the CTAs that leave would still hold back the next cluster
     // (half-empty pairs halved the machine).
-    p->set_chunks(n, n_rounds > 1 ? -1 : (knobs.chunks > 0 ? 0 : (n == 2 ? 10 : 5)));
-    p->tree_blocks = kTreeBlocks;
+    p->set_chunks(n, n_rounds > 1 ? -1 : whole(n));
     p->ranked = (bt.B > 1 && bt.B <= 64 && base * n > sms) ? 1 : 0;
     return true;
 }
@@ -640,6 +654,7 @@ static void narrow_plan(AttnPlan* plan, const sd_batch& bt, int sms, const TestK
     }
     if (knobs.chunks > 0 && knobs.chunks <= max_tiles && (knobs.chunks & (knobs.chunks - 1)) == 0) n = knobs.chunks;     // test hook
     p.set_chunks(n, -1);
+    p.tree_blocks = 0;
     p.ranked = (bt.B > 1 && bt.B <= 64 && (long long)base * n > slots) ? 1 : 0;
 }
 
