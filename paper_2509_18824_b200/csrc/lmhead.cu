@@ -27,7 +27,7 @@ constexpr int kEpiChunks = 4;       // chunks of 32 columns per epilogue warp, a
 __host__ __device__ constexpr int epi_threads(int par) { return par * 128; }
 __host__ __device__ constexpr int lm_threads(int par) { return epi_threads(par) + 32 + 1; }
 constexpr int kMaxCols = kLmMaxCols; // hidden rows per launch (TMEM columns)
-constexpr int kMaxCtas = 256;
+constexpr int kMaxCtas = kLmMaxCtas;
 constexpr int kMaxStages = 8;
 constexpr int kSmemBudget = 227 * 1024 - 2048;
 
@@ -86,12 +86,6 @@ __device__ __forceinline__ int32_t ordered_key(uint32_t bits) {
     int32_t b = (int32_t)bits;
     b = (b < 0) ? (b ^ 0x7fffffff) : b;
     return (b == -1) ? 0 : b;            // -0.0f maps to -1 above; fold it onto +0.0f
-}
-
-__device__ __forceinline__ float redux_max_f32(float v) {
-    float d;
-    asm volatile("redux.sync.max.f32 %0, %1, 0xffffffff;" : "=f"(d) : "f"(v));
-    return d;
 }
 
 // element `lane` of a 32-entry register array, by a binary tree of selects on the lane's bits
@@ -664,18 +658,18 @@ lmhead_merge_kernel(const int32_t* __restrict__ part_key, const int32_t* __restr
     }
 }
 
-// the same merge plus log sum exp(logit / temperature) of every hidden row (natural log);
-// eight threads per row share the CTAs' partials and combine through shuffles (fixed order)
+// the same merge plus log sum exp(logit / temperature) of every hidden row (natural log), one warp per row
 __global__ void __launch_bounds__(256)
 lmhead_merge_stats_kernel(const int32_t* __restrict__ part_key, const int32_t* __restrict__ part_idx,
                           const float* __restrict__ part_ref, const float* __restrict__ part_sum,
                           int n_ctas, int rows, int row0, float c2, int32_t* __restrict__ argmax,
                           float* __restrict__ maxlogit, float* __restrict__ lse) {
     begin_dependent(part_key, part_idx, part_ref, part_sum);
-    const int col = blockIdx.x * 32 + (threadIdx.x >> 3), sub = threadIdx.x & 7;
+    const int col = blockIdx.x * 8 + (threadIdx.x >> 5), lane = threadIdx.x & 31;
+    if (col >= rows) return;
     int32_t k, i;
-    const float row_lse = merge_row_stats(part_key, part_idx, part_ref, part_sum, n_ctas, kMaxCols, col, col < rows, sub, c2, k, i);
-    if (col < rows && sub == 0) {
+    const float row_lse = merge_row_stats(part_key, part_idx, part_ref, part_sum, n_ctas, kMaxCols, col, lane, c2, k, i);
+    if (lane == 0) {
         if (argmax) argmax[row0 + col] = i;
         if (maxlogit) maxlogit[row0 + col] = key_to_float(k);
         lse[row0 + col] = row_lse;
@@ -807,8 +801,8 @@ static sd_status launch_lmhead_impl(const void* hidden, const void* W, int M, in
             return SD_OK;
         }
         if (mass_out) continue;                      // nothing to merge: the epilogue stored the probabilities
-        const dim3 mgrid((p.rows + 31) / 32);
-        const sd_status ms = lse ? launch_dependent(lmhead_merge_stats_kernel, mgrid, 256, 0, 1, st, p.part_key, p.part_idx, p.part_ref,
+        const dim3 mgrid((p.rows + 31) / 32), sgrid((p.rows + 7) / 8);
+        const sd_status ms = lse ? launch_dependent(lmhead_merge_stats_kernel, sgrid, 256, 0, 1, st, p.part_key, p.part_idx, p.part_ref,
                                                     p.part_sum, grid, p.rows, p.row0, p.c2, argmax, maxlogit, lse)
                                  : launch_dependent(lmhead_merge_kernel, mgrid, 256, 0, 1, st, p.part_key, p.part_idx, grid, p.rows,
                                                     p.row0, argmax, maxlogit);

@@ -105,25 +105,36 @@ __device__ __forceinline__ void warp_dots_bf16(const uint4* (&a)[NR], const uint
     }
 }
 
-// Probability, under its parent's target distribution, of the token drafted at node j of sequence b
-// (0 for the root and for unused nodes); one warp.  lse: log sum exp of the LM-head rows.
+// Logit, behind its parent, of the token drafted at node j of sequence b; one warp.  false for the root and for unused
+// nodes (probability 0), and for nodes that are no tree's (reported).
+__device__ __forceinline__ bool child_logit(const sd_batch& bt, int b, int j, int lane, const uint16_t* __restrict__ hidden,
+                                            const uint16_t* __restrict__ W, int Hd, int V, const int32_t* __restrict__ draft,
+                                            int32_t* status, int& parent, float& logit) {
+    const int T = bt.T_max;
+    const int n = bt.n_nodes[b];
+    const int par = bt.parents[(size_t)b * T + j];         // (j < T; loaded whether used or not: one latency for all three)
+    const int tok = draft[(size_t)b * T + j];
+    if (!(j >= 1 && j < n && n <= T)) return false;
+    if (par < 0 || par >= j || tok < 0 || tok >= V) {
+        if (lane == 0) set_status(status, par < 0 || par >= j ? SD_ERR_INVALID_TREE : SD_ERR_BOUNDS);
+        return false;
+    }
+    parent = par;
+    const uint4* wrow[1] = {reinterpret_cast<const uint4*>(W + (size_t)tok * Hd)};
+    float l[1];
+    warp_dots_bf16<1>(wrow, reinterpret_cast<const uint4*>(hidden + (size_t)(b * T + par) * Hd), Hd / 8, lane, l);
+    logit = l[0];
+    return true;
+}
+
+// ... and its probability under the parent's target distribution.  lse: log sum exp of the LM-head rows.
 __device__ __forceinline__ float child_prob(const sd_batch& bt, int b, int j, int lane, const uint16_t* __restrict__ hidden,
                                             const uint16_t* __restrict__ W, int Hd, int V, float inv_temp, const float* lse,
                                             const int32_t* __restrict__ draft, int32_t* status) {
-    const int T = bt.T_max;
-    const int n = bt.n_nodes[b];
-    if (!(j >= 1 && j < n && n <= T)) return 0.f;
-    const int par = bt.parents[(size_t)b * T + j];
-    const int tok = draft[(size_t)b * T + j];
-    if (par < 0 || par >= j || tok < 0 || tok >= V) {
-        if (lane == 0) set_status(status, par < 0 || par >= j ? SD_ERR_INVALID_TREE : SD_ERR_BOUNDS);
-        return 0.f;
-    }
-    const int row = b * T + par;
-    const uint4* wrow[1] = {reinterpret_cast<const uint4*>(W + (size_t)tok * Hd)};
-    float l[1];
-    warp_dots_bf16<1>(wrow, reinterpret_cast<const uint4*>(hidden + (size_t)row * Hd), Hd / 8, lane, l);
-    return __expf(l[0] * inv_temp - lse[row]);
+    int par = 0;
+    float logit = 0.f;
+    if (!child_logit(bt, b, j, lane, hidden, W, Hd, V, draft, status, par, logit)) return 0.f;
+    return __expf(logit * inv_temp - lse[b * bt.T_max + par]);
 }
 
 // one warp per (sequence, node)
@@ -148,13 +159,9 @@ child_prob_kernel(sd_batch bt, const uint16_t* __restrict__ hidden, const uint16
 struct WalkOut { int32_t* path; int32_t* out_tok; int32_t* excl; float* excl_p; };
 struct WalkEnd { int na, stop, n_excl; float R; };
 
-__device__ __forceinline__ WalkEnd sampled_walk(const sd_batch& bt, int b, int lane, const int32_t* __restrict__ draft,
-                                                const float* p_child, const float* __restrict__ u, const WalkOut& o,
-                                                int32_t* status) {
-    const int T = bt.T_max;
-    const int n = bt.n_nodes[b];
-    const int32_t* par = bt.parents + (size_t)b * T;
-    const int32_t* dt = draft + (size_t)b * T;
+// n nodes of at most T; par, dt, p_child, u: the sequence's own (global or shared memory).
+__device__ __forceinline__ WalkEnd sampled_walk(int n, int T, int lane, const int32_t* par, const int32_t* dt, const float* p_child,
+                                                const float* u, const WalkOut& o, int32_t* status) {
     bool bad = (n < 1 || n > T);
     if (!bad)
         for (int i = lane; i < n; i += 32) {
@@ -169,8 +176,8 @@ __device__ __forceinline__ WalkEnd sampled_walk(const sd_batch& bt, int b, int l
     const bool has0 = lane < n, has1 = lane + 32 < n;
     const int pa0 = has0 ? par[lane] : -2, pa1 = has1 ? par[lane + 32] : -2;
     const int tk0 = has0 ? dt[lane] : -1, tk1 = has1 ? dt[lane + 32] : -1;
-    const float pc0 = has0 ? p_child[(size_t)b * T + lane] : 0.f, pc1 = has1 ? p_child[(size_t)b * T + lane + 32] : 0.f;
-    const float u0 = has0 ? u[(size_t)b * T + lane] : 0.f, u1 = has1 ? u[(size_t)b * T + lane + 32] : 0.f;
+    const float pc0 = has0 ? p_child[lane] : 0.f, pc1 = has1 ? p_child[lane + 32] : 0.f;
+    const float u0 = has0 ? u[lane] : 0.f, u1 = has1 ? u[lane + 32] : 0.f;
     int cur = 0, na = 1;
     float R = 1.f;
     if (lane == 0) o.path[0] = 0;
@@ -215,7 +222,8 @@ __global__ void sampled_walk_kernel(sd_batch bt, const int32_t* __restrict__ dra
     const int b = blockIdx.x, lane = threadIdx.x;
     const int T = bt.T_max;
     const WalkOut o{path + (size_t)b * T, out_tok + (size_t)b * T, excl + (size_t)b * 64, excl_p + (size_t)b * 64};
-    const WalkEnd e = sampled_walk(bt, b, lane, draft, p_child, u, o, status);
+    const size_t at = (size_t)b * T;
+    const WalkEnd e = sampled_walk(bt.n_nodes[b], T, lane, bt.parents + at, draft + at, p_child + at, u + at, o, status);
     if (lane == 0) {
         n_acc[b] = e.na;
         n_excl[b] = e.n_excl;
@@ -351,13 +359,16 @@ residual_pick_kernel(sd_batch bt, int V, const float* __restrict__ w, const floa
 constexpr int kPickMaxGroups = 8192;   // vocabularies up to 262144 tokens
 // kClusterCtas > 1: the CTAs of the cluster share the reading of the table (each entry sits in a
 // sector of its own, so one SM's load path is the limit) and push the masses into the shared memory
-// of the cluster's first CTA, which alone goes on; every CTA of the cluster must make the call.
-template <int kClusterCtas>
+// of the cluster's first CTA, which finds the group; its logits are recomputed by all CTAs again (one SM took
+// 5.9 us for the 32 rows of W, now 2.8), four tokens each, and the first CTA goes on.  Every CTA of the cluster
+// must make the call; while the first one searches, the others do `meanwhile`.
+template <int kClusterCtas, typename Meanwhile>
 __device__ __forceinline__ void residual_pick_groups(const uint16_t* __restrict__ hidden, const uint16_t* __restrict__ W,
                                                      int Hd, int V, float inv_temp, float row_lse, int M, int row,
                                                      const float2* __restrict__ group_stats, int n_groups, float wb,
                                                      int ne, const int32_t* excl, const float* excl_p,
-                                                     int32_t* out_slot, int32_t* status) {
+                                                     int32_t* out_slot, int32_t* status, Meanwhile meanwhile) {
+    static_assert(kClusterCtas == 1 || kClusterCtas == 8, "four tokens of a group of 32 per CTA");
     __shared__ float s_g[kPickMaxGroups];
     __shared__ float s_part[256];                                      // sums of the threads' runs of groups
     __shared__ float s_m[32];
@@ -368,9 +379,16 @@ __device__ __forceinline__ void residual_pick_groups(const uint16_t* __restrict_
     const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
     const float c2 = inv_temp * 1.4426950408889634f;
     const float lse2 = row_lse * 1.4426950408889634f;
+    const int rank = kClusterCtas > 1 ? (int)sm100::cluster_ctarank() : 0;
+    const uint4* hrow = reinterpret_cast<const uint4*>(hidden + (size_t)row * Hd);
+    // probability of token t in the residual, its dot product with the row given; one warp
+    auto prob = [&](int t, float dot, const int32_t* ex) {
+        bool hit = false;
+        for (int e = lane; e < ne; e += 32) hit |= (ex[e] == t);
+        return (t >= V || __any_sync(0xffffffffu, hit)) ? 0.f : __expf(dot * inv_temp - row_lse);
+    };
     {
         // (one 8-byte entry per group, a table row apart: the loads of a batch are issued together)
-        const int rank = kClusterCtas > 1 ? (int)sm100::cluster_ctarank() : 0;
         const int per_cta = (n_groups + kClusterCtas - 1) / kClusterCtas;
         const int g_end = min(n_groups, (rank + 1) * per_cta);
         const uint32_t dst = kClusterCtas > 1 ? sm100::map_dsmem(sm100::smem_u32(s_g), 0) : 0;
@@ -395,8 +413,29 @@ __device__ __forceinline__ void residual_pick_groups(const uint16_t* __restrict_
         if (kClusterCtas > 1) {
             sm100::cluster_arrive_release();
             sm100::cluster_wait_acquire();
-            if (rank != 0) return;
         }
+    }
+    // the first CTA tells the others the group, and they send it their probabilities
+    auto together = [&] {
+        const int t = s_k * 32 + rank * 4 + warp;
+        if (warp < 4) {
+            const uint4* wrow[1] = {reinterpret_cast<const uint4*>(W + (size_t)min(t, V - 1) * Hd)};
+            float l[1];
+            warp_dots_bf16<1>(wrow, hrow, Hd / 8, lane, l);
+            const float m = prob(t, l[0], excl);
+            if (lane == 0) sm100::st_dsmem_f32(sm100::map_dsmem(sm100::smem_u32(&s_m[rank * 4 + warp]), 0), m);
+        }
+        __syncwarp();
+        sm100::cluster_arrive_release();
+        sm100::cluster_wait_acquire();
+    };
+    if (kClusterCtas > 1 && rank != 0) {
+        sm100::cluster_arrive_relaxed();
+        meanwhile();
+        __syncwarp();
+        sm100::cluster_wait_acquire();
+        together();
+        return;
     }
     if (threadIdx.x < ne) { s_ex[threadIdx.x] = excl[threadIdx.x]; s_exp[threadIdx.x] = excl_p[threadIdx.x]; }
     __syncthreads();
@@ -435,7 +474,14 @@ __device__ __forceinline__ void residual_pick_groups(const uint16_t* __restrict_
         if (lane == 0) { s_acc = acc; s_target = target; s_k = k; s_pick = -1; s_last = -1; }
     }
     __syncthreads();
-    const uint4* hrow = reinterpret_cast<const uint4*>(hidden + (size_t)row * Hd);
+    if (kClusterCtas > 1) {
+        if (threadIdx.x > 0 && threadIdx.x < kClusterCtas)
+            sm100::st_dsmem_f32(sm100::map_dsmem(sm100::smem_u32(&s_k), threadIdx.x), __int_as_float(s_k));
+        __syncwarp();
+        sm100::cluster_arrive_release();
+        sm100::cluster_wait_acquire();
+        together();
+    }
     // the 32 probabilities of group k, recomputed into s_m: eight warps, four tokens each
     auto recompute_group = [&](int k) {
         const int t0 = k * 32 + warp * 4;
@@ -446,16 +492,13 @@ __device__ __forceinline__ void residual_pick_groups(const uint16_t* __restrict_
         warp_dots_bf16<4>(wrow, hrow, Hd / 8, lane, l);
 #pragma unroll
         for (int i = 0; i < 4; ++i) {
-            const int t = t0 + i;
-            bool hit = false;
-            for (int e = lane; e < ne; e += 32) hit |= (s_ex[e] == t);
-            const float m = (t >= V || __any_sync(0xffffffffu, hit)) ? 0.f : __expf(l[i] * inv_temp - row_lse);
+            const float m = prob(t0 + i, l[i], s_ex);
             if (lane == 0) s_m[warp * 4 + i] = m;
         }
         __syncthreads();
     };
     for (int k = s_k; k < n_groups; ++k) {
-        recompute_group(k);
+        if (kClusterCtas == 1 || k > s_k) recompute_group(k);
         if (threadIdx.x < 32) {
             float acc = s_acc;
             int lastp = -1;
@@ -498,7 +541,7 @@ residual_pick_groups_kernel(sd_batch bt, const uint16_t* __restrict__ hidden, co
     if (na < 1 || na > bt.T_max) return;                               // bad tree: already reported
     const int row = stop_row[b];
     residual_pick_groups<1>(hidden, W, Hd, V, inv_temp, lse[row], bt.B * bt.T_max, row, group_stats, n_groups, w[b], n_excl[b],
-                            excl + (size_t)b * 64, excl_p + (size_t)b * 64, out_tok + (size_t)b * bt.T_max + na - 1, status);
+                            excl + (size_t)b * 64, excl_p + (size_t)b * 64, out_tok + (size_t)b * bt.T_max + na - 1, status, [] {});
 }
 
 // Chains drafted by SAMPLING from a draft distribution (one warp per sequence): node j's token is kept
@@ -595,63 +638,86 @@ sd_status launch_accept_chain_sampled(const sd_batch& bt, const void* hidden, co
 
 // ---------------------------------------------------------------------------
 // Tail of a verify step at a sampling temperature, behind the LM-head tiles of a statistics pass: one
-// cluster of eight CTAs per sequence.
-//   1. every CTA merges the per-CTA soft-max partials of eight of the sequence's LM-head rows -> lse
-//   2. every warp of the cluster computes one node's probability under its parent's distribution
-//   3. every CTA repeats the (cheap) rejection walk into its own shared memory
-//   4. the cluster's first CTA writes the outputs and draws the last token from the group table
-//   5. every CTA copies the accepted nodes' K/V into the caches of its share of the layers
-// Steps 1 and 2 hand their results on through global memory across a cluster barrier.  The arithmetic
-// is that of the stand-alone kernels (the same device functions), so the results are the same bits.
+// cluster of eight CTAs per sequence, each of whose 64 warps looks after one node.
+//   1. every warp computes the logit of its node's token behind the parent (a row of W), and merges the per-CTA
+//      soft-max partials of the node's LM-head row -> lse; both go to the shared memory of all eight CTAs
+//   2. every CTA turns them into probabilities and repeats the (cheap) rejection walk
+//   3. the cluster's first CTA writes the outputs and draws the last token from the group table
+//   4. the other CTAs copy the accepted nodes' K/V into the caches, in part while the first one searches
+// The arithmetic is that of the stand-alone kernels (the same device functions), so the results are the same bits.
+// Latency is what bounds it: 8 sequences of 60 nodes, vocabulary 152064, hidden size 3584, 28 layers take 16.4 us.  It was 28.8 with
+// the merge by two warps per CTA (4.4 us) in front of the logits (3.6), results exchanged through global memory and the walk
+// loading the tree behind them (6.7), one SM recomputing the group's logits (5.9) and then copying its layers (3.0).
 // ---------------------------------------------------------------------------
 constexpr int kTailCluster = 8;
 __global__ void __launch_bounds__(256)
 sampled_tail_kernel(sd_batch bt, const __grid_constant__ CompactLayers ly, int L, LmTables tb, float c2,
                     const uint16_t* __restrict__ hidden, const uint16_t* __restrict__ W, int Hd, int V, float inv_temp,
                     const float2* __restrict__ group_stats, int n_groups, const int32_t* __restrict__ draft,
-                    const float* __restrict__ u, const float* __restrict__ w, float* lse, float* p_child,
+                    const float* __restrict__ u, const float* __restrict__ w, float* lse,
                     int32_t* n_acc, int32_t* path, int32_t* out_tok, int32_t* new_len, int32_t* status) {
+    static_assert(kMaxT == kTailCluster * 8, "one warp of the cluster per node");
     __shared__ int32_t s_path[kMaxT], s_tok[kMaxT], s_excl[64];
     __shared__ float s_excl_p[64];
+    __shared__ int32_t s_par[kMaxT], s_dt[kMaxT];
+    __shared__ float s_u[kMaxT], s_p[kMaxT];
+    __shared__ float s_logit[kMaxT], s_lse[kMaxT];                     // of every node, from the warps of all eight CTAs
     __shared__ WalkEnd s_end;
-    begin_dependent(bt, tb.part_key, tb.part_idx, tb.part_ref, tb.part_sum, hidden, W, group_stats, draft, u, w, lse, p_child);
+    begin_dependent(bt, tb.part_key, tb.part_idx, tb.part_ref, tb.part_sum, hidden, W, group_stats, draft, u, w, lse);
     const int b = blockIdx.x / kTailCluster;
     const int rank = (int)sm100::cluster_ctarank();
     const int T = bt.T_max, warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
-    // 1. lse of rows rank * 8 .. + 7 (of every 64): eight lanes per row, the first two warps
-    if (warp < 2)
-        for (int r0 = 0; r0 < T; r0 += 8 * kTailCluster) {
-            const int node = r0 + rank * 8 + (threadIdx.x >> 3), sub = threadIdx.x & 7;
-            int32_t k, i;
-            const float row_lse = merge_row_stats(tb.part_key, tb.part_idx, tb.part_ref, tb.part_sum, tb.n_ctas, kLmMaxCols,
-                                                  b * T + node, node < T, sub, c2, k, i);
-            if (node < T && sub == 0) lse[b * T + node] = row_lse;
-        }
-    sm100::cluster_arrive_release();
-    sm100::cluster_wait_acquire();
-    // 2. probabilities of the drafted tokens: node rank * 8 + warp (of every 64)
-    for (int j0 = 0; j0 < T; j0 += 8 * kTailCluster) {
-        const int j = j0 + rank * 8 + warp;
-        if (j < T) {
-            const float p = child_prob(bt, b, j, lane, hidden, W, Hd, V, inv_temp, lse, draft, status);
-            if (lane == 0) p_child[(size_t)b * T + j] = p;
-        }
+    const int n = bt.n_nodes[b];
+    if (threadIdx.x < T) {
+        const size_t at = (size_t)b * T + threadIdx.x;
+        s_par[threadIdx.x] = bt.parents[at]; s_dt[threadIdx.x] = draft[at]; s_u[threadIdx.x] = u[at];
     }
+    __syncwarp();
+    sm100::cluster_arrive_relaxed();                                   // every CTA of the cluster is there to be written to
+    const int node = rank * 8 + warp;
+    float logit = -INFINITY, row_lse = 0.f;                            // (no child of a tree: probability 0)
+    if (node < T) {
+        int par, k, i;
+        const bool child = child_logit(bt, b, node, lane, hidden, W, Hd, V, draft, status, par, logit);
+        row_lse = merge_row_stats(tb.part_key, tb.part_idx, tb.part_ref, tb.part_sum, tb.n_ctas, kLmMaxCols, b * T + node, lane, c2, k, i);
+        if (lane == 0) lse[b * T + node] = row_lse;
+        if (!child) logit = -INFINITY;
+    }
+    __syncwarp();
+    sm100::cluster_wait_acquire();
+    if (node < T && lane < kTailCluster) {
+        sm100::st_dsmem_f32(sm100::map_dsmem(sm100::smem_u32(&s_logit[node]), lane), logit);
+        sm100::st_dsmem_f32(sm100::map_dsmem(sm100::smem_u32(&s_lse[node]), lane), row_lse);
+    }
+    __syncwarp();
     sm100::cluster_arrive_release();
     sm100::cluster_wait_acquire();
-    // 3. the walk
+    // 2. the walk
+    if (threadIdx.x < T)
+        s_p[threadIdx.x] = s_logit[threadIdx.x] == -INFINITY ? 0.f
+                                                             : __expf(s_logit[threadIdx.x] * inv_temp - s_lse[s_par[threadIdx.x]]);
+    __syncthreads();
     if (warp == 0) {
         const WalkOut o{s_path, s_tok, s_excl, s_excl_p};
-        const WalkEnd e = sampled_walk(bt, b, lane, draft, p_child, u, o, status);
+        const WalkEnd e = sampled_walk(n, T, lane, s_par, s_dt, s_p, s_u, o, status);
         if (lane == 0) s_end = e;
     }
     __syncthreads();
     const WalkEnd e = s_end;
-    // 4. outputs and the last token (the whole cluster reads the group table, the first CTA draws)
+    // 3. outputs and the last token (the whole cluster reads the group table, the first CTA draws)
     if (rank == 0 && threadIdx.x == 0) {
         n_acc[b] = e.na;
         if (e.na > 0) new_len[b] = bt.len[b] + e.na;
     }
+    // 4. accepted rows into the caches: this CTA's consecutive layers, the next `count` of them
+    const int each = (L + kTailCluster - 2) / (kTailCluster - 1);
+    int l = (rank - 1) * each;
+    const int l_end = rank > 0 ? min(L, l + each) : l;
+    auto copy_layers = [&](int count) {
+        const int n_layers = max(min(count, l_end - l), 0);
+        compact_sequence(bt, ly, l, n_layers, b, e.na, s_path, threadIdx.x, blockDim.x, status);
+        l += n_layers;
+    };
     if (e.na > 0) {                                                    // (the same in every CTA of the cluster)
         if (rank == 0)
             for (int k = threadIdx.x; k < T; k += blockDim.x) {
@@ -659,12 +725,11 @@ sampled_tail_kernel(sd_batch bt, const __grid_constant__ CompactLayers ly, int L
                 if (k != e.na - 1) out_tok[(size_t)b * T + k] = s_tok[k];
             }
         const int row = b * T + e.stop;
-        residual_pick_groups<kTailCluster>(hidden, W, Hd, V, inv_temp, lse[row], bt.B * T, row, group_stats, n_groups, w[b],
-                                           e.n_excl, s_excl, s_excl_p, out_tok + (size_t)b * T + e.na - 1, status);
+        residual_pick_groups<kTailCluster>(hidden, W, Hd, V, inv_temp, s_lse[e.stop], bt.B * T, row, group_stats, n_groups, w[b],
+                                           e.n_excl, s_excl, s_excl_p, out_tok + (size_t)b * T + e.na - 1, status,
+                                           [&] { copy_layers(4); });
     }
-    // 5. accepted rows into the caches; the first CTA, busy with the draw, takes the smallest share
-    for (int l = kTailCluster - 1 - rank; l < L; l += kTailCluster)
-        compact_sequence(bt, ly, l, 1, b, e.na, s_path, threadIdx.x, blockDim.x, status);
+    if (rank != 0) copy_layers(L);
 }
 
 sd_status launch_lmhead_accept_sampled_compact(const sd_batch& bt, const void* hidden, const void* W, int Hd, int V,
@@ -698,8 +763,8 @@ sd_status launch_lmhead_accept_sampled_compact(const sd_batch& bt, const void* h
     const float c2 = inv_temp * 1.4426950408889634f;
     const int n_groups = (V + 31) / 32;
     return launch_dependent(sampled_tail_kernel, dim3(B * kTailCluster), 256, 0, kTailCluster, st, bt, ly, L, tb, c2, hidden, W, Hd, V,
-                            inv_temp, reinterpret_cast<const float2*>(group_stats), n_groups, draft, u, w, lse, s.p_child, n_acc, path,
-                            out_tok, new_len, dev_status);
+                            inv_temp, reinterpret_cast<const float2*>(group_stats), n_groups, draft, u, w, lse, n_acc, path, out_tok,
+                            new_len, dev_status);
 }
 
 sd_status launch_accept_sampled(const sd_batch& bt, const void* hidden, const void* W, int Hd, int V, float inv_temp,

@@ -73,50 +73,55 @@ __device__ __forceinline__ void merge_row_argmax(const int32_t* part_key, const 
     }
 }
 
-// Candidates and soft-max partials of one hidden row (column `col` of the per-CTA tables), merged by the
-// eight consecutive lanes that share the row: lane `sub` takes the CTAs sub, sub + 8, ..., then three
-// exchange steps combine the eight (always lower lane first, so all eight end with the same bits).
-// Every lane of the warp must call this; rows beyond the problem pass active = false.  Returns the
-// row's log sum exp(logit / temperature) (natural log); k, i: the arg-max candidate (key, index).
+// maximum over the warp (numbers win over NaN)
+__device__ __forceinline__ float redux_max_f32(float v) {
+    float d;
+    asm volatile("redux.sync.max.f32 %0, %1, 0xffffffff;" : "=f"(d) : "f"(v));
+    return d;
+}
+
+// Candidates and soft-max partials of one hidden row (column `col` of the per-CTA tables), merged by one warp:
+// lane l takes the CTAs l, l + 32, ... (all of its loads in flight together), the sums are brought to the
+// largest reference of the row and added up in a fixed order.  Every lane must call this and gets the row's
+// log sum exp(logit / temperature) (natural log) and the arg-max candidate (key, index).
+// (Latency is what it takes: with eight lanes per row, 19 partials one after the other in each, the sampled tail of 480
+// rows spent 4.4 us here, and the merge kernel took 6.5 us; see sampled_tail_kernel and lmhead_merge_stats_kernel.)
+constexpr int kLmMaxCtas = 256;          // CTAs of an LM-head pass
 __device__ __forceinline__ float merge_row_stats(const int32_t* __restrict__ part_key, const int32_t* __restrict__ part_idx,
                                                  const float* __restrict__ part_ref, const float* __restrict__ part_sum,
-                                                 int n_ctas, int row_stride, int col, bool active, int sub, float c2,
-                                                 int32_t& k, int32_t& i) {
+                                                 int n_ctas, int row_stride, int col, int lane, float c2, int32_t& k, int32_t& i) {
+    constexpr int kPer = kLmMaxCtas / 32;
     k = INT32_MIN; i = 0x7fffffff;
-    float rf = -INFINITY, sm = 0.f;
-    if (active) {
-        // (the loads of a batch are issued together, then merged in CTA order: latency-bound)
-        constexpr int kAhead = 20;                  // 148 CTAs: 19 per lane
-        for (int c0 = sub; c0 < n_ctas; c0 += 8 * kAhead) {
-            int32_t pk[kAhead], pi[kAhead];
-            float pr[kAhead], ps[kAhead];
+    int32_t pk[kPer], pi[kPer];
+    float pr[kPer], ps[kPer];
 #pragma unroll
-            for (int a = 0; a < kAhead; ++a) {
-                const int c = c0 + 8 * a;
-                if (c < n_ctas) {
-                    pk[a] = __ldg(part_key + (size_t)c * row_stride + col);
-                    pi[a] = __ldg(part_idx + (size_t)c * row_stride + col);
-                    pr[a] = __ldg(part_ref + (size_t)c * row_stride + col);
-                    ps[a] = __ldg(part_sum + (size_t)c * row_stride + col);
-                }
-            }
-#pragma unroll
-            for (int a = 0; a < kAhead; ++a)
-                if (c0 + 8 * a < n_ctas) {
-                    take_better(k, i, pk[a], pi[a]);
-                    merge_sumexp(rf, sm, pr[a], ps[a], c2);
-                }
+    for (int a = 0; a < kPer; ++a) {
+        const int c = lane + 32 * a;
+        pk[a] = INT32_MIN; pi[a] = 0x7fffffff; pr[a] = -INFINITY; ps[a] = 0.f;
+        if (c < n_ctas) {
+            pk[a] = __ldcg(part_key + (size_t)c * row_stride + col);
+            pi[a] = __ldcg(part_idx + (size_t)c * row_stride + col);
+            pr[a] = __ldcg(part_ref + (size_t)c * row_stride + col);
+            ps[a] = __ldcg(part_sum + (size_t)c * row_stride + col);
         }
     }
+    float rf = -INFINITY;
 #pragma unroll
-    for (int d = 1; d <= 4; d <<= 1) {
+    for (int a = 0; a < kPer; ++a) {
+        take_better(k, i, pk[a], pi[a]);
+        if (!(ps[a] > 0.f)) pr[a] = -INFINITY;             // (partials without mass, and those that are no numbers, do not count)
+        rf = fmaxf(rf, pr[a]);
+    }
+    rf = redux_max_f32(rf);
+    float sm = 0.f;
+#pragma unroll
+    for (int a = 0; a < kPer; ++a)
+        if (ps[a] > 0.f) sm += pr[a] == rf ? ps[a] : ps[a] * ex2_lm((pr[a] - rf) * c2);
+#pragma unroll
+    for (int d = 1; d < 32; d <<= 1) {
         const int32_t k2 = __shfl_xor_sync(0xffffffffu, k, d), i2 = __shfl_xor_sync(0xffffffffu, i, d);
-        const float rf2 = __shfl_xor_sync(0xffffffffu, rf, d), sm2 = __shfl_xor_sync(0xffffffffu, sm, d);
         take_better(k, i, k2, i2);
-        float ra = (sub & d) ? rf2 : rf, sa = (sub & d) ? sm2 : sm;
-        const float rb = (sub & d) ? rf : rf2, sb = (sub & d) ? sm : sm2;
-        merge_sumexp(ra, sa, rb, sb, c2);
-        rf = ra; sm = sa;
+        sm += __shfl_xor_sync(0xffffffffu, sm, d);
     }
     return (rf * c2 + log2f(sm)) * 0.6931471805599453f;
 }
@@ -266,21 +271,24 @@ __device__ __forceinline__ void compact_sequence(const sd_batch& bt, const Compa
                 src[u] = (((size_t)b * T + node) * bt.Hkv + kvh) * vec_per_head + c;
                 dst[u] = (((size_t)(blk[u] < 0 ? 0 : blk[u]) * bt.Hkv + kvh) * kBlock + (t % kBlock)) * vec_per_head + c;
             }
-            for (int l = l0; l < l0 + n_layers; ++l) {
-                const uint4* from = is_v ? ly.vt[l] : ly.kt[l];
-                uint4* to = is_v ? ly.vc[l] : ly.kc[l];
-                const int nb = ly.num_blocks[l];
-                uint4 val[kUnroll];
-                bool live[kUnroll];
+            // (two layers at a time, loaded together before either is stored: four layers of five rows 4.7 -> 3 us)
+            for (int l = l0; l < l0 + n_layers; l += 2) {
+                uint4 val[2][kUnroll];
+                bool live[2][kUnroll];
 #pragma unroll
-                for (int u = 0; u < kUnroll; ++u) {
-                    live[u] = has[u] && blk[u] >= 0 && blk[u] < nb;
-                    if (has[u] && !live[u]) set_status(status, SD_ERR_BOUNDS);
-                    if (live[u]) val[u] = from[src[u]];
-                }
+                for (int i = 0; i < 2; ++i)
 #pragma unroll
-                for (int u = 0; u < kUnroll; ++u)
-                    if (live[u]) to[dst[u]] = val[u];
+                    for (int u = 0; u < kUnroll; ++u) {
+                        const bool due = has[u] && l + i < l0 + n_layers;
+                        live[i][u] = due && blk[u] >= 0 && blk[u] < ly.num_blocks[l + i];
+                        if (due && !live[i][u]) set_status(status, SD_ERR_BOUNDS);
+                        if (live[i][u]) val[i][u] = (is_v ? ly.vt[l + i] : ly.kt[l + i])[src[u]];
+                    }
+#pragma unroll
+                for (int i = 0; i < 2; ++i)
+#pragma unroll
+                    for (int u = 0; u < kUnroll; ++u)
+                        if (live[i][u]) (is_v ? ly.vc[l + i] : ly.kc[l + i])[dst[u]] = val[i][u];
             }
         }
         return;
