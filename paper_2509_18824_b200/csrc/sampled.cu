@@ -639,8 +639,8 @@ sd_status launch_accept_chain_sampled(const sd_batch& bt, const void* hidden, co
 // ---------------------------------------------------------------------------
 // Tail of a verify step at a sampling temperature, behind the LM-head tiles of a statistics pass: one
 // cluster of eight CTAs per sequence, each of whose 64 warps looks after one node.
-//   1. every warp computes the logit of its node's token behind the parent (a row of W), and merges the per-CTA
-//      soft-max partials of the node's LM-head row -> lse; both go to the shared memory of all eight CTAs
+//   1. every warp computes the logit of its node's token behind the parent (a row of W), and every CTA merges the per-CTA
+//      soft-max partials of its eight nodes' LM-head rows -> lse; both go to the shared memory of all eight CTAs
 //   2. every CTA turns them into probabilities and repeats the (cheap) rejection walk
 //   3. the cluster's first CTA writes the outputs and draws the last token from the group table
 //   4. the other CTAs copy the accepted nodes' K/V into the caches, in part while the first one searches
@@ -662,6 +662,7 @@ sampled_tail_kernel(sd_batch bt, const __grid_constant__ CompactLayers ly, int L
     __shared__ int32_t s_par[kMaxT], s_dt[kMaxT];
     __shared__ float s_u[kMaxT], s_p[kMaxT];
     __shared__ float s_logit[kMaxT], s_lse[kMaxT];                     // of every node, from the warps of all eight CTAs
+    __shared__ MergeShared s_merge;
     __shared__ WalkEnd s_end;
     begin_dependent(bt, tb.part_key, tb.part_idx, tb.part_ref, tb.part_sum, hidden, W, group_stats, draft, u, w, lse);
     const int b = blockIdx.x / kTailCluster;
@@ -676,13 +677,11 @@ sampled_tail_kernel(sd_batch bt, const __grid_constant__ CompactLayers ly, int L
     sm100::cluster_arrive_relaxed();                                   // every CTA of the cluster is there to be written to
     const int node = rank * 8 + warp;
     float logit = -INFINITY, row_lse = 0.f;                            // (no child of a tree: probability 0)
-    if (node < T) {
-        int par, k, i;
-        const bool child = child_logit(bt, b, node, lane, hidden, W, Hd, V, draft, status, par, logit);
-        row_lse = merge_row_stats(tb.part_key, tb.part_idx, tb.part_ref, tb.part_sum, tb.n_ctas, kLmMaxCols, b * T + node, lane, c2, k, i);
-        if (lane == 0) lse[b * T + node] = row_lse;
-        if (!child) logit = -INFINITY;
-    }
+    int par, k, i;
+    if (node < T && !child_logit(bt, b, node, lane, hidden, W, Hd, V, draft, status, par, logit)) logit = -INFINITY;
+    row_lse = merge_rows_stats(s_merge, tb.part_key, tb.part_idx, tb.part_ref, tb.part_sum, tb.n_ctas, kLmMaxCols, b * T + rank * 8,
+                               (b + 1) * T, c2, k, i);
+    if (node < T && lane == 0) lse[b * T + node] = row_lse;
     __syncwarp();
     sm100::cluster_wait_acquire();
     if (node < T && lane < kTailCluster) {
@@ -715,7 +714,7 @@ sampled_tail_kernel(sd_batch bt, const __grid_constant__ CompactLayers ly, int L
     const int l_end = rank > 0 ? min(L, l + each) : l;
     auto copy_layers = [&](int count) {
         const int n_layers = max(min(count, l_end - l), 0);
-        compact_sequence(bt, ly, l, n_layers, b, e.na, s_path, threadIdx.x, blockDim.x, status);
+        compact_sequence<2>(bt, ly, l, n_layers, b, e.na, s_path, threadIdx.x, blockDim.x, status);
         l += n_layers;
     };
     if (e.na > 0) {                                                    // (the same in every CTA of the cluster)

@@ -73,57 +73,93 @@ __device__ __forceinline__ void merge_row_argmax(const int32_t* part_key, const 
     }
 }
 
-// maximum over the warp (numbers win over NaN)
-__device__ __forceinline__ float redux_max_f32(float v) {
-    float d;
-    asm volatile("redux.sync.max.f32 %0, %1, 0xffffffff;" : "=f"(d) : "f"(v));
-    return d;
+// Arg-max candidates of up to 64 hidden rows (columns col0 .. + rows - 1), merged by a CTA of 512 threads: lanes along the
+// columns, so that a load touches one or two lines of a table, an eighth of the CTAs' candidates per warp (all eight threads of a row
+// in one warp, eight lines per load: 3.1 us of the tail kernel, now 1.8).  Threads 0 .. rows - 1 return row threadIdx.x's.
+struct ArgmaxShared { int32_t key[8][64], idx[8][64]; };
+__device__ __forceinline__ void merge_rows_argmax(ArgmaxShared& sh, const int32_t* part_key, const int32_t* part_idx, int n_ctas,
+                                                  int row_stride, int col0, int rows, int32_t& k, int32_t& i) {
+    const int row = threadIdx.x & 63, part = threadIdx.x >> 6;
+    k = INT32_MIN; i = 0x7fffffff;
+    if (row < rows) {
+        // (the loads of a batch are issued together: one memory latency instead of a chain of them)
+        constexpr int kAhead = 20;                         // 148 CTAs: 19 per thread
+        for (int c0 = part; c0 < n_ctas; c0 += 8 * kAhead) {
+            int32_t pk[kAhead], pi[kAhead];
+#pragma unroll
+            for (int a = 0; a < kAhead; ++a) {
+                const int c = c0 + 8 * a;
+                if (c < n_ctas) {
+                    pk[a] = part_key[(size_t)c * row_stride + col0 + row];
+                    pi[a] = part_idx[(size_t)c * row_stride + col0 + row];
+                }
+            }
+#pragma unroll
+            for (int a = 0; a < kAhead; ++a)
+                if (c0 + 8 * a < n_ctas) take_better(k, i, pk[a], pi[a]);
+        }
+    }
+    sh.key[part][row] = k; sh.idx[part][row] = i;
+    __syncthreads();
+    if ((int)threadIdx.x < rows)
+        for (int w = 1; w < 8; ++w) take_better(k, i, sh.key[w][row], sh.idx[w][row]);
 }
 
-// Candidates and soft-max partials of one hidden row (column `col` of the per-CTA tables), merged by one warp:
-// lane l takes the CTAs l, l + 32, ... (all of its loads in flight together), the sums are brought to the
-// largest reference of the row and added up in a fixed order.  Every lane must call this and gets the row's
-// log sum exp(logit / temperature) (natural log) and the arg-max candidate (key, index).
-// (Latency is what it takes: with eight lanes per row, 19 partials one after the other in each, the sampled tail of 480
-// rows spent 4.4 us here, and the merge kernel took 6.5 us; see sampled_tail_kernel and lmhead_merge_stats_kernel.)
+// Candidates and soft-max partials of eight hidden rows (columns col0 .. + 7 of the per-CTA tables; those from col_end on
+// are not read), merged by a CTA of 256 threads.  Lanes 0 .. 7 of a warp, 8 .. 15, ... read one table row each, so that
+// a load touches four lines of the tables and not 32; all loads of a thread are in flight together; the sums are
+// brought to the largest reference of the row and added up in a fixed order.  Warp w returns row w's log sum
+// exp(logit / temperature) (natural log) and arg-max candidate (key, index) in all lanes.  Every thread must call this.
+// (Latency and the load path are what it takes: with eight lanes per row, 19 partials one after the other in each, the
+// sampled tail of 480 rows spent 4.4 us here, and the merge kernel took 6.5; see sampled_tail_kernel.)
 constexpr int kLmMaxCtas = 256;          // CTAs of an LM-head pass
-__device__ __forceinline__ float merge_row_stats(const int32_t* __restrict__ part_key, const int32_t* __restrict__ part_idx,
-                                                 const float* __restrict__ part_ref, const float* __restrict__ part_sum,
-                                                 int n_ctas, int row_stride, int col, int lane, float c2, int32_t& k, int32_t& i) {
+struct MergeShared { float ref[8][8], sum[8][8]; int32_t key[8][8], idx[8][8]; };      // [warp][row]
+__device__ __forceinline__ float merge_rows_stats(MergeShared& sh, const int32_t* __restrict__ part_key, const int32_t* __restrict__ part_idx,
+                                                  const float* __restrict__ part_ref, const float* __restrict__ part_sum,
+                                                  int n_ctas, int row_stride, int col0, int col_end, float c2, int32_t& k, int32_t& i) {
     constexpr int kPer = kLmMaxCtas / 32;
-    k = INT32_MIN; i = 0x7fffffff;
+    const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31, col = col0 + (lane & 7);
+    // one row's (reference, sum) from several: those without mass, or that are no numbers, do not count
+    auto rescaled = [&](float r, float sum, float ref) { return !(sum > 0.f) ? 0.f : (r == ref ? sum : sum * ex2_lm((r - ref) * c2)); };
     int32_t pk[kPer], pi[kPer];
     float pr[kPer], ps[kPer];
 #pragma unroll
     for (int a = 0; a < kPer; ++a) {
-        const int c = lane + 32 * a;
+        const int c = warp * 4 + (lane >> 3) + 32 * a;
         pk[a] = INT32_MIN; pi[a] = 0x7fffffff; pr[a] = -INFINITY; ps[a] = 0.f;
-        if (c < n_ctas) {
-            pk[a] = __ldcg(part_key + (size_t)c * row_stride + col);
-            pi[a] = __ldcg(part_idx + (size_t)c * row_stride + col);
-            pr[a] = __ldcg(part_ref + (size_t)c * row_stride + col);
-            ps[a] = __ldcg(part_sum + (size_t)c * row_stride + col);
+        if (c < n_ctas && col < col_end) {
+            const size_t at = (size_t)c * row_stride + col;
+            pk[a] = __ldcg(part_key + at); pi[a] = __ldcg(part_idx + at);
+            pr[a] = __ldcg(part_ref + at); ps[a] = __ldcg(part_sum + at);
         }
     }
-    float rf = -INFINITY;
+    k = INT32_MIN; i = 0x7fffffff;
+    float rf = -INFINITY, sm = 0.f;
 #pragma unroll
     for (int a = 0; a < kPer; ++a) {
         take_better(k, i, pk[a], pi[a]);
-        if (!(ps[a] > 0.f)) pr[a] = -INFINITY;             // (partials without mass, and those that are no numbers, do not count)
-        rf = fmaxf(rf, pr[a]);
+        if (ps[a] > 0.f) rf = fmaxf(rf, pr[a]);
     }
-    rf = redux_max_f32(rf);
-    float sm = 0.f;
 #pragma unroll
-    for (int a = 0; a < kPer; ++a)
-        if (ps[a] > 0.f) sm += pr[a] == rf ? ps[a] : ps[a] * ex2_lm((pr[a] - rf) * c2);
+    for (int d = 8; d <= 16; d <<= 1) rf = fmaxf(rf, __shfl_xor_sync(0xffffffffu, rf, d));
 #pragma unroll
-    for (int d = 1; d < 32; d <<= 1) {
+    for (int a = 0; a < kPer; ++a) sm += rescaled(pr[a], ps[a], rf);
+    auto across = [&](int d) {
         const int32_t k2 = __shfl_xor_sync(0xffffffffu, k, d), i2 = __shfl_xor_sync(0xffffffffu, i, d);
         take_better(k, i, k2, i2);
         sm += __shfl_xor_sync(0xffffffffu, sm, d);
-    }
-    return (rf * c2 + log2f(sm)) * 0.6931471805599453f;
+    };
+    across(8); across(16);
+    if (lane < 8) { sh.ref[warp][lane] = rf; sh.sum[warp][lane] = sm; sh.key[warp][lane] = k; sh.idx[warp][lane] = i; }
+    __syncthreads();
+    const int w = lane & 7;                                // this warp's row, warp w's share of it
+    rf = sh.ref[w][warp]; sm = sh.sum[w][warp]; k = sh.key[w][warp]; i = sh.idx[w][warp];
+    float top = sm > 0.f ? rf : -INFINITY;
+#pragma unroll
+    for (int d = 1; d <= 4; d <<= 1) top = fmaxf(top, __shfl_xor_sync(0xffffffffu, top, d));
+    sm = rescaled(rf, sm, top);
+    across(1); across(2); across(4);
+    return (top * c2 + log2f(sm)) * 0.6931471805599453f;
 }
 
 // Where the running sum *acc_io + v[0] + v[1] + ... first reaches `target`, among the elements with
@@ -173,16 +209,15 @@ __device__ __forceinline__ int warp_find_crossing(const float* v, int n, float t
     }
 }
 
-// Greedy acceptance for one sequence, executed by one warp.  par/dt/tg point at the sequence's
-// parents, draft tokens and target arg-max (tg may be shared memory).  Returns the number of
+// Greedy acceptance for one sequence of n nodes and len cached tokens, executed by one warp.  par/dt/tg: the
+// sequence's parents, draft tokens and target arg-max, in shared memory (from global memory every step of the walks
+// towards the root is a trip to the cache: 2.9 us of the tail kernel's 8, now 2.4).  Returns the number of
 // accepted nodes (0 for a bad tree, which is reported through *status) and, in lane 0, has written
 // n_acc, new_len, path and out_tok; `path_out` (nullable, e.g. shared memory) receives the path too.
-__device__ __forceinline__ int accept_sequence(const sd_batch& bt, int b, int lane, const int32_t* par,
+__device__ __forceinline__ int accept_sequence(int T, int b, int lane, int n, int len, const int32_t* par,
                                                const int32_t* dt, const int32_t* tg,
                                                int32_t* n_acc, int32_t* path, int32_t* out_tok, int32_t* new_len,
                                                int32_t* path_out, int32_t* status) {
-    const int T = bt.T_max;
-    const int n = bt.n_nodes[b];
     bool bad = (n < 1 || n > T);
     if (!bad)
         for (int i = lane; i < n; i += 32) {
@@ -193,20 +228,17 @@ __device__ __forceinline__ int accept_sequence(const sd_batch& bt, int b, int la
         if (lane == 0) set_status(status, SD_ERR_INVALID_TREE);
         return 0;
     }
-    // key = depth * 64 + (63 - index) for valid nodes: max key = deepest, lowest index
-    int best_key = -1;
-    for (int i = lane; i < n; i += 32) {
-        bool ok = true;
-        int depth = 0;
-        int j = i;
-        for (int step = 0; step < kMaxT && j > 0; ++step) {
-            int p = par[j];
-            ok = ok && (dt[j] == tg[p]);
-            ++depth;
-            j = p;
-        }
-        if (ok) best_key = max(best_key, depth * 64 + (63 - i));
+    // key = depth * 64 + (63 - index) for valid nodes: max key = deepest, lowest index.  A lane walks up from its
+    // two nodes at the same time.
+    int j0 = lane < n ? lane : 0, j1 = lane + 32 < n ? lane + 32 : 0;
+    int d0 = 0, d1 = 0;
+    bool ok0 = lane < n, ok1 = lane + 32 < n;
+    for (int step = 0; step < kMaxT && (j0 > 0 || j1 > 0); ++step) {
+        if (j0 > 0) { const int p = par[j0]; ok0 = ok0 && dt[j0] == tg[p]; ++d0; j0 = p; }
+        if (j1 > 0) { const int p = par[j1]; ok1 = ok1 && dt[j1] == tg[p]; ++d1; j1 = p; }
     }
+    int best_key = ok0 ? d0 * 64 + (63 - lane) : -1;
+    if (ok1) best_key = max(best_key, d1 * 64 + (31 - lane));
     best_key = __reduce_max_sync(0xffffffffu, best_key);   // node 0 is always valid
     const int best = 63 - (best_key & 63);
     const int na = (best_key >> 6) + 1;
@@ -215,7 +247,7 @@ __device__ __forceinline__ int accept_sequence(const sd_batch& bt, int b, int la
     for (int k = na + lane; k < T; k += 32) { pa[k] = -1; ot[k] = -1; }
     if (lane == 0) {
         n_acc[b] = na;
-        new_len[b] = bt.len[b] + na;
+        new_len[b] = len + na;
         int j = best;
         for (int k = na - 1; k >= 0; --k) {
             pa[k] = j;
@@ -231,6 +263,7 @@ __device__ __forceinline__ int accept_sequence(const sd_batch& bt, int b, int la
 // Copies the accepted rows of sequence b in layers [l0, l0 + n_layers): work items idx = tid, tid + stride, ...
 // One item = one 16-byte vector of one (layer, accepted node, K or V, KV head).  `path` holds the
 // sequence's accepted nodes (global or shared memory).
+template <int kLayers = 1>
 __device__ __forceinline__ void compact_sequence(const sd_batch& bt, const CompactLayers& ly, int l0, int n_layers, int b,
                                                  int na, const int32_t* path, int tid, int stride,
                                                  int32_t* status) {
@@ -271,12 +304,13 @@ __device__ __forceinline__ void compact_sequence(const sd_batch& bt, const Compa
                 src[u] = (((size_t)b * T + node) * bt.Hkv + kvh) * vec_per_head + c;
                 dst[u] = (((size_t)(blk[u] < 0 ? 0 : blk[u]) * bt.Hkv + kvh) * kBlock + (t % kBlock)) * vec_per_head + c;
             }
-            // (two layers at a time, loaded together before either is stored: four layers of five rows 4.7 -> 3 us)
-            for (int l = l0; l < l0 + n_layers; l += 2) {
-                uint4 val[2][kUnroll];
-                bool live[2][kUnroll];
+            // (kLayers at a time, loaded together before any is stored.  A CTA with several layers: two at a time, four layers
+            // of five rows 4.7 -> 3 us; with one layer the longer code only takes longer to fetch, 1.4 -> 1.9 us.)
+            for (int l = l0; l < l0 + n_layers; l += kLayers) {
+                uint4 val[kLayers][kUnroll];
+                bool live[kLayers][kUnroll];
 #pragma unroll
-                for (int i = 0; i < 2; ++i)
+                for (int i = 0; i < kLayers; ++i)
 #pragma unroll
                     for (int u = 0; u < kUnroll; ++u) {
                         const bool due = has[u] && l + i < l0 + n_layers;
@@ -285,7 +319,7 @@ __device__ __forceinline__ void compact_sequence(const sd_batch& bt, const Compa
                         if (live[i][u]) val[i][u] = (is_v ? ly.vt[l + i] : ly.kt[l + i])[src[u]];
                     }
 #pragma unroll
-                for (int i = 0; i < 2; ++i)
+                for (int i = 0; i < kLayers; ++i)
 #pragma unroll
                     for (int u = 0; u < kUnroll; ++u)
                         if (live[i][u]) (is_v ? ly.vc[l + i] : ly.kc[l + i])[dst[u]] = val[i][u];
