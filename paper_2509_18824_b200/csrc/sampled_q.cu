@@ -21,6 +21,7 @@ constexpr int kQCluster = 8;
 constexpr int kQThreads = 512;
 constexpr int kQWarps = kQThreads / 32;
 constexpr int kQPer = 40;                              // entries per thread
+static_assert(kQPer == 40, "draw_token sums 32 and 8 rows");
 constexpr int kQMaxSlice = kQThreads * kQPer;          // vocabulary entries per CTA: V <= 163840
 
 // mute: test hook, the CTA of a cluster that keeps its sums to itself (-1: none)
@@ -42,6 +43,25 @@ __device__ __forceinline__ float warp_sum_f32(float v) {
 #pragma unroll
     for (int d = 16; d >= 1; d >>= 1) v += __shfl_xor_sync(0xffffffffu, v, d);
     return v;
+}
+
+// Sums over the warp of N values per lane (N = 8 or 32): lane j, modulo N, gets value j's, added up in the order that
+// warp_sum_f32 adds in.  Lanes that hold the same values hand half of them over in each step: 31 and 23 exchanges
+// instead of 160 and 40 (a draw's 40 sums took 200).
+template <int N>
+__device__ __forceinline__ float warp_sums(float* x, int lane) {
+#pragma unroll
+    for (int d = 16; d >= N; d >>= 1)
+#pragma unroll
+        for (int i = 0; i < N; ++i) x[i] += __shfl_xor_sync(0xffffffffu, x[i], d);
+#pragma unroll
+    for (int h = N / 2; h >= 1; h >>= 1)
+#pragma unroll
+        for (int i = 0; i < h; ++i) {
+            const float keep = (lane & h) ? x[i + h] : x[i], send = (lane & h) ? x[i] : x[i + h];
+            x[i] = keep + __shfl_xor_sync(0xffffffffu, send, h);
+        }
+    return x[0];
 }
 
 // This CTA's part of the vocabulary behind one node
@@ -124,10 +144,13 @@ __device__ __forceinline__ void draw_token(QShared& sh, const VocabSlice& v, flo
     if (rank != owner) return;
     // which 32 consecutive entries, then which of them
     const int rows = (v.len + kQThreads - 1) / kQThreads;
+    {
+        float x[kQPer];
 #pragma unroll
-    for (int k = 0; k < kQPer; ++k) {
-        const float s = warp_sum_f32(v.at(k, a));
-        if (lane == 0) sh.run_sum[k * kQWarps + warp] = s;
+        for (int k = 0; k < kQPer; ++k) x[k] = v.at(k, a);
+        const float s = warp_sums<32>(x, lane), s8 = warp_sums<8>(x + 32, lane);
+        sh.run_sum[lane * kQWarps + warp] = s;
+        if (lane < 8) sh.run_sum[(32 + lane) * kQWarps + warp] = s8;
     }
     __syncthreads();
     if (warp == 0) {
@@ -190,11 +213,12 @@ tree_walk_q_kernel(sd_batch bt, int V, float inv_temp, const float* lse, const f
     const int n = bt.n_nodes[b];
     // the tree, checked by every CTA in the same way
     const bool n_ok = n >= 1 && n <= T;
-    if (n_ok && tid < n) {
+    if (tid < T) {                                     // (unused nodes too: the loads need not wait for n)
         const size_t at = (size_t)b * T + tid;
         const int p = bt.parents[at], x = draft[at];
         sh.par[tid] = p; sh.tok[tid] = x; sh.u[tid] = u[at];
-        if (tid == 0 ? (p != -1) : (p < 0 || p >= tid)) sh.bad = SD_ERR_INVALID_TREE;
+        if (!n_ok || tid >= n) {}
+        else if (tid == 0 ? (p != -1) : (p < 0 || p >= tid)) sh.bad = SD_ERR_INVALID_TREE;
         else if (tid > 0 && (x < 0 || x >= V)) atomicCAS(&sh.bad, 0, (int)SD_ERR_BOUNDS);
     }
     __syncthreads();
@@ -281,17 +305,18 @@ chain_walk_q_logits_kernel(sd_batch bt, int V, float inv_temp, const float* lse,
     const bool n_ok = n >= 1 && n <= T;
     if (tid < 64) {
         bool rejected = false;
-        if (n_ok && tid < n) {
+        if (tid < T) {                                 // (unused nodes too: the loads need not wait for n)
             const size_t at = (size_t)b * T + tid;
             const int p = bt.parents[at], x = draft[at];
+            const float uq = u[at], qt = q_tok[at], plse = tid > 0 ? lse[at - 1] : 0.f;
+            const bool x_ok = x >= 0 && x < V;
+            const float px = tid > 0 && x_ok ? __expf(__ldg(logits + (at - 1) * V + x) * inv_temp - plse) : 0.f;
             sh.tok[tid] = x;
-            if (tid == 0 ? (p != -1) : (p < 0 || p >= tid)) sh.bad = SD_ERR_INVALID_TREE;
-            else if (tid > 0 && p != tid - 1) atomicCAS(&sh.bad, 0, (int)SD_ERR_UNSUPPORTED);      // the tree branches
-            if (tid > 0) {
-                float px = 0.f;
-                if (x >= 0 && x < V) px = __expf(__ldg(logits + (at - 1) * V + x) * inv_temp - lse[at - 1]);
-                else set_status(status, SD_ERR_BOUNDS);
-                rejected = !(u[at] * q_tok[at] < px);
+            if (n_ok && tid < n) {
+                if (tid == 0 ? (p != -1) : (p < 0 || p >= tid)) sh.bad = SD_ERR_INVALID_TREE;
+                else if (tid > 0 && p != tid - 1) atomicCAS(&sh.bad, 0, (int)SD_ERR_UNSUPPORTED);      // the tree branches
+                if (tid > 0 && !x_ok) set_status(status, SD_ERR_BOUNDS);
+                rejected = tid > 0 && !(uq * qt < px);
             }
         }
         const uint32_t m = __ballot_sync(0xffffffffu, rejected);
