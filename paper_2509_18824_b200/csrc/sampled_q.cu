@@ -11,7 +11,7 @@
 // decisions.  The last token is found by inverse CDF in vocabulary order by the CTA whose slice holds the
 // crossing.  What bounds it is latency: per node one round of loads, per rejection one exchange.  (With the
 // slices in shared memory, 256 threads and two cluster barriers' worth of synchronisation per exchange 8 trees of 60
-// nodes took 51 to 65 us at a vocabulary of 152064, now 26 to 29; 8 chains of 10 drafts 31 in four kernels, now 10.5.)
+// nodes took 51 to 65 us at a vocabulary of 152064, now 24 to 27; 8 chains of 10 drafts 31 in four kernels, now 7.5.)
 #include "tree_device.cuh"
 #include "sm100.cuh"
 
@@ -20,9 +20,11 @@ namespace sdv {
 constexpr int kQCluster = 8;
 constexpr int kQThreads = 512;
 constexpr int kQWarps = kQThreads / 32;
-constexpr int kQPer = 40;                              // entries per thread
-static_assert(kQPer == 40, "draw_token sums 32 and 8 rows");
-constexpr int kQMaxSlice = kQThreads * kQPer;          // vocabulary entries per CTA: V <= 163840
+// Entries per thread, PER: 40 (V <= 163840), and 16 and 8 where they hold the vocabulary.  The code is unrolled over them, and
+// with 40 the way through it is as long however few of them there are.  8 against 40: trees of 60 nodes, 4 sequences, vocabulary
+// 4099, the whole tail 38.1 -> 31.6 us, 2 sequences, 32000 68.5 -> 62.3; 16 against 40: 8 sequences, 50257 131.1 -> 127.5.
+constexpr int kQPerMax = 40;
+constexpr int kQMaxSlice = kQThreads * kQPerMax;       // vocabulary entries per CTA
 
 // mute: test hook, the CTA of a cluster that keeps its sums to itself (-1: none)
 struct QWaits { long long cycles; int mute; };
@@ -31,7 +33,7 @@ struct QShared {
     uint64_t bar[2];                                   // two exchanges in turn: a CTA may start the next while a peer still
     float cta_sum[2][kQCluster];                       // waits for this one (it cannot get two ahead)
     float warp_sum[kQWarps];
-    float run_sum[kQPer * kQWarps];                    // the draw: sums of 32 consecutive entries
+    float run_sum[kQPerMax * kQWarps];                    // the draw: sums of 32 consecutive entries
     float run[32];
     int32_t path[kMaxT], par[kMaxT], tok[kMaxT];
     float u[kMaxT], px[kMaxT], qx[kMaxT];
@@ -45,7 +47,7 @@ __device__ __forceinline__ float warp_sum_f32(float v) {
     return v;
 }
 
-// Sums over the warp of N values per lane (N = 8 or 32): lane j, modulo N, gets value j's, added up in the order that
+// Sums over the warp of N values per lane (N = 8, 16 or 32): lane j, modulo N, gets value j's, added up in the order that
 // warp_sum_f32 adds in.  Lanes that hold the same values hand half of them over in each step: 31 and 23 exchanges
 // instead of 160 and 40 (a draw's 40 sums took 200).
 template <int N>
@@ -65,32 +67,34 @@ __device__ __forceinline__ float warp_sums(float* x, int lane) {
 }
 
 // This CTA's part of the vocabulary behind one node
+template <int PER>
 struct VocabSlice {
-    float p[kQPer], q[kQPer];
+    float p[PER], q[PER];
     int len;
     // q: null for a node whose q is not needed
     __device__ __forceinline__ void load(const float* logits, const float* qrow, float inv_temp, float lse, int tid) {
 #pragma unroll
-        for (int k = 0; k < kQPer; ++k) {
+        for (int k = 0; k < PER; ++k) {
             const int i = k * kQThreads + tid;
             p[k] = i < len ? __ldg(logits + i) : -INFINITY;
             q[k] = (qrow && i < len) ? __ldg(qrow + i) : 0.f;
         }
 #pragma unroll
-        for (int k = 0; k < kQPer; ++k) p[k] = __expf(p[k] * inv_temp - lse);
+        for (int k = 0; k < PER; ++k) p[k] = __expf(p[k] * inv_temp - lse);
     }
     __device__ __forceinline__ float at(int k, float a) const { return fmaxf(p[k] - a * q[k], 0.f); }
     __device__ __forceinline__ float thread_sum(float a) const {
         float s[4] = {0.f, 0.f, 0.f, 0.f};
 #pragma unroll
-        for (int k = 0; k < kQPer; ++k) s[k & 3] += at(k, a);
+        for (int k = 0; k < PER; ++k) s[k & 3] += at(k, a);
         return (s[0] + s[1]) + (s[2] + s[3]);
     }
 };
 
 // Sum of max(p - a q, 0) over the whole vocabulary, the same bits in every CTA of the cluster; n_red counts the
 // exchanges so far.  sh.cta_sum[(n_red - 1) & 1] keeps the eight parts.  false: a peer's part did not arrive.
-__device__ __forceinline__ bool reduce_all(QShared& sh, const VocabSlice& v, float a, int rank, int tid, const QWaits& waits, int& n_red,
+template <int PER>
+__device__ __forceinline__ bool reduce_all(QShared& sh, const VocabSlice<PER>& v, float a, int rank, int tid, const QWaits& waits, int& n_red,
                                            float& all) {
     const int set = n_red & 1;
     const uint32_t phase = (uint32_t)(n_red >> 1) & 1u;
@@ -120,7 +124,8 @@ __device__ __forceinline__ bool reduce_all(QShared& sh, const VocabSlice& v, flo
 
 // The token at which the cumulative mass of max(p - a q, 0), in vocabulary order, reaches w * (total mass); the
 // latest exchange summed exactly this distribution.  Every CTA calls it, the owner of the crossing writes.
-__device__ __forceinline__ void draw_token(QShared& sh, const VocabSlice& v, float a, float w, float total, int n_red, int rank,
+template <int PER>
+__device__ __forceinline__ void draw_token(QShared& sh, const VocabSlice<PER>& v, float a, float w, float total, int n_red, int rank,
                                            int tid, int v0, int32_t* out_slot, int32_t* status) {
     const float* parts = sh.cta_sum[(n_red - 1) & 1];
     const int warp = tid >> 5, lane = tid & 31;
@@ -145,12 +150,17 @@ __device__ __forceinline__ void draw_token(QShared& sh, const VocabSlice& v, flo
     // which 32 consecutive entries, then which of them
     const int rows = (v.len + kQThreads - 1) / kQThreads;
     {
-        float x[kQPer];
+        float x[PER];
 #pragma unroll
-        for (int k = 0; k < kQPer; ++k) x[k] = v.at(k, a);
-        const float s = warp_sums<32>(x, lane), s8 = warp_sums<8>(x + 32, lane);
-        sh.run_sum[lane * kQWarps + warp] = s;
-        if (lane < 8) sh.run_sum[(32 + lane) * kQWarps + warp] = s8;
+        for (int k = 0; k < PER; ++k) x[k] = v.at(k, a);
+        constexpr int kFirst = PER > 32 ? 32 : PER;
+        static_assert(kFirst == PER || PER == 40, "32 rows and 8");
+        const float s = warp_sums<kFirst>(x, lane);
+        if (lane < kFirst) sh.run_sum[lane * kQWarps + warp] = s;
+        if constexpr (PER > 32) {
+            const float s8 = warp_sums<8>(x + 32, lane);
+            if (lane < 8) sh.run_sum[(32 + lane) * kQWarps + warp] = s8;
+        }
     }
     __syncthreads();
     if (warp == 0) {
@@ -164,7 +174,7 @@ __device__ __forceinline__ void draw_token(QShared& sh, const VocabSlice& v, flo
     const int t = sh.pick;
     if (warp == (t & (kQWarps - 1))) {
 #pragma unroll
-        for (int k = 0; k < kQPer; ++k)
+        for (int k = 0; k < PER; ++k)
             if (k == t / kQWarps) sh.run[lane] = v.at(k, a);
         __syncwarp();
         float acc = sh.acc;
@@ -195,6 +205,7 @@ __device__ __forceinline__ void q_end(QShared& sh) {
     if (*reinterpret_cast<volatile int*>(&sh.abort_flag)) sm100::unwind_pause();
 }
 
+template <int PER>
 __global__ void __launch_bounds__(kQThreads, 1)
 tree_walk_q_kernel(sd_batch bt, int V, float inv_temp, const float* lse, const float* logits, const int32_t* draft,
                    const float* q_rows, const float* u, const float* w, int32_t* n_acc, int32_t* path, int32_t* out_tok,
@@ -208,7 +219,7 @@ tree_walk_q_kernel(sd_batch bt, int V, float inv_temp, const float* lse, const f
     const int T = bt.T_max;
     const int slice = (V + kQCluster - 1) / kQCluster;
     const int v0 = min(V, rank * slice);
-    VocabSlice v;
+    VocabSlice<PER> v;
     v.len = min(V, v0 + slice) - v0;
     const int n = bt.n_nodes[b];
     // the tree, checked by every CTA in the same way
@@ -285,6 +296,7 @@ tree_walk_q_kernel(sd_batch bt, int V, float inv_temp, const float* lse, const f
 // Chains: node j's token is kept iff u * q(token) < p(token), p and q behind node j - 1; the walk stops at the
 // first rejection, and the last token comes from max(p - q, 0) there, or from p of the leaf.  Only the stop
 // node's row of p and q is needed, so the whole rule is one kernel with one exchange.
+template <int PER>
 __global__ void __launch_bounds__(kQThreads, 1)
 chain_walk_q_logits_kernel(sd_batch bt, int V, float inv_temp, const float* lse, const float* logits, const int32_t* draft,
                            const float* q_tok, const float* q_rows, const float* u, const float* w, int32_t* n_acc, int32_t* path,
@@ -299,7 +311,7 @@ chain_walk_q_logits_kernel(sd_batch bt, int V, float inv_temp, const float* lse,
     const int T = bt.T_max;
     const int slice = (V + kQCluster - 1) / kQCluster;
     const int v0 = min(V, rank * slice);
-    VocabSlice v;
+    VocabSlice<PER> v;
     v.len = min(V, v0 + slice) - v0;
     const int n = bt.n_nodes[b];
     const bool n_ok = n >= 1 && n <= T;
@@ -362,7 +374,9 @@ sd_status launch_accept_tree_sampled_q(const sd_batch& bt, int V, float inv_temp
                                        int32_t* n_acc, int32_t* path, int32_t* out_tok, int32_t* new_len,
                                        int32_t* dev_status, cudaStream_t st) {
     if (!q_kernels_hold(V)) return SD_ERR_UNSUPPORTED;
-    return launch_dependent(tree_walk_q_kernel, dim3(bt.B * kQCluster), kQThreads, 0, kQCluster, st, bt, V, inv_temp, lse, logits, draft,
+    const int slice = (V + kQCluster - 1) / kQCluster;
+    auto kern = slice <= 8 * kQThreads ? tree_walk_q_kernel<8> : (slice <= 16 * kQThreads ? tree_walk_q_kernel<16> : tree_walk_q_kernel<kQPerMax>);
+    return launch_dependent(kern, dim3(bt.B * kQCluster), kQThreads, 0, kQCluster, st, bt, V, inv_temp, lse, logits, draft,
                             q_rows, u, w, n_acc, path, out_tok, new_len, dev_status, q_waits());
 }
 
@@ -370,7 +384,10 @@ sd_status launch_accept_chain_logits(const sd_batch& bt, int V, float inv_temp, 
                                      const int32_t* draft, const float* q_tok, const float* q_rows, const float* u, const float* w,
                                      int32_t* n_acc, int32_t* path, int32_t* out_tok, int32_t* new_len, int32_t* dev_status,
                                      cudaStream_t st) {
-    return launch_dependent(chain_walk_q_logits_kernel, dim3(bt.B * kQCluster), kQThreads, 0, kQCluster, st, bt, V, inv_temp, lse, logits,
+    const int slice = (V + kQCluster - 1) / kQCluster;
+    auto kern = slice <= 8 * kQThreads ? chain_walk_q_logits_kernel<8>
+                                       : (slice <= 16 * kQThreads ? chain_walk_q_logits_kernel<16> : chain_walk_q_logits_kernel<kQPerMax>);
+    return launch_dependent(kern, dim3(bt.B * kQCluster), kQThreads, 0, kQCluster, st, bt, V, inv_temp, lse, logits,
                             draft, q_tok, q_rows, u, w, n_acc, path, out_tok, new_len, dev_status, q_waits());
 }
 
