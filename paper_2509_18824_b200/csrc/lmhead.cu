@@ -649,18 +649,19 @@ lmhead_umma_pair_kernel(const __grid_constant__ CUtensorMap tmW, const __grid_co
     }
 }
 
-// merge of the per-CTA candidates (lowest index on ties), eight threads per hidden row
-__global__ void __launch_bounds__(256)
+// merge of the per-CTA candidates (lowest index on ties), 64 hidden rows per CTA
+__global__ void __launch_bounds__(512)
 lmhead_merge_kernel(const int32_t* __restrict__ part_key, const int32_t* __restrict__ part_idx,
                                     int n_ctas, int rows, int row0, int32_t* __restrict__ argmax,
                                     float* __restrict__ maxlogit) {
+    __shared__ ArgmaxShared sh;
     begin_dependent(part_key, part_idx);
-    const int col = blockIdx.x * 32 + (threadIdx.x >> 3), sub = threadIdx.x & 7;
+    const int col0 = blockIdx.x * 64, here = min(rows - col0, 64);
     int32_t k, i;
-    merge_row_argmax(part_key, part_idx, n_ctas, kMaxCols, col, col < rows, sub, k, i);
-    if (col < rows && sub == 0) {
-        argmax[row0 + col] = i;
-        if (maxlogit) maxlogit[row0 + col] = key_to_float(k);
+    merge_rows_argmax(sh, part_key, part_idx, n_ctas, kMaxCols, col0, here, k, i);
+    if ((int)threadIdx.x < here) {
+        argmax[row0 + col0 + threadIdx.x] = i;
+        if (maxlogit) maxlogit[row0 + col0 + threadIdx.x] = key_to_float(k);
     }
 }
 
@@ -807,10 +808,10 @@ static sd_status launch_lmhead_impl(const void* hidden, const void* W, int M, in
             return SD_OK;
         }
         if (mass_out) continue;                      // nothing to merge: the epilogue stored the probabilities
-        const dim3 mgrid((p.rows + 31) / 32), sgrid((p.rows + 7) / 8);
+        const dim3 mgrid((p.rows + 63) / 64), sgrid((p.rows + 7) / 8);
         const sd_status ms = lse ? launch_dependent(lmhead_merge_stats_kernel, sgrid, 256, 0, 1, st, p.part_key, p.part_idx, p.part_ref,
                                                     p.part_sum, grid, p.rows, p.row0, p.c2, argmax, maxlogit, lse)
-                                 : launch_dependent(lmhead_merge_kernel, mgrid, 256, 0, 1, st, p.part_key, p.part_idx, grid, p.rows,
+                                 : launch_dependent(lmhead_merge_kernel, mgrid, 512, 0, 1, st, p.part_key, p.part_idx, grid, p.rows,
                                                     p.row0, argmax, maxlogit);
         if (ms != SD_OK) return ms;
     }

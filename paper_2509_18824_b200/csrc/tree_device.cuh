@@ -43,44 +43,30 @@ __device__ __forceinline__ void merge_sumexp(float& ref, float& sum, float ref2,
     else            { sum += sum2 * ex2_lm((ref2 - ref) * c2); }
 }
 
-// Arg-max candidate of one hidden row (column `col` of the per-CTA tables), merged by the eight consecutive
-// lanes that share the row; all of them return the result.  Every lane of the warp must call this.
-__device__ __forceinline__ void merge_row_argmax(const int32_t* part_key, const int32_t* part_idx, int n_ctas, int row_stride,
-                                                 int col, bool active, int sub, int32_t& k, int32_t& i) {
-    k = INT32_MIN; i = 0x7fffffff;
-    if (active) {
-        // (the loads of a batch are issued together: one memory latency instead of a chain of them)
-        constexpr int kAhead = 20;                  // 148 CTAs: 19 per lane
-        for (int c0 = sub; c0 < n_ctas; c0 += 8 * kAhead) {
-            int32_t pk[kAhead], pi[kAhead];
-#pragma unroll
-            for (int a = 0; a < kAhead; ++a) {
-                const int c = c0 + 8 * a;
-                if (c < n_ctas) {
-                    pk[a] = part_key[(size_t)c * row_stride + col];
-                    pi[a] = part_idx[(size_t)c * row_stride + col];
-                }
-            }
-#pragma unroll
-            for (int a = 0; a < kAhead; ++a)
-                if (c0 + 8 * a < n_ctas) take_better(k, i, pk[a], pi[a]);
-        }
-    }
-#pragma unroll
-    for (int d = 1; d <= 4; d <<= 1) {
-        const int32_t k2 = __shfl_xor_sync(0xffffffffu, k, d), i2 = __shfl_xor_sync(0xffffffffu, i, d);
-        take_better(k, i, k2, i2);
-    }
-}
-
 // Arg-max candidates of up to 64 hidden rows (columns col0 .. + rows - 1), merged by a CTA of 512 threads: lanes along the
 // columns, so that a load touches one or two lines of a table, an eighth of the CTAs' candidates per warp (all eight threads of a row
 // in one warp, eight lines per load: 3.1 us of the tail kernel, now 1.8).  Threads 0 .. rows - 1 return row threadIdx.x's.
 struct ArgmaxShared { int32_t key[8][64], idx[8][64]; };
 __device__ __forceinline__ void merge_rows_argmax(ArgmaxShared& sh, const int32_t* part_key, const int32_t* part_idx, int n_ctas,
                                                   int row_stride, int col0, int rows, int32_t& k, int32_t& i) {
-    const int row = threadIdx.x & 63, part = threadIdx.x >> 6;
     k = INT32_MIN; i = 0x7fffffff;
+    if (n_ctas <= 8) {                                     // one candidate per lane: eight lanes to a row after all
+        const int row = threadIdx.x >> 3, c = threadIdx.x & 7;
+        if (row < rows && c < n_ctas) {
+            k = part_key[(size_t)c * row_stride + col0 + row];
+            i = part_idx[(size_t)c * row_stride + col0 + row];
+        }
+#pragma unroll
+        for (int d = 1; d <= 4; d <<= 1) {
+            const int32_t k2 = __shfl_xor_sync(0xffffffffu, k, d), i2 = __shfl_xor_sync(0xffffffffu, i, d);
+            take_better(k, i, k2, i2);
+        }
+        if (c == 0) { sh.key[0][row] = k; sh.idx[0][row] = i; }
+        __syncthreads();
+        k = sh.key[0][threadIdx.x & 63]; i = sh.idx[0][threadIdx.x & 63];
+        return;
+    }
+    const int row = threadIdx.x & 63, part = threadIdx.x >> 6;
     if (row < rows) {
         // (the loads of a batch are issued together: one memory latency instead of a chain of them)
         constexpr int kAhead = 20;                         // 148 CTAs: 19 per thread
@@ -313,7 +299,7 @@ __device__ __forceinline__ void compact_sequence(const sd_batch& bt, const Compa
                 for (int i = 0; i < kLayers; ++i)
 #pragma unroll
                     for (int u = 0; u < kUnroll; ++u) {
-                        const bool due = has[u] && l + i < l0 + n_layers;
+                        const bool due = has[u] && (kLayers == 1 || l + i < l0 + n_layers);
                         live[i][u] = due && blk[u] >= 0 && blk[u] < ly.num_blocks[l + i];
                         if (due && !live[i][u]) set_status(status, SD_ERR_BOUNDS);
                         if (live[i][u]) val[i][u] = (is_v ? ly.vt[l + i] : ly.kt[l + i])[src[u]];
