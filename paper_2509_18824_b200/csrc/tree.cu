@@ -46,17 +46,11 @@ __global__ void accept_kernel(sd_batch bt, const int32_t* __restrict__ draft,
                               const int32_t* __restrict__ target,
                               int32_t* n_acc, int32_t* path, int32_t* out_tok, int32_t* new_len,
                               int32_t* status) {
-    __shared__ int32_t s_par[kMaxT], s_dt[kMaxT], s_tg[kMaxT];
     begin_dependent(bt, draft, target);
     const int b = blockIdx.x;
     const int T = bt.T_max;
-    for (int i = threadIdx.x; i < T; i += 32) {
-        const size_t at = (size_t)b * T + i;
-        s_par[i] = bt.parents[at]; s_dt[i] = draft[at]; s_tg[i] = target[at];
-    }
-    const int n = bt.n_nodes[b], len = bt.len[b];
-    __syncwarp();
-    accept_sequence(T, b, threadIdx.x, n, len, s_par, s_dt, s_tg, n_acc, path, out_tok, new_len, nullptr, status);
+    accept_sequence(T, b, threadIdx.x, bt.n_nodes[b], bt.len[b], bt.parents + (size_t)b * T, draft + (size_t)b * T, target + (size_t)b * T,
+                    n_acc, path, out_tok, new_len, nullptr, status);
 }
 
 sd_status launch_tree_prepare(const sd_batch& bt, int32_t* dev_status, cudaStream_t st) {

@@ -196,8 +196,8 @@ __device__ __forceinline__ int warp_find_crossing(const float* v, int n, float t
 }
 
 // Greedy acceptance for one sequence of n nodes and len cached tokens, executed by one warp.  par/dt/tg: the
-// sequence's parents, draft tokens and target arg-max, in shared memory (from global memory every step of the walks
-// towards the root is a trip to the cache: 2.9 us of the tail kernel's 8, now 2.4).  Returns the number of
+// sequence's parents, draft tokens and target arg-max, in global or shared memory (in the tail kernel, where they can be
+// brought there meanwhile, 2.9 -> 2.4 us; the stand-alone kernel, which would wait for them, takes 3.6 instead of 4.0 without).  Returns the number of
 // accepted nodes (0 for a bad tree, which is reported through *status) and, in lane 0, has written
 // n_acc, new_len, path and out_tok; `path_out` (nullable, e.g. shared memory) receives the path too.
 __device__ __forceinline__ int accept_sequence(int T, int b, int lane, int n, int len, const int32_t* par,
@@ -293,6 +293,16 @@ __device__ __forceinline__ void compact_sequence(const sd_batch& bt, const Compa
             // (kLayers at a time, loaded together before any is stored.  A CTA with several layers: two at a time, four layers
             // of five rows 4.7 -> 3 us; with one layer the longer code only takes longer to fetch, 1.4 -> 1.9 us.)
             for (int l = l0; l < l0 + n_layers; l += kLayers) {
+                const uint4* from[kLayers];
+                uint4* to[kLayers];
+                int nb[kLayers];
+#pragma unroll
+                for (int i = 0; i < kLayers; ++i) {
+                    const int at = kLayers == 1 ? l : min(l + i, l0 + n_layers - 1);
+                    from[i] = is_v ? ly.vt[at] : ly.kt[at];
+                    to[i] = is_v ? ly.vc[at] : ly.kc[at];
+                    nb[i] = ly.num_blocks[at];
+                }
                 uint4 val[kLayers][kUnroll];
                 bool live[kLayers][kUnroll];
 #pragma unroll
@@ -300,15 +310,15 @@ __device__ __forceinline__ void compact_sequence(const sd_batch& bt, const Compa
 #pragma unroll
                     for (int u = 0; u < kUnroll; ++u) {
                         const bool due = has[u] && (kLayers == 1 || l + i < l0 + n_layers);
-                        live[i][u] = due && blk[u] >= 0 && blk[u] < ly.num_blocks[l + i];
+                        live[i][u] = due && blk[u] >= 0 && blk[u] < nb[i];
                         if (due && !live[i][u]) set_status(status, SD_ERR_BOUNDS);
-                        if (live[i][u]) val[i][u] = (is_v ? ly.vt[l + i] : ly.kt[l + i])[src[u]];
+                        if (live[i][u]) val[i][u] = from[i][src[u]];
                     }
 #pragma unroll
                 for (int i = 0; i < kLayers; ++i)
 #pragma unroll
                     for (int u = 0; u < kUnroll; ++u)
-                        if (live[i][u]) (is_v ? ly.vc[l + i] : ly.kc[l + i])[dst[u]] = val[i][u];
+                        if (live[i][u]) to[i][dst[u]] = val[i][u];
             }
         }
         return;
