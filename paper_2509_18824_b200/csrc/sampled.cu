@@ -441,8 +441,8 @@ __device__ __forceinline__ void residual_pick_groups(const uint16_t* __restrict_
     __syncthreads();
     if (threadIdx.x == 0)                                              // drafted children carry no mass (fixed order)
         for (int e = 0; e < ne; ++e) {
-            const int g = s_ex[e] >> 5;
-            s_g[g] = fmaxf(s_g[g] - s_exp[e], 0.f);
+            const int g = s_ex[e] >> 5;                                // (a token outside [0, V), reported by now, is in no group)
+            if ((unsigned)g < (unsigned)n_groups) s_g[g] = fmaxf(s_g[g] - s_exp[e], 0.f);
         }
     __syncthreads();
     // every thread sums a run of consecutive groups; the search goes over the 256 sums, then inside one run
