@@ -21,7 +21,7 @@
 // The launch is a programmatic dependent launch: barriers, tensor memory and
 // tensor-map prefetch are set up before the kernel waits for the kernel ahead of
 // it in the stream, so consecutive per-layer calls overlap their ends.
-#include "attention_shared.cuh"
+#include "attention_plan.cuh"
 
 namespace sdv {
 
@@ -559,66 +559,12 @@ static AttnPlan common_plan(const sd_batch& bt, int n_layers, const TestKnobs& k
     return p;
 }
 
-// The 128-key kernel (attention_wide.cu) runs one CTA per SM.  One round of it takes 5 us, or about 6 with a merge of
-// chunks, plus 0.02 us per CTA (they share the memory that the first copies come from), plus 0.4 us per cache block
-// of its longest chunk, in tiles of two, plus about 0.5 us where the next call's CTAs find no free SMs to set up on
-// while this one runs: fitted to calls of 1 to 16 sequences of 200 to 8192 tokens, trees of 11, 28 and 60 nodes, 1 to 8
-// chunks, of which it picks one within 1.5 % of the fastest on average (12 % at most).  With 8 us and 2.8 to 3.8 us for
-// the merge, which it took before, middling sequences stayed whole or in two for too long: two of 900 tokens and 60 nodes
-// 11.2 us instead of 10.0, four of 1100 13.0 instead of 11.7, eight of 1300 and 28 nodes 14.4 instead of 12.8.  In
-// launches of several rounds, where nothing overlaps a round's ends, each takes 11 us, the merge, and 0.36 us per block.
-// Measured per call in us for 1 to 8 chunks: one sequence of 2048 tokens and 60 nodes 16.4 12.7 10.9 9.9 9.9 10.1 15.6
-// 15.2 (16 clusters of seven or eight are more than fit at a time), of 8192 50.8 29.7 22.1 18.3 17.1 16.0 25.1 23.7, one
-// chain of 11 nodes over 4096 27.8 18.0 14.3 12.2 11.5 11.0 10.5 9.9.  Chunk counts that are no powers of two fill SMs that
-// those leave idle: ten such
-// chains 19.3 us with three chunks (21.4 with two), five sequences of 2000 tokens with 16 heads 13.0 (14.6).
-// The table's width stands for the longest length here, which the host does not know: a table that is far wider
-// makes long launches look longer than they are (in a table of 512 blocks 256 CTAs of 1000 tokens take 26.4 instead
-// of 22.7 us, 160 of 2048 54.6 instead of 35), but what a single round's sequences are cut into follows from
-// their own lengths.
-// The 64-key kernel's two CTAs per SM overlap each other's ends: a round of twice as many CTAs takes about
-// 0.9 us per block plus 13 us.  It is left for launches of several rounds in which those ends weigh more
-// (256 CTAs of 1000 tokens: 28.7 against 33.9 us; of 4096: 71.4 against 69.9; 1792 CTAs of 4096 tokens under the
-// power cap, where 64-key tiles cost more energy: 569 against 544).
+// The plan of a call that the 128-key kernel takes (attention_plan.cuh); false: the 64-key kernel is faster.
 static bool wide_plan(AttnPlan* p, const sd_batch& bt, int dev, int sms, const TestKnobs& knobs) {
     const long long base = (long long)p->n_layers * bt.B * bt.Hkv * p->row_tiles;
-    const int blocks = bt.max_blocks_per_seq;
-    const double merge[kMaxChunks] = {0.0, 2.8, 3.2, 3.2, 3.3, 3.4, 3.6, 3.8};
-    int n = 1;
-    long long n_rounds = 1;
-    double best = 1e30;
-    p->tree_blocks = kTreeBlocks;
-    const bool forced = knobs.chunks > 0 && knobs.chunks <= blocks;
-    auto whole = [&](int c) { return forced ? 0 : (c == 2 ? 10 : 5); };   // blocks of a sequence that is not cut, see below
-    for (int c = 1; c <= kMaxChunks && c <= blocks; ++c) {
-        if (c > 1 && blocks <= whole(c)) continue;         // (CTAs without work: eight chains of 200 tokens 7.6 instead of 7.0 us)
-        const int resident = wide_resident_clusters(dev, sms, c);
-        const long long rounds = (base + resident - 1) / resident;
-        double us = rounds * (11.0 + merge[c - 1] + 0.36 * ((blocks + c - 1) / c));
-        if (rounds == 1) {                                 // blocks of the longest chunk, of a sequence and its tree that fill the table
-            p->set_chunks(c, whole(c));
-            const ChunkRange last = chunk_range(*p, (min(blocks, 1 << 24) - 1) * kBlock, blocks, c - 1);
-            const int per = max(last.tpc, last.t1 - last.t0 + 1);
-            us = (c == 1 ? 5.0 : 5.8 + 0.1 * c) + 0.02 * base * c + (2 * base * c > sms ? 0.52 : 0.0) + 0.28 * per + 0.25 * ((per + 1) / 2);
-        }
-        if (forced ? c == knobs.chunks : us < best - 1e-9) { best = us; n = c; n_rounds = rounds; }
-    }
-    if (n_rounds > 1) {
-        const double rounds = base <= 2 * sms ? 1.0 : (double)base / (2 * sms) + 0.25;     // a partial round, cut into chunks
-        if (best > 1.05 * rounds * (13.0 + 0.9 * blocks)) return false;
-    }
-    // Where all clusters run at once, a sequence so short that the merge costs more than the split saves stays whole
-    // (us per call uncut, in two, three, four, six chunks, one sequence and 60 nodes: 4 blocks 7.1 7.6 7.6 7.6, 6 blocks
-    // 8.1 8.2 8.1 7.9 7.9, 8 blocks 8.6 8.6 8.0 7.9 7.7, 12 blocks 10.0 9.5 9.0 9.0 8.1); the others are cut as far as the
-    // cluster goes.  This must not follow from the table's width, of which a chunk's size was once a share: then one
-    // sequence of 2048 tokens in a table of 512 blocks ran whole (16.3 us, now 9.8; 10.2 in a table of 33), eight chains
-    // of 4096 took 28.7 (17.0), one of 8192 in 2048 blocks 50.7 (16.0).  The other side: in a batch of very different
-    // lengths the short sequences take memory bandwidth from the longest (eight chains over 200 to 8192 tokens
-    // 20.4 us, 19.8 with chunks as long as the longest's; 100 to 3000 tokens 11.4 against 11.7).
-    // In several rounds every sequence is cut alike: the CTAs that leave would still hold back the next cluster
-    // (half-empty pairs halved the machine).
-    p->set_chunks(n, n_rounds > 1 ? -1 : whole(n));
-    p->ranked = (bt.B > 1 && bt.B <= 64 && base * n > sms) ? 1 : 0;
+    if (!choose_wide(p, base, bt.max_blocks_per_seq, sms, knobs.chunks, [&](int c) { return wide_resident_clusters(dev, sms, c); }))
+        return false;
+    p->ranked = (bt.B > 1 && bt.B <= 64 && base * p->n_chunks > sms) ? 1 : 0;
     return true;
 }
 
