@@ -33,8 +33,8 @@ struct QShared {
     uint64_t bar[2];                                   // two exchanges in turn: a CTA may start the next while a peer still
     float cta_sum[2][kQCluster];                       // waits for this one (it cannot get two ahead)
     float warp_sum[kQWarps];
-    float run_sum[kQPerMax * kQWarps];                    // the draw: sums of 32 consecutive entries
-    float run[32];
+    float run_sum[kQPerMax * kQWarps];                 // the draw: sums of 32 consecutive entries
+    float run[kQPerMax][32];                           // the entries of one warp
     int32_t path[kMaxT], par[kMaxT], tok[kMaxT];
     float u[kMaxT], px[kMaxT], qx[kMaxT];
     float acc;
@@ -173,13 +173,15 @@ __device__ __forceinline__ void draw_token(QShared& sh, const VocabSlice<PER>& v
     __syncthreads();
     const int t = sh.pick;
     if (warp == (t & (kQWarps - 1))) {
+        // All rows, not only the one looked for: with 8 and 16 entries the compiler took a selected one for an indexed array,
+        // which put the slice into local memory (per call, 8 sequences of 60 nodes: V 32000 8.9 -> 8.0 us, 50257 10.5 -> 8.8,
+        // chains of 11 5.7 -> 4.7 and 6.8 -> 5.5; with 40, 152064, 16.3 -> 16.2 and 7.4 -> 6.8).
 #pragma unroll
-        for (int k = 0; k < PER; ++k)
-            if (k == t / kQWarps) sh.run[lane] = v.at(k, a);
+        for (int k = 0; k < PER; ++k) sh.run[k][lane] = v.at(k, a);
         __syncwarp();
         float acc = sh.acc;
         int lastp = -1;
-        int e = warp_find_crossing(sh.run, 32, target, &acc, &lastp, lane);
+        int e = warp_find_crossing(sh.run[t / kQWarps], 32, target, &acc, &lastp, lane);
         if (e < 0) e = max(lastp, 0);
         if (lane == 0) *out_slot = v0 + t * 32 + e;
     }
