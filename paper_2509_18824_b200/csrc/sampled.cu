@@ -676,9 +676,9 @@ sampled_tail_kernel(sd_batch bt, const __grid_constant__ CompactLayers ly, int L
     __syncwarp();
     sm100::cluster_arrive_relaxed();                                   // every CTA of the cluster is there to be written to
     const int node = rank * 8 + warp;
-    float logit = -INFINITY, row_lse = 0.f;                            // (no child of a tree: probability 0)
+    float logit = 0.f, row_lse = 0.f;
     int par, k, i;
-    if (node < T && !child_logit(bt, b, node, lane, hidden, W, Hd, V, draft, status, par, logit)) logit = -INFINITY;
+    if (node < T) child_logit(bt, b, node, lane, hidden, W, Hd, V, draft, status, par, logit);
     row_lse = merge_rows_stats(s_merge, tb.part_key, tb.part_idx, tb.part_ref, tb.part_sum, tb.n_ctas, kLmMaxCols, b * T + rank * 8,
                                (b + 1) * T, c2, k, i);
     if (node < T && lane == 0) lse[b * T + node] = row_lse;
@@ -692,9 +692,11 @@ sampled_tail_kernel(sd_batch bt, const __grid_constant__ CompactLayers ly, int L
     sm100::cluster_arrive_release();
     sm100::cluster_wait_acquire();
     // 2. the walk
-    if (threadIdx.x < T)
-        s_p[threadIdx.x] = s_logit[threadIdx.x] == -INFINITY ? 0.f
-                                                             : __expf(s_logit[threadIdx.x] * inv_temp - s_lse[s_par[threadIdx.x]]);
+    if (threadIdx.x < T) {                                             // (what child_logit takes for a child; a logit may be anything)
+        const int j = threadIdx.x, p = s_par[j], x = s_dt[j];
+        const bool child = j >= 1 && j < n && n <= T && p >= 0 && p < j && x >= 0 && x < V;
+        s_p[j] = child ? __expf(s_logit[j] * inv_temp - s_lse[p]) : 0.f;
+    }
     __syncthreads();
     if (warp == 0) {
         const WalkOut o{s_path, s_tok, s_excl, s_excl_p};
