@@ -14,7 +14,7 @@ constexpr float kSumLimit = 1.0995e12f;        // 2^40: a tile's sum above this 
 constexpr float kRaiseAbove = 32.f;            // log2 units: ... where the maximum itself is looked at (128 x 2^32 < 2^40)
 constexpr int kMaxChunks = 8;                  // = portable cluster size
 constexpr int kStartBlocks = 5;                // cache blocks that fit the 128-key kernel's ring at once beside the tree's
-constexpr int kTreeBlocks = 3;                 // blocks that the tree counts for in its longer chunks, see chunk_range
+constexpr int kTreeBlocks = 3;                 // blocks that the tree counts for in longer chunks, see chunk_range
 constexpr int kSplitRounds = 8;                // launches of fewer whole rounds get their remainder as a chunked launch
 
 __device__ __forceinline__ float max3(float a, float b, float c) {
@@ -127,14 +127,23 @@ __device__ __forceinline__ int sequence_of_rank(const sd_batch& bt, int rank, in
 // tokens.  Us per call with the tree counted as 0, 1, 2, 3, 4 blocks: eight chains of 4096 tokens 16.8 16.4 16.4 16.4
 // 16.4, four sequences of 2048 and 60 nodes 13.9 14.3 14.4 14.0 14.0, one chain of 8192 13.1 12.6 12.6 12.6 12.6, 28 layers
 // of one sequence of 2048 (and the LM head) 468 456 456 456 456; in shorter chunks it gains nothing (15 blocks in four
-// chunks: 8.05 8.17 9.01 9.04 8.97: an odd block is half a tile).
+// chunks: 8.05 8.17 9.01 9.04 8.97: an odd block is half a tile).  Nor does it where the even split leaves the last chunk four
+// blocks or fewer, which with the tree are no more than the others have: two sequences of 1369 tokens and 55 nodes (22 blocks in
+// four, 6 6 6 4 or 7 7 7 1) 9.85 and 10.74, five such splits 2 to 7 % slower.  Over 436 splits with a longer last
+// chunk (trees of 2 to 64 nodes, 1 to 16 sequences) three blocks against none are 2.7 % faster on average, 10 % at best; 5 %
+// slower at worst.  Where a boundary lies also decides the scores that a chunk's reference comes
+// from, and so where P rounds to bf16: with other boundaries outputs differ by about 2.5e-3 relative, no more than either is
+// from fp64 (2.295e-3 on average over twelve sequences of 2048 to 3148 tokens evenly split, 2.293e-3 so).
 struct ChunkRange { int n_chunks, tiles_total, tpc, t0, t1; };
 __host__ __device__ __forceinline__ ChunkRange chunk_range(const AttnPlan& plan, int len, int max_blocks, int chunk) {
     ChunkRange r;
     r.tiles_total = min((len + kBlock - 1) / kBlock, max_blocks);
     const bool whole = plan.n_chunks == 1 || r.tiles_total <= max(plan.whole_blocks, 0);
-    const int counted = r.tiles_total + (r.tiles_total > kStartBlocks * plan.n_chunks ? plan.tree_blocks : 0);
-    r.tpc = whole ? r.tiles_total : (int)(((uint64_t)(uint32_t)(counted + plan.n_chunks - 1) * plan.chunk_magic) >> 32);
+    const auto share = [&](int blocks) { return (int)(((uint64_t)(uint32_t)(blocks + plan.n_chunks - 1) * plan.chunk_magic) >> 32); };
+    const int even = share(r.tiles_total), behind = r.tiles_total - (plan.n_chunks - 1) * even;
+    const int last = behind > 0 ? behind : behind + even;      // (more than kStartBlocks each: at most one chunk stays empty)
+    const int counted = r.tiles_total + (even > kStartBlocks && last >= kStartBlocks ? plan.tree_blocks : 0);
+    r.tpc = whole ? r.tiles_total : share(counted);
     r.n_chunks = whole ? 1 : plan.n_chunks;
     if (plan.whole_blocks >= 0 && !whole) {
         r.n_chunks = 2;

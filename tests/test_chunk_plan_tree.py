@@ -1,6 +1,7 @@
 """The split of a sequence into key chunks where the tree's keys, in the last chunk, count for several cache blocks
 (csrc/attention_shared.cuh), compiled for the host: the chunks cover the sequence once, the last is shorter by what the
-tree counts for, and sequences whose chunks hold at most kStartBlocks are cut as without a tree."""
+tree counts for, and sequences whose chunks hold at most kStartBlocks, or whose last one is shorter than that anyway, are
+cut as without a tree."""
 import os
 import subprocess
 
@@ -24,7 +25,10 @@ int main() {
                 p.tree_blocks = kTreeBlocks;
                 const int len = blocks * kBlock;
                 const ChunkRange first = chunk_range(p, len, 4000, 0), was = chunk_range(plain, len, 4000, 0);
-                const bool counts = n > 1 && blocks > whole && blocks > n * kStartBlocks;
+                const int even = (blocks + n - 1) / n;
+                int left = blocks;                                     // of the last chunk that an even split uses
+                while (left > even) left -= even;
+                const bool counts = n > 1 && blocks > whole && blocks > n * kStartBlocks && left >= kStartBlocks;
                 bool ok = first.tiles_total == blocks && first.n_chunks >= 1 && first.n_chunks <= n;
                 if (!counts) ok = ok && first.tpc == was.tpc && first.n_chunks == was.n_chunks;
                 else ok = ok && first.tpc == (blocks + kTreeBlocks + n - 1) / n && first.n_chunks * first.tpc >= blocks + kTreeBlocks;
