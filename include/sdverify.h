@@ -423,8 +423,8 @@ sd_status sd_accept_tree_sampled_q(const sd_batch *batch, int32_t V, float inv_t
  * but behind the LM-head tiles a single kernel does the rest: one cluster of eight
  * CTAs per sequence merges the rows' soft-max statistics, computes the drafted
  * tokens' probabilities, walks the tree, draws the last token from the group table
- * and copies the accepted K/V rows (each CTA a share of the layers) - two launches
- * instead of six.  Arguments as in the three calls:
+ * and copies the accepted K/V rows (the seven CTAs that do not draw, each a share of the
+ * layers) - two launches instead of six.  Arguments as in the three calls:
  *   lse         : dev f32 [B * T_max], output
  *   group_stats : dev f32 [ceil(V / 32)][B * T_max][2], 8-byte aligned, scratch that the
  *                 call fills and reads (required here)

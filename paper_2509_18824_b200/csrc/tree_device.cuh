@@ -44,7 +44,7 @@ __device__ __forceinline__ void merge_sumexp(float& ref, float& sum, float ref2,
 }
 
 // Arg-max candidates of up to 64 hidden rows (columns col0 .. + rows - 1), merged by a CTA of 512 threads: lanes along the
-// columns, so that a load touches one or two lines of a table, an eighth of the CTAs' candidates per warp (all eight threads of a row
+// columns, so that a load touches one or two lines of a table, an eighth of the CTAs' candidates per two warps (all eight threads of a row
 // in one warp, eight lines per load: 3.1 us of the tail kernel, now 1.8).  Threads 0 .. rows - 1 return row threadIdx.x's.
 struct ArgmaxShared { int32_t key[8][64], idx[8][64]; };
 __device__ __forceinline__ void merge_rows_argmax(ArgmaxShared& sh, const int32_t* part_key, const int32_t* part_idx, int n_ctas,

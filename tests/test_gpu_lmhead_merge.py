@@ -1,5 +1,6 @@
-"""GPU: the merges of the LM head's per-CTA candidates and soft-max partials: one CTA's candidates to eight, nine, and all SMs',
-rows that fill the merging CTAs' 8 and 64 rows and one more or less."""
+"""GPU: the merges of the LM head's per-CTA candidates and soft-max partials: the candidates of 1, 2, 8, 10 and of all
+SMs' CTAs (a pair of CTAs from 129 vocabulary rows on: their number is even), rows that fill the merging CTAs' 8 and 64
+rows and one more or less."""
 import pytest
 
 from test_gpu_lmhead_pieces import test_pieces as compare
