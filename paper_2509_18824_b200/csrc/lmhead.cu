@@ -864,6 +864,9 @@ sd_status launch_lmhead(const void* hidden, const void* W, int M, int Hd, int V,
 // Replaces three launches (candidate merge, acceptance, compaction).
 // What depends on nothing else (tree, tokens, length, the block table's entries) is loaded while the candidates
 // are, all rows at a time.  60 nodes, hidden size 3584, 28 layers: one sequence 8.0 -> 5.9 us, eight 9.7 -> 7.0.
+// 64 registers, at which the compiler spills 8 bytes, let two CTAs share an SM.  With 72 and no spill up to 148 CTAs are 0.2 to
+// 0.4 us faster, more of them 3 us slower (the call with a vocabulary of 18944 and hidden size 64, replayed from a graph: one
+// sequence of 60 nodes, 28 layers 9.66 and 9.22 us, eight 13.65 and 16.91, of 11 nodes 10.0 and 12.8).
 // ---------------------------------------------------------------------------
 constexpr int kTailThreads = 512;
 __global__ void __launch_bounds__(kTailThreads)

@@ -11,7 +11,8 @@
 // decisions.  The last token is found by inverse CDF in vocabulary order by the CTA whose slice holds the
 // crossing.  What bounds it is latency: per node one round of loads, per rejection one exchange.  (With the
 // slices in shared memory, 256 threads and two cluster barriers' worth of synchronisation per exchange 8 trees of 60
-// nodes took 51 to 65 us at a vocabulary of 152064, now 24 to 27; 8 chains of 10 drafts 31 in four kernels, now 7.5.)
+// nodes took 51 to 65 us at a vocabulary of 152064, now 24 to 25; 8 chains of 10 drafts 31 in four kernels, now 8.  Calls one
+// behind another; replayed from a graph, as the figures in draw_token are, 23 to 24 and 6.9.)
 #include "tree_device.cuh"
 #include "sm100.cuh"
 
