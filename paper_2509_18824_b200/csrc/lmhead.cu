@@ -32,8 +32,9 @@ constexpr int kMaxStages = 8;
 constexpr int kSmemBudget = 227 * 1024 - 2048;
 
 struct LmParams {
-    int rows;          // hidden rows handled by this launch (<= 512)
+    int rows;          // hidden rows of a row block (<= 512); the launch's last one has what is left of them
     int row0;          // index of the first one
+    int blocks;        // row blocks of this launch, 1 or 2 (pair kernel): as many equal parts of its CTAs, see the launch
     int Hd, V;
     int n_parts;       // MMA instructions along N per k-step (1 or 2)
     int part_n;        // N of each (multiple of 16, <= 256)
@@ -456,12 +457,18 @@ struct LmItems {
 template <int BK, int NPARTS>
 __global__ void __launch_bounds__(lm_threads(2 * NPARTS) + 31, 1)
 lmhead_umma_pair_kernel(const __grid_constant__ CUtensorMap tmW, const __grid_constant__ CUtensorMap tmH,
-                        const __grid_constant__ CUtensorMap tmS, const LmParams p, int32_t* status) {
+                        const __grid_constant__ CUtensorMap tmS, const LmParams p0, int32_t* status) {
     constexpr int kPar = 2 * NPARTS, kTmaWarpLm = 4 * kPar, kMmaWarpLm = kTmaWarpLm + 1;
     constexpr int kSwz = BK * 2;
     constexpr int kGroup = 8 * kSwz;
     extern __shared__ uint8_t smem_raw[];
     uint8_t* smem = reinterpret_cast<uint8_t*>((reinterpret_cast<uintptr_t>(smem_raw) + 1023) & ~(uintptr_t)1023);
+    const int n_pairs = (gridDim.x >> 1) / p0.blocks;
+    const int rb = (int)(blockIdx.x >> 1) / n_pairs;          // row block
+    const int pair = (int)(blockIdx.x >> 1) - rb * n_pairs;
+    LmParams p = p0;
+    p.row0 += rb * p0.rows;
+    p.rows = min(p0.rows, p0.M_total - p.row0);
     const int a_bytes = kBM * kSwz;
     const int half_n = p.part_n / 2;                          // hidden rows of one MMA held by this CTA
     const int stage_bytes = a_bytes + p.n_parts * half_n * kSwz;
@@ -477,8 +484,6 @@ lmhead_umma_pair_kernel(const __grid_constant__ CUtensorMap tmW, const __grid_co
     const int warp = __shfl_sync(0xffffffffu, (int)(threadIdx.x >> 5), 0);   // warp-uniform for the compiler
     const int lane = threadIdx.x & 31;
     const uint32_t rank = cluster_ctarank();                  // 0 = leader
-    const int pair = blockIdx.x >> 1;
-    const int n_pairs = gridDim.x >> 1;
     const int kblocks = p.Hd / BK;
     constexpr bool kCut = NPARTS == 2;
     const LmItems<kCut> items(p, pair, n_pairs);                    // tiles of 256 vocabulary rows
@@ -691,18 +696,19 @@ static int round_up(int x, int m) { return (x + m - 1) / m * m; }
 // pair once again, and fills and drains the pipeline.  480 rows, hidden size 3584: vocabulary of 4099 39.1 -> 24.7 us,
 // 152064 (594 tiles, 74 pairs) 377 -> 368; cutting the 49 tiles left over at 50257 took 82 instead of 78, and up to
 // 256 rows, where streaming W is what takes the time, pieces are as slow as whole tiles.
-static bool plan_slices(LmParams* p, int pairs) {
+// Returns the rounds that the call takes.
+static double plan_slices(LmParams* p, int pairs) {
     const int n_chunks = (p->n_pad + 31) / 32, rest = p->n_tiles % pairs;
     p->rounds = p->n_tiles / pairs;
     p->slices = 0;
-    double best = 0.9;                                 // of a round
+    double best = rest > 0 ? 0.9 : 0.0;                // of a round
     for (int w = 1; w < n_chunks && w <= 8 && rest > 0; ++w) {      // 32 w <= 256: one MMA
         const int s = (n_chunks + w - 1) / w;
         const int each = (rest * s + pairs - 1) / pairs;
         const double cost = each * ((double)w / n_chunks + 0.25);
         if (cost < best) { best = cost; p->slices = s; p->slice_chunks = w; }
     }
-    return p->slices > 0;
+    return p->rounds + (p->slices > 0 || rest == 0 ? best : 1.0);
 }
 
 // tiles_only_ctas != nullptr (M <= 512 required): launch only the tile kernel and report how many
@@ -721,10 +727,11 @@ static sd_status launch_lmhead_impl(const void* hidden, const void* W, int M, in
 
     const int n_blocks = (M + kMaxCols - 1) / kMaxCols;
     const int rows_per_block = round_up((M + n_blocks - 1) / n_blocks, 16);
-    for (int rb = 0; rb < n_blocks; ++rb) {
+    for (int rb = 0, blocks = 1; rb < n_blocks; rb += blocks) {
         LmParams p;
         p.row0 = rb * rows_per_block;
         p.rows = (M - p.row0 < rows_per_block) ? (M - p.row0) : rows_per_block;
+        blocks = 1;
         p.Hd = Hd; p.V = V;
         const int n16 = round_up(p.rows, 16);
         p.n_parts = (n16 > 256) ? 2 : 1;
@@ -776,7 +783,19 @@ static sd_status launch_lmhead_impl(const void* hidden, const void* W, int M, in
             grid &= ~1;
             p.rounds = p.slices = p.slice_chunks = 0;
             tmS = tmH;
-            if (p.n_pad > 256 && plan_slices(&p, grid / 2)) {
+            if (p.n_pad > 256) {
+                // Two row blocks in one launch, side by side: each has half of the pairs, and a tile of W that both come to at about
+                // the same time crosses HBM once (in launches one behind the other, twice).  Such calls run at the
+                // power limit, so that what is not moved comes back as time: 960 rows, hidden size 3584, vocabulary of 152064
+                // 751 -> 707 us, in runs of a second 893 -> 825.  Not where half as many pairs with twice the rounds leave
+                // a longer last one.
+                const double alone = plan_slices(&p, grid / 2);
+                if (rb + 1 < n_blocks && grid >= 4) {
+                    LmParams both = p;
+                    if (plan_slices(&both, grid / 4) <= 2.0 * alone) { p = both; blocks = 2; grid = grid / 4 * 2; }
+                }
+            }
+            if (p.slices > 0) {
                 if (!encode_tmap_bf16_2d(&tmS, hidden, (uint64_t)M, (uint64_t)Hd, (uint64_t)Hd * 2, (uint32_t)bk,
                                          (uint32_t)(p.slice_chunks * 16), bk * 2))
                     return SD_ERR_CUDA;
@@ -791,10 +810,11 @@ static sd_status launch_lmhead_impl(const void* hidden, const void* W, int M, in
                 const int pairs = grid / 2, rounds = (p.n_tiles + pairs - 1) / pairs;
                 if (p.n_pad > 128 || (rounds > 3 && 2 * (p.n_tiles % pairs) <= pairs)) grid = 2 * ((p.n_tiles + rounds - 1) / rounds);
             }
+            p.blocks = blocks;
             auto kern = (bk == 64) ? (p.n_parts == 2 ? lmhead_umma_pair_kernel<64, 2> : lmhead_umma_pair_kernel<64, 1>)
                                    : (p.n_parts == 2 ? lmhead_umma_pair_kernel<32, 2> : lmhead_umma_pair_kernel<32, 1>);
             if (!allow_dynamic_smem(kern, (int)dyn)) return SD_ERR_CUDA;
-            const sd_status ls = launch_dependent(kern, dim3(grid), lm_threads(2 * p.n_parts) + 31, dyn, 2, st, tmW, tmH, tmS, p, dev_status);
+            const sd_status ls = launch_dependent(kern, dim3(blocks * grid), lm_threads(2 * p.n_parts) + 31, dyn, 2, st, tmW, tmH, tmS, p, dev_status);
             if (ls != SD_OK) return ls;
         } else {
             if (grid > p.n_tiles) grid = p.n_tiles;
@@ -808,12 +828,16 @@ static sd_status launch_lmhead_impl(const void* hidden, const void* W, int M, in
             return SD_OK;
         }
         if (mass_out) continue;                      // nothing to merge: the epilogue stored the probabilities
-        const dim3 mgrid((p.rows + 63) / 64), sgrid((p.rows + 7) / 8);
-        const sd_status ms = lse ? launch_dependent(lmhead_merge_stats_kernel, sgrid, 256, 0, 1, st, p.part_key, p.part_idx, p.part_ref,
-                                                    p.part_sum, grid, p.rows, p.row0, p.c2, argmax, maxlogit, lse)
-                                 : launch_dependent(lmhead_merge_kernel, mgrid, 512, 0, 1, st, p.part_key, p.part_idx, grid, p.rows,
-                                                    p.row0, argmax, maxlogit);
-        if (ms != SD_OK) return ms;
+        for (int i = 0; i < blocks; ++i) {
+            const int row0 = p.row0 + i * rows_per_block, rows = (M - row0 < p.rows) ? (M - row0) : p.rows;
+            const size_t at = (size_t)i * grid * kMaxCols;            // this row block's CTAs
+            const dim3 mgrid((rows + 63) / 64), sgrid((rows + 7) / 8);
+            const sd_status ms = lse ? launch_dependent(lmhead_merge_stats_kernel, sgrid, 256, 0, 1, st, p.part_key + at, p.part_idx + at,
+                                                        p.part_ref + at, p.part_sum + at, grid, rows, row0, p.c2, argmax, maxlogit, lse)
+                                     : launch_dependent(lmhead_merge_kernel, mgrid, 512, 0, 1, st, p.part_key + at, p.part_idx + at, grid,
+                                                        rows, row0, argmax, maxlogit);
+            if (ms != SD_OK) return ms;
+        }
     }
     return SD_OK;
 }
