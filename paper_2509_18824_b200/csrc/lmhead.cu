@@ -52,6 +52,7 @@ struct LmParams {
     int32_t* part_idx; // [gridDim.x][kMaxCols]
     // soft-max statistics (sampling at a temperature): c2 = log2(e) / temperature, 0 = not wanted
     float c2;
+    bool index;        // of a statistics pass: the arg-max is wanted too
     float* part_ref;   // [gridDim.x][kMaxCols] reference logit of the partial sum
     float* part_sum;   // [gridDim.x][kMaxCols] sum over the CTA's vocabulary rows of 2^((logit - ref) * c2)
     // probability output (residual draw of the sampled acceptance): when mass_out is set, the epilogue
@@ -111,16 +112,19 @@ __device__ __forceinline__ T pick_lane(const T (&x)[32], int lane) {
     return (lane & 1) ? d[1] : d[0];
 }
 
+// (a tile in which the vocabulary ends: what stands behind it counts as -inf)
+__device__ __forceinline__ void hide_rows(float (&v)[32], bool v_ok) {
+#pragma unroll
+    for (int j = 0; j < 32; ++j) v[j] = v_ok ? v[j] : -INFINITY;
+}
+
 // Arg-max over the 32 lanes (vocabulary rows) of each of 32 accumulator columns (hidden rows):
 // lane j ends up with column j's maximum and the lowest vocabulary row attaining it.  The passes
 // are kept apart on purpose: 32 independent warp reductions are in flight together, then 32
 // independent votes; interleaved per column, every reduction's latency (and then every vote's)
 // would be paid one after the other.
-__device__ __forceinline__ void column_argmax32(const uint32_t (&r)[32], bool v_ok, int v_base, int lane,
-                                                float& cv, int32_t& ci) {
-    float v[32], mx[32];
-#pragma unroll
-    for (int j = 0; j < 32; ++j) v[j] = v_ok ? __uint_as_float(r[j]) : -INFINITY;
+__device__ __forceinline__ void column_argmax32(const float (&v)[32], int v_base, int lane, float& cv, int32_t& ci) {
+    float mx[32];
 #pragma unroll
     for (int j = 0; j < 32; ++j) mx[j] = redux_max_f32(v[j]);
     uint32_t who[32];
@@ -159,24 +163,29 @@ __device__ __forceinline__ float transpose_sum32(const float (&x)[32], int lane)
     return keep + __shfl_xor_sync(0xffffffffu, send, 1);
 }
 
-// The same arg-max plus, per column, sum over the 32 vocabulary rows of 2^((logit - column max) * c2):
+// (Above 256 rows the epilogue stands between the tiles, so its instructions count: without a select per logit for the vocabulary's
+// end, a test per exponential and an index that nobody wants the tail for top-k trees takes 398 instead of 406 us at 480 rows, 471
+// instead of 485 in runs of a second at the power limit; the greedy LM head 440 instead of 444 there, with 960 rows 808 instead of 829.)
+// The same maximum, the arg-max if wanted, and, per column, sum over the 32 vocabulary rows of 2^((logit - column max) * c2):
 // lane j receives column j's sum in cs.
-__device__ __forceinline__ void column_argmax_stats32(const uint32_t (&r)[32], bool v_ok, int v_base, int lane,
-                                                      float c2, float& cv, int32_t& ci, float& cs) {
-    float v[32], mx[32];
-#pragma unroll
-    for (int j = 0; j < 32; ++j) v[j] = v_ok ? __uint_as_float(r[j]) : -INFINITY;
+__device__ __forceinline__ void column_stats32(const float (&v)[32], int v_base, int lane, float c2, bool index,
+                                               float& cv, int32_t& ci, float& cs) {
+    float mx[32];
 #pragma unroll
     for (int j = 0; j < 32; ++j) mx[j] = redux_max_f32(v[j]);
-    uint32_t who[32];
-#pragma unroll
-    for (int j = 0; j < 32; ++j) who[j] = __ballot_sync(0xffffffffu, v[j] == mx[j]);
     cv = pick_lane(mx, lane);
-    ci = v_base + (__ffs(pick_lane(who, lane)) - 1);
+    ci = 0x7fffffff;
+    if (index) {
+        uint32_t who[32];
+#pragma unroll
+        for (int j = 0; j < 32; ++j) who[j] = __ballot_sync(0xffffffffu, v[j] == mx[j]);
+        ci = v_base + (__ffs(pick_lane(who, lane)) - 1);
+    }
     float e[32];
 #pragma unroll
-    for (int j = 0; j < 32; ++j) e[j] = (v[j] == -INFINITY) ? 0.f : ex2_lm((v[j] - mx[j]) * c2);
+    for (int j = 0; j < 32; ++j) e[j] = ex2_lm((v[j] - mx[j]) * c2);     // (2^-inf = 0; not a number where all are -inf)
     cs = transpose_sum32(e, lane);
+    if (cv == -INFINITY) cs = 0.f;
 }
 
 // ---------------------------------------------------------------------------
@@ -213,6 +222,9 @@ __device__ __forceinline__ void epi_tile(const LmParams& p, EpiState& e, uint32_
             tmem_ld_wait();
             float cv;
             int32_t ci;
+            float v[32];
+#pragma unroll
+            for (int j = 0; j < 32; ++j) v[j] = __uint_as_float(r[j]);
             if (p.mass_out) {
                 if (v_ok) {
 #pragma unroll
@@ -235,14 +247,16 @@ __device__ __forceinline__ void epi_tile(const LmParams& p, EpiState& e, uint32_
                         dst += p.V;
                     }
                 }
+                if (v_base + 32 > p.V) hide_rows(v, v_ok);
                 float cs;
-                column_argmax_stats32(r, v_ok, v_base, lane, p.c2, cv, ci, cs);
+                column_stats32(v, v_base, lane, p.c2, p.index, cv, ci, cs);
                 merge_sumexp(e.run_ref[h], e.run_sum[h], cv, cs, p.c2);
                 if (p.group_stats && v_base < p.V && c * 32 + lane < p.rows)
                     p.group_stats[(size_t)(v_base >> 5) * p.M_total + p.row0 + c * 32 + lane] = make_float2(cv, cs);
 
             } else {
-                column_argmax32(r, v_ok, v_base, lane, cv, ci);
+                if (v_base + 32 > p.V) hide_rows(v, v_ok);
+                column_argmax32(v, v_base, lane, cv, ci);
             }
             if (cv > e.best_val[h]) { e.best_val[h] = cv; e.best_idx[h] = ci; }
         }
@@ -761,6 +775,7 @@ static sd_status launch_lmhead_impl(const void* hidden, const void* W, int M, in
         p.stages = stages;
         p.part_key = static_cast<int32_t*>(ws);
         p.part_idx = p.part_key + (size_t)kMaxCtas * kMaxCols;
+        p.index = argmax != nullptr;
         p.c2 = lse ? inv_temp * 1.4426950408889634f : 0.f;
         p.part_ref = reinterpret_cast<float*>(static_cast<char*>(ws) + tail_workspace_bytes(M, V));
         p.part_sum = p.part_ref + (size_t)kMaxCtas * kMaxCols;
