@@ -380,7 +380,7 @@ def main():
         lm_s = per_call_ms["tail"] * 1e-3
         lm_tflops = work["lm_flops"] / lm_s / 1e12
         traffic = ATTENTION_DRAM_BYTES_PER_LAUNCH.get(args.config)
-        roofline = {"kernel": "sd_verify_attention, one layer per launch (attn_wide_kernel<1>)", "bound": "tensor",
+        roofline = {"kernel": "sd_verify_attention, one layer per launch (attn_wide_kernel<1, false>)", "bound": "tensor",
                     "achieved": att_tflops, "peak": peaks["tensor_sustained"], "unit": "TFLOP/s",
                     "frac": att_tflops / peaks["tensor_sustained"],
                     "frac_of_burst_peak": att_tflops / peaks["tensor_burst"], "burst_peak": peaks["tensor_burst"],

@@ -80,4 +80,14 @@ inline bool choose_wide(AttnPlan* p, long long base, int blocks, int sms, int fo
     return true;
 }
 
+// Whether the 128-key kernel's first copies go first: calls of one round with a single row tile per KV head (bound by the K/V
+// stream and latencies) or short chunks.  Twenty-eight calls in a row, us, without and with: 11 nodes, eight sequences of 500 tokens 270
+// 267, of 1500 326 321, of 4096 482 478, of 10000 949 939; 60 nodes, one sequence of 300 221 218, of 2048 286 283 (9 blocks
+// a chunk), of 8192 456 453 (22); eight of 1000 380 381 (16), of 1500 496 499 (24), of 2200 645 653 (35); one of 16000
+// 669 679 (42), eight of 4096 1055 1065 (64).
+constexpr int kEarlyBlocks = 22;
+inline bool copies_first(const AttnPlan& p, int blocks) {
+    return !p.ranked && (p.row_tiles == 1 || (blocks + p.n_chunks - 1) / p.n_chunks <= kEarlyBlocks);
+}
+
 }  // namespace sdv

@@ -11,11 +11,15 @@
 // the one O, which works because a row's reference stays where its first scores put it (see kSumLimit): the
 // rare tile that raises it is serialised through a per-warp commit barrier that every tile passes anyway.
 #include <atomic>
+#include "attention_plan.cuh"
 #include "attention_wide.cuh"
 
 namespace sdv {
 
-template <int NL>
+// EARLY: the first K and V copies go in front of everything else that stands between the wait for the kernel ahead and the tile
+// loop (bounds check, zeros of unused rows, set-up of the exchange), about 300 cycles.  Calls whose time is latencies and copies
+// gain from it (copies_first); in long calls the tile loop, as it is then compiled, is 40 to 80 of 1270 cycles a tile slower.
+template <int NL, bool EARLY>
 __global__ void __launch_bounds__(kWThreads, 1)
 attn_wide_kernel(const __grid_constant__ AttnLayers<NL> layers, const sd_batch bt,
                  const float scale_log2, const AttnPlan plan, int32_t* status) {
@@ -102,7 +106,10 @@ attn_wide_kernel(const __grid_constant__ AttnLayers<NL> layers, const sd_batch b
     n = wk.n; len = wk.len;
     const int rows = n * G;                                // rows of this sequence's own nodes
     const bool m64 = (rows - rt * tile_rows) <= 64;        // last row tile of at most 64 rows: M = 64 (lanes 0..15 of a quadrant)
-    if ((len + kBlock - 1) / kBlock > bt.max_blocks_per_seq && threadIdx.x == 0) set_status(status, SD_ERR_BOUNDS);
+    auto check_length = [&] {
+        if ((len + kBlock - 1) / kBlock > bt.max_blocks_per_seq && threadIdx.x == 0) set_status(status, SD_ERR_BOUNDS);
+    };
+    if constexpr (!EARLY) check_length();
     const int n_chunks = wk.n_chunks, n_pref = wk.n_pref, nb = wk.nb, t0 = wk.t0;
     const int nt = (nb + 1) / 2;
     const bool has_rows = rt * tile_rows < rows && chunk < n_chunks;   // (CTAs beyond have nothing to do)
@@ -114,7 +121,6 @@ attn_wide_kernel(const __grid_constant__ AttnLayers<NL> layers, const sd_batch b
     // divergence, and eight copies a tile made the producer the kernel's bound).  Its lanes hold the
     // block table: 32 entries in `even` (blocks 64 w ..) and 32 in `odd` (blocks 64 w + 32 ..), fetched a
     // window ahead, handed out by shuffles.
-    int jk = 0, jv = 0;
     auto window = [&](int i0) { return i0 + lane < n_pref ? __ldg(table + i0 + lane) : 0; };
     auto block_of = [&](int i) {
         int blk = __shfl_sync(0xffffffffu, (i & 32) ? odd : even, i & 31);
@@ -155,7 +161,25 @@ attn_wide_kernel(const __grid_constant__ AttnLayers<NL> layers, const sd_batch b
         }
         __syncwarp();
     };
-    if (chunk == 0) zero_unused_rows(bt, plan, ly, b, rt, kvh, rows, (int)threadIdx.x, kWThreads);
+    auto first_copies = [&] {
+        if (t0 != t0_read) {
+            even = window(0);
+            odd = window(32);
+        }
+#pragma unroll
+        for (int i = 0; i < kWStages; ++i)
+            if (i < nt) {
+                issue(i, i, false);
+                issue(i, i, true);
+            }
+    };
+    if constexpr (EARLY) {
+        if (active && warp == kWTmaWarp) first_copies();
+        check_length();
+        if (chunk == 0 && warp < 8) zero_unused_rows(bt, plan, ly, b, rt, kvh, rows, (int)threadIdx.x, 256);
+    } else {
+        if (chunk == 0) zero_unused_rows(bt, plan, ly, b, rt, kvh, rows, (int)threadIdx.x, kWThreads);
+    }
     float m_used = -INFINITY, l = 0.f;                     // this thread's row: reference, sum over its group's tiles
     bool rows_ready = false;
     const RowExchange x{bt, plan, ly, smem_u32(k_smem), smem_u32(x_full), chunk, n_chunks, rt, b, kvh, rows, wk.tpc, wk.tiles_total};
@@ -171,17 +195,8 @@ attn_wide_kernel(const __grid_constant__ AttnLayers<NL> layers, const sd_batch b
     if (active) {
     if (warp == kWTmaWarp) {
         // ------------------------------------------------------------ TMA producer
-        if (t0 != t0_read) {
-            even = window(0);
-            odd = window(32);
-        }
-#pragma unroll
-        for (int i = 0; i < kWStages; ++i)
-            if (i < nt) {
-                issue(i, i, false);
-                issue(i, i, true);
-                jk = jv = i + 1;
-            }
+        if constexpr (!EARLY) first_copies();
+        int jk = min(nt, kWStages), jv = jk;
         // (K slot j % 3 is free once the scores of tile j - 3 are complete: the score barrier tells both)
         bool ok = true;
         long long t_last = clock64();
@@ -395,7 +410,10 @@ attn_wide_kernel(const __grid_constant__ AttnLayers<NL> layers, const sd_batch b
 template <int NL>
 sd_status launch_wide(const AttnLayers<NL>& layers, const sd_batch& bt, float scale, const AttnPlan& plan,
                       int z_count, int32_t* dev_status, cudaStream_t st) {
-    return launch_attn(attn_wide_kernel<NL>, kWThreads, kWSmem, layers, bt, scale, plan, z_count, dev_status, st);
+    if constexpr (NL == 1)
+        if (copies_first(plan, bt.max_blocks_per_seq))
+            return launch_attn(attn_wide_kernel<NL, true>, kWThreads, kWSmem, layers, bt, scale, plan, z_count, dev_status, st);
+    return launch_attn(attn_wide_kernel<NL, false>, kWThreads, kWSmem, layers, bt, scale, plan, z_count, dev_status, st);
 }
 template sd_status launch_wide<1>(const AttnLayers<1>&, const sd_batch&, float, const AttnPlan&, int, int32_t*, cudaStream_t);
 template sd_status launch_wide<kMaxLayersPerLaunch>(const AttnLayers<kMaxLayersPerLaunch>&, const sd_batch&, float,
@@ -421,8 +439,8 @@ int wide_resident_clusters(int dev, int sms, int n_chunks) {
     cfg.attrs = attr;
     cfg.numAttrs = 1;
     int n = 0;
-    if (cudaFuncSetAttribute(attn_wide_kernel<1>, cudaFuncAttributeMaxDynamicSharedMemorySize, kWSmem) != cudaSuccess ||
-        cudaOccupancyMaxActiveClusters(&n, attn_wide_kernel<1>, &cfg) != cudaSuccess || n < 1)
+    if (cudaFuncSetAttribute(attn_wide_kernel<1, false>, cudaFuncAttributeMaxDynamicSharedMemorySize, kWSmem) != cudaSuccess ||
+        cudaOccupancyMaxActiveClusters(&n, attn_wide_kernel<1, false>, &cfg) != cudaSuccess || n < 1)
         n = max(1, sms / n_chunks - n_chunks);             // (no answer: a cautious guess, and ask again next time)
     else if (dev >= 0 && dev < kDevs)
         cache[dev][n_chunks].store(n, std::memory_order_relaxed);
