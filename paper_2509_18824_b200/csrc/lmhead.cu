@@ -29,6 +29,7 @@ __host__ __device__ constexpr int lm_threads(int par) { return epi_threads(par) 
 constexpr int kMaxCols = kLmMaxCols; // hidden rows per launch (TMEM columns)
 constexpr int kMaxCtas = kLmMaxCtas;
 constexpr int kMaxStages = 8;
+constexpr int kAheadSteps = 8;      // k-steps of 64 that a waiting CTA has brought to L2
 constexpr int kSmemBudget = 227 * 1024 - 2048;
 
 struct LmParams {
@@ -36,6 +37,7 @@ struct LmParams {
     int row0;          // index of the first one
     int blocks;        // row blocks of this launch, 1 or 2 (pair kernel): as many equal parts of its CTAs, see the launch
     int Hd, V;
+    const uint8_t* W;  // (for prefetches)
     int n_parts;       // MMA instructions along N per k-step (1 or 2)
     int part_n;        // N of each (multiple of 16, <= 256)
     int n_pad;         // n_parts * part_n
@@ -520,6 +522,17 @@ lmhead_umma_pair_kernel(const __grid_constant__ CUtensorMap tmW, const __grid_co
     cluster_wait_acquire();
     tc_fence_after_sync();
     const uint32_t tmem_base = tmem_base_slot;
+    // A CTA that is there before the kernel ahead is done has W's first k-steps brought to L2 meanwhile, by the warps that have nothing
+    // to do yet.  (Into L2 only: what the kernel ahead may still write to W is not missed by the copies behind the wait.)  Calls in
+    // a row, us: vocabulary of 32000 and hidden size 4096, 60 rows 49.5 -> 48.3, the top-k tail with 50257 and 2048 50.5 -> 48.7, chains' tail with
+    // 152064 and 3584 208.8 -> 208.2; three k-steps give half of that.
+    if (warp < kTmaWarpLm) {
+        const int v0 = (pair * 2 + (int)rank) * kBM;
+        for (int i = threadIdx.x; i < kAheadSteps * kBM; i += epi_threads(kPar)) {
+            const int row = v0 + (i & (kBM - 1)), step = i / kBM;
+            if (row < p.V && step * 64 < p.Hd) asm volatile("prefetch.global.L2 [%0];" ::"l"(p.W + ((size_t)row * p.Hd + step * 64) * 2));
+        }
+    }
     griddep_wait();                    // set-up done: global memory from here on
 
     if (warp == kTmaWarpLm) {
@@ -747,6 +760,7 @@ static sd_status launch_lmhead_impl(const void* hidden, const void* W, int M, in
         p.rows = (M - p.row0 < rows_per_block) ? (M - p.row0) : rows_per_block;
         blocks = 1;
         p.Hd = Hd; p.V = V;
+        p.W = static_cast<const uint8_t*>(W);
         const int n16 = round_up(p.rows, 16);
         p.n_parts = (n16 > 256) ? 2 : 1;
         p.part_n = round_up((n16 + p.n_parts - 1) / p.n_parts, 16);
