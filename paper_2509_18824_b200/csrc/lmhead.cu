@@ -8,6 +8,7 @@
 // lanes (max + lowest index) and keep a running best per hidden row; only
 // (max, index) pairs per CTA reach memory, and a tiny kernel merges them.
 #include <atomic>
+#include "lmhead_plan.cuh"
 #include "tree_device.cuh"
 #include "sm100.cuh"
 
@@ -35,7 +36,7 @@ constexpr int kSmemBudget = 227 * 1024 - 2048;
 struct LmParams {
     int rows;          // hidden rows of a row block (<= 512); the launch's last one has what is left of them
     int row0;          // index of the first one
-    int blocks;        // row blocks of this launch, 1 or 2 (pair kernel): as many equal parts of its CTAs, see the launch
+    int blocks;        // row blocks of this launch, 1 or 2 (pair kernel): as many equal parts of its CTAs, see side_by_side
     int Hd, V;
     const uint8_t* W;  // (for prefetches)
     int n_parts;       // MMA instructions along N per k-step (1 or 2)
@@ -737,27 +738,6 @@ lmhead_merge_stats_kernel(const int32_t* __restrict__ part_key, const int32_t* _
 
 static int round_up(int x, int m) { return (x + m - 1) / m * m; }
 
-// More than 256 hidden rows, where the tensor cores bound a tile: if few tiles are left over after whole rounds of
-// all pairs (or there are few tiles at all), they are cut along the hidden rows into pieces that are dealt out to
-// all pairs.  A piece costs its share of a tile and about a quarter more: it streams its tile's W through the
-// pair once again, and fills and drains the pipeline.  480 rows, hidden size 3584: vocabulary of 4099 39.1 -> 24.7 us,
-// 152064 (594 tiles, 74 pairs) 377 -> 368; cutting the 49 tiles left over at 50257 took 82 instead of 78, and up to
-// 256 rows, where streaming W is what takes the time, pieces are as slow as whole tiles.
-// Returns the rounds that the call takes.
-static double plan_slices(LmParams* p, int pairs) {
-    const int n_chunks = (p->n_pad + 31) / 32, rest = p->n_tiles % pairs;
-    p->rounds = p->n_tiles / pairs;
-    p->slices = 0;
-    double best = rest > 0 ? 0.9 : 0.0;                // of a round
-    for (int w = 1; w < n_chunks && w <= 8 && rest > 0; ++w) {      // 32 w <= 256: one MMA
-        const int s = (n_chunks + w - 1) / w;
-        const int each = (rest * s + pairs - 1) / pairs;
-        const double cost = each * ((double)w / n_chunks + 0.25);
-        if (cost < best) { best = cost; p->slices = s; p->slice_chunks = w; }
-    }
-    return p->rounds + (p->slices > 0 || rest == 0 ? best : 1.0);
-}
-
 // tiles_only_ctas != nullptr (M <= 512 required): launch only the tile kernel and report how many
 // CTAs filled the candidate tables; the caller merges them itself (the fused tail kernel).
 static sd_status launch_lmhead_impl(const void* hidden, const void* W, int M, int Hd, int V,
@@ -781,10 +761,10 @@ static sd_status launch_lmhead_impl(const void* hidden, const void* W, int M, in
         blocks = 1;
         p.Hd = Hd; p.V = V;
         p.W = static_cast<const uint8_t*>(W);
-        const int n16 = round_up(p.rows, 16);
-        p.n_parts = (n16 > 256) ? 2 : 1;
-        p.part_n = round_up((n16 + p.n_parts - 1) / p.n_parts, 16);
-        p.n_pad = p.n_parts * p.part_n;
+        const LmColumns columns = lm_columns(p.rows);
+        p.n_parts = columns.n_parts;
+        p.part_n = columns.part_n;
+        p.n_pad = columns.padded();
         p.buf_stride = round_up(p.n_pad, 32);
         p.acc_bufs = (2 * p.buf_stride <= kMaxCols) ? 2 : 1;
         int cols = 32;
@@ -794,10 +774,7 @@ static sd_status launch_lmhead_impl(const void* hidden, const void* W, int M, in
         // Two-CTA tiles whenever a pair has work (the common case); rows per MMA part must then
         // split evenly over the two CTAs in whole 8-row swizzle groups.
         const bool pair = (sms >= 2) && (V > kBM);
-        if (pair) {
-            p.part_n = round_up(p.part_n, 16);
-            p.n_tiles = (V + 2 * kBM - 1) / (2 * kBM);
-        }
+        if (pair) p.n_tiles = (V + 2 * kBM - 1) / (2 * kBM);
         const int b_rows = pair ? p.n_pad / 2 : p.n_pad;      // hidden rows staged per CTA and k-step
         // contraction step: 64 (128-byte swizzle) while at least four stages fit, else 32
         const int stage64 = (kBM + b_rows) * 128;
@@ -833,16 +810,12 @@ static sd_status launch_lmhead_impl(const void* hidden, const void* W, int M, in
             p.rounds = p.slices = p.slice_chunks = 0;
             tmS = tmH;
             if (p.n_pad > 256) {
-                // Two row blocks in one launch, side by side: each has half of the pairs, and a tile of W that both come to at about
-                // the same time crosses HBM once (in launches one behind the other, twice).  Such calls run at the
-                // power limit, so that what is not moved comes back as time: 960 rows, hidden size 3584, vocabulary of 152064
-                // 751 -> 707 us, in runs of a second 893 -> 825.  Not where half as many pairs with twice the rounds leave
-                // a longer last one.
-                const double alone = plan_slices(&p, grid / 2);
-                if (rb + 1 < n_blocks && grid >= 4) {
-                    LmParams both = p;
-                    if (plan_slices(&both, grid / 4) <= 2.0 * alone) { p = both; blocks = 2; grid = grid / 4 * 2; }
+                if (rb + 1 < n_blocks && side_by_side(p.rows, min(rows_per_block, M - p.row0 - rows_per_block), Hd, p.n_tiles, grid / 2)) {
+                    blocks = 2;
+                    grid = grid / 4 * 2;
                 }
+                const LmSlices cut = plan_slices(p.n_tiles, grid / 2, p.n_pad);
+                p.rounds = cut.rounds; p.slices = cut.slices; p.slice_chunks = cut.slice_chunks;
             }
             if (p.slices > 0) {
                 if (!encode_tmap_bf16_2d(&tmS, hidden, (uint64_t)M, (uint64_t)Hd, (uint64_t)Hd * 2, (uint32_t)bk,

@@ -38,3 +38,34 @@ def test_row_blocks(M, Hd, V):
     assert (np.abs(kept.cpu().numpy() - logits) <= bound + 1e-6).all()
     _, rlse = smp.softmax_rows(logits, inv_temp)
     np.testing.assert_allclose(lse.cpu().numpy(), rlse, rtol=0, atol=3e-4)
+
+
+# row blocks of 272 and 241 rows one behind the other; of 400, 400, 400 and 337: two side by side, then one and one
+@pytest.mark.parametrize("M,rows", [(513, 272), (1537, 400)])
+def test_row_blocks_one_behind_the_other(M, rows):
+    """The same bits as calls for the rows of each block alone."""
+    V, Hd = 128256, 2048
+    g = torch.Generator(device="cuda").manual_seed(M)
+    h = torch.randn((M, Hd), device="cuda", generator=g).to(torch.bfloat16)
+    W = torch.randn((V, Hd), device="cuda", generator=g).to(torch.bfloat16)
+    ws = torch.empty(sd.sd_workspace_bytes(None, M, V), dtype=torch.uint8, device="cuda")
+    st = sd.new_status()
+
+    def call(x):
+        n = x.shape[0]
+        am = torch.full((n,), -5, dtype=torch.int32, device="cuda")
+        mx, lse, kept = torch.zeros(n, device="cuda"), torch.zeros(n, device="cuda"), torch.full((n, V), float("nan"), device="cuda")
+        sd.sd_lmhead_stats_logits(x, W, 1.0 / 32, am, mx, lse, kept, ws, st)
+        am2 = torch.full((n,), -5, dtype=torch.int32, device="cuda")
+        sd.sd_lmhead_argmax(x, W, am2, None, ws, st)
+        assert torch.equal(am, am2)
+        return am, mx, lse, kept
+
+    whole = call(h)
+    for r in range(0, M, rows):
+        part = call(h[r:r + rows].contiguous())
+        for k in (0, 1, 3):
+            assert torch.equal(whole[k][r:r + rows], part[k])
+        # (sums of V fp32 terms, brought together from other CTAs' parts: a few 2^-24 of the sum in each of some ten merges)
+        assert (whole[2][r:r + rows] - part[2]).abs().max().item() <= 1e-5
+    assert int(st.item()) == 0
