@@ -30,7 +30,6 @@ __host__ __device__ constexpr int lm_threads(int par) { return epi_threads(par) 
 constexpr int kMaxCols = kLmMaxCols; // hidden rows per launch (TMEM columns)
 constexpr int kMaxCtas = kLmMaxCtas;
 constexpr int kMaxStages = 8;
-constexpr int kAheadSteps = 8;      // k-steps of 64 that a waiting CTA has brought to L2
 constexpr int kSmemBudget = 227 * 1024 - 2048;
 
 struct LmParams {
@@ -39,6 +38,7 @@ struct LmParams {
     int blocks;        // row blocks of this launch, 1 or 2 (pair kernel): as many equal parts of its CTAs, see side_by_side
     int Hd, V;
     const uint8_t* W;  // (for prefetches)
+    int ahead;         // hidden dimensions that a waiting CTA has brought to L2, in k-steps of 64 (at most kAheadSteps), 0: none
     int n_parts;       // MMA instructions along N per k-step (1 or 2)
     int part_n;        // N of each (multiple of 16, <= 256)
     int n_pad;         // n_parts * part_n
@@ -523,15 +523,17 @@ lmhead_umma_pair_kernel(const __grid_constant__ CUtensorMap tmW, const __grid_co
     cluster_wait_acquire();
     tc_fence_after_sync();
     const uint32_t tmem_base = tmem_base_slot;
-    // A CTA that is there before the kernel ahead is done has W's first k-steps brought to L2 meanwhile, by the warps that have nothing
-    // to do yet.  (Into L2 only: what the kernel ahead may still write to W is not missed by the copies behind the wait.)  Calls in
-    // a row, us: vocabulary of 32000 and hidden size 4096, 60 rows 49.5 -> 48.3, the top-k tail with 50257 and 2048 50.5 -> 48.7, chains' tail with
-    // 152064 and 3584 208.8 -> 208.2; three k-steps give half of that.
+    // A CTA that is there before the kernel ahead is done has W's first k-steps brought to L2 meanwhile (brings_ahead), by the warps that
+    // have nothing to do yet.  (Into L2 only: what the kernel ahead may still write to W is not missed by the copies behind the wait.
+    // With no kernel ahead the copies follow at once: no gain, no loss beyond the noise.)  Where there are no whole rounds and the
+    // tiles are cut, the CTAs do it for one another: a CTA's own piece is of tile pair / slices, and finding it costs a
+    // division and asks for a tile once per piece (480 rows, hidden size 1024, vocabulary of 4099 12.0 us without, 11.6 so, 12.1 with the own
+    // pieces).  Of two row blocks the first does it for both: twice, 960 rows there take 4 % longer than without.
     if (warp < kTmaWarpLm) {
-        const int v0 = (pair * 2 + (int)rank) * kBM;
+        const int v0 = (pair * 2 + (int)rank) * kBM, ahead = kCut && rb > 0 ? 0 : p.ahead;
         for (int i = threadIdx.x; i < kAheadSteps * kBM; i += epi_threads(kPar)) {
             const int row = v0 + (i & (kBM - 1)), step = i / kBM;
-            if (row < p.V && step * 64 < p.Hd) asm volatile("prefetch.global.L2 [%0];" ::"l"(p.W + ((size_t)row * p.Hd + step * 64) * 2));
+            if (row < p.V && step * 64 < ahead) asm volatile("prefetch.global.L2 [%0];" ::"l"(p.W + ((size_t)row * p.Hd + step * 64) * 2));
         }
     }
     griddep_wait();                    // set-up done: global memory from here on
@@ -817,6 +819,7 @@ static sd_status launch_lmhead_impl(const void* hidden, const void* W, int M, in
                 const LmSlices cut = plan_slices(p.n_tiles, grid / 2, p.n_pad);
                 p.rounds = cut.rounds; p.slices = cut.slices; p.slice_chunks = cut.slice_chunks;
             }
+            p.ahead = brings_ahead(Hd, p.n_tiles, grid / 2) ? Hd : 0;
             if (p.slices > 0) {
                 if (!encode_tmap_bf16_2d(&tmS, hidden, (uint64_t)M, (uint64_t)Hd, (uint64_t)Hd * 2, (uint32_t)bk,
                                          (uint32_t)(p.slice_chunks * 16), bk * 2))

@@ -60,4 +60,13 @@ inline bool side_by_side(int rows, int next_rows, int Hd, int n_tiles, int pairs
     return both <= 1.02 * (alone + next);
 }
 
+// Whether a CTA has the first eight k-steps of 64 of its first tile of W brought to L2 while the kernel ahead runs.  Calls in a row, W from HBM, us without
+// and with: 60 rows, hidden size 4096 and vocabulary of 32000 47.1 45.3, 2048 and 50257 37.8 36.2, 768 and 32000 14.4 13.1; chains'
+// tail at 3584 and 152064 208.8 208.2; 480 rows, 1024 and 1025 10.9 10.6; three k-steps give half of that.  Not where a CTA has no
+// second tile and eight k-steps are much or all of the one it has, which its copies ask for at once anyway: 60 rows, 512 and 6000
+// 7.2 7.6, 4099 7.0 7.4; 384 and 6000 6.9 7.2; 480 rows, 256 and 6000 9.3 9.7.  (A hidden size of 128 has so little W that it gains
+// again: 60 rows and 6000 6.0 5.9.)
+constexpr int kAheadSteps = 8;
+inline bool brings_ahead(int Hd, int n_tiles, int pairs) { return Hd < 256 || Hd >= 1024 || n_tiles >= pairs; }
+
 }  // namespace sdv

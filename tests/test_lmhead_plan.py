@@ -34,6 +34,7 @@ static int cover() {                                       // every (tile, chunk
 }
 int main(int argc, char** argv) {
     if (argc == 1) return cover();
+    if (argc == 3) { printf("%d\n", (int)brings_ahead(atoi(argv[1]), (atoi(argv[2]) + 255) / 256, 74)); return 0; }
     const int M = atoi(argv[1]), V = atoi(argv[2]), Hd = atoi(argv[3]);       // how the row blocks of a call share launches, 74 pairs
     const int n = (M + 511) / 512, rows = ((M + n - 1) / n + 15) / 16 * 16;
     for (int rb = 0; rb < n;) {
@@ -72,3 +73,9 @@ def test_pieces_cover_the_tiles(plan):
     (577, 128256, 4096, "11"), (769, 128256, 4096, "11"), (961, 128256, 4096, "11"), (1537, 128256, 4096, "211")])
 def test_row_blocks_share_a_launch_where_it_is_faster(plan, M, V, Hd, launches):
     assert plan(M, V, Hd) == launches
+
+
+@pytest.mark.parametrize("Hd,V,ahead", [(4096, 32000, 1), (2048, 50257, 1), (768, 32000, 1), (3584, 152064, 1), (1024, 1025, 1), (128, 6000, 1),
+                                        (512, 6000, 0), (512, 4099, 0), (384, 6000, 0), (256, 6000, 0)])
+def test_k_steps_brought_to_l2(plan, Hd, V, ahead):
+    assert int(plan(Hd, V)) == ahead
