@@ -80,14 +80,23 @@ inline bool choose_wide(AttnPlan* p, long long base, int blocks, int sms, int fo
     return true;
 }
 
-// Whether the 128-key kernel's first copies go first: calls of one round with a single row tile per KV head (bound by the K/V
-// stream and latencies) or short chunks.  Twenty-eight calls in a row, us, without and with: 11 nodes, eight sequences of 500 tokens 270
-// 267, of 1500 326 321, of 4096 482 478, of 10000 949 939; 60 nodes, one sequence of 300 221 218, of 2048 286 283 (9 blocks
-// a chunk), of 8192 456 453 (22); eight of 1000 380 381 (16), of 1500 496 499 (24), of 2200 645 653 (35); one of 16000
-// 669 679 (42), eight of 4096 1055 1065 (64).
-constexpr int kEarlyBlocks = 22;
+// Whether the 128-key kernel's first copies go first.  Calls of several rounds keep the other order: nothing waits for their
+// later CTAs' copies (72 chains of 1000 tokens, eight calls 248.1 248.7; 256 row tiles of one sequence of 4000 545 561).  In one round
+// latencies count, 1 to 3 % of the calls below, but a row tile's loop takes 40 to 80 of 1270 cycles a tile longer, which shows
+// where several row tiles share K and V: the line is the blocks of a chunk, fitted for each number of chunks.  Fourteen calls in a row,
+// us, without and with, sequences of 60 nodes and their blocks a chunk: one chunk, eight of 1250 (20) 204.0 203.6, 1300
+// (22) 206.0 204.8, 1350 (23) 214.3 215.9, six of 1500 (25) 222.7 225.9; two chunks, four of 2100 (17) 195.8 193.9, 2200 (18) 201.8
+// 204.3, 2700 (22) 222.6 227.8, three of 2200 (18) 1.3 % longer; three chunks, two of 1000 (6) 1.1 % shorter, three of 2500 (14) 214.1
+// 215.9, 4000 (22) 274.4 281.0; four, two of 5500 (22) 224.4 222.2, 6500 (26) 243.5 242.5; six, one of 8192 (22) 1.2 % shorter, 12000 (32)
+// 0.4 % longer.  With one or two row tiles the line may be anywhere from 22 up (four sequences of 28 nodes and 2900 tokens 2.2 %
+// shorter, eight of 2700 in two chunks of 22 233.1 233.9); chains, one row tile, gain at every length (eight of 10000 1 %).
+// The blocks are the table's width, which stands for the longest length as above: in a table that is far wider a call keeps the
+// order that is right for long sequences and misses the gain (28 calls, one sequence of 2048 tokens in 33 blocks 269, in 512 275).
 inline bool copies_first(const AttnPlan& p, int blocks) {
-    return !p.ranked && (p.row_tiles == 1 || (blocks + p.n_chunks - 1) / p.n_chunks <= kEarlyBlocks);
+    constexpr int kLine = 22, kLineShared[kMaxChunks] = {kLine, 17, 12, kLine, kLine, kLine, kLine, kLine};
+    if (p.whole_blocks < 0) return false;                  // several rounds
+    const int per = (blocks + p.n_chunks - 1) / p.n_chunks;
+    return p.row_tiles == 1 || per <= (p.row_tiles == 2 ? kLine : kLineShared[p.n_chunks - 1]);
 }
 
 }  // namespace sdv

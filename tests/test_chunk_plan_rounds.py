@@ -53,3 +53,44 @@ def test_a_wider_table_does_not_bring_several_rounds(tmp_path):
     r = subprocess.run([str(exe)], capture_output=True, text=True)
     assert r.returncode == 0, r.stdout
     assert int(r.stdout) > 13000
+
+
+FIRST_COPIES = r"""
+#include <cstdio>
+#include <cstdlib>
+#include "attention_plan.cuh"
+using namespace sdv;
+int main(int argc, char** argv) {                          // B, KV heads, row tiles, width of the table
+    const int B = atoi(argv[1]), Hkv = atoi(argv[2]), blocks = atoi(argv[4]), sms = 148;
+    AttnPlan p;
+    p.row_tiles = atoi(argv[3]);
+    const int base = B * Hkv * p.row_tiles;
+    if (!choose_wide(&p, base, blocks, sms, 0, [&](int c) { return c <= 2 ? sms / c : c < 7 ? sms / c - 1 : 15; })) { printf("64\n"); return 0; }
+    p.ranked = B > 1 && B <= 64 && base * p.n_chunks > sms;
+    printf("%d %d\n", p.n_chunks, (int)copies_first(p, blocks));
+}
+"""
+
+
+@pytest.fixture(scope="module")
+def first_copies(tmp_path_factory):
+    nvcc = build._nvcc()
+    if not os.path.exists(nvcc):
+        pytest.skip("no nvcc")
+    d = tmp_path_factory.mktemp("first_copies")
+    (d / "first.cu").write_text(FIRST_COPIES)
+    subprocess.run([nvcc, "-std=c++17", "-O1", "-gencode", "arch=compute_100a,code=sm_100a", "-I", build.INCLUDE, "-I", build.CSRC,
+                    str(d / "first.cu"), "-o", str(d / "first")], check=True)
+    return lambda *a: subprocess.run([str(d / "first"), *map(str, a)], capture_output=True, text=True, check=True).stdout.split()
+
+
+# (chunks, whether the first copies go first), as measured where the comment at copies_first says so
+@pytest.mark.parametrize("B,Hkv,row_tiles,blocks,plan", [
+    (1, 4, 4, 2, (1, 1)), (1, 4, 4, 33, (4, 1)), (1, 4, 4, 129, (6, 1)), (1, 4, 4, 251, (6, 0)),
+    (8, 4, 4, 22, (1, 1)), (8, 4, 4, 23, (1, 0)), (8, 4, 4, 65, (1, 0)), (4, 4, 4, 34, (2, 1)), (4, 4, 4, 36, (2, 0)), (4, 4, 4, 43, (2, 0)),
+    (3, 4, 4, 41, (3, 0)), (2, 4, 4, 17, (3, 1)), (2, 4, 4, 87, (4, 1)), (8, 4, 2, 43, (2, 1)), (16, 4, 2, 25, (1, 0)),
+    (8, 4, 1, 65, (4, 1)), (8, 4, 1, 200, (4, 1)), (37, 4, 1, 16, (1, 1)),
+    # several rounds, of one and of more row tiles, more sequences than are ranked by length, and one sequence
+    (72, 4, 1, 65, (1, 0)), (100, 4, 1, 32, (1, 0)), (1, 64, 4, 64, (1, 0)), (16, 4, 4, 257, (1, 0))])
+def test_first_copies_go_first(first_copies, B, Hkv, row_tiles, blocks, plan):
+    assert tuple(int(x) for x in first_copies(B, Hkv, row_tiles, blocks)) == plan
