@@ -435,7 +435,7 @@ def test_lmhead_small_shapes_crisp(M, Hd, V):
 
 
 def test_lmhead_more_rows_than_one_pass():
-    """More than 512 rows are processed in several passes over the vocabulary."""
+    """More than 512 rows are processed in row blocks: three here, two of them side by side in one pass over the vocabulary."""
     g = np.random.default_rng(11)
     M, Hd, V = 1100, 128, 2500
     h = wl.f32_to_bf16_bits(g.standard_normal((M, Hd)).astype(np.float32))

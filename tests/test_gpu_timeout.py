@@ -103,8 +103,9 @@ def test_lmhead_wait_runs_out_and_the_next_call_is_fine(monkeypatch):
     check_argmax(am2, mx2, ram, t1, t2)
 
 
-# one pair of CTAs, pairs with one and several tiles, two MMAs a step (one accumulator), leftover tiles cut into pieces
-@pytest.mark.parametrize("M,V", [(8, 200), (60, 4099), (60, 60000), (300, 4099), (480, 25000)])
+# one pair of CTAs, pairs with one and several tiles, two MMAs a step (one accumulator), leftover tiles cut into pieces, two row
+# blocks in a launch, and a third one behind them
+@pytest.mark.parametrize("M,V", [(8, 200), (60, 4099), (60, 60000), (300, 4099), (480, 25000), (700, 4099), (1100, 25000)])
 def test_lmhead_pair_wait_runs_out_and_the_next_call_is_fine(monkeypatch, M, V):
     g = np.random.default_rng(M)
     Hd = 128
