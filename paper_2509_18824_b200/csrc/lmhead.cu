@@ -480,12 +480,16 @@ lmhead_umma_pair_kernel(const __grid_constant__ CUtensorMap tmW, const __grid_co
     constexpr int kGroup = 8 * kSwz;
     extern __shared__ uint8_t smem_raw[];
     uint8_t* smem = reinterpret_cast<uint8_t*>((reinterpret_cast<uintptr_t>(smem_raw) + 1023) & ~(uintptr_t)1023);
-    const int n_pairs = (gridDim.x >> 1) / p0.blocks;
-    const int rb = (int)(blockIdx.x >> 1) / n_pairs;          // row block
+    constexpr bool kCut = NPARTS == 2;                        // more than 256 rows: tiles may be cut, two row blocks side by side
+    // (no division: the set-up of a small call is part of its time)
+    const int n_pairs = kCut ? gridDim.x >> p0.blocks : gridDim.x >> 1;
+    const int rb = kCut && (int)(blockIdx.x >> 1) >= n_pairs ? 1 : 0;             // row block
     const int pair = (int)(blockIdx.x >> 1) - rb * n_pairs;
     LmParams p = p0;
-    p.row0 += rb * p0.rows;
-    p.rows = min(p0.rows, p0.M_total - p.row0);
+    if (kCut && p0.blocks == 2) {
+        p.row0 += rb * p0.rows;
+        p.rows = min(p0.rows, p0.M_total - p.row0);
+    }
     const int a_bytes = kBM * kSwz;
     const int half_n = p.part_n / 2;                          // hidden rows of one MMA held by this CTA
     const int stage_bytes = a_bytes + p.n_parts * half_n * kSwz;
@@ -502,7 +506,6 @@ lmhead_umma_pair_kernel(const __grid_constant__ CUtensorMap tmW, const __grid_co
     const int lane = threadIdx.x & 31;
     const uint32_t rank = cluster_ctarank();                  // 0 = leader
     const int kblocks = p.Hd / BK;
-    constexpr bool kCut = NPARTS == 2;
     const LmItems<kCut> items(p, pair, n_pairs);                    // tiles of 256 vocabulary rows
 
     if (threadIdx.x == 0) {
