@@ -55,7 +55,6 @@ struct LmParams {
     int32_t* part_idx; // [gridDim.x][kMaxCols]
     // soft-max statistics (sampling at a temperature): c2 = log2(e) / temperature, 0 = not wanted
     float c2;
-    bool index;        // of a statistics pass: the arg-max is wanted too
     float* part_ref;   // [gridDim.x][kMaxCols] reference logit of the partial sum
     float* part_sum;   // [gridDim.x][kMaxCols] sum over the CTA's vocabulary rows of 2^((logit - ref) * c2)
     // probability output (residual draw of the sampled acceptance): when mass_out is set, the epilogue
@@ -166,24 +165,21 @@ __device__ __forceinline__ float transpose_sum32(const float (&x)[32], int lane)
     return keep + __shfl_xor_sync(0xffffffffu, send, 1);
 }
 
+// The same arg-max plus, per column, sum over the 32 vocabulary rows of 2^((logit - column max) * c2): lane j receives column j's sum in cs.
 // (Above 256 rows the epilogue stands between the tiles, so its instructions count: without a select per logit for the vocabulary's
-// end, a test per exponential and an index that nobody wants the tail for top-k trees takes 398 instead of 406 us at 480 rows, 471
-// instead of 485 in runs of a second at the power limit; the greedy LM head 440 instead of 444 there, with 960 rows 808 instead of 829.)
-// The same maximum, the arg-max if wanted, and, per column, sum over the 32 vocabulary rows of 2^((logit - column max) * c2):
-// lane j receives column j's sum in cs.
-__device__ __forceinline__ void column_stats32(const float (&v)[32], int v_base, int lane, float c2, bool index,
-                                               float& cv, int32_t& ci, float& cs) {
+// end and a test per exponential the tail for top-k trees takes 411 instead of 416 us at 480 rows, 483 instead of 487 in runs of a
+// second at the power limit; with a vocabulary of 50257 and hidden size 2048 98 instead of 100.5; statistics of 264 rows, 512 and
+// 256, 7.3 instead of 7.8.  Leaving the index out where nobody asks for it gains nothing (411 and 483 again) and costs the others: its
+// branch stands between the votes and the exponentials, 5.45 instead of 5.33 us for 8 rows, 7.6 instead of 7.3 for 264.)
+__device__ __forceinline__ void column_stats32(const float (&v)[32], int v_base, int lane, float c2, float& cv, int32_t& ci, float& cs) {
     float mx[32];
 #pragma unroll
     for (int j = 0; j < 32; ++j) mx[j] = redux_max_f32(v[j]);
-    cv = pick_lane(mx, lane);
-    ci = 0x7fffffff;
-    if (index) {
-        uint32_t who[32];
+    uint32_t who[32];
 #pragma unroll
-        for (int j = 0; j < 32; ++j) who[j] = __ballot_sync(0xffffffffu, v[j] == mx[j]);
-        ci = v_base + (__ffs(pick_lane(who, lane)) - 1);
-    }
+    for (int j = 0; j < 32; ++j) who[j] = __ballot_sync(0xffffffffu, v[j] == mx[j]);
+    cv = pick_lane(mx, lane);
+    ci = v_base + (__ffs(pick_lane(who, lane)) - 1);
     float e[32];
 #pragma unroll
     for (int j = 0; j < 32; ++j) e[j] = ex2_lm((v[j] - mx[j]) * c2);     // (2^-inf = 0; not a number where all are -inf)
@@ -252,7 +248,7 @@ __device__ __forceinline__ void epi_tile(const LmParams& p, EpiState& e, uint32_
                 }
                 if (v_base + 32 > p.V) hide_rows(v, v_ok);
                 float cs;
-                column_stats32(v, v_base, lane, p.c2, p.index, cv, ci, cs);
+                column_stats32(v, v_base, lane, p.c2, cv, ci, cs);
                 merge_sumexp(e.run_ref[h], e.run_sum[h], cv, cs, p.c2);
                 if (p.group_stats && v_base < p.V && c * 32 + lane < p.rows)
                     p.group_stats[(size_t)(v_base >> 5) * p.M_total + p.row0 + c * 32 + lane] = make_float2(cv, cs);
@@ -791,7 +787,6 @@ static sd_status launch_lmhead_impl(const void* hidden, const void* W, int M, in
         p.stages = stages;
         p.part_key = static_cast<int32_t*>(ws);
         p.part_idx = p.part_key + (size_t)kMaxCtas * kMaxCols;
-        p.index = argmax != nullptr;
         p.c2 = lse ? inv_temp * 1.4426950408889634f : 0.f;
         p.part_ref = reinterpret_cast<float*>(static_cast<char*>(ws) + tail_workspace_bytes(M, V));
         p.part_sum = p.part_ref + (size_t)kMaxCtas * kMaxCols;
