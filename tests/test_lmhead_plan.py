@@ -69,7 +69,7 @@ def test_pieces_cover_the_tiles(plan):
     (600, 128256, 4096, "2"), (960, 128256, 4096, "2"), (513, 50257, 2048, "2"), (960, 50257, 2048, "2"), (2048, 32000, 4096, "22"),
     (513, 4099, 1024, "2"), (600, 200, 1024, "2"), (1537, 4099, 3584, "22"),
     # a second block whose own columns are fewer, where W's tiles take many rounds
-    (513, 152064, 3584, "11"), (520, 128256, 4096, "11"), (528, 94000, 3584, "11"), (513, 110000, 3584, "11"),
+    (513, 152064, 3584, "11"), (513, 152064, 1024, "11"), (520, 128256, 4096, "11"), (528, 94000, 3584, "11"), (513, 110000, 3584, "11"),
     (577, 128256, 4096, "11"), (769, 128256, 4096, "11"), (961, 128256, 4096, "11"), (1537, 128256, 4096, "211")])
 def test_row_blocks_share_a_launch_where_it_is_faster(plan, M, V, Hd, launches):
     assert plan(M, V, Hd) == launches
