@@ -1,5 +1,5 @@
-"""GPU: the 128-key attention kernel with its first copies in front (chunks of up to 22 blocks of the table's width, or a single row
-tile) and behind the bounds check and zeros: both sides of the line against the fp64 checker, and the same bits."""
+"""GPU: the 128-key attention kernel with its first copies in front (two row tiles and chunks of up to 22 blocks of the table's width,
+or a single row tile; test_chunk_plan_rounds.py has which plans take which order) and behind the bounds check and zeros: both sides of the line against the fp64 checker, and the same bits."""
 import numpy as np
 import pytest
 
