@@ -35,7 +35,7 @@ constexpr int kSmemBudget = 227 * 1024 - 2048;
 struct LmParams {
     int rows;          // hidden rows of a row block (<= 512); the launch's last one has what is left of them
     int row0;          // index of the first one
-    int blocks;        // row blocks of this launch, 1 or 2 (pair kernel): as many equal parts of its CTAs, see side_by_side
+    int blocks;        // row blocks of this launch, 1 or 2 (pair kernel): as many equal parts of its CTAs, see the launch
     int Hd, V;
     const uint8_t* W;  // (for prefetches)
     int ahead;         // hidden dimensions that a waiting CTA has brought to L2, in k-steps of 64 (at most kAheadSteps), 0: none
@@ -810,7 +810,15 @@ static sd_status launch_lmhead_impl(const void* hidden, const void* W, int M, in
             p.rounds = p.slices = p.slice_chunks = 0;
             tmS = tmH;
             if (p.n_pad > 256) {
-                if (rb + 1 < n_blocks && side_by_side(p.rows, min(rows_per_block, M - p.row0 - rows_per_block), Hd, p.n_tiles, grid / 2)) {
+                // Two row blocks in one launch, side by side: each has half of the pairs, and a tile of W that both come to at about
+                // the same time crosses HBM once (in launches one behind the other, twice; DRAM reads of 960 rows, vocabulary 65536 and hidden
+                // size 3584: 476.8 MB for 476.7 of W and hidden rows).  One behind the other and side by side, us, single calls behind a
+                // pause and in runs of a second at the power limit, vocabulary 152064 and hidden size 3584: 600 rows 518 472, 636 569;
+                // 960 rows 717 671, 866 817; 513 rows, whose second block is multiplied with 288 columns and not its own 256, 449 433, 564
+                // 527; 1537 rows 1251 1196, 1508 1423; 128256 and 4096, 769 rows 585 566, 715 683; 50257 and 2048, 960 rows 162 142, 181 162;
+                // 4099 and 1024, 600 rows 21.3 11.5.  The one size that lost: 513 rows, 152064 and 1024, 148 157, 178 177.
+                // (Short bursts of both in turn, at clocks that had not settled, said otherwise for the larger vocabularies.)
+                if (rb + 1 < n_blocks && grid >= 4) {
                     blocks = 2;
                     grid = grid / 4 * 2;
                 }

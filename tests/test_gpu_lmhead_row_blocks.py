@@ -1,4 +1,4 @@
-"""GPU: LM head above 512 rows, where two row blocks may share a launch: a last block that is narrower, an odd number of blocks,
+"""GPU: LM head above 512 rows, where two row blocks share a launch: a last block that is narrower, an odd number of blocks,
 whole tiles alone, tiles cut into pieces, fewer tiles than pairs; arg-max, statistics with and without it, group statistics, kept
 logits and the probabilities of more than 512 stop rows."""
 import copy
@@ -44,9 +44,9 @@ def test_row_blocks(M, Hd, V):
     np.testing.assert_allclose(lse.cpu().numpy(), rlse, rtol=0, atol=3e-4)
 
 
-# row blocks of 272 and 241 rows one behind the other; of 400, 400, 400 and 337: two side by side, then one and one
-@pytest.mark.parametrize("M,rows", [(513, 272), (1537, 400)])
-def test_row_blocks_one_behind_the_other(M, rows):
+# row blocks of 272 and 241 rows, the latter with fewer columns of its own; of 368, 368 and 364: two side by side, then one
+@pytest.mark.parametrize("M,rows", [(513, 272), (1100, 368)])
+def test_row_blocks_and_calls_for_each(M, rows):
     """The same bits as calls for the rows of each block alone."""
     V, Hd = 128256, 2048
     g = torch.Generator(device="cuda").manual_seed(M)

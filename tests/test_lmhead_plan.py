@@ -1,5 +1,5 @@
-"""How an LM-head call is dealt out (csrc/lmhead_plan.cuh), compiled for the host: tiles cut into pieces are covered once, and two
-row blocks share a launch where that was measured to be faster and not where it was slower."""
+"""How an LM-head call is dealt out (csrc/lmhead_plan.cuh), compiled for the host: tiles cut into pieces are covered once, and W
+is brought to L2 ahead where that was measured to be faster and not where it was slower."""
 import os
 import subprocess
 
@@ -25,7 +25,7 @@ static int cover() {                                       // every (tile, chunk
                 const LmSlices s = plan_slices(tiles, pairs, n_pad);
                 const int n_chunks = (n_pad + 31) / 32;
                 const bool cut = s.slices > 0;
-                if (s.rounds != tiles / pairs || s.cost < s.rounds || s.cost > s.rounds + 1.0) { printf("cost %d %d %d\n", n_pad, pairs, tiles); return 1; }
+                if (s.rounds != tiles / pairs) { printf("rounds %d %d %d\n", n_pad, pairs, tiles); return 1; }
                 if (cut && (s.slices * s.slice_chunks < n_chunks || (s.slices - 1) * s.slice_chunks >= n_chunks || s.slice_chunks > 8)) { printf("pieces %d %d %d\n", n_pad, pairs, tiles); return 1; }
                 if (cut == (tiles % pairs == 0) && cut) { printf("nothing left %d %d %d\n", n_pad, pairs, tiles); return 1; }
             }
@@ -34,15 +34,7 @@ static int cover() {                                       // every (tile, chunk
 }
 int main(int argc, char** argv) {
     if (argc == 1) return cover();
-    if (argc == 3) { printf("%d\n", (int)brings_ahead(atoi(argv[1]), (atoi(argv[2]) + 255) / 256, 74)); return 0; }
-    const int M = atoi(argv[1]), V = atoi(argv[2]), Hd = atoi(argv[3]);       // how the row blocks of a call share launches, 74 pairs
-    const int n = (M + 511) / 512, rows = ((M + n - 1) / n + 15) / 16 * 16;
-    for (int rb = 0; rb < n;) {
-        const bool two = rb + 1 < n && side_by_side(rows, M - (rb + 1) * rows < rows ? M - (rb + 1) * rows : rows, Hd, (V + 255) / 256, 74);
-        printf("%d", two ? 2 : 1);
-        rb += two ? 2 : 1;
-    }
-    printf("\n");
+    printf("%d\n", (int)brings_ahead(atoi(argv[1]), (atoi(argv[2]) + 255) / 256, 74));
 }
 """
 
@@ -61,18 +53,6 @@ def plan(tmp_path_factory):
 
 def test_pieces_cover_the_tiles(plan):
     assert int(plan()) == 8 * 6 * 700
-
-
-# "2": side by side, "11": one behind the other.  Measured where the comment at side_by_side says so.
-@pytest.mark.parametrize("M,V,Hd,launches", [
-    (544, 152064, 3584, "2"), (600, 152064, 3584, "2"), (960, 152064, 3584, "2"), (1025, 152064, 3584, "21"),
-    (600, 128256, 4096, "2"), (960, 128256, 4096, "2"), (513, 50257, 2048, "2"), (960, 50257, 2048, "2"), (2048, 32000, 4096, "22"),
-    (513, 4099, 1024, "2"), (600, 200, 1024, "2"), (1537, 4099, 3584, "22"),
-    # a second block whose own columns are fewer, where W's tiles take many rounds
-    (513, 152064, 3584, "11"), (513, 152064, 1024, "11"), (520, 128256, 4096, "11"), (528, 94000, 3584, "11"), (513, 110000, 3584, "11"),
-    (577, 128256, 4096, "11"), (769, 128256, 4096, "11"), (961, 128256, 4096, "11"), (1537, 128256, 4096, "211")])
-def test_row_blocks_share_a_launch_where_it_is_faster(plan, M, V, Hd, launches):
-    assert plan(M, V, Hd) == launches
 
 
 @pytest.mark.parametrize("Hd,V,ahead", [(4096, 32000, 1), (2048, 50257, 1), (768, 32000, 1), (3584, 152064, 1), (1024, 1025, 1), (128, 6000, 1),
